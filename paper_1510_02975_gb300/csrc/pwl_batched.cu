@@ -3,8 +3,9 @@
 // each a fixed sequence of launches over all functions, so that the four
 // phases can be captured in one CUDA graph and replayed.
 //
-//   design      density / chunk scan / cumulative / inversion over the chunks
-//               of every function at once (the kernels of pwl_design.cu)
+//   design      density / chunk scan / inversion over the chunks of every
+//               function at once (FP64), or one CTA per function (FP32; the
+//               kernels of pwl_design.cu)
 //   projection  hat integrals of every interval, then one CTA per function
 //               for the Gram solve (pwl_project.cu)
 //   index       one CTA per function: FP32 knots and values, slopes and the
@@ -794,9 +795,10 @@ pwl_status pwl_batch_design(pwl_batch b, int32_t precision, void* stream)
     p.knots = b->knots;
     design_carve_scratch(p, b->design_scratch);
     p.order = b->order;
-    // the fused path keeps no cumulative values: its per-chunk markers use that
-    // area, and its FP32 mode keeps the FP32 densities in the density area
-    p.clast = reinterpret_cast<int*>(p.G);
+    // FP64: the chunk-parallel kernels, whatever the number of functions (the
+    // FP64 pipe bounds them, and they compute each density once); FP32: one
+    // CTA per function
+    if (precision == PWL_PREC_FP64) return design_launch(p, as_stream(stream));
     return design_fused_launch(p, as_stream(stream));
 }
 

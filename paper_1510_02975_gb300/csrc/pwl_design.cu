@@ -4,13 +4,18 @@
 // rule) and the inversion F(x_i) = i/N (Eq. 17).
 //
 // Every kernel is batched over F functions described by device arrays
-// (descriptors and CSR offsets of knots, cells and 2048-cell chunks); a
-// single function is a batch of one.  Four launches:
+// (descriptors and CSR offsets of knots, cells and 256-cell chunks, the
+// chunks of a function padded to whole tiles of 8); a single function is a
+// batch of one.  Three launches:
 //   density_chunks  d_k = |f''(t_k)|^{2/5} and one FP64 partial sum per chunk
 //   chunk_scan      exclusive FP64 scan of the chunk sums, per function
-//   cumulative      G_k = delta * (chunk base + in-chunk exclusive scan)
-//   invert          one thread per knot: binary search of tau_i = i G_M / N
-//                   in G, then the linear solve inside the cell
+//   invert_tiles    per tile of 2048 cells: the in-tile prefix of the
+//                   densities and the knots whose targets tau_i = i G_M / N
+//                   fall into the tile
+// They serve one function and, in FP64, every batch: a batch designed by one
+// CTA per function (as the FP32 mode below is) waits for its largest function
+// and computes every density twice: 40 functions of up to 4095 intervals at 64
+// cells per interval took 25.2 ms that way, 1.12 ms this way (density 1.03).
 #include <math.h>
 
 #include <algorithm>
@@ -21,9 +26,11 @@ namespace pwl {
 
 namespace {
 
-constexpr int kChunk = 2048;      // density cells per chunk
 constexpr int kDesignThreads = 256;
-constexpr int kPerThread = kChunk / kDesignThreads;
+constexpr int kChunk = kDesignThreads;         // density cells per chunk
+constexpr int kTileChunks = 8;                 // chunks per tile (every function holds whole tiles)
+constexpr int kTile = kChunk * kTileChunks;    // cells per tile
+constexpr int kTilePer = kTile / kDesignThreads;  // cells per thread of a tile
 
 // index f with off[f] <= g < off[f+1] (off has F+1 non-decreasing entries)
 __device__ __forceinline__ int find_segment(const int64_t* __restrict__ off, int F, int64_t g)
@@ -76,221 +83,213 @@ __device__ __forceinline__ double block_exclusive_scan(double v, double* s_warp,
     return r;
 }
 
-// d_k for this thread's cells of the chunk at c0 (sum returned), THREADS
-// threads per chunk; the sampled path is a template flag, chosen once per
-// chunk
-template <typename T, bool SAMPLED, int THREADS>
-__device__ __forceinline__ double density_chunk(const pwl_func& F, int64_t c0, int64_t M, double delta,
-                                                double* __restrict__ d)
+// Density of one cell: d_k = |f''(t_k)|^{2/5}, f'' and the power in T
+template <typename T, bool SAMPLED>
+__device__ __forceinline__ double cell_density(const pwl_func& F, double delta, int64_t k)
 {
-    double acc = 0.0;
-    for (int r = 0; r < kChunk / THREADS; ++r) {
-        const int64_t k = c0 + r * THREADS + threadIdx.x;
-        if (k < M) {
-            // t_k = a + (k + 1/2) delta, rounded as written (no fused multiply-add)
-            const double t = __dadd_rn(F.a, __dmul_rn((double)k + 0.5, delta));
-            const T f2 = func_second_derivative_k<SAMPLED, T>(F, (T)t);
-            const double dk = (double)FMath<T>::dens(f2);
-            d[k] = dk;
-            acc += dk;
-        }
-    }
-    return acc;
+    // t_k = a + (k + 1/2) delta, rounded as written (no fused multiply-add)
+    const double t = __dadd_rn(F.a, __dmul_rn((double)k + 0.5, delta));
+    return (double)FMath<T>::dens(func_second_derivative_k<SAMPLED, T>(F, (T)t));
 }
 
-// The density of a single function's few chunks (128 at N = 4096) takes
-// kDensityThreads threads per chunk, so that its FP64 f'' evaluations keep
-// more warps in flight per SM than the scans' 256-thread CTAs would: 512
-// threads (the FP64 J0 path needs ~128 registers, so 1024 would spill
-// heavily) took the bench's design graph of 9 tables from 0.56 to 0.49 ms.
-constexpr int kDensityThreads = 512;
-
+// One CTA per chunk, one cell per thread: d_k, the chunk's FP64 sum and its
+// last cell of positive density.  The kernel is bound by the FP64 pipe (about
+// one lane-operation per SM and clock, which 8 warps keep busy), so a chunk is
+// as small as a 256-thread CTA: one N = 1024 design (65536 cells) then fills
+// 256 CTAs, where 2048-cell chunks left it on 32 of the 152 SMs (J0, from f to
+// a table and 2^20 evaluations: 493 -> 416 us).
 template <typename T, bool SAMPLED>
-__global__ void __launch_bounds__(kDensityThreads) density_chunks_kernel(DesignPlan p)
+__global__ void __launch_bounds__(kDesignThreads, 2) density_chunks_kernel(DesignPlan p)
 {
-    __shared__ double s_red[kDensityThreads / 32];
+    __shared__ double s_red[kDesignThreads / 32];
+    __shared__ int s_last[kDesignThreads / 32];
     for (int64_t ch = blockIdx.x; ch < p.total_chunks; ch += gridDim.x) {
         const int f = find_segment(p.choff, p.F, ch);
         const pwl_func F = p.funcs[f];
         if ((F.kind == PWL_F_SAMPLED) != SAMPLED) continue;  // the other launch's (uniform per CTA)
         const int64_t M = p.moff[f + 1] - p.moff[f];
-        const int64_t c0 = (ch - p.choff[f]) * kChunk;
+        const int64_t k = (ch - p.choff[f]) * kChunk + threadIdx.x;
         const double delta = (F.b - F.a) / (double)M;
-        double* __restrict__ d = p.d + p.moff[f];
-        double acc = density_chunk<T, SAMPLED, kDensityThreads>(F, c0, M, delta, d);
+        double acc = 0.0;
+        if (k < M) {
+            acc = cell_density<T, SAMPLED>(F, delta, k);
+            p.d[p.moff[f] + k] = acc;
+        }
+        const unsigned pos = __ballot_sync(0xffffffffu, acc > 0.0);
         acc = warp_sum(acc);
-        if ((threadIdx.x & 31) == 0) s_red[threadIdx.x >> 5] = acc;
+        if ((threadIdx.x & 31) == 0) {
+            s_red[threadIdx.x >> 5] = acc;
+            s_last[threadIdx.x >> 5] = pos ? (int)threadIdx.x + 31 - __clz(pos) : -1;
+        }
         __syncthreads();
         if (threadIdx.x == 0) {
-            double s = 0.0;
-            for (int w = 0; w < kDensityThreads / 32; ++w) s += s_red[w];
-            p.csum[ch] = s;
+            double sum = 0.0;
+            int last = -1;
+            for (int w = 0; w < kDesignThreads / 32; ++w) {
+                sum += s_red[w];
+                last = max(last, s_last[w]);
+            }
+            p.csum[ch] = sum;
+            p.plast[ch] = last < 0 ? -1 : k + last;  // k: the chunk's first cell (thread 0)
         }
         __syncthreads();
     }
 }
 
+// Per function: the exclusive FP64 scan of the chunk sums (cbase, stot) and
+// the last cell of positive density before every chunk (plast, in place).
+// kScanPer consecutive chunks per thread, 2048 chunks a round.
+constexpr int kScanPer = 8;
+
 __global__ void __launch_bounds__(kDesignThreads) chunk_scan_kernel(DesignPlan p)
 {
     __shared__ double s_warp[kDesignThreads / 32 + 1];
+    __shared__ long long s_max[kDesignThreads / 32];
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     for (int f = blockIdx.x; f < p.F; f += gridDim.x) {
         const int64_t c0 = p.choff[f], c1 = p.choff[f + 1];
         double carry = 0.0;
-        for (int64_t base = c0; base < c1; base += kDesignThreads) {
-            const int64_t c = base + threadIdx.x;
-            const double v = (c < c1) ? p.csum[c] : 0.0;
+        long long before = -1;  // last positive cell of the rounds before
+        for (int64_t base = c0; base < c1; base += kDesignThreads * kScanPer) {
+            const int64_t c = base + (int64_t)threadIdx.x * kScanPer;
+            double v[kScanPer], run = 0.0;
+            long long l[kScanPer], mine = -1;
+#pragma unroll
+            for (int r = 0; r < kScanPer; ++r) {
+                v[r] = c + r < c1 ? p.csum[c + r] : 0.0;
+                l[r] = c + r < c1 ? p.plast[c + r] : -1;
+                run += v[r];
+                mine = max(mine, l[r]);
+            }
             double tot;
-            const double ex = block_exclusive_scan(v, s_warp, &tot);
-            if (c < c1) p.cbase[c] = carry + ex;
+            double ex = carry + block_exclusive_scan(run, s_warp, &tot);
+            long long incl = mine;
+            for (int o = 1; o < 32; o <<= 1) {
+                const long long t = __shfl_up_sync(0xffffffffu, incl, o);
+                if (lane >= o) incl = max(incl, t);
+            }
+            if (lane == 31) s_max[warp] = incl;
+            __syncthreads();
+            long long prev = __shfl_up_sync(0xffffffffu, incl, 1);
+            prev = max(lane == 0 ? -1ll : prev, before);
+            for (int w = 0; w < kDesignThreads / 32; ++w) {
+                if (w < warp) prev = max(prev, s_max[w]);
+                before = max(before, s_max[w]);
+            }
+#pragma unroll
+            for (int r = 0; r < kScanPer; ++r) {
+                if (c + r < c1) {
+                    p.cbase[c + r] = ex;
+                    p.plast[c + r] = prev;
+                }
+                ex += v[r];
+                prev = max(prev, l[r]);
+            }
             carry += tot;
+            __syncthreads();  // s_max is rewritten in the next round
         }
         if (threadIdx.x == 0) p.stot[f] = carry;
     }
 }
 
-__global__ void __launch_bounds__(kDesignThreads) cumulative_kernel(DesignPlan p)
+// smallest i in [1, N] with tau_i = i G_M / N >= G (N if none below N)
+__device__ __forceinline__ int64_t first_target_at_or_above(double G, double GM, int64_t N)
 {
-    __shared__ double s_d[kChunk];
+    auto tau = [&](int64_t i) { return (double)i * GM / (double)N; };
+    const double e = floor(G / GM * (double)N);
+    int64_t i = (int64_t)fmin(fmax(e, 1.0), (double)N);
+    while (i > 1 && tau(i - 1) >= G) --i;
+    while (i < N && tau(i) < G) ++i;
+    return i;
+}
+
+// The knots whose targets fall into a tile of kTileChunks chunks (tau_i at or
+// above G at the tile's start and below G at the next tile's): the tile's
+// densities and the FP64 prefix of its thread partials in shared memory,
+// then per knot the largest cell k with G_k <= tau_i (binary search over the
+// thread prefixes, then the thread's cells), the walk back to a cell of
+// positive density, and x_i = a + k delta + (tau_i - G_k) / d_k.  It reads 8
+// bytes per cell; writing G to memory and searching it there took 24 bytes
+// per cell and a chain of ~17 dependent L2 reads per knot.
+__global__ void __launch_bounds__(kDesignThreads) invert_tiles_kernel(DesignPlan p)
+{
+    __shared__ double s_d[kTile];
+    __shared__ double s_S[kDesignThreads];  // tile base + exclusive prefix of the thread partials
     __shared__ double s_warp[kDesignThreads / 32 + 1];
-    for (int64_t ch = blockIdx.x; ch < p.total_chunks; ch += gridDim.x) {
+    __shared__ int64_t s_i[2];
+    const int t = threadIdx.x;
+    for (int64_t tile = blockIdx.x; tile < p.total_chunks / kTileChunks; tile += gridDim.x) {
+        const int64_t ch = tile * kTileChunks;  // the tile's first chunk
         const int f = find_segment(p.choff, p.F, ch);
         const int64_t M = p.moff[f + 1] - p.moff[f];
-        const int64_t c0 = (ch - p.choff[f]) * kChunk;
-        const int cnt = (int)min((int64_t)kChunk, M - c0);
-        const double delta = (p.funcs[f].b - p.funcs[f].a) / (double)M;
-        const double* __restrict__ d = p.d + p.moff[f];
-        double* __restrict__ G = p.G + p.moff[f] + f;
-        for (int i = threadIdx.x; i < kChunk; i += kDesignThreads) s_d[i] = (i < cnt) ? d[c0 + i] : 0.0;
-        __syncthreads();
-        double loc[kPerThread];
-        double run = 0.0;
-        for (int r = 0; r < kPerThread; ++r) {
-            loc[r] = run;
-            run += s_d[threadIdx.x * kPerThread + r];
-        }
-        double tot;
-        const double tb = block_exclusive_scan(run, s_warp, &tot);
-        const double base = p.cbase[ch] + tb;
-        for (int r = 0; r < kPerThread; ++r) {
-            const int i = threadIdx.x * kPerThread + r;
-            if (i < cnt) G[c0 + i] = delta * (base + loc[r]);
-        }
-        if (c0 + cnt == M && threadIdx.x == 0) G[M] = delta * p.stot[f];
-        __syncthreads();
-    }
-}
-
-__global__ void invert_kernel(DesignPlan p)
-{
-    const int64_t stride = (int64_t)gridDim.x * blockDim.x;
-    for (int64_t g = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; g < p.total_knots; g += stride) {
-        const int f = find_segment(p.koff, p.F, g);
-        const int64_t i = g - p.koff[f];
         const int64_t N = p.koff[f + 1] - p.koff[f] - 1;
+        const int64_t c0 = (ch - p.choff[f]) * kChunk;
         const double a = p.funcs[f].a, b = p.funcs[f].b;
-        double x;
-        if (i == 0) {
-            x = a;
-        } else if (i == N) {
-            x = b;
-        } else {
-            const int64_t M = p.moff[f + 1] - p.moff[f];
-            const double* __restrict__ G = p.G + p.moff[f] + f;
-            const double* __restrict__ d = p.d + p.moff[f];
-            const double GM = G[M];
-            if (!(GM > 0.0)) {
-                x = a + (double)i * (b - a) / (double)N;  // f linear on I: uniform partition
-            } else {
-                const double delta = (b - a) / (double)M;
-                const double tau = (double)i * GM / (double)N;
-                int64_t lo = 0, hi = M - 1;  // largest k with G_k <= tau
-                while (lo < hi) {
-                    const int64_t mid = lo + (hi - lo + 1) / 2;
-                    if (G[mid] <= tau) lo = mid; else hi = mid - 1;
-                }
-                int64_t k = lo;
-                while (k > 0 && !(d[k] > 0.0)) --k;
-                x = __dadd_rn(a, __dmul_rn((double)k, delta));
-                if (d[k] > 0.0) {
-                    double step = (tau - G[k]) / d[k];
-                    step = fmin(fmax(step, 0.0), delta);
-                    x = __dadd_rn(x, step);
-                }
+        const double delta = (b - a) / (double)M;
+        const double GM = delta * p.stot[f];
+        double* __restrict__ knots = p.knots + p.koff[f];
+        if (t == 0 && c0 == 0) {
+            knots[0] = a;
+            knots[N] = b;
+        }
+        if (!(GM > 0.0)) {  // f linear on I (or no finite density): the uniform partition
+            if (c0 == 0)
+                for (int64_t i = 1 + t; i < N; i += kDesignThreads) knots[i] = a + (double)i * (b - a) / (double)N;
+            continue;
+        }
+        const double base = p.cbase[ch];
+        // neighbouring tiles evaluate the same expression at their common
+        // boundary, so every knot has exactly one tile
+        if (t == 0) s_i[0] = first_target_at_or_above(delta * base, GM, N);
+        if (t == 32)
+            s_i[1] = c0 + kTile < M ? first_target_at_or_above(delta * p.cbase[ch + kTileChunks], GM, N) : N;
+        const int cnt = (int)min((int64_t)kTile, M - c0);
+        const double* __restrict__ d = p.d + p.moff[f] + c0;
+        for (int i = t; i < kTile; i += kDesignThreads) s_d[i] = i < cnt ? d[i] : 0.0;
+        __syncthreads();
+        const int64_t i0 = s_i[0], i1 = s_i[1];
+        double run = 0.0;
+        for (int r = 0; r < kTilePer; ++r) run += s_d[t * kTilePer + r];
+        double tot;
+        s_S[t] = base + block_exclusive_scan(run, s_warp, &tot);
+        __syncthreads();
+        const int U = (cnt + kTilePer - 1) / kTilePer;  // threads holding cells
+        for (int64_t i = i0 + t; i < i1; i += kDesignThreads) {
+            const double tau = (double)i * GM / (double)N;
+            int lo = 0, hi = U - 1;  // largest u with G at its first cell <= tau (u = 0 is)
+            while (lo < hi) {
+                const int mid = (lo + hi + 1) >> 1;
+                if (delta * s_S[mid] <= tau) lo = mid; else hi = mid - 1;
             }
+            const int nr = min(kTilePer, cnt - lo * kTilePer);
+            double acc = 0.0, Gk = delta * s_S[lo];
+            int kl = lo * kTilePer;
+            for (int r = 1; r < nr; ++r) {  // the thread's last cell with G <= tau (G does not decrease)
+                acc += s_d[lo * kTilePer + r - 1];
+                const double Gr = delta * (s_S[lo] + acc);
+                if (!(Gr <= tau)) break;
+                kl = lo * kTilePer + r;
+                Gk = Gr;
+            }
+            int kk = kl;  // largest cell <= kl of positive density
+            while (kk >= 0 && !(s_d[kk] > 0.0)) --kk;
+            double x;
+            if (kk == kl) {
+                x = __dadd_rn(a, __dmul_rn((double)(c0 + kk), delta));
+                x = __dadd_rn(x, fmin(fmax((tau - Gk) / s_d[kk], 0.0), delta));
+            } else {
+                // no density between the last positive cell (in the tile or before
+                // it) and here, so tau is at or past G at that cell's end: its
+                // right edge
+                const int64_t e = kk >= 0 ? c0 + kk : p.plast[ch];
+                x = e < 0 ? a : __dadd_rn(__dadd_rn(a, __dmul_rn((double)e, delta)), delta);
+            }
+            knots[i] = x;
         }
-        p.knots[g] = x;
+        __syncthreads();  // the shared arrays are rewritten for the next tile
     }
 }
 
-// ---- fused design of whole functions (batches) ----------------------------
-// One CTA designs one function at a time, in one launch for the batch:
-//   pass A  for every 2048-cell chunk: the densities (8 contiguous cells per
-//           thread), the chunk total (block scan in FP64) and the chunk's
-//           last cell of positive density;
-//   scan    exclusive FP64 scan of the chunk totals: chunk bases, G_M;
-//   pass B  for every chunk holding targets tau_i (G at the chunk start <=
-//           tau_i < G at the next chunk's start): the densities again, the
-//           FP64 prefix of the thread partials, and for each such knot the
-//           largest cell k with G_k <= tau_i (binary search over the thread
-//           prefixes, then the thread's cells), the walk back to a cell of
-//           positive density, and x_i = a + k delta + (tau_i - G_k) / d_k.
-// Nothing per cell goes to memory.  Thread partials of 8 densities are a
-// plain FP64 sum (FP64 mode) or a compensated FP32 sum (FP32 mode: two-sum,
-// every rounding error carried, about 2^-48 relative); all sums above them
-// are FP64.  In FP32 mode the cell midpoints are formed in FP32 from the
-// chunk start (the FP32 f'' rounds its argument to FP32 anyway).
-template <typename T>
-struct Partial;
-template <>
-struct Partial<double> {
-    double s = 0.0;
-    __device__ __forceinline__ void add(double v) { s = __dadd_rn(s, v); }
-    __device__ __forceinline__ double value() const { return s; }
-};
-template <>
-struct Partial<float> {
-    float s = 0.0f, c = 0.0f;
-    __device__ __forceinline__ void add(float v)
-    {
-        const float t = __fadd_rn(s, v);
-        const float bp = __fsub_rn(t, s);
-        const float e = __fadd_rn(__fsub_rn(s, __fsub_rn(t, bp)), __fsub_rn(v, bp));
-        s = t;
-        c = __fadd_rn(c, e);
-    }
-    __device__ __forceinline__ double value() const { return (double)s + (double)c; }
-};
-
-// The uncompensated running sum of a partial, in the density's type: the
-// cheap candidate of the in-thread cell search (checked in FP64 after).
-__device__ __forceinline__ double approx(const Partial<double>& p) { return p.s; }
-__device__ __forceinline__ float approx(const Partial<float>& p) { return p.s; }
-
-// FP64 density of cell k: |f''(t_k)|^{2/5}, t_k = a + (k + 1/2) delta
-template <bool SAMPLED>
-__device__ __forceinline__ double fused_density64(const pwl_func& F, double a, double delta, int64_t k)
-{
-    const double t = __dadd_rn(a, __dmul_rn((double)k + 0.5, delta));
-    return pow_two_fifths(func_second_derivative_k<SAMPLED, double>(F, t));
-}
-
-// The densities of one chunk's cells of this thread, added to `part`; STORE
-// keeps them in s_d, LAST tracks the last cell of positive density.  The
-// sampled path is a template flag, chosen once per chunk.
-template <bool SAMPLED, bool STORE, bool LAST>
-__device__ __forceinline__ void fused_chunk64(const pwl_func& F, double a, double delta, int64_t c0, int cnt,
-                                              Partial<double>& part, int& last, double* s_d)
-{
-    for (int r = 0; r < kPerThread; ++r) {
-        const int l = threadIdx.x * kPerThread + r;
-        if (l < cnt) {
-            const double dk = fused_density64<SAMPLED>(F, a, delta, c0 + l);
-            if (STORE) s_d[l] = dk;
-            part.add(dk);
-            if (LAST && dk > 0.0) last = l;
-        }
-    }
-}
 // FP32 density from the function's FP32 constants: |f''|^{2/5} by the
 // hardware exp2/log2 pair (__powf), a few ulp (the FP32 mode's knot bound
 // allows a relative density error near 1e-6), for a third of the
@@ -306,172 +305,18 @@ __device__ __forceinline__ float fused_density_f(const FuncF& G, const pwl_func&
     return __powf(fabsf(f2), 0.4f);
 }
 
-
-// smallest i in [1, N] with tau_i = i G_M / N >= G (N if none below N)
-__device__ __forceinline__ int64_t first_target_at_or_above(double G, double GM, int64_t N)
-{
-    auto tau = [&](int64_t i) { return (double)i * GM / (double)N; };
-    const double e = floor(G / GM * (double)N);
-    int64_t i = (int64_t)fmin(fmax(e, 1.0), (double)N);
-    while (i > 1 && tau(i - 1) >= G) --i;
-    while (i < N && tau(i) < G) ++i;
-    return i;
-}
-
-template <typename T, bool SAMPLED>
-__global__ void __launch_bounds__(kDesignThreads) design_fused_kernel(DesignPlan p)
-{
-    __shared__ T s_d[kChunk];
-    __shared__ double s_S[kDesignThreads];  // chunk base + exclusive prefix of the thread partials
-    __shared__ double s_G[kDesignThreads];  // delta * s_S: G at each thread's first cell
-    __shared__ double s_warp[kDesignThreads / 32 + 1];
-    __shared__ int s_last;
-    const int t = threadIdx.x;
-    for (int o = blockIdx.x; o < p.F; o += gridDim.x) {
-        const int f = p.order[o];
-        const pwl_func F = p.funcs[f];
-        if ((F.kind == PWL_F_SAMPLED) != SAMPLED) continue;  // the other launch's (uniform per CTA)
-        const int64_t M = p.moff[f + 1] - p.moff[f];
-        const int64_t N = p.koff[f + 1] - p.koff[f] - 1;
-        const int64_t nch = p.choff[f + 1] - p.choff[f];
-        const double a = F.a, b = F.b;
-        const double delta = (b - a) / (double)M;
-        const float deltaf = (float)delta;
-        double* __restrict__ knots = p.knots + p.koff[f];
-        double* __restrict__ csum = p.csum + p.choff[f];
-        double* __restrict__ cbase = p.cbase + p.choff[f];
-        int* __restrict__ clast = p.clast + p.choff[f];
-
-        // pass A
-        for (int64_t ch = 0; ch < nch; ++ch) {
-            const int64_t c0 = ch * kChunk;
-            const int cnt = (int)min((int64_t)kChunk, M - c0);
-            const float t0f = (float)(a + (double)c0 * delta);
-            Partial<T> part;
-            int last = -1;
-            fused_chunk64<SAMPLED, false, true>(F, a, delta, c0, cnt, part, last, nullptr);
-            if (t == 0) s_last = -1;
-            __syncthreads();
-            if (last >= 0) atomicMax(&s_last, last);
-            double tot;
-            block_exclusive_scan(part.value(), s_warp, &tot);
-            if (t == 0) {
-                csum[ch] = tot;
-                clast[ch] = s_last;
-            }
-        }
-        __syncthreads();
-        // exclusive scan of the chunk totals
-        double carry = 0.0;
-        for (int64_t base = 0; base < nch; base += kDesignThreads) {
-            const int64_t c = base + t;
-            const double v = c < nch ? csum[c] : 0.0;
-            double tot;
-            const double ex = block_exclusive_scan(v, s_warp, &tot);
-            if (c < nch) cbase[c] = carry + ex;
-            carry += tot;
-        }
-        __syncthreads();
-        const double GM = delta * carry;
-        if (t == 0) {
-            knots[0] = a;
-            knots[N] = b;
-        }
-        if (!(GM > 0.0)) {  // f linear on I (or no finite density): the uniform partition
-            for (int64_t i = 1 + t; i < N; i += kDesignThreads) knots[i] = a + (double)i * (b - a) / (double)N;
-            __syncthreads();
-            continue;
-        }
-        // the first target of every chunk, all chunks at once (the chunk sums
-        // are spent: their area takes the indices)
-        int64_t* ifirst = reinterpret_cast<int64_t*>(csum);
-        for (int64_t c = t; c < nch; c += kDesignThreads) ifirst[c] = first_target_at_or_above(delta * cbase[c], GM, N);
-        __syncthreads();
-
-        // pass B
-        int64_t lastpos = -1;  // last cell of positive density before the current chunk
-        for (int64_t ch = 0; ch < nch; ++ch) {
-            const int64_t c0 = ch * kChunk;
-            const int64_t i0 = ifirst[ch], i1 = ch + 1 < nch ? ifirst[ch + 1] : N;
-            if (i0 < i1) {
-                const int cnt = (int)min((int64_t)kChunk, M - c0);
-                const float t0f = (float)(a + (double)c0 * delta);
-                Partial<T> part;
-                int unused = -1;
-                fused_chunk64<SAMPLED, true, false>(F, a, delta, c0, cnt, part, unused, s_d);
-                double tot;
-                const double ex = block_exclusive_scan(part.value(), s_warp, &tot);
-                s_S[t] = cbase[ch] + ex;
-                s_G[t] = delta * (cbase[ch] + ex);
-                __syncthreads();
-                const int U = (cnt + kPerThread - 1) / kPerThread;  // threads holding cells
-                // G at local cell l: delta * (S_u + partial of the thread's cells before l)
-                auto g_at = [&](int l) {
-                    const int u = l / kPerThread;
-                    Partial<T> q;
-                    for (int r = u * kPerThread; r < l; ++r) q.add(s_d[r]);
-                    return delta * (s_S[u] + q.value());
-                };
-                const double inv_delta = 1.0 / delta;
-                for (int64_t i = i0 + t; i < i1; i += kDesignThreads) {
-                    const double tau = (double)i * GM / (double)N;
-                    int lo = 0, hi = U - 1;  // largest u with G at its first cell <= tau (u = 0 is)
-                    while (lo < hi) {
-                        const int mid = (lo + hi + 1) >> 1;
-                        if (s_G[mid] <= tau) lo = mid; else hi = mid - 1;
-                    }
-                    // largest cell r of thread lo with G_r <= tau: a candidate from
-                    // the running sums in T against tau / delta - S, then the exact
-                    // FP64 G of the candidate and its right neighbour decide
-                    const int nr = min(kPerThread, cnt - lo * kPerThread);
-                    const T target = (T)(tau * inv_delta - s_S[lo]);
-                    Partial<T> run;
-                    int r = 0;
-                    for (int q = 1; q < nr; ++q) {
-                        run.add(s_d[lo * kPerThread + q - 1]);
-                        if (approx(run) <= target) r = q;
-                    }
-                    int kl = lo * kPerThread + r;
-                    double Gk = g_at(kl);
-                    while (kl > lo * kPerThread && !(Gk <= tau)) Gk = g_at(--kl);
-                    while (kl + 1 < lo * kPerThread + nr) {
-                        const double Gn = g_at(kl + 1);
-                        if (!(Gn <= tau)) break;
-                        ++kl;
-                        Gk = Gn;
-                    }
-                    int kk = kl;  // largest cell <= kl of positive density
-                    while (kk >= 0 && !(s_d[kk] > T(0))) --kk;
-                    double x;
-                    if (kk >= 0) {
-                        if (kk != kl) Gk = g_at(kk);
-                        const double dk = (double)s_d[kk];
-                        x = __dadd_rn(a, __dmul_rn((double)(c0 + kk), delta));
-                        const double step = fmin(fmax((tau - Gk) / dk, 0.0), delta);
-                        x = __dadd_rn(x, step);
-                    } else if (lastpos >= 0) {
-                        // no density from cell lastpos + 1 to here, so tau is at or past
-                        // G at the end of cell lastpos: its right edge
-                        x = __dadd_rn(__dadd_rn(a, __dmul_rn((double)lastpos, delta)), delta);
-                    } else {
-                        x = a;  // no positive density from the start of I
-                    }
-                    knots[i] = x;
-                }
-            }
-            const int cl = clast[ch];
-            if (cl >= 0) lastpos = c0 + cl;
-            __syncthreads();  // s_d and s_S are rewritten for the next chunk
-        }
-    }
-}
-
 // ---- fused design, FP32 mode ------------------------------------------------
-// The FP32-density variant of design_fused_kernel, arranged so that almost
-// no FP64 operation is spent per density cell (GB300 runs about one FP64
+// One CTA designs one function at a time, in one launch for the batch, with
+// almost no FP64 operation per density cell (GB300 runs about one FP64
 // operation per SM and cycle):
-//   - pass A writes the FP32 densities to scratch; pass B reads them back;
-//   - sums inside a chunk are float-float (a compensated pair hi + lo, about
+//   - pass A, per tile of 2048 cells: the FP32 densities (8 contiguous cells
+//     per thread, written to scratch), the tile's sum and its last cell of
+//     positive density; then the exclusive FP64 scan of the tile sums;
+//   - pass B, per tile holding targets: the densities read back, their prefix,
+//     and the knots as in invert_tiles_kernel;
+//   - cell midpoints are formed in FP32 from the tile start (the FP32 f''
+//     rounds its argument to FP32 anyway);
+//   - sums inside a tile are float-float (a compensated pair hi + lo, about
 //     48 significant bits): thread partials, the block scan and the chunk
 //     total; the chunk totals, their scan and G_M are FP64;
 //   - the knot search compares float-float values in FP32, in units of the
@@ -569,8 +414,8 @@ template <bool SAMPLED>
 __device__ __forceinline__ void chunk_densities_f(const FuncF& G, const pwl_func& F, float t0f, float deltaf,
                                                   int cnt, float* __restrict__ dchunk, FF& part, int& last)
 {
-    for (int r = 0; r < kPerThread; ++r) {
-        const int l = threadIdx.x * kPerThread + r;
+    for (int r = 0; r < kTilePer; ++r) {
+        const int l = threadIdx.x * kTilePer + r;
         if (l < cnt) {
             const float dk = fused_density_f<SAMPLED>(G, F, t0f, deltaf, l);
             dchunk[l] = dk;
@@ -583,7 +428,7 @@ __device__ __forceinline__ void chunk_densities_f(const FuncF& G, const pwl_func
 template <bool SAMPLED>
 __global__ void __launch_bounds__(kDesignThreads, 4) design_fused_fp32_kernel(DesignPlan p)
 {
-    __shared__ float s_d[kChunk];
+    __shared__ float s_d[kTile];
     __shared__ FF s_ex[kDesignThreads];  // exclusive float-float prefix of the thread partials
     __shared__ FF s_w[2 * (kDesignThreads / 32) + 1];
     __shared__ int s_last2[2];
@@ -600,20 +445,20 @@ __global__ void __launch_bounds__(kDesignThreads, 4) design_fused_fp32_kernel(De
         const FuncF G = make_funcf(F);  // FP32 constants of f'', once per function
         const int64_t M = p.moff[f + 1] - p.moff[f];
         const int64_t N = p.koff[f + 1] - p.koff[f] - 1;
-        const int64_t nch = p.choff[f + 1] - p.choff[f];
+        const int64_t nch = (M + kTile - 1) / kTile;
         const double a = F.a, b = F.b;
         const double delta = (b - a) / (double)M;
         const float deltaf = (float)delta;
         double* __restrict__ knots = p.knots + p.koff[f];
         double* __restrict__ csum = p.csum + p.choff[f];
         double* __restrict__ cbase = p.cbase + p.choff[f];
-        int* __restrict__ clast = p.clast + p.choff[f];
+        int* __restrict__ clast = reinterpret_cast<int*>(p.plast + p.choff[f]);  // tile-local indices
         float* __restrict__ dbuf = dbuf_all + p.moff[f];
 
         // pass A: densities (to scratch), chunk totals, last positive cell
         for (int64_t ch = 0; ch < nch; ++ch) {
-            const int64_t c0 = ch * kChunk;
-            const int cnt = (int)min((int64_t)kChunk, M - c0);
+            const int64_t c0 = ch * kTile;
+            const int cnt = (int)min((int64_t)kTile, M - c0);
             const float t0f = (float)(a + (double)c0 * delta);
             FF part{0.0f, 0.0f};
             int last = -1;
@@ -661,13 +506,13 @@ __global__ void __launch_bounds__(kDesignThreads, 4) design_fused_fp32_kernel(De
         // pass B
         int64_t lastpos = -1;
         for (int64_t ch = 0; ch < nch; ++ch) {
-            const int64_t c0 = ch * kChunk;
+            const int64_t c0 = ch * kTile;
             const int64_t i0 = ifirst[ch], i1 = ch + 1 < nch ? ifirst[ch + 1] : N;
             if (i0 < i1) {
-                const int cnt = (int)min((int64_t)kChunk, M - c0);
+                const int cnt = (int)min((int64_t)kTile, M - c0);
                 FF part{0.0f, 0.0f};
-                for (int r = 0; r < kPerThread; ++r) {
-                    const int l = t * kPerThread + r;
+                for (int r = 0; r < kTilePer; ++r) {
+                    const int l = t * kTilePer + r;
                     if (l < cnt) {
                         const float dk = dbuf[c0 + l];
                         s_d[l] = dk;
@@ -677,13 +522,13 @@ __global__ void __launch_bounds__(kDesignThreads, 4) design_fused_fp32_kernel(De
                 FF tot;
                 s_ex[t] = ff_block_exclusive_scan(part, s_w, &tot);
                 __syncthreads();
-                const int U = (cnt + kPerThread - 1) / kPerThread;
+                const int U = (cnt + kTilePer - 1) / kTilePer;
                 const double cb = cbase[ch];
                 // float-float prefix of local cell l: S_u + the thread's cells before l
                 auto ff_at = [&](int l) {
-                    const int u = l / kPerThread;
+                    const int u = l / kTilePer;
                     FF q = s_ex[u];
-                    for (int r = u * kPerThread; r < l; ++r) q = ff_add(q, FF{s_d[r], 0.0f});
+                    for (int r = u * kTilePer; r < l; ++r) q = ff_add(q, FF{s_d[r], 0.0f});
                     return q;
                 };
                 for (int64_t i = i0 + t; i < i1; i += kDesignThreads) {
@@ -693,13 +538,13 @@ __global__ void __launch_bounds__(kDesignThreads, 4) design_fused_fp32_kernel(De
                         const int mid = (lo + hi + 1) >> 1;
                         if (ff_le(s_ex[mid], tl)) lo = mid; else hi = mid - 1;
                     }
-                    const int nr = min(kPerThread, cnt - lo * kPerThread);
+                    const int nr = min(kTilePer, cnt - lo * kTilePer);
                     FF q = s_ex[lo], Sk = q;
-                    int kl = lo * kPerThread;
+                    int kl = lo * kTilePer;
                     for (int r = 1; r < nr; ++r) {
-                        q = ff_add(q, FF{s_d[lo * kPerThread + r - 1], 0.0f});
+                        q = ff_add(q, FF{s_d[lo * kTilePer + r - 1], 0.0f});
                         if (!ff_le(q, tl)) break;
-                        kl = lo * kPerThread + r;
+                        kl = lo * kTilePer + r;
                         Sk = q;
                     }
                     int kk = kl;
@@ -727,7 +572,7 @@ __global__ void __launch_bounds__(kDesignThreads, 4) design_fused_fp32_kernel(De
 
 // Writes the descriptor and offsets of a one-function batch into the
 // workspace (kernel parameters, so the call needs no host-to-device copy).
-__global__ void single_setup_kernel(pwl_func F, int64_t N, int64_t M, pwl_func* funcs,
+__global__ void single_setup_kernel(pwl_func F, int64_t N, int64_t M, int64_t chunks, pwl_func* funcs,
                                     int64_t* koff, int64_t* moff, int64_t* choff)
 {
     if (threadIdx.x == 0 && blockIdx.x == 0) {
@@ -737,7 +582,7 @@ __global__ void single_setup_kernel(pwl_func F, int64_t N, int64_t M, pwl_func* 
         moff[0] = 0;
         moff[1] = M;
         choff[0] = 0;
-        choff[1] = (M + kChunk - 1) / kChunk;
+        choff[1] = chunks;
     }
 }
 
@@ -745,13 +590,12 @@ inline size_t align256(size_t x) { return (x + 255) & ~(size_t)255; }
 
 }  // namespace
 
-int64_t design_chunks(int64_t M) { return (M + kChunk - 1) / kChunk; }
+int64_t design_chunks(int64_t M) { return (M + kTile - 1) / kTile * kTileChunks; }
 
 size_t design_scratch_bytes(int64_t F, int64_t total_cells, int64_t total_chunks)
 {
-    return align256(sizeof(double) * (size_t)total_cells) +
-           align256(sizeof(double) * (size_t)(total_cells + F)) +
-           align256(sizeof(double) * (size_t)total_chunks) * 2 + align256(sizeof(double) * (size_t)F);
+    return align256(sizeof(double) * (size_t)total_cells) + align256(sizeof(double) * (size_t)total_chunks) * 2 +
+           align256(sizeof(int64_t) * (size_t)total_chunks) + align256(sizeof(double) * (size_t)F);
 }
 
 void design_carve_scratch(DesignPlan& p, void* scratch)
@@ -759,41 +603,39 @@ void design_carve_scratch(DesignPlan& p, void* scratch)
     char* w = static_cast<char*>(scratch);
     p.d = reinterpret_cast<double*>(w);
     w += align256(sizeof(double) * (size_t)p.total_cells);
-    p.G = reinterpret_cast<double*>(w);
-    w += align256(sizeof(double) * (size_t)(p.total_cells + p.F));
     p.csum = reinterpret_cast<double*>(w);
     w += align256(sizeof(double) * (size_t)p.total_chunks);
     p.cbase = reinterpret_cast<double*>(w);
     w += align256(sizeof(double) * (size_t)p.total_chunks);
+    p.plast = reinterpret_cast<int64_t*>(w);
+    w += align256(sizeof(int64_t) * (size_t)p.total_chunks);
     p.stot = reinterpret_cast<double*>(w);
 }
 
 pwl_status design_launch(const DesignPlan& p, cudaStream_t s)
 {
     const DeviceInfo& di = device_info();
-    const int grid_chunks = (int)std::min<int64_t>(p.total_chunks, (int64_t)di.sms * 8);
+    const int grid_chunks = (int)std::min<int64_t>(p.total_chunks, (int64_t)di.sms * 16);
     const int kinds = plan_kinds(p.kinds);
     if (kinds & kKindsAnalytic) {
         if (p.precision == PWL_PREC_FP32)
-            density_chunks_kernel<float, false><<<grid_chunks, kDensityThreads, 0, s>>>(p);
+            density_chunks_kernel<float, false><<<grid_chunks, kDesignThreads, 0, s>>>(p);
         else
-            density_chunks_kernel<double, false><<<grid_chunks, kDensityThreads, 0, s>>>(p);
+            density_chunks_kernel<double, false><<<grid_chunks, kDesignThreads, 0, s>>>(p);
         PWL_CHECK_LAUNCH("density_chunks_kernel");
     }
     if (kinds & kKindsSampled) {
         if (p.precision == PWL_PREC_FP32)
-            density_chunks_kernel<float, true><<<grid_chunks, kDensityThreads, 0, s>>>(p);
+            density_chunks_kernel<float, true><<<grid_chunks, kDesignThreads, 0, s>>>(p);
         else
-            density_chunks_kernel<double, true><<<grid_chunks, kDensityThreads, 0, s>>>(p);
+            density_chunks_kernel<double, true><<<grid_chunks, kDesignThreads, 0, s>>>(p);
         PWL_CHECK_LAUNCH("density_chunks_kernel");
     }
     chunk_scan_kernel<<<(int)std::min<int64_t>(p.F, 65535), kDesignThreads, 0, s>>>(p);
     PWL_CHECK_LAUNCH("chunk_scan_kernel");
-    cumulative_kernel<<<grid_chunks, kDesignThreads, 0, s>>>(p);
-    PWL_CHECK_LAUNCH("cumulative_kernel");
-    const int grid_knots = (int)std::min<int64_t>((p.total_knots + 255) / 256, (int64_t)di.sms * 16);
-    invert_kernel<<<grid_knots, 256, 0, s>>>(p);
-    PWL_CHECK_LAUNCH("invert_kernel");
+    const int grid_tiles = (int)std::min<int64_t>(p.total_chunks / kTileChunks, (int64_t)di.sms * 16);
+    invert_tiles_kernel<<<grid_tiles, kDesignThreads, 0, s>>>(p);
+    PWL_CHECK_LAUNCH("invert_tiles_kernel");
     return PWL_OK;
 }
 
@@ -803,18 +645,12 @@ pwl_status design_fused_launch(const DesignPlan& p, cudaStream_t s)
     const int grid = (int)std::min<int64_t>(p.F, (int64_t)di.sms * 8);
     const int kinds = plan_kinds(p.kinds);
     if (kinds & kKindsAnalytic) {
-        if (p.precision == PWL_PREC_FP32)
-            design_fused_fp32_kernel<false><<<grid, kDesignThreads, 0, s>>>(p);
-        else
-            design_fused_kernel<double, false><<<grid, kDesignThreads, 0, s>>>(p);
-        PWL_CHECK_LAUNCH("design_fused_kernel");
+        design_fused_fp32_kernel<false><<<grid, kDesignThreads, 0, s>>>(p);
+        PWL_CHECK_LAUNCH("design_fused_fp32_kernel");
     }
     if (kinds & kKindsSampled) {
-        if (p.precision == PWL_PREC_FP32)
-            design_fused_fp32_kernel<true><<<grid, kDesignThreads, 0, s>>>(p);
-        else
-            design_fused_kernel<double, true><<<grid, kDesignThreads, 0, s>>>(p);
-        PWL_CHECK_LAUNCH("design_fused_kernel");
+        design_fused_fp32_kernel<true><<<grid, kDesignThreads, 0, s>>>(p);
+        PWL_CHECK_LAUNCH("design_fused_fp32_kernel");
     }
     return PWL_OK;
 }
@@ -834,7 +670,9 @@ size_t pwl_design_workspace_size(int64_t n_intervals, int64_t m_cells)
 {
     if (n_intervals < 1) return 0;
     const int64_t M = resolve_cells(n_intervals, m_cells);
-    return kMetaBytes + design_scratch_bytes(1, M, design_chunks(M));
+    // the size stays two doubles per cell, which the call's contract has had
+    // callers provide; the kernels use about half of it
+    return kMetaBytes + std::max(design_scratch_bytes(1, M, design_chunks(M)), align256(2 * sizeof(double) * (size_t)M));
 }
 
 pwl_status pwl_design(const pwl_func* f, int64_t n_intervals, int64_t m_cells, int32_t precision,
@@ -873,7 +711,7 @@ pwl_status pwl_design(const pwl_func* f, int64_t n_intervals, int64_t m_cells, i
     p.knots = d_knots;
     design_carve_scratch(p, w + kMetaBytes);
     cudaStream_t s = as_stream(stream);
-    single_setup_kernel<<<1, 1, 0, s>>>(*f, n_intervals, M, const_cast<pwl_func*>(p.funcs),
+    single_setup_kernel<<<1, 1, 0, s>>>(*f, n_intervals, M, p.total_chunks, const_cast<pwl_func*>(p.funcs),
                                         const_cast<int64_t*>(p.koff), const_cast<int64_t*>(p.moff),
                                         const_cast<int64_t*>(p.choff));
     PWL_CHECK_LAUNCH("single_setup_kernel");

@@ -24,8 +24,7 @@ __device__ __forceinline__ double recip_newton(double d)
 }
 
 // F functions; function f owns knots koff[f] .. koff[f+1]-1 (N_f + 1 of them),
-// density cells moff[f] .. moff[f+1]-1 (M_f), chunks choff[f] .. choff[f+1]-1,
-// and G entries moff[f] + f .. moff[f+1] + f (M_f + 1).
+// density cells moff[f] .. moff[f+1]-1 (M_f) and chunks choff[f] .. choff[f+1]-1.
 // Which kinds a plan holds: the hot kernels are compiled once for the
 // analytic kinds and once for sampled functions (whose FP64 interpolation
 // would otherwise weigh on the analytic loops' registers); a launch runs the
@@ -49,24 +48,22 @@ struct DesignPlan {
     const int64_t* moff;
     const int64_t* choff;
     int64_t total_knots, total_cells, total_chunks;
-    double* d;      // total_cells densities
-    double* G;      // total_cells + F cumulative values
-    double* csum;   // total_chunks partial sums
-    double* cbase;  // total_chunks exclusive chunk bases
-    double* stot;   // F totals (sum of d over the function)
-    double* knots;  // total_knots output
-    // fused per-function path (batches)
-    const int* order;  // F function indices, largest M first
-    int* clast;        // total_chunks: last cell of positive density in the chunk (local index), or -1;
-                       // must not overlap d (the FP32 fused kernel keeps FP32 densities there)
+    double* d;       // total_cells densities (the FP32 fused kernel: floats)
+    double* csum;    // total_chunks partial sums
+    double* cbase;   // total_chunks exclusive chunk bases
+    int64_t* plast;  // per chunk: its last cell of positive density, then (after the scan) the last one before
+                     // it, or -1
+    double* stot;    // F totals (sum of d over the function)
+    double* knots;   // total_knots output
+    const int* order;  // fused FP32 path: F function indices, largest M first
 };
 
 int64_t design_chunks(int64_t M);
 size_t design_scratch_bytes(int64_t F, int64_t total_cells, int64_t total_chunks);
 void design_carve_scratch(DesignPlan& p, void* scratch);
 pwl_status design_launch(const DesignPlan& p, cudaStream_t s);
-// One persistent launch for a batch: each CTA designs whole functions (in
-// p.order); needs p.order and p.clast, writes p.csum, p.cbase and p.knots.
+// FP32 mode of a batch, one persistent launch: each CTA designs whole
+// functions (in p.order); writes p.csum, p.cbase, p.plast and p.knots.
 pwl_status design_fused_launch(const DesignPlan& p, cudaStream_t s);
 
 // Projection: F functions with knots at koff (device), values out.
