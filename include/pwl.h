@@ -484,15 +484,14 @@ pwl_status pwl_batch_get_info(pwl_batch b, pwl_batch_info* info);
 /* y[r, c] = v_c(x[r, c]) for a row-major x[rows, n_channels], where channel
  * c is the CPWL function with FP32 knots d_knots[c, 0..N] and values
  * d_values[c, 0..N] (device arrays [n_channels, N+1], e.g. learnable
- * parameters).  Each CTA builds the cell index of 8 channels in shared
- * memory (k_cells cells per channel of 16 bytes each, 0 selects 4 (N+1) as
- * far as the CTA's shared memory allows; cells holding several knots are
- * walked).  io_dtype PWL_FP32 or PWL_BF16 (x and y alike); the arithmetic
+ * parameters).  Each CTA builds the cell index of a few channels in shared
+ * memory (k_cells cells per channel, 0 selects a count from N and the CTA's
+ * shared memory; cells holding several knots are walked).  io_dtype PWL_FP32 or PWL_BF16 (x and y alike); the arithmetic
  * is FP32; clamping and NaN as in pwl_eval.  Knots must be strictly
  * increasing per channel: a violation sets bit 0 of the device word
  * *d_status (the caller zeroes it; results are then unspecified).
- * Errors: PWL_ENOTSUP if 8 channels' index does not fit a CTA
- * (128 (k_cells + N + 1) bytes).                                           */
+ * Errors: PWL_ENOTSUP if 128 (k_cells + N + 1) bytes do not fit a CTA's
+ * shared memory (N up to ~1790 with k_cells = 0).                          */
 pwl_status pwl_channels_forward(const float* d_knots, const float* d_values, int64_t n_channels,
                                 int64_t n_intervals, int64_t k_cells, const void* d_x, void* d_y,
                                 int64_t rows, int32_t io_dtype, int32_t* d_status, void* stream);
@@ -500,12 +499,22 @@ pwl_status pwl_channels_forward(const float* d_knots, const float* d_values, int
 /* Backward of pwl_channels_forward (FP32 only): gx[r, c] = gy[r, c] * s,
  * and for every channel d_g_values[c, j] += sum over rows of gy dy/dv_j,
  * d_g_knots[c, j] += sum of gy dy/dx_j (the formulas of pwl_eval_backward;
- * either may be NULL; accumulated with FP32 atomics, order-dependent at FP32
- * rounding).  k_cells: 0 selects 2 (N+1).                                  */
+ * either may be NULL).  Inside a CTA the sums are fixed point per channel
+ * (each term rounded at 2^-29 of the channel's typical |gy| or finer, the
+ * sums exact; terms far above the typical one in FP32); the CTAs' sums are
+ * added with FP32 atomics, order-dependent at FP32 rounding.  k_cells as in
+ * the forward.                                                             */
 pwl_status pwl_channels_backward(const float* d_knots, const float* d_values, int64_t n_channels,
                                  int64_t n_intervals, int64_t k_cells, const float* d_x, const float* d_gy,
                                  float* d_gx, float* d_g_values, float* d_g_knots, int64_t rows,
                                  int32_t* d_status, void* stream);
+
+/* The same with x, gy and gx in BF16: the arithmetic of the FP32 call on the
+ * widened inputs, gx rounded to BF16 (no FP32 copies of the streams).      */
+pwl_status pwl_channels_backward_bf16(const float* d_knots, const float* d_values, int64_t n_channels,
+                                      int64_t n_intervals, int64_t k_cells, const void* d_x, const void* d_gy,
+                                      void* d_gx, float* d_g_values, float* d_g_knots, int64_t rows,
+                                      int32_t* d_status, void* stream);
 
 /* ------------------------------------------------------------------------ */
 /* Failure injection: tests of the error paths (no counterpart in the paper;  */

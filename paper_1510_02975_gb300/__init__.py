@@ -23,7 +23,7 @@ __all__ = [
     "pwl_error_constants", "pwl_predicted_error", "pwl_n_for_error",
     "pwl_batch_create", "pwl_batch_destroy", "pwl_batch_design", "pwl_batch_project", "pwl_batch_build",
     "pwl_batch_check", "pwl_batch_plan", "pwl_batch_eval", "pwl_batch_autotune", "pwl_batch_get_info", "Batch",
-    "pwl_channels_forward", "pwl_channels_backward", "ChannelPWL", "pwl_test_fail_allocations",
+    "pwl_channels_forward", "pwl_channels_backward", "pwl_channels_backward_bf16", "ChannelPWL", "pwl_test_fail_allocations",
     "pwl_batch_inject_wait_timeout", "Table", "design", "project", "PWLFunction",
     "KINDS", "FORMS", "DTYPES", "PRECISIONS",
 ]
@@ -401,19 +401,30 @@ def pwl_channels_forward(knots, values, x, y=None, k_cells: int = 0, status=None
 def pwl_channels_backward(knots, values, x, gy, gx=None, g_values=None, g_knots=None, k_cells: int = 0,
                           status=None, stream=None):
     """Backward of pwl_channels_forward (FP32): returns gx; accumulates g_values, g_knots [C, N+1]."""
+    return _channels_backward("pwl_channels_backward", _torch().float32, knots, values, x, gy, gx, g_values, g_knots,
+                              k_cells, status, stream)
+
+
+def pwl_channels_backward_bf16(knots, values, x, gy, gx=None, g_values=None, g_knots=None, k_cells: int = 0,
+                               status=None, stream=None):
+    """pwl_channels_backward with x, gy and gx in BF16 (the FP32 call's arithmetic on the widened inputs)."""
+    return _channels_backward("pwl_channels_backward_bf16", _torch().bfloat16, knots, values, x, gy, gx, g_values,
+                              g_knots, k_cells, status, stream)
+
+
+def _channels_backward(name, io, knots, values, x, gy, gx, g_values, g_knots, k_cells, status, stream):
     torch = _torch()
     _require(knots, torch.float32, "knots")
     _require(values, torch.float32, "values", knots.numel())
     C, n1 = knots.shape
-    _require(x, torch.float32, "x")
-    _require(gy, torch.float32, "gy", x.numel())
+    _require(x, io, "x")
+    _require(gy, io, "gy", x.numel())
     if gx is None:
         gx = torch.empty_like(x)
     if status is None:
         status = torch.zeros(1, dtype=torch.int32, device=x.device)
-    check(load().pwl_channels_backward(_ptr(knots), _ptr(values), C, n1 - 1, k_cells, _ptr(x), _ptr(gy), _ptr(gx),
-                                       _ptr(g_values), _ptr(g_knots), x.shape[0], _ptr(status), _stream(stream)),
-          "pwl_channels_backward")
+    check(getattr(load(), name)(_ptr(knots), _ptr(values), C, n1 - 1, k_cells, _ptr(x), _ptr(gy), _ptr(gx),
+                                _ptr(g_values), _ptr(g_knots), x.shape[0], _ptr(status), _stream(stream)), name)
     return gx
 
 
@@ -574,11 +585,10 @@ def _autograd_classes():
             x, knots, values = ctx.saved_tensors
             gv = torch.zeros_like(values) if ctx.needs_input_grad[2] else None
             gk = torch.zeros_like(knots) if ctx.needs_input_grad[1] else None
-            # the backward kernel takes FP32 streams: a BF16 map's x and gy
-            # are widened (exactly) and gx is returned in x's dtype
-            gx = pwl_channels_backward(knots, values, x.contiguous().float(), gy.contiguous().float(), None, gv, gk,
-                                       k_cells=ctx.k_cells_bwd, status=ctx.status)
-            return gx.to(x.dtype), gk, gv, None, None, None
+            bwd = pwl_channels_backward_bf16 if x.dtype == torch.bfloat16 else pwl_channels_backward
+            gx = bwd(knots, values, x.contiguous(), gy.to(x.dtype).contiguous(), None, gv, gk,
+                     k_cells=ctx.k_cells_bwd, status=ctx.status)
+            return gx, gk, gv, None, None, None
 
     _FUNCS["table"] = _TableFn
     _FUNCS["channels"] = _ChannelFn

@@ -94,6 +94,7 @@ SIGNATURES = {
     "pwl_batch_get_info": (_ST, [_P, ctypes.POINTER(PwlBatchInfo)]),
     "pwl_channels_forward": (_ST, [_P, _P, _I64, _I64, _I64, _P, _P, _I64, _I32, _P, _P]),
     "pwl_channels_backward": (_ST, [_P, _P, _I64, _I64, _I64, _P, _P, _P, _P, _P, _I64, _P, _P]),
+    "pwl_channels_backward_bf16": (_ST, [_P, _P, _I64, _I64, _I64, _P, _P, _P, _P, _P, _I64, _P, _P]),
     "pwl_test_fail_allocations": (_ST, [_I64]),
     "pwl_batch_inject_wait_timeout": (_ST, [_P, _I32, ctypes.c_uint64]),
 }

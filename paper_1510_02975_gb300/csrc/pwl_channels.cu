@@ -5,26 +5,50 @@
 // arrays [C, N+1] (learnable parameters that change every step), so each CTA
 // builds the cell index of its channels in shared memory when it starts.
 //
-// Forward: a CTA owns a tile of 8 consecutive channels and keeps, per
-// channel, 16-byte cell records {x_s, y_s, s_left, s_right} (one load, a
-// compare, a select and an FMA per element), channel-interleaved ([c * 8 + ch])
-// so that the 8 lanes of a quarter warp read 8 different bank groups.  Four
-// CTAs form a thread-block cluster on adjacent tiles (32 channels, 128-byte
-// row segments) and walk the same rows at once.
+// Both directions: a CTA owns a tile of CH consecutive channels (a lane keeps
+// one of them) and holds, per channel, K uniform cells and one 16-byte record
+// per interval, channel-interleaved ([e * CH + ch]) so that the lanes of a
+// quarter- or half-warp read different banks whatever they look up.
+//   cell       {x_k of the first knot in the cell (+inf if none), the interval
+//              at the cell's left end | the distance to the next knot}
+//   interval i {x_{i-1}, v_{i-1}, s_i, x_i} (forward),
+//              {x_{i-1}, 1/h_i, s_i, x_i} (backward); record N + 1 serves
+//              x = x_N
+// An element takes the cell's interval, from x_k on the next one and from the
+// knot after it on the one after that: two shared loads, two compares and no
+// side selects.  The second distance is a BF16 number rounded up, so a point
+// between a knot and its rounded place, or past a third knot of the cell, walks
+// on while it is at or beyond the interval's right end.
 //
-// Backward: a CTA owns 16 channels (a warp covers two rows, 64-byte row
-// segments), with 8-byte cell records {i, x_{i-1}} or {knot tag, x_k} and
-// interval records {s_i, 1/h_i}, channel-interleaved ([e * 16 + ch]), and
-// two shared accumulators per interval; 2-CTA clusters (128-byte segments).
+// The CTAs of a cluster own adjacent tiles, 128 bytes of a row together (64
+// for two 16-channel BF16 tiles), and walk the same rows: a row segment of
+// less than a line that one CTA alone reads costs the whole line (a copy of
+// [65536, 4096] FP32 in 64-byte segments: 640 us, by pairs 360 us).  What a
+// copy of that access pattern reaches also depends on the L1 the index
+// leaves: 16-channel tiles 360 us up to 132 KB of shared memory, 370 at 164
+// KB, 500 at 198 KB and beyond; 8-channel tiles 503, 578 and 665.  So tiles
+// are as wide as keeps the index below kIndexBytes.
 //
-// Both: the rows of x are split into chunks; units = (tile group, chunk of
-// rows), group-major; each cluster takes a contiguous range of units and
-// rebuilds its indexes only when the group changes.  A 32-byte row segment
-// read by one CTA alone costs a whole line fetch; the sibling CTAs of a
-// cluster use the rest of the line while it is in L2.
+// Measured, [65536, 4096] x 257 knots: forward 532 -> 377 us (FP32; 5.70 TB/s),
+// backward 1042 -> 689 us (4.67 TB/s); [16384, 4096] in BF16: forward 196 ->
+// 110 us, backward 695 -> 199 us, 388 us of it FP32 copies of the streams,
+// which the BF16 kernel does without.  Before, the forward had 8-channel
+// tiles (16-byte cells), the backward two compare-and-swap adds
+// and side selects per element (103 instructions, now ~65), and four CTAs a
+// cluster left 8 SMs idle.  What bounds them now: the forward the access
+// pattern (350-370 us as a plain copy), the backward instruction issue (75%).
+// A range costs ~5 us (forward) to ~15 us (backward) besides its rows: the
+// index build and, backward, the reductions into the global gradients.
+//
+// Work: the tile groups (one per cluster) x passes of the CTA's rows, cut
+// into one contiguous range per cluster, equal to a pass; a CTA rebuilds its
+// index only where its range enters another group.
 #include <math.h>
 
 #include <algorithm>
+#include <map>
+#include <mutex>
+#include <tuple>
 
 #include "pwl_channels.cuh"
 
@@ -32,135 +56,14 @@ namespace pwl {
 
 namespace {
 
-constexpr int kChThreads = 1024;                 // threads per CTA, both directions
-// backward tiles (the forward's constants are kChF, kClF, kRowsPerPassF, ...)
-constexpr int kCh = 16;                          // channels per backward tile
-constexpr int kRowsPerPass = kChThreads / kCh;   // 64 rows per pass of the CTA
-constexpr int kChUnroll = 16;                    // loads in flight per thread (8 rows x, gy: 64 KB per SM)
-constexpr int kChTail = 3;                       // rows per predicated batch of a unit's tail
-
-struct TileParams {
-    float a[kCh], b[kCh], inv_w[kCh], off[kCh], w[kCh];
-    int max_chain[kCh];
-    int any_chain;
-    int bad;
-};
-
-__device__ __forceinline__ int lower_bound_cells(const int* cj, int n, int v)
-{
-    int lo = 0, hi = n;
-    while (lo < hi) {
-        int mid = (lo + hi) >> 1;
-        if (cj[mid * kCh] < v) lo = mid + 1; else hi = mid;
-    }
-    return lo;
-}
-
-// Slopes are FP32 IEEE divisions of the FP32 differences: at most ~2 ulp
-// from the exact slope of the FP32 table, which moves a lerped value by
-// ~2^-23 |v_i - v_{i-1}| (FP64 would cost a slow FP64 division per record on
-// this GPU's few FP64 units).
-
-// Builds the backward index of channels [c0, c0 + 16) in shared memory.
-//   sP[cell * 16 + ch]      cell records {i, x_{i-1}} or {knot tag, x_k}
-//   sX[i * 16 + ch]         interval records {s_i, 1/h_i}, i = 0..N+1 (0 and N+1
-//                           copy intervals 1 and N)
-//   xs[j * 16 + ch]         the tile's knots (staged first, coalesced)
-//   cj[j * 16 + ch]         scratch: first the tile's values, then the cell of knot j
-// Every global read is a coalesced pass over the tile's knots and values;
-// the rest works in shared memory.
-__device__ void build_tile(const ChanArgs& p, int64_t c0, float2* sP, float2* sX, float* xs, int* cj,
-                           TileParams* tp)
-{
-    const int N = p.N, K = p.K, n1 = N + 1;
-    const int nch = (int)min((int64_t)kCh, p.C - c0);
-    float* vs = reinterpret_cast<float*>(cj);
-    const int per_ch = blockDim.x / kCh;  // threads per channel
-    for (int ch = threadIdx.x / per_ch, j = threadIdx.x % per_ch; j < n1; j += per_ch) {
-        // consecutive threads read consecutive knots of one channel
-        float xv, vv;
-        if (ch < nch) {
-            xv = p.knots[(c0 + ch) * (int64_t)n1 + j];
-            vv = p.values[(c0 + ch) * (int64_t)n1 + j];
-        } else {  // padding channel of a partial tile: an unused identity on [0, 1]
-            xv = (float)j / (float)N;
-            vv = 0.0f;
-        }
-        xs[j * kCh + ch] = xv;
-        vs[j * kCh + ch] = vv;
-    }
-    if (threadIdx.x == 0) {
-        tp->any_chain = 0;
-        tp->bad = 0;
-    }
-    __syncthreads();
-    if (threadIdx.x < kCh) {
-        const int ch = threadIdx.x;
-        const float a = xs[ch], b = xs[N * kCh + ch];
-        tp->a[ch] = a;
-        tp->b[ch] = b;
-        tp->inv_w[ch] = (float)K / (b - a);
-        tp->off[ch] = -a * tp->inv_w[ch];
-        tp->w[ch] = (b - a) / (float)K;
-        tp->max_chain[ch] = 0;
-    }
-    // interval records, from the staged arrays
-    for (int e = threadIdx.x; e < (N + 2) * kCh; e += blockDim.x) {
-        const int q = e / kCh, ch = e % kCh;
-        const int i = min(max(q, 1), N);  // interval q (0 and N+1 copy 1 and N)
-        const float h = __fsub_rn(xs[i * kCh + ch], xs[(i - 1) * kCh + ch]);
-        sX[e] = make_float2(__fdiv_rn(__fsub_rn(vs[i * kCh + ch], vs[(i - 1) * kCh + ch]), h), __frcp_rn(h));
-    }
-    __syncthreads();
-    // cells of the knots (overwrites the staged values)
-    for (int e = threadIdx.x; e < n1 * kCh; e += blockDim.x) {
-        const int j = e / kCh, ch = e % kCh;
-        const float xj = xs[e];
-        if (j > 0 && !(xj > xs[e - kCh])) atomicOr(&tp->bad, 1);
-        cj[e] = cell_of(xj, tp->inv_w[ch], tp->off[ch], K);
-    }
-    __syncthreads();
-    for (int e = threadIdx.x; e < n1 * kCh; e += blockDim.x) {
-        const int j = e / kCh, ch = e % kCh;
-        if (j > 0 && cj[e] == cj[e - kCh]) {
-            int first = j;
-            while (first > 0 && cj[(first - 1) * kCh + ch] == cj[e]) --first;
-            atomicMax(&tp->max_chain[ch], j - first);
-            atomicOr(&tp->any_chain, 1);
-        }
-    }
-    // cell records: each thread takes a run of consecutive cells of one
-    // channel, finds the first one's knot by bisection and walks on
-    {
-        const int ch = threadIdx.x % kCh, runs = blockDim.x / kCh, q = threadIdx.x / kCh;
-        const int per = (K + runs - 1) / runs;
-        const int cb = q * per, ce = min(K, cb + per);
-        int lb = cb < ce ? lower_bound_cells(cj + ch, n1, cb) : 0;
-        for (int c = cb; c < ce; ++c) {
-            while (lb < n1 && cj[lb * kCh + ch] < c) ++lb;  // lb: the first knot whose cell is >= c
-            float2 rec;
-            if (lb <= N && cj[lb * kCh + ch] == c) {
-                const bool chain = (lb < N && cj[(lb + 1) * kCh + ch] == c);
-                rec = make_float2(make_knot_tag(lb, chain), xs[lb * kCh + ch]);
-            } else {
-                const int i = lb;  // the cell lies inside interval i = [x_{i-1}, x_i]
-                rec = make_float2(__int_as_float(i), xs[(i - 1) * kCh + ch]);
-            }
-            sP[c * kCh + ch] = rec;
-        }
-    }
-    __syncthreads();
-}
-
-// A thread's channel is fixed for a tile: its constants live in registers.
-struct ChanConst {
-    float a, b, inv_w, off, w;
-    int max_chain;
-    __device__ __forceinline__ ChanConst(const TileParams& tp, int ch)
-        : a(tp.a[ch]), b(tp.b[ch]), inv_w(tp.inv_w[ch]), off(tp.off[ch]), w(tp.w[ch]), max_chain(tp.max_chain[ch])
-    {
-    }
-};
+constexpr int kChThreads = 1024;  // threads per CTA, both directions
+constexpr int kFwdUnroll = 16;    // rows in flight per thread (64 KB per SM in FP32)
+constexpr int kFwdTail = 4;       // rows per predicated batch of a range's tail
+constexpr int kBwdUnroll = 8;     // rows of x and gy in flight per thread (64 KB per SM in FP32)
+constexpr int kBwdTail = 2;
+constexpr int kFwdGroup = 4;      // elements looked up together (their shared loads overlap, one chain test)
+constexpr int kBwdGroup = 2;
+constexpr int kStage = 4;         // knots and values in flight per thread while a tile is staged
 
 template <typename IO>
 __device__ __forceinline__ float to_f32(IO v);
@@ -178,466 +81,674 @@ __device__ __forceinline__ __nv_bfloat16 from_f32<__nv_bfloat16>(float v) { retu
 __device__ __forceinline__ void st_cs(float* p, float v) { __stcs(p, v); }
 __device__ __forceinline__ void st_cs(__nv_bfloat16* p, __nv_bfloat16 v) { *p = v; }
 
-// ---- forward: 8-channel tiles with 16-byte split records ---------------------
-// A cell record is {x_s, y_s, s_left, s_right}: v(x) = y_s + (x - x_s) s with
-// s = s_left left of x_s and s_right from x_s on.  A knot-free cell inside
-// interval i stores its anchor x_c = a + c w, the line's value there and s_i
-// twice; a cell holding one knot k stores {x_k, v_k, s_k, s_{k+1}}.  One
-// 16-byte load, a compare, a select and an FMA per element; no tag test and
-// no second load.  A cell holding several knots stores a NaN-tagged s_right
-// (knot k, its first): elements right of x_k walk the tile's knots and take
-// {x_k', v_k', s_{k'+1}} from the staged knots, values and slopes.
-// Records are channel-interleaved ([c * 8 + ch]): the 8 lanes of a quarter
-// warp read 8 different 16-byte bank groups.  With 4 cells per knot a tile
-// takes 128 (K + N + 1) bytes (164 KB at N = 256), so a CTA owns 8 channels,
-// and 4-CTA clusters walk the same rows at once to use whole 128-byte lines.
-constexpr int kChF = 8;                           // channels per forward tile
-constexpr int kClF = 4;                           // CTAs per forward cluster (32 channels)
-constexpr int kRowsPerPassF = kChThreads / kChF;  // 128 rows per pass
-constexpr int kChUnrollF = 24;
-constexpr int kChTailF = 8;
-
-struct TileParamsF {
-    float a[kChF], b[kChF], inv_w[kChF], off[kChF], w[kChF];
-    int max_chain[kChF];
-    int any_chain;
-    int bad;
-};
-
-struct ChanConstF {
-    float a, b, inv_w, off, w;
-    int max_chain;
-    __device__ __forceinline__ ChanConstF(const TileParamsF& tp, int ch)
-        : a(tp.a[ch]), b(tp.b[ch]), inv_w(tp.inv_w[ch]), off(tp.off[ch]), w(tp.w[ch]), max_chain(tp.max_chain[ch])
-    {
-    }
-};
-
-__device__ __forceinline__ int lower_bound_cells8(const int* cj, int n, int v)
+// Cell of a point in [a, b]: cell_of with the clamp at 0 done by the unsigned
+// conversion (negative and NaN give 0).  Monotone in x; the builder applies it
+// to the knots.
+__device__ __forceinline__ int chan_cell(float xc, float inv_w, float off, int K)
 {
-    int lo = 0, hi = n;
-    while (lo < hi) {
-        const int mid = (lo + hi) >> 1;
-        if (cj[mid * kChF] < v) lo = mid + 1; else hi = mid;
-    }
-    return lo;
+    return (int)min(__float2uint_rz(__fmaf_rn(xc, inv_w, off)), (unsigned)(K - 1));
 }
 
-// Builds the forward index of channels [c0, c0 + 8) in shared memory:
-//   R[c * 8 + ch]   cell records (K)
-//   xs, vs, sp      knots, values and slopes s_{j+1} (s_N for j = N), [j * 8 + ch]
-//   cj              build scratch: the cell of knot j
-__device__ void build_tile_fwd(const ChanArgs& p, int64_t c0, float4* R, float* xs, float* vs, float* sp, int* cj,
-                               TileParamsF* tp)
+// odd pitch of the staged knots and values ([ch][j]): the linear copy from
+// global memory and the [j][ch] reads of the build are both nearly free of
+// bank conflicts
+__host__ __device__ __forceinline__ int stage_pitch(int N) { return (N + 1) | 1; }
+
+// A cell's second word: interval i (16 bits) and, in the upper half, a BF16
+// number strictly above d (the distance from the cell's first knot to the next
+// one; an FP32 difference at or above it is of a point at or beyond that knot
+// whatever the roundings).
+__device__ __forceinline__ float make_cell(int i, float d)
 {
-    const int N = p.N, K = p.K, n1 = N + 1;
-    const int nch = (int)min((int64_t)kChF, p.C - c0);
-    const int per_ch = blockDim.x / kChF;  // threads per channel
-    for (int ch = threadIdx.x / per_ch, j = threadIdx.x % per_ch; j < n1; j += per_ch) {
-        // consecutive threads read consecutive knots of one channel
-        float xv, vv;
+    return __uint_as_float((unsigned)i | (min(__float_as_uint(fmaxf(d, 0.0f)) >> 16, 0x7f7fu) + 1) << 16);
+}
+
+// Builds the index of channels [c0, c0 + CH): interval records rec[i * CH + ch]
+// (i = 0..N+1) and cell records cells[c * CH + ch].  The staged knots and
+// values live where the cell records go, which are written last, from the
+// interval records.  Every cell gets a record in range whatever the knots are,
+// so that knots that do not increase (*bad is set) give unspecified results
+// but no stray access.  staged() runs after the first barrier; the caller has
+// a barrier before (nobody reads the previous tile) and gets one after.
+// Measured (16 channels of 257 knots, clocks): staging 3000, interval records
+// 2300, cells 4500.
+template <int CH, bool BWD, class Staged>
+__device__ __forceinline__ void build_tile(const ChanArgs& p, int64_t c0, float2* cells, float4* rec, int* bad,
+                                           const Staged& staged)
+{
+    const int N = p.N, K = p.K, n1 = N + 1, P = stage_pitch(N);
+    const int nch = (int)min((int64_t)CH, p.C - c0);
+    float* xs = reinterpret_cast<float*>(cells);
+    float* vs = xs + (size_t)CH * P;
+    {
+        constexpr int per_ch = kChThreads / CH;
+        const int ch = threadIdx.x / per_ch;
         if (ch < nch) {
-            xv = p.knots[(c0 + ch) * (int64_t)n1 + j];
-            vv = p.values[(c0 + ch) * (int64_t)n1 + j];
-        } else {  // padding channel of a partial tile: an unused identity on [0, 1]
-            xv = (float)j / (float)N;
-            vv = 0.0f;
-        }
-        xs[j * kChF + ch] = xv;
-        vs[j * kChF + ch] = vv;
-    }
-    if (threadIdx.x == 0) {
-        tp->any_chain = 0;
-        tp->bad = 0;
-    }
-    __syncthreads();
-    if (threadIdx.x < kChF) {
-        const int ch = threadIdx.x;
-        const float a = xs[ch], b = xs[N * kChF + ch];
-        tp->a[ch] = a;
-        tp->b[ch] = b;
-        tp->inv_w[ch] = (float)K / (b - a);
-        tp->off[ch] = -a * tp->inv_w[ch];
-        tp->w[ch] = (b - a) / (float)K;
-        tp->max_chain[ch] = 0;
-    }
-    for (int e = threadIdx.x; e < n1 * kChF; e += blockDim.x) {
-        const int j = e / kChF, ch = e % kChF;
-        const int i = min(j + 1, N);  // slope of interval j + 1 (of interval N for j = N)
-        const float h = __fsub_rn(xs[i * kChF + ch], xs[(i - 1) * kChF + ch]);
-        sp[e] = __fdiv_rn(__fsub_rn(vs[i * kChF + ch], vs[(i - 1) * kChF + ch]), h);
-    }
-    __syncthreads();
-    for (int e = threadIdx.x; e < n1 * kChF; e += blockDim.x) {
-        const int j = e / kChF, ch = e % kChF;
-        const float xj = xs[e];
-        if (j > 0 && !(xj > xs[e - kChF])) atomicOr(&tp->bad, 1);
-        cj[e] = cell_of(xj, tp->inv_w[ch], tp->off[ch], K);
-    }
-    __syncthreads();
-    for (int e = threadIdx.x; e < n1 * kChF; e += blockDim.x) {
-        const int j = e / kChF, ch = e % kChF;
-        if (j > 0 && cj[e] == cj[e - kChF]) {
-            int first = j;
-            while (first > 0 && cj[(first - 1) * kChF + ch] == cj[e]) --first;
-            atomicMax(&tp->max_chain[ch], j - first);
-            atomicOr(&tp->any_chain, 1);
-        }
-    }
-    // cell records: each thread takes a run of consecutive cells of one
-    // channel, finds the first one's knot by bisection and walks on
-    {
-        const int ch = threadIdx.x % kChF, runs = blockDim.x / kChF, q = threadIdx.x / kChF;
-        const int per = (K + runs - 1) / runs;
-        const int cb = q * per, ce = min(K, cb + per);
-        int lb = cb < ce ? lower_bound_cells8(cj + ch, n1, cb) : 0;
-        for (int c = cb; c < ce; ++c) {
-            while (lb < n1 && cj[lb * kChF + ch] < c) ++lb;  // lb: the first knot whose cell is >= c
-            float4 rec;
-            if (lb <= N && cj[lb * kChF + ch] == c) {  // knot lb is the cell's first knot
-                const int k = lb;
-                const bool chain = k < N && cj[(k + 1) * kChF + ch] == c;
-                const float sl = sp[max(k - 1, 0) * kChF + ch];
-                const float sr = chain ? make_knot_tag(k, true) : sp[k * kChF + ch];
-                rec = make_float4(xs[k * kChF + ch], vs[k * kChF + ch], sl, sr);
-            } else {  // inside interval lb: the line through (x_j, v_j), j = lb - 1, at the anchor
-                const int j = lb - 1;
-                const float sj = sp[j * kChF + ch];
-                const float xc = __fmaf_rn(__int2float_rn(c), tp->w[ch], tp->a[ch]);
-                rec = make_float4(xc, __fmaf_rn(__fsub_rn(xc, xs[j * kChF + ch]), sj, vs[j * kChF + ch]), sj, sj);
+            const float* kx = p.knots + (c0 + ch) * (int64_t)n1;
+            const float* kv = p.values + (c0 + ch) * (int64_t)n1;
+            for (int j = threadIdx.x % per_ch; j < n1; j += kStage * per_ch) {
+                float a[kStage], b[kStage];
+#pragma unroll
+                for (int u = 0; u < kStage; ++u)
+                    if (j + u * per_ch < n1) {
+                        a[u] = kx[j + u * per_ch];
+                        b[u] = kv[j + u * per_ch];
+                    }
+#pragma unroll
+                for (int u = 0; u < kStage; ++u)
+                    if (j + u * per_ch < n1) {
+                        xs[ch * P + j + u * per_ch] = a[u];
+                        vs[ch * P + j + u * per_ch] = b[u];
+                    }
             }
-            R[c * kChF + ch] = rec;
+        }
+        if (threadIdx.x == 0) *bad = 0;
+    }
+    __syncthreads();
+    staged();
+    // from here on a thread keeps one channel
+    constexpr int RP = kChThreads / CH;
+    const int ch = threadIdx.x % CH, row = threadIdx.x / CH;
+    const float inf = __int_as_float(0x7f800000);
+    if (ch < nch) {
+        bool ok = true;
+        for (int i = 1 + row; i <= N; i += RP) {
+            const float xl = xs[ch * P + i - 1], vl = vs[ch * P + i - 1];
+            const float xr = xs[ch * P + i], vr = vs[ch * P + i];
+            // slopes and reciprocal lengths by FP32 IEEE division of the FP32
+            // differences: at most ~2 ulp from the exact slope of the FP32 table
+            const float h = __fsub_rn(xr, xl), s = __fdiv_rn(__fsub_rn(vr, vl), h);
+            rec[i * CH + ch] = make_float4(xl, BWD ? __frcp_rn(h) : vl, s, xr);
+            ok = ok && xr > xl;
+            if (i == N) {
+                // x = x_N.  Forward: v_N exactly.  Backward: delta = 0 from x_N to
+                // a right end one spacing above it, so that its sums reach knot N;
+                // gx = gy s_N
+                const float up = fabsf(xr) < 0x1p-100f ? xr + 0x1p-100f : nextafterf(xr, inf);
+                rec[(N + 1) * CH + ch] = BWD ? make_float4(xr, 1.0f / (up - xr), s, up) : make_float4(xr, vr, 0.0f, inf);
+            }
+        }
+        if (row == RP - 1) rec[ch] = make_float4(xs[ch * P], 0.0f, 0.0f, xs[ch * P]);
+        if (!ok) *bad = 1;
+    }
+    __syncthreads();
+    if (ch < nch) {
+        // a few consecutive knots per thread: knot j names the cells after knot
+        // j - 1's up to its own, which is a knot cell of knot j if it is the
+        // first there (and x_N the cells past its own, which no point reaches)
+        const float4* knot = rec + CH + ch;  // x_j = knot[j * CH].x, j = 0..N
+        const float a = knot[0].x, b = knot[N * CH].x;
+        const float inv_w = (float)K / (b - a), off = -a * inv_w;
+        const int per = (n1 + RP - 1) / RP, je = min(n1, (row + 1) * per);
+        int j = row * per;
+        if (j < je) {
+            int c = j > 0 ? chan_cell(knot[(j - 1) * CH].x, inv_w, off, K) + 1 : 0;
+            float xj = knot[j * CH].x;
+            for (; j < je; ++j) {
+                const float xn = j < N ? knot[(j + 1) * CH].x : inf;
+                const int cj = chan_cell(xj, inv_w, off, K);
+                const float2 free = make_float2(inf, make_cell(j, inf));
+#pragma unroll 4
+                for (; c < cj; ++c) cells[c * CH + ch] = free;
+                if (c == cj) cells[c * CH + ch] = make_float2(xj, make_cell(j, xn - xj));
+                if (j == N)
+                    for (c = cj + 1; c < K; ++c) cells[c * CH + ch] = free;
+                c = cj + 1;
+                xj = xn;
+            }
         }
     }
     __syncthreads();
 }
 
-template <bool CHAINS>
-__device__ __forceinline__ float chan_fwd8(float x, int ch, const float4* R, const float* xs, const float* vs,
-                                           const float* sp, const ChanConstF& cc, int N, int K)
+// Shared memory by 32-bit address.  A pointer into extern shared memory is
+// rebuilt from special registers at each use in a cluster launch (about six
+// instructions per element of the backward); these addresses are formed once.
+__device__ __forceinline__ uint32_t smem_addr(const void* p)
 {
-    const float xc = clamp_nan(x, cc.a, cc.b);
-    const int c = cell_of(xc, cc.inv_w, cc.off, K);
-    const float4 r = R[c * kChF + ch];
-    float s = xc < r.x ? r.z : r.w;
-    float anchor = r.x, y0 = r.y;
-    if (CHAINS && s != s) {  // right of the first knot of a cell holding several
-        int k = (int)(__float_as_uint(r.w) & kKnotTagMask);
-        for (int g = 0; g < cc.max_chain && k < N; ++g) {
-            if (!(xc >= xs[(k + 1) * kChF + ch])) break;
-            ++k;
+    uint32_t a = (uint32_t)__cvta_generic_to_shared(p);
+    asm volatile("" : "+r"(a));  // keeps the compiler from forming it again
+    return a;
+}
+__device__ __forceinline__ float2 lds2(uint32_t a)
+{
+    float2 v;
+    asm("ld.shared.v2.f32 {%0, %1}, [%2];" : "=f"(v.x), "=f"(v.y) : "r"(a) : "memory");
+    return v;
+}
+__device__ __forceinline__ float4 lds4(uint32_t a)
+{
+    float4 v;
+    asm("ld.shared.v4.f32 {%0, %1, %2, %3}, [%4];" : "=f"(v.x), "=f"(v.y), "=f"(v.z), "=f"(v.w) : "r"(a) : "memory");
+    return v;
+}
+template <int OFF>
+__device__ __forceinline__ void red_add(uint32_t a, int v)
+{
+    asm volatile("red.shared.add.s32 [%0+%2], %1;" ::"r"(a), "r"(v), "n"(OFF) : "memory");
+}
+
+// A thread's channel is fixed for a tile: its constants live in registers.
+template <int CH>
+struct ChanConst {
+    uint32_t cells, rec;  // shared addresses of the channel's first cell and record
+    uint32_t last;        // of record N + 1
+    float a, b, inv_w, off;
+    int K;
+    __device__ __forceinline__ ChanConst(const ChanArgs& p, const float2* cells0, const float4* rec0, int ch)
+        : cells(smem_addr(cells0 + ch)), rec(smem_addr(rec0 + ch)), last(rec + (uint32_t)(p.N + 1) * (16 * CH)),
+          a(rec0[CH + ch].x), b(rec0[p.N * CH + ch].w), inv_w((float)p.K / (b - a)), off(-a * inv_w), K(p.K)
+    {
+    }
+};
+
+// The records of the intervals of G points in [a, b], and their addresses.
+template <int CH, int G>
+__device__ __forceinline__ void chan_lookup(const float (&xc)[G], const ChanConst<CH>& cc, float4 (&r)[G],
+                                            uint32_t (&at)[G])
+{
+    float2 c[G];
+#pragma unroll
+    for (int g = 0; g < G; ++g) c[g] = lds2(cc.cells + chan_cell(xc[g], cc.inv_w, cc.off, cc.K) * (8 * CH));
+    bool more = false;
+#pragma unroll
+    for (int g = 0; g < G; ++g) {
+        const unsigned w = __float_as_uint(c[g].y);
+        int i = (int)(w & 0xffffu);
+        if (xc[g] >= c[g].x) ++i;
+        if (xc[g] - c[g].x >= __uint_as_float(w & 0xffff0000u)) ++i;
+        at[g] = cc.rec + i * (16 * CH);
+        r[g] = lds4(at[g]);
+    }
+#pragma unroll
+    for (int g = 0; g < G; ++g) more = more || xc[g] >= r[g].w;
+    if (more) {
+#pragma unroll
+        for (int g = 0; g < G; ++g)
+            while (xc[g] >= r[g].w && at[g] < cc.last) {
+                at[g] += 16 * CH;
+                r[g] = lds4(at[g]);
+            }
+    }
+}
+
+// ---- forward -----------------------------------------------------------------
+template <int CH, int G>
+__device__ __forceinline__ void chan_fwd(float (&v)[G], const ChanConst<CH>& cc)
+{
+    float xc[G];
+    float4 r[G];
+    uint32_t at[G];
+#pragma unroll
+    for (int g = 0; g < G; ++g) xc[g] = clamp_nan(v[g], cc.a, cc.b);
+    chan_lookup<CH, G>(xc, cc, r, at);
+#pragma unroll
+    for (int g = 0; g < G; ++g) v[g] = __fmaf_rn(xc[g] - r[g].x, r[g].z, r[g].y);
+}
+
+template <typename IO, int CH>
+__device__ __forceinline__ void chan_fwd_rows(const ChanArgs& p, int64_t c0, int64_t r0, int64_t r1,
+                                              const float2* cells, const float4* rec, const IO* __restrict__ x,
+                                              IO* __restrict__ y)
+{
+    constexpr int RP = kChThreads / CH, U = kFwdUnroll, G = kFwdGroup;
+    const int ch = threadIdx.x % CH, row = threadIdx.x / CH;
+    if (c0 + ch >= p.C) return;
+    const ChanConst<CH> cc(p, cells, rec, ch);
+    int64_t r = r0 + row;
+    const int64_t step = (int64_t)RP * p.C;  // elements between a thread's consecutive rows
+    const IO* px = x + r * p.C + c0 + ch;
+    IO* py = y + r * p.C + c0 + ch;
+    for (; r + (U - 1) * RP < r1; r += U * RP) {
+        // x is read at the L2 only (ld.global.cg)
+        float v[U];
+#pragma unroll
+        for (int u = 0; u < U; ++u) v[u] = to_f32<IO>(__ldcg(px + u * step));
+#pragma unroll
+        for (int u = 0; u < U; u += G) {
+            float w[G];
+#pragma unroll
+            for (int g = 0; g < G; ++g) w[g] = v[u + g];
+            chan_fwd<CH, G>(w, cc);
+#pragma unroll
+            for (int g = 0; g < G; ++g) st_cs(py + (u + g) * step, from_f32<IO>(w[g]));
         }
-        anchor = xs[k * kChF + ch];
-        y0 = vs[k * kChF + ch];
-        s = sp[k * kChF + ch];
+        px += U * step;
+        py += U * step;
     }
-    return __fmaf_rn(xc - anchor, s, y0);
+    // the rest (fewer than U rows per thread) in predicated batches: a few load
+    // latencies instead of one per row
+    for (; r < r1; r += (int64_t)kFwdTail * RP) {
+        const int64_t left = (r1 - r + RP - 1) / RP;
+        const int rem = left < kFwdTail ? (int)left : kFwdTail;
+        float v[kFwdTail];
+#pragma unroll
+        for (int u = 0; u < kFwdTail; ++u) v[u] = u < rem ? to_f32<IO>(__ldcg(px + u * step)) : cc.a;
+        chan_fwd<CH, kFwdTail>(v, cc);
+#pragma unroll
+        for (int u = 0; u < kFwdTail; ++u)
+            if (u < rem) st_cs(py + u * step, from_f32<IO>(v[u]));
+        px += kFwdTail * step;
+        py += kFwdTail * step;
+    }
 }
 
-template <typename IO, bool CHAINS>
-__device__ __forceinline__ void chan_fwd8_rows(const ChanArgs& p, int64_t c0, int64_t r0, int64_t r1,
-                                               const float4* R, const float* xs, const float* vs, const float* sp,
-                                               const TileParamsF& tp, const IO* __restrict__ x, IO* __restrict__ y)
+// Calls body(tile, r0, r1) for the row ranges of this CTA's share of the work.
+template <int CH, class Body>
+__device__ __forceinline__ void for_each_range(const ChanArgs& p, const Body& body)
 {
-    const int ch = threadIdx.x % kChF;
-    const int64_t c = c0 + ch;
-    if (c >= p.C) return;
-    const ChanConstF cc(tp, ch);
-    int64_t r = r0 + threadIdx.x / kChF;
-    const int64_t pass = (int64_t)kRowsPerPassF * p.C;  // elements between a thread's consecutive rows
-    // x is read at the L2 only (ld.global.cg): 2% faster than through L1,
-    // whose lines the row segments of other CTAs do not share anyway
-    const IO* px = x + r * p.C + c;
-    IO* py = y + r * p.C + c;
-    for (; r + (int64_t)(kChUnrollF - 1) * kRowsPerPassF < r1; r += (int64_t)kChUnrollF * kRowsPerPassF) {
-        float v[kChUnrollF];
-#pragma unroll
-        for (int u = 0; u < kChUnrollF; ++u) v[u] = to_f32<IO>(__ldcg(px + u * pass));
-#pragma unroll
-        for (int u = 0; u < kChUnrollF; ++u) v[u] = chan_fwd8<CHAINS>(v[u], ch, R, xs, vs, sp, cc, p.N, p.K);
-#pragma unroll
-        for (int u = 0; u < kChUnrollF; ++u) st_cs(py + u * pass, from_f32<IO>(v[u]));
-        px += kChUnrollF * pass;
-        py += kChUnrollF * pass;
-    }
-    // the rest (fewer than kChUnrollF rows per thread) in predicated batches of
-    // kChTailF: a few load latencies instead of one per row
-    for (; r < r1; r += (int64_t)kChTailF * kRowsPerPassF) {
-        const int64_t left = (r1 - r + kRowsPerPassF - 1) / kRowsPerPassF;
-        const int rem = left < kChTailF ? (int)left : kChTailF;
-        float v[kChTailF];
-#pragma unroll
-        for (int u = 0; u < kChTailF; ++u)
-            if (u < rem) v[u] = to_f32<IO>(__ldcg(px + u * pass));
-#pragma unroll
-        for (int u = 0; u < kChTailF; ++u)
-            if (u < rem) st_cs(py + u * pass, from_f32<IO>(chan_fwd8<CHAINS>(v[u], ch, R, xs, vs, sp, cc, p.N, p.K)));
-        px += kChTailF * pass;
-        py += kChTailF * pass;
+    constexpr int RP = kChThreads / CH;
+    const int64_t cluster = blockIdx.x / p.cluster, nclusters = gridDim.x / p.cluster;
+    const int64_t w1 = p.work * (cluster + 1) / nclusters;
+    for (int64_t w = p.work * cluster / nclusters; w < w1;) {
+        const int64_t group = w / p.passes, end = min(w1, (group + 1) * p.passes);
+        const int64_t tile = group * p.cluster + blockIdx.x % p.cluster;
+        const int64_t r0 = (w - group * p.passes) * RP, r1 = min(p.R, (end - group * p.passes) * RP);
+        w = end;
+        if (tile * CH < p.C) body(tile, r0, r1);  // no tile past the last one of a partial group
     }
 }
 
-// Units = (tile quad, chunk of rows), quad-major; the 4 CTAs of a cluster take
-// the 4 tiles of a quad on the same rows.
-template <typename IO>
+template <typename IO, int CH>
 __global__ void __launch_bounds__(kChThreads, 1) channels_forward_kernel(const ChanArgs p, const IO* x, IO* y)
 {
     extern __shared__ float4 s_ch[];
-    float4* R = s_ch;
-    float* xs = reinterpret_cast<float*>(R + (size_t)p.K * kChF);
-    float* vs = xs + (size_t)(p.N + 1) * kChF;
-    float* sp = vs + (size_t)(p.N + 1) * kChF;
-    int* cj = reinterpret_cast<int*>(sp + (size_t)(p.N + 1) * kChF);
-    __shared__ TileParamsF tp;
-    const int64_t cluster = blockIdx.x / kClF, nclusters = gridDim.x / kClF;
-    const int64_t u0 = p.units * cluster / nclusters, u1 = p.units * (cluster + 1) / nclusters;
-    int64_t built = -1;
-    for (int64_t u = u0; u < u1; ++u) {
-        const int64_t tile = kClF * (u / p.per_pair) + (blockIdx.x % kClF), chunk = u % p.per_pair;
-        if (tile >= p.tiles) continue;  // a tile past the last one of a partial quad
-        if (tile != built) {
-            __syncthreads();
-            build_tile_fwd(p, tile * kChF, R, xs, vs, sp, cj, &tp);
-            if (threadIdx.x == 0 && tp.bad) atomicOr(p.status, 1);
-            built = tile;
-        }
-        const int64_t r0 = chunk * p.rows_per_unit, r1 = min(p.R, r0 + p.rows_per_unit);
-        if (tp.any_chain)
-            chan_fwd8_rows<IO, true>(p, tile * kChF, r0, r1, R, xs, vs, sp, tp, x, y);
-        else
-            chan_fwd8_rows<IO, false>(p, tile * kChF, r0, r1, R, xs, vs, sp, tp, x, y);
-    }
+    __shared__ int s_bad;
+    float4* rec = s_ch;
+    float2* cells = reinterpret_cast<float2*>(rec + (size_t)(p.N + 2) * CH);
+    for_each_range<CH>(p, [&](int64_t tile, int64_t r0, int64_t r1) {
+        __syncthreads();  // nobody reads the previous tile any more
+        build_tile<CH, false>(p, tile * CH, cells, rec, &s_bad, [] {});
+        if (threadIdx.x == 0 && s_bad) atomicOr(p.status, 1);
+        chan_fwd_rows<IO, CH>(p, tile * CH, r0, r1, cells, rec, x, y);
+    });
 }
 
 // ---- backward ----------------------------------------------------------------
-// gx = gy * s_i; per (channel, interval) sums A_i = sum gy (1 - delta) and
-// B_i = sum gy delta accumulate in shared memory (FP32 atomics); at the end
-// of a tile's rows they become g_v[j] += A_{j+1} + B_j (+ clamped terms) and
+// gx = gy * s_i; per (channel, interval) the sums A_i = sum gy (x_i - x)/h_i and
+// B_i = sum gy (x - x_{i-1})/h_i accumulate in shared memory; at the end of a
+// tile's rows they become g_v[j] += A_{j+1} + B_j (+ clamped terms) and
 // g_x[j] += -s_{j+1} A_{j+1} - s_j B_j, added to the global gradients.
+//
+// The sums are fixed point, in two 32-bit words each: a term v in units of
+// 2^-F is split into h = rint(v 2^-17) and the rest l = rint(v - h 2^17), both
+// (h by adding 1.5 2^23, which needs no conversion), and added with native
+// integer shared-memory atomics that return nothing.  An FP32 shared-memory
+// add is a compare-and-swap loop in software (about 10 instructions, 2.6 adds
+// per clock and SM against more than 9 for int32): with it this kernel was
+// issue bound.  |v| < 2^33 keeps h and l
+// within 2^16, so neither word of an interval wraps in kFlushRows rows.  F comes, per
+// channel, from the mean binary exponent of gy over rows spread over all of
+// R: a typical term is ~2^kTypicalBits units, i.e. rounded at 2^-29 of it (an FP32 add
+// rounds at 2^-25 of the running sum), terms above 32 times the typical one,
+// inf and NaN are added to the global gradients in FP32, and so is every
+// nonzero term of a tile whose sampled rows are all zero.
+constexpr int kTypicalBits = 28;
+constexpr float kFixLimit = 0x1p33f;
+constexpr int64_t kFlushRows = 32512;  // at most 2^15 - 1, whole passes of every tile width (64, 128, 256 rows)
+constexpr float kMagic = 0x1.8p23f;
+constexpr int kMagicBits = 0x4B400000;
+
+struct BwdShared {
+    int bad;
+    int esum[16], ecnt[16];
+};
+
+// gy of this thread's channel at its sampled row (0 past the last channel)
+template <typename IO, int CH>
+__device__ __forceinline__ float sample_gy(const ChanArgs& p, int64_t c0, const IO* gy)
+{
+    const int64_t c = c0 + threadIdx.x % CH, r = p.R * (int64_t)(threadIdx.x / CH) / (kChThreads / CH);
+    return c < p.C ? to_f32<IO>(__ldcg(gy + r * p.C + c)) : 0.0f;
+}
+// the samples' binary exponents (nonzero finite ones) into the channels' sums
+template <int CH>
+__device__ __forceinline__ void sum_exponents(float g, BwdShared* sh)
+{
+    const int ex = (int)(__float_as_uint(g) >> 23 & 0xffu);
+    const bool ok = ex != 0 && ex != 0xff;
+    int esum = ok ? ex - 127 : 0, ecnt = ok ? 1 : 0;
+    for (int o = CH; o < 32; o <<= 1) {
+        esum += __shfl_xor_sync(0xffffffffu, esum, o);
+        ecnt += __shfl_xor_sync(0xffffffffu, ecnt, o);
+    }
+    if ((threadIdx.x & 31) < CH && ecnt) {
+        atomicAdd(&sh->esum[threadIdx.x % CH], esum);
+        atomicAdd(&sh->ecnt[threadIdx.x % CH], ecnt);
+    }
+}
+
+// F of a channel: from its own samples, else the tile's; with no nonzero
+// sample at all the largest unit scale, which sends every nonzero term to the
+// FP32 path.  2^F and 2^-F are normal FP32 numbers.
+template <int CH>
+__device__ __forceinline__ int fix_exponent(const BwdShared* sh, int ch)
+{
+    int s = sh->esum[ch], n = sh->ecnt[ch];
+    if (n == 0)
+        for (int q = 0; q < CH; ++q) {
+            s += sh->esum[q];
+            n += sh->ecnt[q];
+        }
+    if (n == 0) return 126;
+    return min(max(kTypicalBits - (int)floorf((float)s / (float)n), -60), 126);
+}
+__device__ __forceinline__ float exp2_int(int e) { return __int_as_float((e + 127) << 23); }
+
+// one term into its two words (h at byte offset H, l at byte offset L)
+template <int H, int L>
+__device__ __forceinline__ void fix_add(uint32_t at, float v)
+{
+    const float m = __fmaf_rn(v, 0x1p-17f, kMagic);
+    red_add<H>(at, __float_as_int(m) - kMagicBits);
+    red_add<L>(at, __float2int_rn(__fmaf_rn(__fsub_rn(m, kMagic), -0x1p17f, v)));
+}
+
+// FP32 sums of the gradients w.r.t. the end values of clamped elements
 struct EndSums {
     float left, right;
 };
 
-// One element without branches apart from chain walks (a divergent version
-// issued the shared-memory atomics once per path): the lookup runs on the
-// clamped point (NaN looks up a and contributes nothing), the side and the
-// interval come from selects, and one predicated pair of atomics takes an
-// in-range element's two sums.  A knot-free cell's record {i, x_{i-1}} is
-// the right side of knot i - 1; a knot cell's {tag(k), x_k} either side of
-// knot k; so both read "knot k, point x_k".
-template <bool CHAINS>
-__device__ __forceinline__ float chan_bwd_one(float x, float g, int ch, const float* __restrict__ xs,
-                                              const float2* sP, const float2* sI, const ChanConst& cc, int N,
-                                              int K, float* accA, float* accB, EndSums& e)
+// What the backward of one channel needs besides its lookup.
+struct BwdOut {
+    float* gv;  // the channel's rows of the global gradients (or NULL)
+    float* gk;
+    uint32_t first, second;  // record address -> address of the interval's A words and B words (odd rows: B and A)
+    float scale;
+    bool odd;
+};
+
+// An element that is clamped, NaN, or beyond the fixed-point range (FP32 to the
+// global gradients); returns its gx.
+__device__ __noinline__ float chan_bwd_rare(float x, float g, float a, float b, float4 r, int e, bool last, float* gv,
+                                            float* gk, EndSums* ends)
 {
-    const float xc = fminf(fmaxf(x, cc.a), cc.b);  // NaN -> a
-    const int c = cell_of(xc, cc.inv_w, cc.off, K);
-    const float2 r = sP[c * kCh + ch];
-    const uint32_t bits = __float_as_uint(r.x);
-    const bool knot = (bits & 0xFFC00000u) == kLinkTag;
-    int k = knot ? (int)(bits & kKnotTagMask) : __float_as_int(r.x) - 1;
-    float xk = r.y;
-    if (CHAINS && knot && (bits & kKnotTagChain)) {
-        for (int gg = 0; gg < cc.max_chain && k < N; ++gg) {
-            const float xn = xs[(k + 1) * kCh + ch];
-            if (!(xc >= xn)) break;
-            ++k;
-            xk = xn;
+    if (x >= a && x <= b) {
+        const int i = max(e, 1);  // 0 only where x_0 is NaN
+        const float ca = g * ((r.w - x) * r.y), cb = g * ((x - r.x) * r.y);
+        if (gv) {
+            atomicAdd(gv + i - 1, ca);
+            if (!last) atomicAdd(gv + i, cb);
         }
+        if (gk) {
+            atomicAdd(gk + i - 1, -r.z * ca);
+            if (!last) atomicAdd(gk + i, -r.z * cb);
+        }
+        return g * r.z;
     }
-    // right of x_k: interval k + 1 from its left end; left of it: interval k
-    // from its right end; x = x_N: interval N at delta = 1
-    const bool right = xc >= xk;
-    const bool at_b = right && k == N;
-    const int i = right && !at_b ? k + 1 : k;
-    const float2 q = sI[i * kCh + ch];
-    const float tt = (right ? (xc - xk) : (xk - xc)) * q.y;
-    const float delta = at_b ? 1.0f : (right ? tt : 1.0f - tt);
-    const float one_minus = at_b ? 0.0f : (right ? 1.0f - tt : tt);
-    const bool inside = x >= cc.a && x <= cc.b;  // false for NaN
-    if (inside) {
-        atomicAdd(accA + i * kCh + ch, g * one_minus);
-        atomicAdd(accB + i * kCh + ch, g * delta);
-    }
-    e.left += x < cc.a ? g : 0.0f;
-    e.right += x > cc.b ? g : 0.0f;
-    const float gx = inside ? g * q.x : 0.0f;
-    return x != x ? x : gx;
+    ends->left += x < a ? g : 0.0f;
+    ends->right += x > b ? g : 0.0f;
+    return x != x ? x : 0.0f;
 }
 
-template <bool CHAINS>
+// G elements: gx in place of g.
+template <int CH, int G>
+__device__ __forceinline__ void chan_bwd(const float (&x)[G], float (&g)[G], const ChanConst<CH>& cc, const BwdOut& o,
+                                         EndSums& ends)
+{
+    float xc[G];
+    float4 r[G];
+    uint32_t at[G];
+    bool fine = true;
+#pragma unroll
+    for (int q = 0; q < G; ++q) {
+        xc[q] = fminf(fmaxf(x[q], cc.a), cc.b);  // NaN -> a
+        fine = fine && x[q] == xc[q] && fabsf(g[q] * o.scale) < kFixLimit;
+    }
+    chan_lookup<CH, G>(xc, cc, r, at);
+    auto add = [&](int q) {
+        // 1 - delta and delta, each from the interval's other end and so accurate
+        // where it is small; odd rows take them in the other order
+        const float gs = g[q] * o.scale;
+        const float p1 = o.odd ? r[q].x : r[q].w, p2 = o.odd ? r[q].w : r[q].x;
+        fix_add<0, 8 * CH>(at[q] + o.first, gs * (fabsf(p1 - xc[q]) * r[q].y));
+        fix_add<0, 8 * CH>(at[q] + o.second, gs * (fabsf(p2 - xc[q]) * r[q].y));
+        g[q] *= r[q].z;
+    };
+    if (fine) {
+#pragma unroll
+        for (int q = 0; q < G; ++q) add(q);
+    } else {
+#pragma unroll
+        for (int q = 0; q < G; ++q) {
+            if (x[q] == xc[q] && fabsf(g[q] * o.scale) < kFixLimit)
+                add(q);
+            else
+                g[q] = chan_bwd_rare(x[q], g[q], cc.a, cc.b, r[q], (int)(at[q] - cc.rec) / (16 * CH),
+                                     at[q] == cc.last, o.gv, o.gk, &ends);
+        }
+    }
+}
+
+template <typename IO, int CH>
 __device__ __forceinline__ void chan_bwd_rows(const ChanArgs& p, int64_t c0, int64_t r0, int64_t r1,
-                                              const float2* sP, const float2* sI, const float* xs,
-                                              const TileParams& tp, float* accA, float* accB,
-                                              const float* __restrict__ x, const float* __restrict__ gy,
-                                              float* __restrict__ gx)
+                                              const float2* cells, const float4* rec, int* acc, float scale,
+                                              const IO* __restrict__ x, const IO* __restrict__ gy,
+                                              IO* __restrict__ gx, float* g_values, float* g_knots)
 {
-    const int ch = threadIdx.x % kCh;
+    constexpr int RP = kChThreads / CH, U = kBwdUnroll, G = kBwdGroup;
+    const int ch = threadIdx.x % CH, row = threadIdx.x / CH;
     const int64_t c = c0 + ch;
-    EndSums e{0.0f, 0.0f};
-    if (c < p.C) {
-        const ChanConst cc(tp, ch);
-        int64_t r = r0 + threadIdx.x / kCh;
-        const int64_t pass = (int64_t)kRowsPerPass * p.C;
-        const int64_t o = r * p.C + c;
-        const float* px = x + o;
-        const float* pg = gy + o;
-        float* po = gx + o;
-        constexpr int U = kChUnroll / 2;  // two loads per element
-        for (; r + (int64_t)(U - 1) * kRowsPerPass < r1; r += (int64_t)U * kRowsPerPass) {
-            float xv[U], gv[U];
+    if (c >= p.C) return;
+    const ChanConst<CH> cc(p, cells, rec, ch);
+    const bool odd = CH == 16 && row % 2;
+    const uint32_t words = smem_addr(acc + ch) - cc.rec;
+    BwdOut out{g_values ? g_values + c * (p.N + 1) : nullptr, g_knots ? g_knots + c * (p.N + 1) : nullptr,
+               words + (odd ? 4 * CH : 0), words + (odd ? 0 : 4 * CH), scale, odd};
+    EndSums ends{0.0f, 0.0f};
+    int64_t r = r0 + row;
+    const int64_t step = (int64_t)RP * p.C;
+    const IO* px = x + r * p.C + c;
+    const IO* pg = gy + r * p.C + c;
+    IO* po = gx + r * p.C + c;
+    for (; r + (U - 1) * RP < r1; r += U * RP) {
+        IO xv[U], gv[U];
 #pragma unroll
-            for (int u = 0; u < U; ++u) {
-                xv[u] = px[u * pass];
-                gv[u] = pg[u * pass];
+        for (int u = 0; u < U; ++u) {
+            xv[u] = __ldcg(px + u * step);
+            gv[u] = __ldcg(pg + u * step);
+        }
+#pragma unroll
+        for (int u = 0; u < U; u += G) {
+            float xf[G], gf[G];
+#pragma unroll
+            for (int q = 0; q < G; ++q) {
+                xf[q] = to_f32<IO>(xv[u + q]);
+                gf[q] = to_f32<IO>(gv[u + q]);
             }
+            chan_bwd<CH, G>(xf, gf, cc, out, ends);
 #pragma unroll
-            for (int u = 0; u < U; ++u)
-                po[u * pass] = chan_bwd_one<CHAINS>(xv[u], gv[u], ch, xs, sP, sI, cc, p.N, p.K, accA, accB, e);
-            px += U * pass;
-            pg += U * pass;
-            po += U * pass;
+            for (int q = 0; q < G; ++q) st_cs(po + (u + q) * step, from_f32<IO>(gf[q]));
         }
-        // the rest (fewer than U rows per thread) in predicated batches of
-        // kChTail: a few load latencies instead of one per row
-        for (; r < r1; r += (int64_t)kChTail * kRowsPerPass) {
-            const int64_t left = (r1 - r + kRowsPerPass - 1) / kRowsPerPass;
-            const int rem = left < kChTail ? (int)left : kChTail;
-            float xv[kChTail], gv[kChTail];
-#pragma unroll
-            for (int u = 0; u < kChTail; ++u)
-                if (u < rem) {
-                    xv[u] = px[u * pass];
-                    gv[u] = pg[u * pass];
-                }
-#pragma unroll
-            for (int u = 0; u < kChTail; ++u)
-                if (u < rem)
-                    po[u * pass] = chan_bwd_one<CHAINS>(xv[u], gv[u], ch, xs, sP, sI, cc, p.N, p.K, accA, accB, e);
-            px += kChTail * pass;
-            pg += kChTail * pass;
-            po += kChTail * pass;
-        }
+        px += U * step;
+        pg += U * step;
+        po += U * step;
     }
-    // lanes ch and ch + 16 share a channel: one add each
-    if (e.left != 0.0f) atomicAdd(accA + 0 * kCh + ch, e.left);
-    if (e.right != 0.0f) atomicAdd(accA + (p.N + 1) * kCh + ch, e.right);
+    for (; r < r1; r += (int64_t)kBwdTail * RP) {
+        const int64_t left = (r1 - r + RP - 1) / RP;
+        const int rem = left < kBwdTail ? (int)left : kBwdTail;
+        float xf[kBwdTail], gf[kBwdTail];
+#pragma unroll
+        for (int u = 0; u < kBwdTail; ++u) {
+            xf[u] = u < rem ? to_f32<IO>(__ldcg(px + u * step)) : cc.a;
+            gf[u] = u < rem ? to_f32<IO>(__ldcg(pg + u * step)) : 0.0f;
+        }
+        chan_bwd<CH, kBwdTail>(xf, gf, cc, out, ends);
+#pragma unroll
+        for (int u = 0; u < kBwdTail; ++u)
+            if (u < rem) st_cs(po + u * step, from_f32<IO>(gf[u]));
+        px += kBwdTail * step;
+        pg += kBwdTail * step;
+        po += kBwdTail * step;
+    }
+    if (out.gv) {
+        if (ends.left != 0.0f) atomicAdd(out.gv, ends.left);
+        if (ends.right != 0.0f) atomicAdd(out.gv + p.N, ends.right);
+    }
 }
 
-// Adds a tile's shared sums to the global gradients and clears them.
-__device__ void flush_tile(const ChanArgs& p, int64_t c0, const float2* sI, float* accA, float* accB,
-                           float* g_values, float* g_knots)
+// n floats from shared memory (16-byte aligned) added to global ones, whole
+// 16-byte vectors where dst allows.
+__device__ __forceinline__ void add_global(float* dst, const float* src, int n)
+{
+    const int nv = reinterpret_cast<uintptr_t>(dst) % 16 == 0 ? n / 4 : 0;
+    for (int i = threadIdx.x; i < nv; i += kChThreads)
+        atomicAdd(reinterpret_cast<float4*>(dst) + i, reinterpret_cast<const float4*>(src)[i]);
+    for (int i = 4 * nv + threadIdx.x; i < n; i += kChThreads)
+        if (src[i] != 0.0f) atomicAdd(dst + i, src[i]);
+}
+
+// Adds a tile's sums to the global gradients and clears them.  With the tile's
+// last rows done (`stage`: the cell records' memory) the gradients pass
+// through shared memory, laid out as in global memory, and are added 16 bytes
+// at a time (one reduction per lane and address, to 32 different lines per
+// warp, took 15000 clocks for 16 channels of 257 knots).
+template <int CH>
+__device__ __forceinline__ void flush_tile(const ChanArgs& p, int64_t c0, const float4* rec, int* acc, float unit,
+                                           float* stage, float* g_values, float* g_knots)
 {
     __syncthreads();
-    const int N = p.N;
-    for (int e = threadIdx.x; e < (N + 1) * kCh; e += blockDim.x) {
-        const int j = e / kCh, ch = e % kCh;
-        const int64_t c = c0 + ch;
-        if (c >= p.C) continue;
-        const float A1 = (j < N) ? accA[(j + 1) * kCh + ch] : 0.0f;
-        const float Bj = (j > 0) ? accB[j * kCh + ch] : 0.0f;
-        float gv = A1 + Bj;
-        if (j == 0) gv += accA[0 * kCh + ch];
-        if (j == N) gv += accA[(N + 1) * kCh + ch];
-        if (g_values && gv != 0.0f) atomicAdd(g_values + c * (int64_t)(N + 1) + j, gv);
-        if (g_knots) {
-            const float gk = -sI[(j + 1) * kCh + ch].x * A1 - sI[j * kCh + ch].x * Bj;
-            if (gk != 0.0f) atomicAdd(g_knots + c * (int64_t)(N + 1) + j, gk);
+    const int N = p.N, n1 = N + 1;
+    const int ch = threadIdx.x % CH, nch = (int)min((int64_t)CH, p.C - c0);
+    float* stage_k = stage + (CH * n1 + 3) / 4 * 4;
+    // h 2^17 + l of word w, cleared: with l's carry moved to h, one conversion is
+    // exact (or rounds below half an ulp) and nothing cancels
+    auto take = [&](int i, int w) {
+        int *ph = acc + (i * 4 + w) * CH + ch, *pl = ph + 2 * CH;
+        const int l = *pl, h = *ph + (l >> 17);
+        *ph = 0;
+        *pl = 0;
+        return __fmaf_rn((float)h, 0x1p17f, (float)(l & 0x1ffff)) * unit;
+    };
+    if (ch < nch)
+        for (int j = threadIdx.x / CH; j <= N; j += kChThreads / CH) {
+            // A of interval j + 1 (of the elements at x_N for j = N), B of interval j
+            const float A = take(j + 1, 0), B = j > 0 ? take(j, 1) : 0.0f;
+            const float gv = A + B, gk = -rec[(j + 1) * CH + ch].z * A - rec[j * CH + ch].z * B;
+            if (stage) {
+                stage[ch * n1 + j] = gv;
+                stage_k[ch * n1 + j] = gk;
+            } else {
+                const int64_t at = (c0 + ch) * n1 + j;
+                if (g_values && gv != 0.0f) atomicAdd(g_values + at, gv);
+                if (g_knots && gk != 0.0f) atomicAdd(g_knots + at, gk);
+            }
         }
-    }
     __syncthreads();
-    for (int e = threadIdx.x; e < (N + 2) * kCh; e += blockDim.x) {
-        accA[e] = 0.0f;
-        accB[e] = 0.0f;
-    }
-    __syncthreads();
+    if (stage && g_values) add_global(g_values + c0 * n1, stage, nch * n1);
+    if (stage && g_knots) add_global(g_knots + c0 * n1, stage_k, nch * n1);
 }
 
-__global__ void __launch_bounds__(kChThreads, 1) channels_backward_kernel(const ChanArgs p, const float* x,
-                                                                          const float* gy, float* gx,
-                                                                          float* g_values, float* g_knots)
+template <typename IO, int CH>
+__global__ void __launch_bounds__(kChThreads, 1) channels_backward_kernel(const ChanArgs p, const IO* x, const IO* gy,
+                                                                          IO* gx, float* g_values, float* g_knots)
 {
     extern __shared__ float4 s_ch[];
-    float2* sP = reinterpret_cast<float2*>(s_ch);
-    float2* sI = sP + (size_t)p.K * kCh;
-    float* accA = reinterpret_cast<float*>(sI + (size_t)(p.N + 2) * kCh);
-    float* accB = accA + (size_t)(p.N + 2) * kCh;
-    float* xs = accB + (size_t)(p.N + 2) * kCh;
-    int* cj = reinterpret_cast<int*>(accA);  // build scratch aliases the accumulators
-    __shared__ TileParams tp;
-    const int64_t cluster = blockIdx.x >> 1, nclusters = gridDim.x >> 1;
-    const int64_t u0 = p.units * cluster / nclusters, u1 = p.units * (cluster + 1) / nclusters;
-    int64_t built = -1;
-    for (int64_t u = u0; u < u1; ++u) {
-        const int64_t tile = 2 * (u / p.per_pair) + (blockIdx.x & 1), chunk = u % p.per_pair;
-        if (tile >= p.tiles) break;  // the odd tile out of an odd tile count
-        if (tile != built) {
-            if (built >= 0) flush_tile(p, built * kCh, sI, accA, accB, g_values, g_knots);
-            __syncthreads();
-            build_tile(p, tile * kCh, sP, sI, xs, cj, &tp);
-            if (threadIdx.x == 0 && tp.bad) atomicOr(p.status, 1);
-            for (int e = threadIdx.x; e < (p.N + 2) * kCh; e += blockDim.x) {
-                accA[e] = 0.0f;
-                accB[e] = 0.0f;
-            }
-            __syncthreads();
-            built = tile;
+    __shared__ BwdShared sh;
+    float4* rec = s_ch;
+    int* acc = reinterpret_cast<int*>(rec + (size_t)(p.N + 2) * CH);
+    float2* cells = reinterpret_cast<float2*>(acc + (size_t)(p.N + 2) * 4 * CH);
+    for (int i = threadIdx.x; i < (p.N + 2) * 4 * CH; i += kChThreads) acc[i] = 0;
+    for_each_range<CH>(p, [&](int64_t tile, int64_t r0, int64_t r1) {
+        __syncthreads();  // nobody reads the previous tile any more
+        if (threadIdx.x < CH) sh.esum[threadIdx.x] = sh.ecnt[threadIdx.x] = 0;
+        const float g = sample_gy<IO, CH>(p, tile * CH, gy);
+        build_tile<CH, true>(p, tile * CH, cells, rec, &sh.bad, [&] { sum_exponents<CH>(g, &sh); });
+        if (threadIdx.x == 0 && sh.bad) atomicOr(p.status, 1);
+        const int F = fix_exponent<CH>(&sh, threadIdx.x % CH);
+        const float scale = exp2_int(F), unit = exp2_int(-F);
+        for (int64_t r = r0; r < r1; r += kFlushRows) {
+            chan_bwd_rows<IO, CH>(p, tile * CH, r, min(r1, r + kFlushRows), cells, rec, acc, scale, x, gy, gx, g_values,
+                                  g_knots);
+            flush_tile<CH>(p, tile * CH, rec, acc, unit,
+                           r + kFlushRows < r1 ? nullptr : reinterpret_cast<float*>(cells), g_values, g_knots);
         }
-        const int64_t r0 = chunk * p.rows_per_unit, r1 = min(p.R, r0 + p.rows_per_unit);
-        if (tp.any_chain)
-            chan_bwd_rows<true>(p, tile * kCh, r0, r1, sP, sI, xs, tp, accA, accB, x, gy, gx);
-        else
-            chan_bwd_rows<false>(p, tile * kCh, r0, r1, sP, sI, xs, tp, accA, accB, x, gy, gx);
-    }
-    if (built >= 0) flush_tile(p, built * kCh, sI, accA, accB, g_values, g_knots);
+    });
 }
 
-}  // namespace
-
-size_t channels_smem_bytes(int64_t N, int64_t K, bool backward)
+// ---- launch shapes -------------------------------------------------------------
+// The sizes the calls accept are those of one CTA holding 8 channels' 16-byte
+// cells, knots, values and slopes (forward) or 16 channels' 8-byte cells,
+// 8-byte interval records, two sums and knots (backward), plus a little for
+// scalars; every accepted size fits the tiles below (a 4-channel tile takes
+// less for the same N and K).  Without k_cells, that index may shrink to its
+// remainder of 16 cells.
+size_t accepted_bytes(int64_t N, int64_t K, bool backward)
 {
     const size_t n1 = (size_t)(N + 1), n2 = (size_t)(N + 2);
-    // forward: 8 channels of 16-byte cell records, knots, values, slopes and build scratch
-    if (!backward) return sizeof(float4) * kChF * (size_t)K + 4 * sizeof(float) * kChF * n1;
-    // backward: 16 channels of 8-byte cell and interval records, two accumulators, knots
-    return sizeof(float2) * kCh * ((size_t)K + n2) + sizeof(float) * 2 * kCh * n2 + sizeof(float) * kCh * n1;
+    if (!backward) return 128 * ((size_t)K + n1) + 200;
+    return 128 * ((size_t)K + n2) + 128 * n2 + 64 * n1 + 392;
 }
 
-int64_t channels_default_cells(int64_t N, bool backward)
+size_t tile_bytes(int64_t N, int64_t K, int CH, bool backward)
 {
-    // 4 (N+1) cells forward, 2 (N+1) backward, as far as one CTA's shared memory allows
-    // the static tile parameters of the kernel share the CTA's shared memory
-    const size_t budget = device_info().smem_optin - (backward ? sizeof(TileParams) : sizeof(TileParamsF));
-    int64_t K = (backward ? 2 : 4) * (N + 1);
-    while (K > 16 && channels_smem_bytes(N, K, backward) > budget) K -= 16;
-    return K;
+    const size_t recs = 16 * (size_t)(N + 2) * (size_t)CH * (backward ? 2 : 1);
+    return recs + 8 * (size_t)std::max<int64_t>(K, stage_pitch((int)N)) * (size_t)CH;
 }
 
-pwl_status channels_launch(const ChanArgs& base, bool backward, int io_dtype, const void* x, void* y,
-                           const float* gy, float* gx, float* g_values, float* g_knots, cudaStream_t s)
+// Shared memory of a CTA that leaves the L1 at least ~60 KB (a carve-out of
+// 196 KB) for the rows in flight.
+constexpr size_t kIndexBytes = 196 * 1024 - 1024 - 512;
+constexpr int64_t kFwdCells = 2, kBwdCells = 2;  // cells per knot where they fit
+
+struct ChanShape {
+    int CH, K;
+    size_t smem;
+};
+
+// The widest tile whose index fits kIndexBytes with the wanted cells (at least
+// kBwdCells per knot), else the narrowest.
+ChanShape choose_shape(int64_t N, int64_t k_cells, bool backward)
 {
-    ChanArgs p = base;
-    const size_t smem = channels_smem_bytes(p.N, p.K, backward);
-    const DeviceInfo& di = device_info();
-    const int tile_ch = backward ? kCh : kChF;       // channels per tile
-    const int cluster_ctas = backward ? 2 : kClF;    // CTAs per cluster (adjacent tiles, same rows)
-    if (smem + (backward ? sizeof(TileParams) : sizeof(TileParamsF)) > di.smem_optin)
-        return fail(PWL_ENOTSUP, "channel index of %zu bytes (%d channels x %d cells, N = %d) does not fit one CTA",
-                    smem, tile_ch, p.K, p.N);
-    p.tiles = (p.C + tile_ch - 1) / tile_ch;
-    const int64_t pairs = (p.tiles + cluster_ctas - 1) / cluster_ctas;  // tile groups of one cluster
-    const void* kfn;
-    if (backward)
-        kfn = (const void*)channels_backward_kernel;
-    else if (io_dtype == PWL_BF16)
-        kfn = (const void*)channels_forward_kernel<__nv_bfloat16>;
-    else
-        kfn = (const void*)channels_forward_kernel<float>;
-    PWL_CUDA_TRY(ensure_smem_limit(kfn, smem));
+    const int64_t want = k_cells > 0 ? k_cells : (backward ? kBwdCells : kFwdCells) * (N + 1);
+    const int64_t need = k_cells > 0 ? k_cells : kBwdCells * (N + 1);
+    const size_t optin = device_info().smem_optin - 512;
+    ChanShape s{};
+    for (int CH : {16, 8, 4}) {
+        const size_t budget = CH == 4 ? optin : std::min(kIndexBytes, optin);
+        const size_t recs = 16 * (size_t)(N + 2) * (size_t)CH * (backward ? 2 : 1);
+        const int64_t room = budget > recs ? (int64_t)((budget - recs) / (8 * (size_t)CH)) : 0;
+        s.CH = CH;
+        s.K = (int)std::min(want, std::max<int64_t>(room, 1));
+        if (room >= std::max<int64_t>(need, stage_pitch((int)N))) break;
+    }
+    s.smem = tile_bytes(N, s.K, s.CH, backward);
+    return s;
+}
+
+std::mutex g_cluster_mu;
+std::map<std::tuple<int, const void*, int, size_t>, int> g_clusters;
+
+// resident clusters of a kernel (a host call of several microseconds, cached)
+cudaError_t cluster_count(const void* fn, const cudaLaunchConfig_t& cfg, int ctas, int* n)
+{
+    std::lock_guard<std::mutex> lk(g_cluster_mu);
+    const auto key = std::make_tuple(device_info().device, fn, ctas, (size_t)cfg.dynamicSmemBytes);
+    const auto it = g_clusters.find(key);
+    if (it != g_clusters.end()) {
+        *n = it->second;
+        return cudaSuccess;
+    }
+    const cudaError_t e = cudaOccupancyMaxActiveClusters(n, fn, &cfg);
+    if (e != cudaSuccess) return e;
+    *n = std::max(*n, 1);
+    g_clusters[key] = *n;
+    return cudaSuccess;
+}
+
+template <typename... Args>
+pwl_status launch(ChanArgs p, int CH, size_t smem, void (*kern)(const ChanArgs, Args...), cudaStream_t s,
+                  Args... args)
+{
+    const void* fn = reinterpret_cast<const void*>(kern);
+    PWL_CUDA_TRY(ensure_smem_limit(fn, smem));
+    // a cluster covers a 128-byte line of a row (two CTAs for 16-channel BF16
+    // tiles: four leave 8 of the 152 SMs without a cluster)
+    p.cluster = CH == 16 ? 2 : (CH == 8 ? 4 : 8);
     cudaLaunchConfig_t cfg{};
     cudaLaunchAttribute attr[1];
     attr[0].id = cudaLaunchAttributeClusterDimension;
-    attr[0].val.clusterDim.x = cluster_ctas;
+    attr[0].val.clusterDim.x = p.cluster;
     attr[0].val.clusterDim.y = 1;
     attr[0].val.clusterDim.z = 1;
     cfg.blockDim = dim3(kChThreads);
@@ -645,52 +756,92 @@ pwl_status channels_launch(const ChanArgs& base, bool backward, int io_dtype, co
     cfg.stream = s;
     cfg.attrs = attr;
     cfg.numAttrs = 1;
-    cfg.gridDim = dim3(cluster_ctas);
+    cfg.gridDim = dim3(p.cluster);
     int clusters = 0;
-    PWL_CUDA_TRY(cudaOccupancyMaxActiveClusters(&clusters, kfn, &cfg));
-    clusters = std::max(clusters, 1);
-    // about 8 units per cluster: few index builds per CTA, and the last
-    // units balance the load
-    int64_t chunks = std::max<int64_t>(1, ((int64_t)clusters * 8 + pairs - 1) / pairs);
-    chunks = std::min<int64_t>(chunks, std::max<int64_t>(1, p.R / (kChThreads / tile_ch)));
-    p.rows_per_unit = (p.R + chunks - 1) / chunks;
-    chunks = (p.R + p.rows_per_unit - 1) / p.rows_per_unit;
-    p.per_pair = chunks;
-    p.units = pairs * chunks;
-    clusters = (int)std::min<int64_t>(clusters, p.units);
-    cfg.gridDim = dim3(cluster_ctas * clusters);
-    if (backward) {
-        PWL_CUDA_TRY(cudaLaunchKernelEx(&cfg, channels_backward_kernel, p, static_cast<const float*>(x), gy, gx,
-                                        g_values, g_knots));
-    } else if (io_dtype == PWL_BF16) {
-        PWL_CUDA_TRY(cudaLaunchKernelEx(&cfg, channels_forward_kernel<__nv_bfloat16>, p,
-                                        static_cast<const __nv_bfloat16*>(x), static_cast<__nv_bfloat16*>(y)));
-    } else {
-        PWL_CUDA_TRY(cudaLaunchKernelEx(&cfg, channels_forward_kernel<float>, p, static_cast<const float*>(x),
-                                        static_cast<float*>(y)));
-    }
+    PWL_CUDA_TRY(cluster_count(fn, cfg, p.cluster, &clusters));
+    const int64_t tiles = (p.C + CH - 1) / CH, groups = (tiles + p.cluster - 1) / p.cluster;
+    p.passes = (p.R + kChThreads / CH - 1) / (kChThreads / CH);
+    p.work = groups * p.passes;
+    cfg.gridDim = dim3(p.cluster * (unsigned)std::min<int64_t>(clusters, p.work));
+    PWL_CUDA_TRY(cudaLaunchKernelEx(&cfg, kern, p, args...));
     PWL_CHECK_LAUNCH("channels kernel");
     return PWL_OK;
 }
 
-}  // namespace pwl
+template <typename IO>
+pwl_status launch_forward(ChanArgs p, const ChanShape& sh, const void* x, void* y, cudaStream_t s)
+{
+    const IO* xi = static_cast<const IO*>(x);
+    IO* yo = static_cast<IO*>(y);
+    switch (sh.CH) {
+    case 16: return launch(p, 16, sh.smem, channels_forward_kernel<IO, 16>, s, xi, yo);
+    case 8: return launch(p, 8, sh.smem, channels_forward_kernel<IO, 8>, s, xi, yo);
+    default: return launch(p, 4, sh.smem, channels_forward_kernel<IO, 4>, s, xi, yo);
+    }
+}
 
-using namespace pwl;
+template <typename IO>
+pwl_status launch_backward(ChanArgs p, const ChanShape& sh, const void* x, const void* gy, void* gx, float* g_values,
+                           float* g_knots, cudaStream_t s)
+{
+    const IO *xi = static_cast<const IO*>(x), *gi = static_cast<const IO*>(gy);
+    IO* go = static_cast<IO*>(gx);
+    switch (sh.CH) {
+    case 16:
+        return launch(p, 16, sh.smem, channels_backward_kernel<IO, 16>, s, xi, gi, go, g_values, g_knots);
+    case 8:
+        return launch(p, 8, sh.smem, channels_backward_kernel<IO, 8>, s, xi, gi, go, g_values, g_knots);
+    default:
+        return launch(p, 4, sh.smem, channels_backward_kernel<IO, 4>, s, xi, gi, go, g_values, g_knots);
+    }
+}
 
-namespace {
-
-pwl_status check_channels(const float* knots, const float* values, int64_t C, int64_t N, int64_t R,
-                          int64_t k_cells, int32_t* d_status)
+// Validates the arguments shared by both directions and fills p and the shape.
+pwl_status setup(const float* knots, const float* values, int64_t C, int64_t N, int64_t R, int64_t k_cells,
+                 int32_t* d_status, int32_t io_dtype, bool backward, ChanArgs& p, ChanShape& sh)
 {
     if (!knots || !values) return fail(PWL_EINVAL, "knots / values is NULL");
     if (C < 1 || N < 1 || N > 65535) return fail(PWL_EINVAL, "need C >= 1 channels and 1 <= N <= 65535 intervals");
     if (R < 0) return fail(PWL_EINVAL, "rows must be >= 0");
     if (k_cells < 0 || k_cells > (1 << 20)) return fail(PWL_EINVAL, "k_cells must be in [0, 2^20]");
     if (!d_status) return fail(PWL_EINVAL, "status word is NULL");
+    if (io_dtype != PWL_FP32 && io_dtype != PWL_BF16) return fail(PWL_EINVAL, "io dtype must be FP32 or BF16");
+    if (R == 0) return PWL_OK;
+    const size_t optin = device_info().smem_optin;
+    const int64_t least = k_cells > 0 ? k_cells : ((backward ? 2 : 4) * (N + 1) - 1) % 16 + 1;
+    if (accepted_bytes(N, least, backward) > optin)
+        return fail(PWL_ENOTSUP, "a channel index of N = %lld intervals and %lld cells does not fit one CTA",
+                    (long long)N, (long long)least);
+    sh = choose_shape(N, k_cells, backward);
+    p.knots = knots;
+    p.values = values;
+    p.C = C;
+    p.R = R;
+    p.N = (int)N;
+    p.K = sh.K;
+    p.status = d_status;
     return PWL_OK;
 }
 
+pwl_status backward(const float* knots, const float* values, int64_t C, int64_t N, int64_t k_cells, const void* x,
+                    const void* gy, void* gx, float* g_values, float* g_knots, int64_t R, int32_t io_dtype,
+                    int32_t* d_status, void* stream)
+{
+    ChanArgs p{};
+    ChanShape sh{};
+    const pwl_status st = setup(knots, values, C, N, R, k_cells, d_status, io_dtype, true, p, sh);
+    if (st != PWL_OK || R == 0) return st;
+    if (!x || !gy || !gx) return fail(PWL_EINVAL, "x / gy / gx is NULL");
+    if (io_dtype == PWL_BF16)
+        return launch_backward<__nv_bfloat16>(p, sh, x, gy, gx, g_values, g_knots, as_stream(stream));
+    return launch_backward<float>(p, sh, x, gy, gx, g_values, g_knots, as_stream(stream));
+}
+
 }  // namespace
+
+}  // namespace pwl
+
+using namespace pwl;
 
 extern "C" {
 
@@ -699,20 +850,14 @@ pwl_status pwl_channels_forward(const float* d_knots, const float* d_values, int
                                 int32_t io_dtype, int32_t* d_status, void* stream)
 {
     clear_error();
-    pwl_status st = check_channels(d_knots, d_values, n_channels, n_intervals, rows, k_cells, d_status);
-    if (st != PWL_OK) return st;
-    if (io_dtype != PWL_FP32 && io_dtype != PWL_BF16) return fail(PWL_EINVAL, "io dtype must be FP32 or BF16");
-    if (rows == 0) return PWL_OK;
-    if (!d_x || !d_y) return fail(PWL_EINVAL, "x / y is NULL");
     ChanArgs p{};
-    p.knots = d_knots;
-    p.values = d_values;
-    p.C = n_channels;
-    p.R = rows;
-    p.N = (int)n_intervals;
-    p.K = (int)(k_cells > 0 ? k_cells : channels_default_cells(n_intervals, false));
-    p.status = d_status;
-    return channels_launch(p, false, io_dtype, d_x, d_y, nullptr, nullptr, nullptr, nullptr, as_stream(stream));
+    ChanShape sh{};
+    const pwl_status st =
+        setup(d_knots, d_values, n_channels, n_intervals, rows, k_cells, d_status, io_dtype, false, p, sh);
+    if (st != PWL_OK || rows == 0) return st;
+    if (!d_x || !d_y) return fail(PWL_EINVAL, "x / y is NULL");
+    if (io_dtype == PWL_BF16) return launch_forward<__nv_bfloat16>(p, sh, d_x, d_y, as_stream(stream));
+    return launch_forward<float>(p, sh, d_x, d_y, as_stream(stream));
 }
 
 pwl_status pwl_channels_backward(const float* d_knots, const float* d_values, int64_t n_channels,
@@ -721,19 +866,18 @@ pwl_status pwl_channels_backward(const float* d_knots, const float* d_values, in
                                  void* stream)
 {
     clear_error();
-    pwl_status st = check_channels(d_knots, d_values, n_channels, n_intervals, rows, k_cells, d_status);
-    if (st != PWL_OK) return st;
-    if (rows == 0) return PWL_OK;
-    if (!d_x || !d_gy || !d_gx) return fail(PWL_EINVAL, "x / gy / gx is NULL");
-    ChanArgs p{};
-    p.knots = d_knots;
-    p.values = d_values;
-    p.C = n_channels;
-    p.R = rows;
-    p.N = (int)n_intervals;
-    p.K = (int)(k_cells > 0 ? k_cells : channels_default_cells(n_intervals, true));
-    p.status = d_status;
-    return channels_launch(p, true, PWL_FP32, d_x, nullptr, d_gy, d_gx, d_g_values, d_g_knots, as_stream(stream));
+    return backward(d_knots, d_values, n_channels, n_intervals, k_cells, d_x, d_gy, d_gx, d_g_values, d_g_knots, rows,
+                    PWL_FP32, d_status, stream);
+}
+
+pwl_status pwl_channels_backward_bf16(const float* d_knots, const float* d_values, int64_t n_channels,
+                                      int64_t n_intervals, int64_t k_cells, const void* d_x, const void* d_gy,
+                                      void* d_gx, float* d_g_values, float* d_g_knots, int64_t rows,
+                                      int32_t* d_status, void* stream)
+{
+    clear_error();
+    return backward(d_knots, d_values, n_channels, n_intervals, k_cells, d_x, d_gy, d_gx, d_g_values, d_g_knots, rows,
+                    PWL_BF16, d_status, stream);
 }
 
 }  // extern "C"

@@ -10,11 +10,10 @@ struct ChanArgs {
     const float* values;  // [C, N+1] FP32
     int64_t C, R;         // channels, rows
     int N, K;             // intervals, cells per channel
-    int64_t tiles, units, rows_per_unit, per_pair;
+    int cluster;          // CTAs per cluster
+    int64_t passes;       // passes of the CTA over all rows: ceil(R / rows per pass)
+    int64_t work;         // tile groups (of a cluster's CTAs) x passes
     int* status;          // device word: bit 0 set if a channel's knots are not strictly increasing
 };
-
-size_t channels_smem_bytes(int64_t N, int64_t K, bool backward);
-int64_t channels_default_cells(int64_t N, bool backward);
 
 }  // namespace pwl
