@@ -3,9 +3,8 @@
 // each a fixed sequence of launches over all functions, so that the four
 // phases can be captured in one CUDA graph and replayed.
 //
-//   design      density / chunk scan / inversion over the chunks of every
-//               function at once (FP64), or one CTA per function (FP32; the
-//               kernels of pwl_design.cu)
+//   design      density / chunk scan / inversion over the tiles of every
+//               function at once (the kernels of pwl_design.cu)
 //   projection  hat integrals of every interval, then one CTA per function
 //               for the Gram solve (pwl_project.cu)
 //   index       one CTA per function: FP32 knots and values, slopes and the
@@ -535,7 +534,9 @@ struct pwl_batch_s {
     int* cj;
     float2 *recP, *recS;
     int* status;                // device word: bit 2 = an evaluation wait timed out
-    int* order;                 // functions by decreasing density cells (design order)
+    int* order;                 // functions by decreasing intervals (the Gram solves' order)
+    int* tile_func;             // per design tile: its function
+    DesignFunc* ffuncs;         // FP32 design: constants per function (scratch)
     // evaluation plan
     std::vector<int64_t> qoff;  // query offsets of the plan
     void* plan_dev;             // items, then the CTA ranges
@@ -709,11 +710,14 @@ pwl_status pwl_batch_create(const pwl_func* funcs, const int64_t* n_intervals, i
         poff += K;
         soff += N + 2;
     }
-    // design order: the functions with the most density cells first, so that
-    // the persistent design launch ends on small functions
+    // the largest functions first, so that the Gram solves (one warp per
+    // function) end on small ones
     std::vector<int> order(n_funcs);
     for (int64_t f = 0; f < n_funcs; ++f) order[f] = (int)f;
     std::stable_sort(order.begin(), order.end(), [&](int x, int y) { return b->N[x] > b->N[y]; });
+    std::vector<int> tile_func((size_t)(choff[n_funcs] / design_chunks(1)));
+    for (int64_t f = 0; f < n_funcs; ++f)
+        std::fill(tile_func.begin() + choff[f] / design_chunks(1), tile_func.begin() + choff[f + 1] / design_chunks(1), (int)f);
     b->total_knots = b->koff[n_funcs];
     b->total_cells_design = moff[n_funcs];
     b->total_chunks = choff[n_funcs];
@@ -735,11 +739,14 @@ pwl_status pwl_batch_create(const pwl_func* funcs, const int64_t* n_intervals, i
                             align256(8 * (size_t)poff),
                             align256(16 * T),
                             align256(sizeof(int)),
-                            align256(sizeof(int) * F)};
+                            align256(sizeof(int) * F),
+                            align256(sizeof(int) * tile_func.size()),
+                            align256(sizeof(DesignFunc) * F)};
     void** slots[] = {(void**)&b->funcs, (void**)&b->d_koff, (void**)&b->d_moff, (void**)&b->d_choff,
                       (void**)&b->knots, (void**)&b->values, &b->design_scratch, &b->project_scratch,
                       (void**)&b->bf, (void**)&b->xk, (void**)&b->vk, (void**)&b->slope, (void**)&b->cj,
-                      (void**)&b->recP, (void**)&b->recS, (void**)&b->status, (void**)&b->order};
+                      (void**)&b->recP, (void**)&b->recS, (void**)&b->status, (void**)&b->order,
+                      (void**)&b->tile_func, (void**)&b->ffuncs};
     static_assert(sizeof(sizes) / sizeof(sizes[0]) == sizeof(slots) / sizeof(slots[0]), "one size per slot");
     size_t total = 0;
     for (size_t s : sizes) total += s;
@@ -759,7 +766,8 @@ pwl_status pwl_batch_create(const pwl_func* funcs, const int64_t* n_intervals, i
         (e = cudaMemcpy(b->d_choff, choff.data(), 8 * (F + 1), cudaMemcpyHostToDevice)) != cudaSuccess ||
         (e = cudaMemcpy(b->bf, bfh.data(), sizeof(BatchFunc) * F, cudaMemcpyHostToDevice)) != cudaSuccess ||
         (e = cudaMemset(b->status, 0, sizeof(int))) != cudaSuccess ||
-        (e = cudaMemcpy(b->order, order.data(), sizeof(int) * F, cudaMemcpyHostToDevice)) != cudaSuccess) {
+        (e = cudaMemcpy(b->order, order.data(), sizeof(int) * F, cudaMemcpyHostToDevice)) != cudaSuccess ||
+        (e = cudaMemcpy(b->tile_func, tile_func.data(), sizeof(int) * tile_func.size(), cudaMemcpyHostToDevice)) != cudaSuccess) {
         batch_free(b);
         return cuda_fail(e, "batch upload");
     }
@@ -794,12 +802,10 @@ pwl_status pwl_batch_design(pwl_batch b, int32_t precision, void* stream)
     p.total_chunks = b->total_chunks;
     p.knots = b->knots;
     design_carve_scratch(p, b->design_scratch);
-    p.order = b->order;
-    // FP64: the chunk-parallel kernels, whatever the number of functions (the
-    // FP64 pipe bounds them, and they compute each density once); FP32: one
-    // CTA per function
+    p.tile_func = b->tile_func;
+    p.ffuncs = b->ffuncs;
     if (precision == PWL_PREC_FP64) return design_launch(p, as_stream(stream));
-    return design_fused_launch(p, as_stream(stream));
+    return design_batch_f_launch(p, as_stream(stream));
 }
 
 pwl_status pwl_batch_project(pwl_batch b, int32_t form, int32_t quad_points, int32_t precision, void* stream)

@@ -7,15 +7,17 @@
 // (descriptors and CSR offsets of knots, cells and 256-cell chunks, the
 // chunks of a function padded to whole tiles of 8); a single function is a
 // batch of one.  Three launches:
-//   density_chunks  d_k = |f''(t_k)|^{2/5} and one FP64 partial sum per chunk
-//   chunk_scan      exclusive FP64 scan of the chunk sums, per function
-//   invert_tiles    per tile of 2048 cells: the in-tile prefix of the
+//   densities       d_k = |f''(t_k)|^{2/5} and one partial sum per chunk (FP64)
+//                   or tile (FP32 mode of a batch)
+//   scan            exclusive FP64 scan of the partial sums, per function
+//   knots           per tile of 2048 cells: the in-tile prefix of the
 //                   densities and the knots whose targets tau_i = i G_M / N
 //                   fall into the tile
-// They serve one function and, in FP64, every batch: a batch designed by one
-// CTA per function (as the FP32 mode below is) waits for its largest function
-// and computes every density twice: 40 functions of up to 4095 intervals at 64
-// cells per interval took 25.2 ms that way, 1.12 ms this way (density 1.03).
+// No CTA waits for another tile of its function: a batch designed by one CTA
+// per function waits for its largest function and for the barriers of every
+// tile in turn.  40 functions of up to 4095 intervals at 64 cells per
+// interval, FP64: 25.2 ms that way (which also computed the densities twice),
+// 1.12 ms this way (density 1.03).
 #include <math.h>
 
 #include <algorithm>
@@ -31,17 +33,6 @@ constexpr int kChunk = kDesignThreads;         // density cells per chunk
 constexpr int kTileChunks = 8;                 // chunks per tile (every function holds whole tiles)
 constexpr int kTile = kChunk * kTileChunks;    // cells per tile
 constexpr int kTilePer = kTile / kDesignThreads;  // cells per thread of a tile
-
-// index f with off[f] <= g < off[f+1] (off has F+1 non-decreasing entries)
-__device__ __forceinline__ int find_segment(const int64_t* __restrict__ off, int F, int64_t g)
-{
-    int lo = 0, hi = F - 1;
-    while (lo < hi) {
-        int mid = (lo + hi + 1) >> 1;
-        if (__ldg(off + mid) <= g) lo = mid; else hi = mid - 1;
-    }
-    return lo;
-}
 
 __device__ __forceinline__ double warp_sum(double v)
 {
@@ -104,7 +95,7 @@ __global__ void __launch_bounds__(kDesignThreads, 2) density_chunks_kernel(Desig
     __shared__ double s_red[kDesignThreads / 32];
     __shared__ int s_last[kDesignThreads / 32];
     for (int64_t ch = blockIdx.x; ch < p.total_chunks; ch += gridDim.x) {
-        const int f = find_segment(p.choff, p.F, ch);
+        const int f = p.tile_func ? p.tile_func[ch / kTileChunks] : 0;
         const pwl_func F = p.funcs[f];
         if ((F.kind == PWL_F_SAMPLED) != SAMPLED) continue;  // the other launch's (uniform per CTA)
         const int64_t M = p.moff[f + 1] - p.moff[f];
@@ -220,7 +211,7 @@ __global__ void __launch_bounds__(kDesignThreads) invert_tiles_kernel(DesignPlan
     const int t = threadIdx.x;
     for (int64_t tile = blockIdx.x; tile < p.total_chunks / kTileChunks; tile += gridDim.x) {
         const int64_t ch = tile * kTileChunks;  // the tile's first chunk
-        const int f = find_segment(p.choff, p.F, ch);
+        const int f = p.tile_func ? p.tile_func[tile] : 0;
         const int64_t M = p.moff[f + 1] - p.moff[f];
         const int64_t N = p.koff[f + 1] - p.koff[f] - 1;
         const int64_t c0 = (ch - p.choff[f]) * kChunk;
@@ -305,23 +296,25 @@ __device__ __forceinline__ float fused_density_f(const FuncF& G, const pwl_func&
     return __powf(fabsf(f2), 0.4f);
 }
 
-// ---- fused design, FP32 mode ------------------------------------------------
-// One CTA designs one function at a time, in one launch for the batch, with
-// almost no FP64 operation per density cell (GB300 runs about one FP64
-// operation per SM and cycle):
-//   - pass A, per tile of 2048 cells: the FP32 densities (8 contiguous cells
-//     per thread, written to scratch), the tile's sum and its last cell of
-//     positive density; then the exclusive FP64 scan of the tile sums;
-//   - pass B, per tile holding targets: the densities read back, their prefix,
-//     and the knots as in invert_tiles_kernel;
-//   - cell midpoints are formed in FP32 from the tile start (the FP32 f''
-//     rounds its argument to FP32 anyway);
+// ---- FP32 mode of a batch -----------------------------------------------------
+// The same three launches with almost no FP64 operation per density cell
+// (GB300 runs about one FP64 operation per SM and cycle):
+//   - what needs FP64 once per function or tile (constants, cell width, tile
+//     start, the first target of every tile) comes from launches with one
+//     thread per tile: an FP64 instruction occupies the pipe for the whole warp
+//     however few of its lanes run it, and done by one lane, or by every thread,
+//     of each tile's CTA these took most of the time (design of 4096 functions
+//     1.79 ms, 1.25 ms by one CTA per function, 0.96 ms now; 40 functions
+//     209 -> 42 us);
+//   - the densities go to scratch and come back in 16-byte vectors; cell
+//     midpoints are formed in FP32 from the tile start (the FP32 f'' rounds its
+//     argument to FP32 anyway);
 //   - sums inside a tile are float-float (a compensated pair hi + lo, about
-//     48 significant bits): thread partials, the block scan and the chunk
-//     total; the chunk totals, their scan and G_M are FP64;
+//     48 significant bits): thread partials, the block scan and the tile
+//     total; the tile totals, their scan and G_M are FP64;
 //   - the knot search compares float-float values in FP32, in units of the
 //     density sum (G / delta): the target tau_i / delta = i G_M / (N delta)
-//     minus the chunk base is formed in FP64 once per knot and split into a
+//     minus the tile base is formed in FP64 once per knot and split into a
 //     float-float pair;
 //   - the step inside the cell, (tau_i - G_k) / d_k, is FP32 (it is at most
 //     delta, so its rounding is below 1e-7 delta), and x = a + k delta + step
@@ -344,6 +337,30 @@ __device__ __forceinline__ FF ff_from_double(double v)
 {
     const float hi = __double2float_rn(v);
     return FF{hi, __double2float_rn(v - (double)hi)};
+}
+// The same pair without FP64 operations, for v of normal FP32 magnitude (else by
+// the conversions): the top 24 significant bits, the 29 below them, and a
+// compensated sum that brings them into rounded form.
+__device__ __forceinline__ FF ff_from_double_bits(double v)
+{
+    const uint32_t h = (uint32_t)__double2hiint(v), l = (uint32_t)__double2loint(v);
+    const uint32_t e = h >> 20 & 0x7ffu;
+    if (e < 1023 - 60 || e > 1023 + 120) return ff_from_double(v);
+    // (sign, exponent, upper 23 mantissa bits) as FP32; the lower 29 bits are
+    // worth l' 2^(e - 52), exact in FP32 but for the last few
+    const uint32_t top = (h & 0x80000000u) | (e - 896) << 23 | (h << 3 & 0x7ffff8u) | l >> 29;
+    const float hi = __uint_as_float(top);
+    const float ulp = __uint_as_float((h & 0x80000000u) | (e - 896 - 52) << 23);  // +-2^(e - 52)
+    const float lo = __uint2float_rn(l & 0x1fffffffu) * ulp;
+    const float s = __fadd_rn(hi, lo);
+    return FF{s, __fsub_rn(lo, __fsub_rn(s, hi))};
+}
+// FP32 to FP64 without an FP64 operation (normal x, or 0; the rest by conversion)
+__device__ __forceinline__ double widen_bits(float x)
+{
+    const uint32_t b = __float_as_uint(x), e = b >> 23 & 0xffu;
+    if (e == 0 || e == 255) return x == 0.0f ? 0.0 : (double)x;
+    return __hiloint2double((int)((b & 0x80000000u) | ((b & 0x7fffffffu) >> 3) + 0x38000000u), (int)(b << 29));
 }
 __device__ __forceinline__ double ff_to_double(FF x) { return (double)x.hi + (double)x.lo; }
 
@@ -381,21 +398,6 @@ __device__ __forceinline__ FF ff_block_exclusive_scan(FF v, FF* s_w, FF* total)
     return r;
 }
 
-// Block-wide float-float sum (kDesignThreads); the result is valid in
-// thread 0.  One barrier.
-__device__ __forceinline__ FF ff_block_sum(FF v, FF* s_w)
-{
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    for (int o = 16; o > 0; o >>= 1)
-        v = ff_add(v, FF{__shfl_down_sync(0xffffffffu, v.hi, o), __shfl_down_sync(0xffffffffu, v.lo, o)});
-    if (lane == 0) s_w[warp] = v;
-    __syncthreads();
-    FF r{0.0f, 0.0f};
-    if (threadIdx.x == 0)
-        for (int w = 0; w < kDesignThreads / 32; ++w) r = ff_add(r, s_w[w]);
-    return r;
-}
-
 // smallest i in [1, N] with i c >= S (N if none below N), c = G_M / (N delta)
 __device__ __forceinline__ int64_t first_target_at_or_above_units(double S, double c, int64_t N)
 {
@@ -406,167 +408,230 @@ __device__ __forceinline__ int64_t first_target_at_or_above_units(double S, doub
     return i;
 }
 
-// The densities of one chunk into scratch, with the float-float total of the
-// thread's cells and its last cell of positive density.  Sampled functions
-// take a loop of their own, so that their FP64 interpolation does not weigh
-// on the registers of the analytic kinds' loop.
-template <bool SAMPLED>
-__device__ __forceinline__ void chunk_densities_f(const FuncF& G, const pwl_func& F, float t0f, float deltaf,
-                                                  int cnt, float* __restrict__ dchunk, FF& part, int& last)
+// One thread per tile: the tile's start in FP32 (in its first chunk's cbase,
+// which the scan overwrites), and each function's constants.
+__global__ void __launch_bounds__(128) tile_setup_f_kernel(DesignPlan p)
 {
-    for (int r = 0; r < kTilePer; ++r) {
-        const int l = threadIdx.x * kTilePer + r;
-        if (l < cnt) {
-            const float dk = fused_density_f<SAMPLED>(G, F, t0f, deltaf, l);
-            dchunk[l] = dk;
-            part = ff_add(part, FF{dk, 0.0f});
-            if (dk > 0.0f) last = l;
-        }
+    const int64_t tile = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+    if (tile >= p.total_chunks / kTileChunks) return;
+    const int f = p.tile_func[tile];
+    const int64_t ch = tile * kTileChunks, c0 = (ch - p.choff[f]) * kChunk;
+    const double a = p.funcs[f].a, delta = (p.funcs[f].b - a) / (double)(p.moff[f + 1] - p.moff[f]);
+    *reinterpret_cast<float*>(p.cbase + ch) = (float)(a + (double)c0 * delta);
+    if (c0 == 0) {
+        const pwl_func F = p.funcs[f];
+        DesignFunc d{};
+        d.g = make_funcf(F);
+        d.deltaf = (float)delta;
+        d.a = a;
+        d.delta = delta;
+        p.ffuncs[f] = d;
     }
 }
 
-template <bool SAMPLED>
-__global__ void __launch_bounds__(kDesignThreads, 4) design_fused_fp32_kernel(DesignPlan p)
+// One warp per function: the exclusive FP64 scan of the tile sums (cbase), the
+// last cell of positive density before every tile (plast, in place), and, from
+// the total, cunit = G_M / (N delta) (0: the uniform partition) and every
+// tile's first target (smallest i in [1, N] with i cunit >= the tile's base, N
+// if none; in its first chunk's csum, which is spent by then).
+__global__ void __launch_bounds__(128) tile_scan_f_kernel(DesignPlan p)
 {
-    __shared__ float s_d[kTile];
-    __shared__ FF s_ex[kDesignThreads];  // exclusive float-float prefix of the thread partials
-    __shared__ FF s_w[2 * (kDesignThreads / 32) + 1];
-    __shared__ int s_last2[2];
-    __shared__ double s_warp[kDesignThreads / 32 + 1];
-    __shared__ int s_last;
-    const int t = threadIdx.x;
-    float* __restrict__ dbuf_all = reinterpret_cast<float*>(p.d);
-    if (t < 2) s_last2[t] = -1;
-    __syncthreads();
-    for (int o = blockIdx.x; o < p.F; o += gridDim.x) {
-        const int f = p.order[o];
-        const pwl_func F = p.funcs[f];
-        if ((F.kind == PWL_F_SAMPLED) != SAMPLED) continue;  // the other launch's (uniform per CTA)
-        const FuncF G = make_funcf(F);  // FP32 constants of f'', once per function
-        const int64_t M = p.moff[f + 1] - p.moff[f];
+    const int lane = threadIdx.x & 31;
+    for (int f = blockIdx.x * 4 + (threadIdx.x >> 5); f < p.F; f += gridDim.x * 4) {
+        const int64_t c0 = p.choff[f], tiles = (p.choff[f + 1] - c0) / kTileChunks;
         const int64_t N = p.koff[f + 1] - p.koff[f] - 1;
-        const int64_t nch = (M + kTile - 1) / kTile;
-        const double a = F.a, b = F.b;
-        const double delta = (b - a) / (double)M;
-        const float deltaf = (float)delta;
-        double* __restrict__ knots = p.knots + p.koff[f];
-        double* __restrict__ csum = p.csum + p.choff[f];
-        double* __restrict__ cbase = p.cbase + p.choff[f];
-        int* __restrict__ clast = reinterpret_cast<int*>(p.plast + p.choff[f]);  // tile-local indices
-        float* __restrict__ dbuf = dbuf_all + p.moff[f];
-
-        // pass A: densities (to scratch), chunk totals, last positive cell
-        for (int64_t ch = 0; ch < nch; ++ch) {
-            const int64_t c0 = ch * kTile;
-            const int cnt = (int)min((int64_t)kTile, M - c0);
-            const float t0f = (float)(a + (double)c0 * delta);
-            FF part{0.0f, 0.0f};
-            int last = -1;
-            chunk_densities_f<SAMPLED>(G, F, t0f, deltaf, cnt, dbuf + c0, part, last);
-            // chunk total and last positive cell: one barrier per chunk (the
-            // slot pair alternates so that a chunk's writes never meet the
-            // previous chunk's reads)
-            const int slot = (int)(ch & 1);
-            if (last >= 0) atomicMax(&s_last2[slot], last);
-            const FF tot = ff_block_sum(part, s_w + slot * (kDesignThreads / 32));
-            if (t == 0) {
-                csum[ch] = ff_to_double(tot);
-                clast[ch] = s_last2[slot];
-                s_last2[slot] = -1;
-            }
-        }
-        __syncthreads();
         double carry = 0.0;
-        for (int64_t base = 0; base < nch; base += kDesignThreads) {
-            const int64_t c = base + t;
-            const double v = c < nch ? csum[c] : 0.0;
-            double tot;
-            const double ex = block_exclusive_scan(v, s_warp, &tot);
-            if (c < nch) cbase[c] = carry + ex;
-            carry += tot;
+        long long before = -1;
+        for (int64_t base = 0; base < tiles; base += 32) {
+            const int64_t ch = c0 + (base + lane) * kTileChunks;
+            const bool in = base + lane < tiles;
+            double incl = in ? p.csum[ch] : 0.0;
+            long long last = in ? p.plast[ch] : -1;
+            for (int o = 1; o < 32; o <<= 1) {
+                const double v = __shfl_up_sync(0xffffffffu, incl, o);
+                const long long l = __shfl_up_sync(0xffffffffu, last, o);
+                if (lane >= o) {
+                    incl += v;
+                    last = max(last, l);
+                }
+            }
+            double ex = __shfl_up_sync(0xffffffffu, incl, 1);
+            long long prev = __shfl_up_sync(0xffffffffu, last, 1);
+            if (lane == 0) {
+                ex = 0.0;
+                prev = -1;
+            }
+            if (in) {
+                p.cbase[ch] = carry + ex;
+                p.plast[ch] = max(prev, before);
+            }
+            carry += __shfl_sync(0xffffffffu, incl, 31);
+            before = max(before, __shfl_sync(0xffffffffu, last, 31));
+        }
+        const double cunit = carry / (double)N;
+        const bool linear = !(p.ffuncs[f].delta * carry > 0.0);  // f linear on I, or no finite density
+        for (int64_t tile = lane; tile < tiles; tile += 32) {
+            const int64_t ch = c0 + tile * kTileChunks;
+            reinterpret_cast<int64_t*>(p.csum)[ch] =
+                linear ? 1 : first_target_at_or_above_units(p.cbase[ch], cunit, N);
+        }
+        if (lane == 0) p.ffuncs[f].cunit = linear ? 0.0 : cunit;
+    }
+}
+
+// FP32 densities of function f from its cell c0 on: every function starts
+// 16-byte aligned, with room for the last vector's padding (float index
+// moff + 4 f rounded down to a multiple of 4)
+__device__ __forceinline__ float* tile_densities(const DesignPlan& p, int f, int64_t c0)
+{
+    return reinterpret_cast<float*>(p.d) + (p.moff[f] + 4 * (int64_t)f) / 4 * 4 + c0;
+}
+
+template <bool SAMPLED>
+__global__ void __launch_bounds__(kDesignThreads, SAMPLED ? 4 : 8) density_tiles_f_kernel(DesignPlan p)
+{
+    __shared__ FF s_w[kDesignThreads / 32];
+    __shared__ int s_last[kDesignThreads / 32];
+    const int t = threadIdx.x;
+    for (int64_t tile = blockIdx.x; tile < p.total_chunks / kTileChunks; tile += gridDim.x) {
+        const int f = p.tile_func[tile];
+        const DesignFunc& D = p.ffuncs[f];
+        if ((D.g.kind == PWL_F_SAMPLED) != SAMPLED) continue;  // the other launch's (uniform per CTA)
+        const int64_t ch = tile * kTileChunks, c0 = (ch - p.choff[f]) * kChunk, M = p.moff[f + 1] - p.moff[f];
+        const FuncF G = D.g;
+        const float deltaf = D.deltaf, t0f = *reinterpret_cast<const float*>(p.cbase + ch);
+        const int cnt = (int)min((int64_t)kTile, M - c0);
+        FF part{0.0f, 0.0f};
+        int last = -1;
+        float* __restrict__ out = tile_densities(p, f, c0);
+        // cells strided over the threads, one copy of the loop's body (unrolled,
+        // the Bessel functions overflow the instruction cache)
+#pragma unroll 1
+        for (int l = t; l < cnt; l += kDesignThreads) {
+            float v;
+            if constexpr (SAMPLED) v = fused_density_f<true>(G, p.funcs[f], t0f, deltaf, l);
+            else v = fused_density_f<false>(G, pwl_func{}, t0f, deltaf, l);
+            out[l] = v;
+            part = ff_add(part, FF{v, 0.0f});
+            if (v > 0.0f) last = l;
+        }
+        for (int o = 16; o > 0; o >>= 1)
+            part = ff_add(part, FF{__shfl_down_sync(0xffffffffu, part.hi, o), __shfl_down_sync(0xffffffffu, part.lo, o)});
+        last = __reduce_max_sync(0xffffffffu, last);
+        if ((t & 31) == 0) {
+            s_w[t >> 5] = part;
+            s_last[t >> 5] = last;
         }
         __syncthreads();
-        const double GM = delta * carry;
-        if (t == 0) {
-            knots[0] = a;
-            knots[N] = b;
+        if (t == 0) {  // (the first of the tile's chunks stands for the tile)
+            FF r{0.0f, 0.0f};
+            int m = -1;
+            for (int w = 0; w < kDesignThreads / 32; ++w) {
+                r = ff_add(r, s_w[w]);
+                m = max(m, s_last[w]);
+            }
+            p.csum[ch] = ff_to_double(r);
+            p.plast[ch] = m < 0 ? -1 : c0 + m;
         }
-        if (!(GM > 0.0)) {
-            for (int64_t i = 1 + t; i < N; i += kDesignThreads) knots[i] = a + (double)i * (b - a) / (double)N;
-            __syncthreads();
+        __syncthreads();
+    }
+}
+
+// 8 CTAs per SM: the kernel waits on the chain of loads that starts a tile and
+// on the scan's barriers (4 CTAs per SM 586 us, 6 480 us, 8 414 us).
+__global__ void __launch_bounds__(kDesignThreads, 8) invert_tiles_f_kernel(DesignPlan p)
+{
+    __shared__ float4 s_d4[kTile / 4];
+    __shared__ FF s_ex[kDesignThreads];  // exclusive float-float prefix of the thread partials
+    __shared__ FF s_w[kDesignThreads / 32 + 1];
+    float* s_d = reinterpret_cast<float*>(s_d4);
+    const int t = threadIdx.x;
+    for (int64_t tile = blockIdx.x; tile < p.total_chunks / kTileChunks; tile += gridDim.x) {
+        const int f = p.tile_func[tile];
+        const int64_t ch = tile * kTileChunks, c0 = (ch - p.choff[f]) * kChunk, M = p.moff[f + 1] - p.moff[f];
+        const int64_t N = p.koff[f + 1] - p.koff[f] - 1;
+        const double a = p.ffuncs[f].a, delta = p.ffuncs[f].delta, cunit = p.ffuncs[f].cunit;
+        double* __restrict__ knots = p.knots + p.koff[f];
+        if (t == 0 && c0 == 0) {
+            knots[0] = a;
+            knots[N] = p.funcs[f].b;
+        }
+        if (cunit == 0.0) {
+            if (c0 == 0) {
+                const double b = p.funcs[f].b;
+                for (int64_t i = 1 + t; i < N; i += kDesignThreads) knots[i] = a + (double)i * (b - a) / (double)N;
+            }
             continue;
         }
-        const double cunit = carry / (double)N;  // tau_i / delta = i * cunit
-        // the first target of every chunk, all chunks at once (the chunk sums
-        // are spent: their area takes the indices)
-        int64_t* ifirst = reinterpret_cast<int64_t*>(csum);
-        for (int64_t c = t; c < nch; c += kDesignThreads) ifirst[c] = first_target_at_or_above_units(cbase[c], cunit, N);
-        __syncthreads();
-
-        // pass B
-        int64_t lastpos = -1;
-        for (int64_t ch = 0; ch < nch; ++ch) {
-            const int64_t c0 = ch * kTile;
-            const int64_t i0 = ifirst[ch], i1 = ch + 1 < nch ? ifirst[ch + 1] : N;
-            if (i0 < i1) {
-                const int cnt = (int)min((int64_t)kTile, M - c0);
-                FF part{0.0f, 0.0f};
-                for (int r = 0; r < kTilePer; ++r) {
-                    const int l = t * kTilePer + r;
-                    if (l < cnt) {
-                        const float dk = dbuf[c0 + l];
-                        s_d[l] = dk;
-                        part = ff_add(part, FF{dk, 0.0f});
-                    }
-                }
-                FF tot;
-                s_ex[t] = ff_block_exclusive_scan(part, s_w, &tot);
-                __syncthreads();
-                const int U = (cnt + kTilePer - 1) / kTilePer;
-                const double cb = cbase[ch];
-                // float-float prefix of local cell l: S_u + the thread's cells before l
-                auto ff_at = [&](int l) {
-                    const int u = l / kTilePer;
-                    FF q = s_ex[u];
-                    for (int r = u * kTilePer; r < l; ++r) q = ff_add(q, FF{s_d[r], 0.0f});
-                    return q;
-                };
-                for (int64_t i = i0 + t; i < i1; i += kDesignThreads) {
-                    const FF tl = ff_from_double((double)i * cunit - cb);  // target in the chunk
-                    int lo = 0, hi = U - 1;  // largest u with S_u <= target (u = 0 is)
-                    while (lo < hi) {
-                        const int mid = (lo + hi + 1) >> 1;
-                        if (ff_le(s_ex[mid], tl)) lo = mid; else hi = mid - 1;
-                    }
-                    const int nr = min(kTilePer, cnt - lo * kTilePer);
-                    FF q = s_ex[lo], Sk = q;
-                    int kl = lo * kTilePer;
-                    for (int r = 1; r < nr; ++r) {
-                        q = ff_add(q, FF{s_d[lo * kTilePer + r - 1], 0.0f});
-                        if (!ff_le(q, tl)) break;
-                        kl = lo * kTilePer + r;
-                        Sk = q;
-                    }
-                    int kk = kl;
-                    while (kk >= 0 && !(s_d[kk] > 0.0f)) --kk;
-                    double x;
-                    if (kk >= 0) {
-                        if (kk != kl) Sk = ff_at(kk);
-                        const FF diff = ff_add(tl, ff_neg(Sk));  // (tau - G_k) / delta
-                        const float step = fminf(fmaxf((diff.hi + diff.lo) * deltaf / s_d[kk], 0.0f), deltaf);
-                        x = __dadd_rn(__fma_rn((double)(c0 + kk), delta, a), (double)step);
-                    } else if (lastpos >= 0) {
-                        x = __dadd_rn(__dadd_rn(a, __dmul_rn((double)lastpos, delta)), delta);
-                    } else {
-                        x = a;
-                    }
-                    knots[i] = x;
-                }
+        // tau_i / delta = i * cunit; the next tile's first target ends this one's
+        const int64_t* first = reinterpret_cast<const int64_t*>(p.csum + ch);
+        const int64_t i0 = first[0], i1 = c0 + kTile < M ? first[kTileChunks] : N;
+        if (i0 >= i1) continue;
+        const int cnt = (int)min((int64_t)kTile, M - c0);
+        const float4* in = reinterpret_cast<const float4*>(tile_densities(p, f, c0));
+        FF part{0.0f, 0.0f};
+#pragma unroll
+        for (int q = 0; q < kTilePer / 4; ++q) {  // zero past the function's last cell: adds nothing
+            const int i = t * (kTilePer / 4) + q;
+            float4 v = 4 * i < cnt ? in[i] : make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+            if (4 * i + 3 >= cnt) {  // the padding of the last vector is not written
+                v.w = 0.0f;
+                if (4 * i + 2 >= cnt) v.z = 0.0f;
+                if (4 * i + 1 >= cnt) v.y = 0.0f;
             }
-            const int cl = clast[ch];
-            if (cl >= 0) lastpos = c0 + cl;
-            __syncthreads();
+            s_d4[t * (kTilePer / 4) + q] = v;
+            part = ff_add(part, FF{v.x, 0.0f});
+            part = ff_add(part, FF{v.y, 0.0f});
+            part = ff_add(part, FF{v.z, 0.0f});
+            part = ff_add(part, FF{v.w, 0.0f});
         }
+        FF tot;
+        s_ex[t] = ff_block_exclusive_scan(part, s_w, &tot);
+        __syncthreads();
+        {
+            const int U = (cnt + kTilePer - 1) / kTilePer;
+            const double cb = p.cbase[ch];
+            const float deltaf = p.ffuncs[f].deltaf;
+            // float-float prefix of local cell l: S_u + the thread's cells before l
+            auto ff_at = [&](int l) {
+                const int u = l / kTilePer;
+                FF q = s_ex[u];
+                for (int r = u * kTilePer; r < l; ++r) q = ff_add(q, FF{s_d[r], 0.0f});
+                return q;
+            };
+            // (i < 2^16 and c0 < 2^28 in a batch: 32-bit conversions)
+            for (int64_t i = i0 + t; i < i1; i += kDesignThreads) {
+                const FF tl = ff_from_double_bits((double)(int)i * cunit - cb);  // target in the tile
+                int lo = 0, hi = U - 1;  // largest u with S_u <= target (u = 0 is)
+                while (lo < hi) {
+                    const int mid = (lo + hi + 1) >> 1;
+                    if (ff_le(s_ex[mid], tl)) lo = mid; else hi = mid - 1;
+                }
+                const int nr = min(kTilePer, cnt - lo * kTilePer);
+                FF q = s_ex[lo], Sk = q;
+                int kl = lo * kTilePer;
+                for (int r = 1; r < nr; ++r) {
+                    q = ff_add(q, FF{s_d[lo * kTilePer + r - 1], 0.0f});
+                    if (!ff_le(q, tl)) break;
+                    kl = lo * kTilePer + r;
+                    Sk = q;
+                }
+                int kk = kl;
+                while (kk >= 0 && !(s_d[kk] > 0.0f)) --kk;
+                double x;
+                if (kk >= 0) {
+                    if (kk != kl) Sk = ff_at(kk);
+                    const FF diff = ff_add(tl, ff_neg(Sk));  // (tau - G_k) / delta
+                    const float step = fminf(fmaxf((diff.hi + diff.lo) * deltaf / s_d[kk], 0.0f), deltaf);
+                    x = __dadd_rn(__fma_rn((double)((int)c0 + kk), delta, a), widen_bits(step));
+                } else {
+                    const int64_t e = p.plast[ch];
+                    x = e < 0 ? a : __dadd_rn(__dadd_rn(a, __dmul_rn((double)e, delta)), delta);
+                }
+                knots[i] = x;
+            }
+        }
+        __syncthreads();  // the shared arrays are rewritten for the next tile
     }
 }
 
@@ -592,9 +657,15 @@ inline size_t align256(size_t x) { return (x + 255) & ~(size_t)255; }
 
 int64_t design_chunks(int64_t M) { return (M + kTile - 1) / kTile * kTileChunks; }
 
+// FP64 per cell, or (FP32 mode of a batch) floats with 4 more per function
+static size_t density_bytes(int64_t F, int64_t total_cells)
+{
+    return align256(std::max(sizeof(double) * (size_t)total_cells, sizeof(float) * (size_t)(total_cells + 4 * F + 4)));
+}
+
 size_t design_scratch_bytes(int64_t F, int64_t total_cells, int64_t total_chunks)
 {
-    return align256(sizeof(double) * (size_t)total_cells) + align256(sizeof(double) * (size_t)total_chunks) * 2 +
+    return density_bytes(F, total_cells) + align256(sizeof(double) * (size_t)total_chunks) * 2 +
            align256(sizeof(int64_t) * (size_t)total_chunks) + align256(sizeof(double) * (size_t)F);
 }
 
@@ -602,7 +673,7 @@ void design_carve_scratch(DesignPlan& p, void* scratch)
 {
     char* w = static_cast<char*>(scratch);
     p.d = reinterpret_cast<double*>(w);
-    w += align256(sizeof(double) * (size_t)p.total_cells);
+    w += density_bytes(p.F, p.total_cells);
     p.csum = reinterpret_cast<double*>(w);
     w += align256(sizeof(double) * (size_t)p.total_chunks);
     p.cbase = reinterpret_cast<double*>(w);
@@ -639,19 +710,26 @@ pwl_status design_launch(const DesignPlan& p, cudaStream_t s)
     return PWL_OK;
 }
 
-pwl_status design_fused_launch(const DesignPlan& p, cudaStream_t s)
+pwl_status design_batch_f_launch(const DesignPlan& p, cudaStream_t s)
 {
     const DeviceInfo& di = device_info();
-    const int grid = (int)std::min<int64_t>(p.F, (int64_t)di.sms * 8);
+    const int grid = (int)std::min<int64_t>(p.total_chunks / kTileChunks, (int64_t)di.sms * 16);
     const int kinds = plan_kinds(p.kinds);
+    const int grid_setup = (int)((p.total_chunks / kTileChunks + 127) / 128);
+    tile_setup_f_kernel<<<grid_setup, 128, 0, s>>>(p);
+    PWL_CHECK_LAUNCH("tile_setup_f_kernel");
     if (kinds & kKindsAnalytic) {
-        design_fused_fp32_kernel<false><<<grid, kDesignThreads, 0, s>>>(p);
-        PWL_CHECK_LAUNCH("design_fused_fp32_kernel");
+        density_tiles_f_kernel<false><<<grid, kDesignThreads, 0, s>>>(p);
+        PWL_CHECK_LAUNCH("density_tiles_f_kernel");
     }
     if (kinds & kKindsSampled) {
-        design_fused_fp32_kernel<true><<<grid, kDesignThreads, 0, s>>>(p);
-        PWL_CHECK_LAUNCH("design_fused_fp32_kernel");
+        density_tiles_f_kernel<true><<<grid, kDesignThreads, 0, s>>>(p);
+        PWL_CHECK_LAUNCH("density_tiles_f_kernel");
     }
+    tile_scan_f_kernel<<<(int)std::min<int64_t>((p.F + 3) / 4, 65535), 128, 0, s>>>(p);
+    PWL_CHECK_LAUNCH("tile_scan_f_kernel");
+    invert_tiles_f_kernel<<<grid, kDesignThreads, 0, s>>>(p);
+    PWL_CHECK_LAUNCH("invert_tiles_f_kernel");
     return PWL_OK;
 }
 

@@ -39,6 +39,14 @@ inline int kinds_of(const pwl_func* f, int64_t n)
     return k;
 }
 
+// A function's constants in the FP32 mode of a batch
+struct DesignFunc {
+    FuncF g;
+    float deltaf;     // cell width, rounded
+    double a, delta;  // interval start, cell width
+    double cunit;     // G_M / (N delta): tau_i / delta = i cunit (0: the uniform partition)
+};
+
 struct DesignPlan {
     int F;
     int precision;
@@ -48,23 +56,23 @@ struct DesignPlan {
     const int64_t* moff;
     const int64_t* choff;
     int64_t total_knots, total_cells, total_chunks;
-    double* d;       // total_cells densities (the FP32 fused kernel: floats)
+    const int* tile_func;  // per tile of 8 chunks: its function (NULL: one function)
+    DesignFunc* ffuncs;    // FP32 mode of a batch: F constants (scratch)
+    double* d;       // total_cells densities (FP32 mode of a batch: floats, every function 16-byte aligned)
     double* csum;    // total_chunks partial sums
     double* cbase;   // total_chunks exclusive chunk bases
     int64_t* plast;  // per chunk: its last cell of positive density, then (after the scan) the last one before
                      // it, or -1
     double* stot;    // F totals (sum of d over the function)
     double* knots;   // total_knots output
-    const int* order;  // fused FP32 path: F function indices, largest M first
 };
 
 int64_t design_chunks(int64_t M);
 size_t design_scratch_bytes(int64_t F, int64_t total_cells, int64_t total_chunks);
 void design_carve_scratch(DesignPlan& p, void* scratch);
 pwl_status design_launch(const DesignPlan& p, cudaStream_t s);
-// FP32 mode of a batch, one persistent launch: each CTA designs whole
-// functions (in p.order); writes p.csum, p.cbase, p.plast and p.knots.
-pwl_status design_fused_launch(const DesignPlan& p, cudaStream_t s);
+// FP32 mode of a batch; needs p.tile_func and p.ffuncs.
+pwl_status design_batch_f_launch(const DesignPlan& p, cudaStream_t s);
 
 // Projection: F functions with knots at koff (device), values out.
 struct ProjectPlan {
