@@ -536,6 +536,7 @@ struct pwl_batch_s {
     int* status;                // device word: bit 2 = an evaluation wait timed out
     int* order;                 // functions by decreasing intervals (the Gram solves' order)
     int* tile_func;             // per design tile: its function
+    FuncValueF* funcs_f;        // the functions' FP32 parameters
     DesignFunc* ffuncs;         // FP32 design: constants per function (scratch)
     // evaluation plan
     std::vector<int64_t> qoff;  // query offsets of the plan
@@ -718,6 +719,12 @@ pwl_status pwl_batch_create(const pwl_func* funcs, const int64_t* n_intervals, i
     std::vector<int> tile_func((size_t)(choff[n_funcs] / design_chunks(1)));
     for (int64_t f = 0; f < n_funcs; ++f)
         std::fill(tile_func.begin() + choff[f] / design_chunks(1), tile_func.begin() + choff[f + 1] / design_chunks(1), (int)f);
+    std::vector<FuncValueF> funcs_f((size_t)n_funcs);
+    std::vector<pwl_func> funcs_d((size_t)n_funcs);
+    for (int64_t f = 0; f < n_funcs; ++f) {
+        funcs_f[(size_t)f] = func_value_params(funcs[f]);
+        funcs_d[(size_t)f] = prepared(funcs[f]);
+    }
     b->total_knots = b->koff[n_funcs];
     b->total_cells_design = moff[n_funcs];
     b->total_chunks = choff[n_funcs];
@@ -741,12 +748,13 @@ pwl_status pwl_batch_create(const pwl_func* funcs, const int64_t* n_intervals, i
                             align256(sizeof(int)),
                             align256(sizeof(int) * F),
                             align256(sizeof(int) * tile_func.size()),
-                            align256(sizeof(DesignFunc) * F)};
+                            align256(sizeof(DesignFunc) * F),
+                            align256(sizeof(FuncValueF) * F)};
     void** slots[] = {(void**)&b->funcs, (void**)&b->d_koff, (void**)&b->d_moff, (void**)&b->d_choff,
                       (void**)&b->knots, (void**)&b->values, &b->design_scratch, &b->project_scratch,
                       (void**)&b->bf, (void**)&b->xk, (void**)&b->vk, (void**)&b->slope, (void**)&b->cj,
                       (void**)&b->recP, (void**)&b->recS, (void**)&b->status, (void**)&b->order,
-                      (void**)&b->tile_func, (void**)&b->ffuncs};
+                      (void**)&b->tile_func, (void**)&b->ffuncs, (void**)&b->funcs_f};
     static_assert(sizeof(sizes) / sizeof(sizes[0]) == sizeof(slots) / sizeof(slots[0]), "one size per slot");
     size_t total = 0;
     for (size_t s : sizes) total += s;
@@ -760,13 +768,14 @@ pwl_status pwl_batch_create(const pwl_func* funcs, const int64_t* n_intervals, i
         *slots[i] = p;
         p += sizes[i];
     }
-    if ((e = cudaMemcpy(b->funcs, funcs, sizeof(pwl_func) * F, cudaMemcpyHostToDevice)) != cudaSuccess ||
+    if ((e = cudaMemcpy(b->funcs, funcs_d.data(), sizeof(pwl_func) * F, cudaMemcpyHostToDevice)) != cudaSuccess ||
         (e = cudaMemcpy(b->d_koff, b->koff.data(), 8 * (F + 1), cudaMemcpyHostToDevice)) != cudaSuccess ||
         (e = cudaMemcpy(b->d_moff, moff.data(), 8 * (F + 1), cudaMemcpyHostToDevice)) != cudaSuccess ||
         (e = cudaMemcpy(b->d_choff, choff.data(), 8 * (F + 1), cudaMemcpyHostToDevice)) != cudaSuccess ||
         (e = cudaMemcpy(b->bf, bfh.data(), sizeof(BatchFunc) * F, cudaMemcpyHostToDevice)) != cudaSuccess ||
         (e = cudaMemset(b->status, 0, sizeof(int))) != cudaSuccess ||
         (e = cudaMemcpy(b->order, order.data(), sizeof(int) * F, cudaMemcpyHostToDevice)) != cudaSuccess ||
+        (e = cudaMemcpy(b->funcs_f, funcs_f.data(), sizeof(FuncValueF) * F, cudaMemcpyHostToDevice)) != cudaSuccess ||
         (e = cudaMemcpy(b->tile_func, tile_func.data(), sizeof(int) * tile_func.size(), cudaMemcpyHostToDevice)) != cudaSuccess) {
         batch_free(b);
         return cuda_fail(e, "batch upload");
@@ -825,6 +834,7 @@ pwl_status pwl_batch_project(pwl_batch b, int32_t form, int32_t quad_points, int
     p.total_knots = b->total_knots;
     p.total_intervals = b->total_knots - b->F;
     p.funcs = b->funcs;
+    p.funcs_f = b->funcs_f;
     p.koff = b->d_koff;
     p.knots = b->knots;
     p.values = b->values;

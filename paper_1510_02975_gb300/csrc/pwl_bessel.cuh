@@ -8,8 +8,10 @@
 // alpha >= 3 on [0, 50].  There the modulus-phase form (DLMF 10.17)
 //     J_nu(x) = sqrt(2 / (pi x)) (P_nu(x) cos chi - Q_nu(x) sin chi),
 //     chi = x - (2 nu + 1) pi / 4,
-// is evaluated with Chebyshev series of P_nu and (x/8) Q_nu in
-// w = 2 (8/x)^2 - 1 (pwl_bessel_tables.cuh, from gen_bessel_pq.py), and with
+// is evaluated with polynomials of P_nu and (x/8) Q_nu in u = (8/x)^2
+// (pwl_bessel_tables.cuh, from gen_bessel_pq.py; one FP64 operation per term,
+// where Clenshaw's sum of the same polynomial takes two: the FP64 pipe bounds
+// every user of these functions), and with
 //     cos chi0 = (cos x + sin x) / sqrt 2,   sin chi0 = (sin x - cos x) / sqrt 2,
 //     cos chi1 = (sin x - cos x) / sqrt 2,   sin chi1 = -(sin x + cos x) / sqrt 2:
 // absolute error ~3e-16.
@@ -21,27 +23,23 @@
 
 namespace pwl {
 
-// Clenshaw sum of c_0 T_0(w) + ... + c_{N-1} T_{N-1}(w)
-template <typename T, int N>
-__device__ __forceinline__ T chebyshev_sum(const T* c, T w)
+// c_0 + c_1 u + ... + c_{N-1} u^{N-1}
+template <int N>
+__device__ __forceinline__ double polynomial(const double* c, double u)
 {
-    T b1 = T(0), b2 = T(0);
+    double r = c[N - 1];
 #pragma unroll
-    for (int j = N - 1; j >= 1; --j) {
-        const T b0 = T(2) * w * b1 - b2 + c[j];
-        b2 = b1;
-        b1 = b0;
-    }
-    return w * b1 - b2 + c[0];
+    for (int j = N - 2; j >= 0; --j) r = fma(r, u, c[j]);
+    return r;
 }
 
 __device__ __forceinline__ double bessel_j0(double x)
 {
     const double ax = fabs(x);
     if (ax < 8.0) return j0(x);
-    const double t = 8.0 / ax, w = 2.0 * t * t - 1.0;
-    const double p = chebyshev_sum<double, 16>(kBesselP0, w);
-    const double q = t * chebyshev_sum<double, 16>(kBesselQ0, w);
+    const double t = 8.0 / ax, u = t * t;
+    const double p = polynomial<16>(kBesselP0, u);
+    const double q = t * polynomial<16>(kBesselQ0, u);
     double s, c;
     sincos(ax, &s, &c);
     return (p * (c + s) - q * (s - c)) * rsqrt(3.14159265358979323846 * ax);
@@ -51,9 +49,9 @@ __device__ __forceinline__ double bessel_j1(double x)
 {
     const double ax = fabs(x);
     if (ax < 8.0) return j1(x);
-    const double t = 8.0 / ax, w = 2.0 * t * t - 1.0;
-    const double p = chebyshev_sum<double, 16>(kBesselP1, w);
-    const double q = t * chebyshev_sum<double, 16>(kBesselQ1, w);
+    const double t = 8.0 / ax, u = t * t;
+    const double p = polynomial<16>(kBesselP1, u);
+    const double q = t * polynomial<16>(kBesselQ1, u);
     double s, c;
     sincos(ax, &s, &c);
     const double r = (p * (s - c) + q * (s + c)) * rsqrt(3.14159265358979323846 * ax);
@@ -65,27 +63,33 @@ __device__ __forceinline__ double bessel_j1(double x)
 __device__ __forceinline__ float bessel_j0(float x) { return j0f(x); }
 __device__ __forceinline__ float bessel_j1(float x) { return j1f(x); }
 
-// J0 and J1 at the same point (f'' needs both): one sincos and one square
-// root for the two.
-__device__ __forceinline__ void bessel_j01(double x, double& j0v, double& j1v)
+// J0(x) and J1(x)/x (f'' needs both; 1/2 - x^2/16 near 0): one sincos and one
+// square root for the two, and 1/x = t/8.
+__device__ __forceinline__ void bessel_j0_j1x(double x, double& j0v, double& j1x)
 {
     const double ax = fabs(x);
     if (ax < 8.0) {
         j0v = j0(x);
-        j1v = j1(x);
+        j1x = ax < 1e-8 ? 0.5 - x * x / 16.0 : j1(x) / x;
         return;
     }
-    const double t = 8.0 / ax, w = 2.0 * t * t - 1.0;
-    const double p0 = chebyshev_sum<double, 16>(kBesselP0, w), q0 = t * chebyshev_sum<double, 16>(kBesselQ0, w);
-    const double p1 = chebyshev_sum<double, 16>(kBesselP1, w), q1 = t * chebyshev_sum<double, 16>(kBesselQ1, w);
+    const double t = 8.0 / ax, u = t * t;
+    const double p0 = polynomial<16>(kBesselP0, u), q0 = t * polynomial<16>(kBesselQ0, u);
+    const double p1 = polynomial<16>(kBesselP1, u), q1 = t * polynomial<16>(kBesselQ1, u);
     double s, c;
     sincos(ax, &s, &c);
     const double r = rsqrt(3.14159265358979323846 * ax);
     j0v = (p0 * (c + s) - q0 * (s - c)) * r;
-    const double j1a = (p1 * (s - c) + q1 * (s + c)) * r;
-    j1v = x < 0.0 ? -j1a : j1a;
+    j1x = (p1 * (s - c) + q1 * (s + c)) * r * (0.125 * t);
 }
 
+__device__ __forceinline__ void bessel_j0_j1x(float x, float& j0v, float& j1x)
+{
+    j0v = j0f(x);
+    j1x = fabsf(x) < 1e-8f ? 0.5f - x * x / 16.0f : j1f(x) / x;
+}
+
+// J0 and J1 at the same point, FP32
 __device__ __forceinline__ void bessel_j01(float x, float& j0v, float& j1v)
 {
     j0v = j0f(x);

@@ -159,6 +159,30 @@ __device__ __forceinline__ double sampled_second_derivative(const pwl_func& F, d
     return dj + c.t * (dk - dj);
 }
 
+// Descriptors as the kernels get them: a Gaussian or Lorentzian carries 1/s and
+// 1/s^2 in p[6], p[7] (unused by these kinds; 0 where they are not normal
+// numbers), formed once on the host.
+inline pwl_func prepared(const pwl_func& f)
+{
+    pwl_func g = f;
+    if (f.kind == PWL_F_GAUSSIAN || f.kind == PWL_F_LORENTZIAN) {
+        const double s = f.p[2], r = 1.0 / s, r2 = 1.0 / (s * s);
+        const bool ok = isfinite(r) && isfinite(r2) && fabs(r) > 1e-290 && r2 > 1e-290 && fabs(s) < 1e145;
+        g.p[6] = ok ? r : 0.0;
+        g.p[7] = ok ? r2 : 0.0;
+    }
+    return g;
+}
+// a / s from r = 1/s rounded: the product and one correction by its remainder,
+// three FP64 operations (a division's rounding, for about ten)
+__device__ __forceinline__ double ratio(double a, double s, double r)
+{
+    if (__double2hiint(r) == 0) return a / s;
+    const double q = a * r;
+    return fma(fma(-q, s, a), r, q);
+}
+__device__ __forceinline__ float ratio(float a, float s, double) { return a / s; }
+
 // f(x) for the analytic kinds of pwl_kind.
 template <typename T>
 __device__ __forceinline__ T func_value_analytic(const pwl_func& F, T x)
@@ -166,11 +190,11 @@ __device__ __forceinline__ T func_value_analytic(const pwl_func& F, T x)
     using M = FMath<T>;
     switch (F.kind) {
     case PWL_F_GAUSSIAN: {
-        T u = (x - (T)F.p[1]) / (T)F.p[2];
+        T u = ratio(x - (T)F.p[1], (T)F.p[2], F.p[6]);
         return (T)F.p[0] * M::ex(T(-0.5) * u * u);
     }
     case PWL_F_LORENTZIAN: {
-        T u = (x - (T)F.p[1]) / (T)F.p[2];
+        T u = ratio(x - (T)F.p[1], (T)F.p[2], F.p[6]);
         return (T)F.p[0] / (T(1) + u * u);
     }
     case PWL_F_BESSEL_J0:
@@ -196,21 +220,20 @@ __device__ __forceinline__ T func_second_derivative_analytic(const pwl_func& F, 
     switch (F.kind) {
     case PWL_F_GAUSSIAN: {
         T s = (T)F.p[2];
-        T u = (x - (T)F.p[1]) / s;
-        return (T)F.p[0] * (u * u - T(1)) / (s * s) * M::ex(T(-0.5) * u * u);
+        T u = ratio(x - (T)F.p[1], s, F.p[6]);
+        return ratio((T)F.p[0] * (u * u - T(1)), s * s, F.p[7]) * M::ex(T(-0.5) * u * u);
     }
     case PWL_F_LORENTZIAN: {
         T g = (T)F.p[2];
-        T u = (x - (T)F.p[1]) / g;
+        T u = ratio(x - (T)F.p[1], g, F.p[6]);
         T q = T(1) + u * u;
         return (T)F.p[0] * (T(6) * u * u - T(2)) / (g * g * q * q * q);
     }
     case PWL_F_BESSEL_J0: {
         T al = (T)F.p[1];
         T z = al * x;
-        T b0, b1;
-        bessel_j01(z, b0, b1);
-        T r = (fabs(z) < T(1e-8)) ? T(0.5) - z * z / T(16) : b1 / z;
+        T b0, r;
+        bessel_j0_j1x(z, b0, r);
         return (T)F.p[0] * al * al * (r - b0);
     }
     case PWL_F_POLY: {
@@ -249,6 +272,63 @@ template <typename T>
 __device__ __forceinline__ T func_second_derivative(const pwl_func& F, T x)
 {
     return F.kind == PWL_F_SAMPLED ? func_second_derivative_k<true, T>(F, x) : func_second_derivative_k<false, T>(F, x);
+}
+
+// FP32 evaluation of f (the FP32 mode of P_T) from parameters rounded to FP32
+// on the host: the arithmetic of func_value_analytic<float>, without its
+// conversions on the FP64 pipe.
+struct FuncValueF {
+    int kind;
+    float p[8];
+};
+inline FuncValueF func_value_params(const pwl_func& F)
+{
+    FuncValueF g;
+    g.kind = F.kind;
+    for (int k = 0; k < 8; ++k) g.p[k] = (float)F.p[k];
+    return g;
+}
+__device__ __forceinline__ float func_value_f(const FuncValueF& F, float x)
+{
+    switch (F.kind) {
+    case PWL_F_GAUSSIAN: {
+        const float u = (x - F.p[1]) / F.p[2];
+        return F.p[0] * expf(-0.5f * u * u);
+    }
+    case PWL_F_LORENTZIAN: {
+        const float u = (x - F.p[1]) / F.p[2];
+        return F.p[0] / (1.0f + u * u);
+    }
+    case PWL_F_BESSEL_J0:
+        return F.p[0] * bessel_j0(F.p[1] * x);
+    case PWL_F_POLY: {
+        float s = 0.0f;
+        for (int k = 7; k >= 0; --k) s = s * x + F.p[k];
+        return s;
+    }
+    case PWL_F_EXP:
+        return F.p[0] * expf(F.p[1] * x);
+    }
+    return 0.0f;
+}
+
+// FP64 <-> FP32 without the FP64 pipe (normal FP32 magnitudes and zero by bit
+// arithmetic, the rest by conversion): narrowing rounds to nearest even.
+__device__ __forceinline__ float narrow_bits(double v)
+{
+    const uint32_t h = (uint32_t)__double2hiint(v), l = (uint32_t)__double2loint(v);
+    const uint32_t e = h >> 20 & 0x7ffu;
+    if (e < 897 || e > 1149) return (h << 1 | l) == 0 ? 0.0f : __double2float_rn(v);
+    const uint32_t m = (e - 896) << 23 | (h << 3 & 0x7ffff8u) | l >> 29;
+    const uint32_t rest = l << 3;  // the 29 bits below, at the top
+    const uint32_t up = rest > 0x80000000u || (rest == 0x80000000u && (m & 1u)) ? 1u : 0u;
+    return __uint_as_float((h & 0x80000000u) | (m + up));
+}
+__device__ __forceinline__ double widen_bits(float x)
+{
+    const uint32_t b = __float_as_uint(x), e = b >> 23 & 0xffu;
+    if (e == 0 || e == 255) return x == 0.0f ? 0.0 : (double)x;
+    return __hiloint2double((int)((b & 0x80000000u) | (((b & 0x7fffffffu) >> 3) + 0x38000000u)), (int)(b << 29));
 }
 
 // FP32 evaluation of f'' (the FP32 design mode) from constants converted

@@ -355,13 +355,6 @@ __device__ __forceinline__ FF ff_from_double_bits(double v)
     const float s = __fadd_rn(hi, lo);
     return FF{s, __fsub_rn(lo, __fsub_rn(s, hi))};
 }
-// FP32 to FP64 without an FP64 operation (normal x, or 0; the rest by conversion)
-__device__ __forceinline__ double widen_bits(float x)
-{
-    const uint32_t b = __float_as_uint(x), e = b >> 23 & 0xffu;
-    if (e == 0 || e == 255) return x == 0.0f ? 0.0 : (double)x;
-    return __hiloint2double((int)((b & 0x80000000u) | ((b & 0x7fffffffu) >> 3) + 0x38000000u), (int)(b << 29));
-}
 __device__ __forceinline__ double ff_to_double(FF x) { return (double)x.hi + (double)x.lo; }
 
 // Block-wide exclusive scan of one float-float per thread (kDesignThreads);
@@ -789,7 +782,7 @@ pwl_status pwl_design(const pwl_func* f, int64_t n_intervals, int64_t m_cells, i
     p.knots = d_knots;
     design_carve_scratch(p, w + kMetaBytes);
     cudaStream_t s = as_stream(stream);
-    single_setup_kernel<<<1, 1, 0, s>>>(*f, n_intervals, M, p.total_chunks, const_cast<pwl_func*>(p.funcs),
+    single_setup_kernel<<<1, 1, 0, s>>>(prepared(*f), n_intervals, M, p.total_chunks, const_cast<pwl_func*>(p.funcs),
                                         const_cast<int64_t*>(p.koff), const_cast<int64_t*>(p.moff),
                                         const_cast<int64_t*>(p.choff));
     PWL_CHECK_LAUNCH("single_setup_kernel");

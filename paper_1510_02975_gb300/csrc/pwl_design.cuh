@@ -8,19 +8,17 @@ namespace pwl {
 
 constexpr int kMaxIntervals = 1048575;
 
-// 1/d for a positive normal FP64 d by Newton's method for the reciprocal,
-// r <- r + r (1 - d r), from the hardware's approximate reciprocal
-// (rcp.approx.ftz.f64); each step doubles the correct bits, two reach FP64
-// rounding.  Five FP64 operations against about twice that for a division
-// (the Gram solves and the table build's slopes and reciprocal lengths).
+// 1/d for a positive normal FP64 d from the hardware's approximate reciprocal
+// (rcp.approx.ftz.f64, relative error e below 2^-19.9) by one step of third
+// order, r (1 + e + e^2) with e = 1 - d r: what remains, e^3, is below FP64
+// rounding.  Three FP64 operations against about ten for a division (the Gram
+// solves and the table build's slopes and reciprocal lengths).
 __device__ __forceinline__ double recip_newton(double d)
 {
     double r;
     asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(r) : "d"(d));
-    double e = fma(-d, r, 1.0);
-    r = fma(r, e, r);
-    e = fma(-d, r, 1.0);
-    return fma(r, e, r);
+    const double e = fma(-d, r, 1.0);
+    return fma(r, fma(e, e, e), r);
 }
 
 // F functions; function f owns knots koff[f] .. koff[f+1]-1 (N_f + 1 of them),
@@ -84,11 +82,12 @@ struct ProjectPlan {
     int64_t total_knots;
     int64_t total_intervals;
     const pwl_func* funcs;
+    const FuncValueF* funcs_f;  // the functions' FP32 parameters (FP32 mode of P_T)
     const int64_t* koff;
     const double* knots;
     double* values;
     double2* lr;           // per interval: (int f phi_left, int f phi_right)
-    double* cr;            // 4 * total_knots doubles of solver scratch (used when rows do not fit smem)
+    double* cr;            // solver scratch: 4 doubles per knot and 128 per function
     int solver;            // 0: cyclic reduction, one CTA per function; 1: partitioned Thomas, one warp per function
     const int* order;      // solver 1: the order in which warps take the functions (NULL: 0..F-1)
 };

@@ -92,9 +92,9 @@ pwl_status pwl_error_constants(const pwl_func* f, int64_t m_cells, double* d_out
     PWL_CUDA_TRY(cudaMemsetAsync(d_out, 0, 2 * sizeof(double), s));
     const int64_t blocks = std::min<int64_t>((M + kConstThreads - 1) / kConstThreads, (int64_t)device_info().sms * 8);
     if (f->kind == PWL_F_SAMPLED)
-        error_constants_kernel<true><<<(int)blocks, kConstThreads, 0, s>>>(*f, M, d_out);
+        error_constants_kernel<true><<<(int)blocks, kConstThreads, 0, s>>>(prepared(*f), M, d_out);
     else
-        error_constants_kernel<false><<<(int)blocks, kConstThreads, 0, s>>>(*f, M, d_out);
+        error_constants_kernel<false><<<(int)blocks, kConstThreads, 0, s>>>(prepared(*f), M, d_out);
     PWL_CHECK_LAUNCH("error_constants_kernel");
     return PWL_OK;
 }

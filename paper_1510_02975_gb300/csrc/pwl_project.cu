@@ -46,6 +46,10 @@ __device__ __forceinline__ int find_knot_owner(const int64_t* __restrict__ koff,
     return lo;
 }
 
+// Start of function f's solver scratch: 4 doubles per row and 32 rows of padding
+// per function (the planes of gram_spike_kernel hold whole rows of 32 lanes)
+__device__ __forceinline__ int64_t solver_scratch(int64_t k0, int f) { return 4 * (k0 + 32 * (int64_t)f); }
+
 template <typename T, bool SAMPLED>
 __global__ void interp_values_kernel(ProjectPlan p)
 {
@@ -65,18 +69,94 @@ __global__ void interp_values_kernel(ProjectPlan p)
 // division per node.  FP64 mode: t_q and the sums in FP64.  FP32 mode: t_q
 // and f(t_q) in FP32 (the argument of an FP32 f is rounded to FP32 anyway),
 // the sums in FP64.
-// sum_q wl_q f(t_q) and sum_q wr_q f(t_q) over one interval (the half-length
-// factor applied by the caller); the sampled path is a template flag,
-// chosen once per interval
-template <typename T, bool SAMPLED>
-__device__ __forceinline__ void hat_sums(const pwl_func& F, const GaussLegendre& gl, double mid, double half,
-                                         double& L, double& R)
+//
+// The function of global interval g: a search for the CTA's first interval,
+// which all lanes make on the same addresses, then on from there (functions
+// are longer than a CTA's 128 intervals, or it steps through a few).
+__device__ __forceinline__ int interval_owner(const ProjectPlan& p, int64_t g)
 {
-    if constexpr (sizeof(T) == 4) {
-        // sums of w f(t) as float-float pairs: each product exact (the
-        // weight split hi + lo, the rounding error of hi f recovered by an
-        // FMA), each addition compensated; FP64 once per interval
-        const float midf = (float)mid, halff = (float)half;
+    int f = p.F > 1 ? find_interval_owner(p.koff, p.F, g - threadIdx.x) : 0;
+    while (f + 1 < p.F && __ldg(p.koff + f + 1) - (f + 1) <= g) ++f;
+    return f;
+}
+
+// FP64: one thread per interval.  Bound by the FP64 pipe for thousands of
+// intervals; see hat_nodes_kernel for few.
+template <bool SAMPLED>
+__global__ void hat_integrals_kernel(ProjectPlan p, const __grid_constant__ GaussLegendre gl)
+{
+    const int64_t stride = (int64_t)gridDim.x * blockDim.x;
+    for (int64_t g = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; g < p.total_intervals;
+         g += stride) {
+        const int f = interval_owner(p, g);
+        const int64_t j = g - (p.koff[f] - f) + 1;  // interval index 1..N_f
+        const double* x = p.knots + p.koff[f];
+        const double xl = x[j - 1], xr = x[j];
+        const double mid = 0.5 * (xl + xr), half = 0.5 * (xr - xl);
+        const pwl_func F = p.funcs[f];
+        if ((F.kind == PWL_F_SAMPLED) != SAMPLED) continue;  // the other launch's
+        double L = 0.0, R = 0.0;
+        for (int q = 0; q < gl.Q; ++q) {
+            const double fv = func_value_k<SAMPLED, double>(F, __fma_rn(half, gl.x[q], mid));
+            L = __fma_rn(gl.wl[q], fv, L);
+            R = __fma_rn(gl.wr[q], fv, R);
+        }
+        p.lr[g] = make_double2(half * L, half * R);
+    }
+}
+
+// FP64, few intervals: 16 lanes per interval, one node each, so that a single
+// table still spreads over the chip (J0, 1023 intervals: 38 us with one thread
+// per interval, on 8 CTAs, 6.3 us so).
+template <bool SAMPLED>
+__global__ void __launch_bounds__(128) hat_nodes_kernel(ProjectPlan p, const __grid_constant__ GaussLegendre gl)
+{
+    const int q = threadIdx.x % 16;
+    const int64_t stride = (int64_t)gridDim.x * (blockDim.x / 16);
+    for (int64_t g = blockIdx.x * (int64_t)(blockDim.x / 16) + threadIdx.x / 16; g < p.total_intervals; g += stride) {
+        const int f = p.F > 1 ? find_interval_owner(p.koff, p.F, g) : 0;
+        const int64_t j = g - (p.koff[f] - f) + 1;
+        const double* x = p.knots + p.koff[f];
+        const double xl = x[j - 1], xr = x[j];
+        const double mid = 0.5 * (xl + xr), half = 0.5 * (xr - xl);
+        const pwl_func F = p.funcs[f];
+        if ((F.kind == PWL_F_SAMPLED) != SAMPLED) continue;  // the other launch's (the same for the 16 lanes)
+        double L = 0.0, R = 0.0;
+        if (q < gl.Q) {
+            const double fv = func_value_k<SAMPLED, double>(F, __fma_rn(half, gl.x[q], mid));
+            L = gl.wl[q] * fv;
+            R = gl.wr[q] * fv;
+        }
+        const unsigned lanes = 0xffffu << (threadIdx.x & 16);
+        for (int o = 8; o > 0; o >>= 1) {
+            L += __shfl_xor_sync(lanes, L, o);
+            R += __shfl_xor_sync(lanes, R, o);
+        }
+        if (q == 0) p.lr[g] = make_double2(half * L, half * R);
+    }
+}
+
+// FP32 mode: nodes and f in FP32, the sums of w f(t) as float-float pairs: each
+// product exact (the weight split hi + lo, the rounding error of hi f
+// recovered by an FMA), each addition compensated.  The FP64 pipe (one
+// instruction takes it for 16 clocks or more per warp) was 78% busy with
+// conversions, of the function's parameters above all: those are FP32 in
+// memory now and the rest go by bit arithmetic, which leaves eight FP64
+// operations per interval (4096 functions, 8.4 M intervals: 388 -> 312 us).
+template <bool SAMPLED>
+__global__ void __launch_bounds__(128) hat_integrals_f_kernel(ProjectPlan p, const __grid_constant__ GaussLegendre gl)
+{
+    const int64_t stride = (int64_t)gridDim.x * blockDim.x;
+    for (int64_t g = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; g < p.total_intervals;
+         g += stride) {
+        const int f = interval_owner(p, g);
+        const FuncValueF& G = p.funcs_f[f];
+        if ((G.kind == PWL_F_SAMPLED) != SAMPLED) continue;  // the other launch's
+        const int64_t j = g - (p.koff[f] - f) + 1;  // interval index 1..N_f
+        const double* x = p.knots + p.koff[f];
+        const double xl = x[j - 1], xr = x[j];
+        const double half = 0.5 * (xr - xl);
+        const float midf = narrow_bits(0.5 * (xl + xr)), halff = narrow_bits(half);
         float Lh = 0.0f, Ll = 0.0f, Rh = 0.0f, Rl = 0.0f;
         auto acc = [](float& h, float& l, float wh, float wlo, float fv) {
             const float p = __fmul_rn(wh, fv);
@@ -87,40 +167,16 @@ __device__ __forceinline__ void hat_sums(const pwl_func& F, const GaussLegendre&
             h = s;
             l = __fadd_rn(l, __fadd_rn(e, pe));
         };
+#pragma unroll 1
         for (int q = 0; q < gl.Q; ++q) {
-            const float fv = func_value_k<SAMPLED, float>(F, __fmaf_rn(halff, gl.xf[q], midf));
+            const float t = __fmaf_rn(halff, gl.xf[q], midf);
+            float fv;
+            if constexpr (SAMPLED) fv = (float)sampled_value(p.funcs[f], (double)t);
+            else fv = func_value_f(G, t);
             acc(Lh, Ll, gl.wlh[q], gl.wll[q], fv);
             acc(Rh, Rl, gl.wrh[q], gl.wrl[q], fv);
         }
-        L = (double)Lh + (double)Ll;
-        R = (double)Rh + (double)Rl;
-    } else {
-        L = 0.0;
-        R = 0.0;
-        for (int q = 0; q < gl.Q; ++q) {
-            const double fv = func_value_k<SAMPLED, double>(F, __fma_rn(half, gl.x[q], mid));
-            L = __fma_rn(gl.wl[q], fv, L);
-            R = __fma_rn(gl.wr[q], fv, R);
-        }
-    }
-}
-
-template <typename T, bool SAMPLED>
-__global__ void hat_integrals_kernel(ProjectPlan p, const __grid_constant__ GaussLegendre gl)
-{
-    const int64_t stride = (int64_t)gridDim.x * blockDim.x;
-    for (int64_t g = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; g < p.total_intervals;
-         g += stride) {
-        const int f = find_interval_owner(p.koff, p.F, g);
-        const int64_t j = g - (p.koff[f] - f) + 1;  // interval index 1..N_f
-        const double* x = p.knots + p.koff[f];
-        const double xl = x[j - 1], xr = x[j];
-        const double mid = 0.5 * (xl + xr), half = 0.5 * (xr - xl);
-        const pwl_func F = p.funcs[f];
-        if ((F.kind == PWL_F_SAMPLED) != SAMPLED) continue;  // the other launch's
-        double L, R;
-        hat_sums<T, SAMPLED>(F, gl, mid, half, L, R);
-        p.lr[g] = make_double2(half * L, half * R);
+        p.lr[g] = make_double2(half * (widen_bits(Lh) + widen_bits(Ll)), half * (widen_bits(Rh) + widen_bits(Rl)));
     }
 }
 
@@ -141,7 +197,17 @@ __global__ void hat_integrals_kernel(ProjectPlan p, const __grid_constant__ Gaus
 //  3. every lane reconstructs its rows.
 // The rows are assembled on the fly (M_{i,i-1} = h_i/6, M_ii = (h_i +
 // h_{i+1})/3, M_{i,i+1} = h_{i+1}/6, b_i = R_i + L_{i+1}).  About 20 FP64
-// operations per row, one division; no barrier beyond the warp.
+// operations per row; no barrier beyond the warp.
+// Blocks of some dozen rows or more are as good as decoupled beyond their
+// neighbours: the spikes fall by 0.27 per row of a uniform partition, and once
+// every w at its block's first row and v at its last is below kSpikeGone, the
+// two unknowns at each boundary follow from two equations per lane, without
+// the recurrence over the lanes (about 25 FP64 operations of the whole warp
+// per block, as many as a row and a half of elimination).
+// The scratch (c', y, v, w per row) is laid out by planes, row-in-block major:
+// the 32 lanes' accesses are consecutive, where rows of 32 bytes at a stride of
+// a block touched a sector each.  4096 functions, 8.4 M rows: 703 -> 477 us.
+constexpr double kSpikeGone = 1e-30;
 
 __global__ void __launch_bounds__(64) gram_spike_kernel(ProjectPlan p, const int* __restrict__ order)
 {
@@ -155,8 +221,12 @@ __global__ void __launch_bounds__(64) gram_spike_kernel(ProjectPlan p, const int
         const int N = n - 1;
         const double* __restrict__ x = p.knots + k0;
         const double2* __restrict__ lr = p.lr + (k0 - f);
-        double* __restrict__ sc = p.cr + 4 * k0;  // per row: c', then y, v, w
         const int P = min(32, max(1, n / 2));
+        const int plane = (n + P - 1) / P * P;
+        double* __restrict__ sc = p.cr + solver_scratch(k0, f) + lane;  // planes c', y, v, w: [row in block][lane]
+        double* __restrict__ sy = sc + plane;
+        double* __restrict__ sv = sy + plane;
+        double* __restrict__ sw = sv + plane;
         double y0 = 0.0, v0 = 0.0, w0 = 0.0, yL = 0.0, vL = 0.0, wL = 0.0;
         const int r0 = (int)((int64_t)lane * n / P), r1 = (int)((int64_t)(lane + 1) * n / P);
         if (lane < P) {
@@ -177,9 +247,10 @@ __global__ void __launch_bounds__(64) gram_spike_kernel(ProjectPlan p, const int
                 const double vv = ((i == r0 ? hl * kSixth : 0.0) - lower * vprev) * r;
                 cprev = i + 1 < r1 ? upper * r : 0.0;
                 if (i + 1 == r1) wlast = upper * r;  // w'_{m-1}: the coupling to the next block
-                sc[4 * i] = cprev;
-                sc[4 * i + 1] = yv;
-                sc[4 * i + 2] = vv;
+                const int at = (i - r0) * P;
+                sc[at] = cprev;
+                sy[at] = yv;
+                sv[at] = vv;
                 yprev = yv;
                 vprev = vv;
                 hl = hr;
@@ -189,13 +260,14 @@ __global__ void __launch_bounds__(64) gram_spike_kernel(ProjectPlan p, const int
             double yn = 0.0, vn = 0.0, wn = 0.0;
 #pragma unroll 4
             for (int i = r1 - 1; i >= r0; --i) {
-                const double c = sc[4 * i];
-                const double yv = sc[4 * i + 1] - c * yn;
-                const double vv = sc[4 * i + 2] - c * vn;
+                const int at = (i - r0) * P;
+                const double c = sc[at];
+                const double yv = sy[at] - c * yn;
+                const double vv = sv[at] - c * vn;
                 const double wv = (i == r1 - 1 ? wlast : 0.0) - c * wn;
-                sc[4 * i + 1] = yv;
-                sc[4 * i + 2] = vv;
-                sc[4 * i + 3] = wv;
+                sy[at] = yv;
+                sv[at] = vv;
+                sw[at] = wv;
                 yn = yv;
                 vn = vv;
                 wn = wv;
@@ -209,49 +281,63 @@ __global__ void __launch_bounds__(64) gram_spike_kernel(ProjectPlan p, const int
             v0 = vn;
             w0 = wn;
         }
-        // boundary unknowns, forward over the blocks in lane order.  Every lane
-        // runs the same recurrence on shuffled (uniform) inputs; lane q keeps
-        // block q's coefficients.  Carried: L_{q-1} = alpha + beta F_q.
-        double alpha = 0.0, beta = 0.0;
-        double gq_own = 0.0, dq_own = 0.0, aq_own = 0.0, bq_own = 0.0;
-        for (int q = 0; q < P; ++q) {
-            const double y0q = __shfl_sync(0xffffffffu, y0, q), v0q = __shfl_sync(0xffffffffu, v0, q);
-            const double w0q = __shfl_sync(0xffffffffu, w0, q), yLq = __shfl_sync(0xffffffffu, yL, q);
-            const double vLq = __shfl_sync(0xffffffffu, vL, q), wLq = __shfl_sync(0xffffffffu, wL, q);
-            // F_q = y0 - v0 L_{q-1} - w0 F_{q+1}  ->  F_q = g + d F_{q+1}
-            const double piv = 1.0 / (1.0 + v0q * beta);
-            const double g = (y0q - v0q * alpha) * piv;
-            const double d = -w0q * piv;
-            // L_q = yL - vL L_{q-1} - wL F_{q+1}  ->  L_q = an + bn F_{q+1}
-            const double an = yLq - vLq * (alpha + beta * g);
-            const double bn = -(vLq * beta * d + wLq);
-            if (lane == q) {
-                gq_own = g;
-                dq_own = d;
-                aq_own = an;
-                bq_own = bn;
+        double Lprev, Fafter;  // the unknowns before and after this lane's block
+        if (__all_sync(0xffffffffu, fabs(w0) < kSpikeGone && fabs(vL) < kSpikeGone)) {
+            // F_p = y0 - v0 L_{p-1} and L_{p-1} = yL_{p-1} - wL_{p-1} F_p
+            const double yb = __shfl_up_sync(0xffffffffu, yL, 1), wb = __shfl_up_sync(0xffffffffu, wL, 1);
+            const double F = lane > 0 ? (y0 - v0 * yb) / (1.0 - v0 * wb) : y0;
+            Lprev = lane > 0 ? yb - wb * F : 0.0;
+            Fafter = __shfl_down_sync(0xffffffffu, F, 1);
+            if (lane >= P - 1) Fafter = 0.0;
+        } else {
+            // forward over the blocks in lane order.  Every lane runs the same
+            // recurrence on shuffled (uniform) inputs; lane q keeps block q's
+            // coefficients.  Carried: L_{q-1} = alpha + beta F_q.
+            double alpha = 0.0, beta = 0.0;
+            double gq_own = 0.0, dq_own = 0.0, aq_own = 0.0, bq_own = 0.0;
+            for (int q = 0; q < P; ++q) {
+                const double y0q = __shfl_sync(0xffffffffu, y0, q), v0q = __shfl_sync(0xffffffffu, v0, q);
+                const double w0q = __shfl_sync(0xffffffffu, w0, q), yLq = __shfl_sync(0xffffffffu, yL, q);
+                const double vLq = __shfl_sync(0xffffffffu, vL, q), wLq = __shfl_sync(0xffffffffu, wL, q);
+                // F_q = y0 - v0 L_{q-1} - w0 F_{q+1}  ->  F_q = g + d F_{q+1}
+                const double piv = 1.0 / (1.0 + v0q * beta);
+                const double g = (y0q - v0q * alpha) * piv;
+                const double d = -w0q * piv;
+                // L_q = yL - vL L_{q-1} - wL F_{q+1}  ->  L_q = an + bn F_{q+1}
+                const double an = yLq - vLq * (alpha + beta * g);
+                const double bn = -(vLq * beta * d + wLq);
+                if (lane == q) {
+                    gq_own = g;
+                    dq_own = d;
+                    aq_own = an;
+                    bq_own = bn;
+                }
+                alpha = an;
+                beta = bn;
             }
-            alpha = an;
-            beta = bn;
-        }
-        // backward from F_P = 0: F_q = g_q + d_q F_{q+1}, L_q = a_q + b_q F_{q+1}
-        double Fnext = 0.0, Fq = 0.0, Lq = 0.0;
-        for (int q = P - 1; q >= 0; --q) {
-            const double gq = __shfl_sync(0xffffffffu, gq_own, q), dq = __shfl_sync(0xffffffffu, dq_own, q);
-            const double aq = __shfl_sync(0xffffffffu, aq_own, q), bq = __shfl_sync(0xffffffffu, bq_own, q);
-            if (lane == q) {
-                Fq = Fnext;  // F_{q+1}, the unknown after this lane's block
-                Lq = aq + bq * Fnext;
+            // backward from F_P = 0: F_q = g_q + d_q F_{q+1}, L_q = a_q + b_q F_{q+1}
+            double Fnext = 0.0, Lq = 0.0;
+            Fafter = 0.0;
+            for (int q = P - 1; q >= 0; --q) {
+                const double gq = __shfl_sync(0xffffffffu, gq_own, q), dq = __shfl_sync(0xffffffffu, dq_own, q);
+                const double aq = __shfl_sync(0xffffffffu, aq_own, q), bq = __shfl_sync(0xffffffffu, bq_own, q);
+                if (lane == q) {
+                    Fafter = Fnext;  // F_{q+1}
+                    Lq = aq + bq * Fnext;
+                }
+                Fnext = gq + dq * Fnext;
             }
-            Fnext = gq + dq * Fnext;
+            // L_{p-1} from the previous lane (0 before the first block)
+            Lprev = __shfl_up_sync(0xffffffffu, Lq, 1);
+            if (lane == 0) Lprev = 0.0;
         }
-        // L_{p-1} from the previous lane (0 before the first block)
-        double Lprev = __shfl_up_sync(0xffffffffu, Lq, 1);
-        if (lane == 0) Lprev = 0.0;
         if (lane < P) {
             double* __restrict__ v = p.values + k0;
 #pragma unroll 4
-            for (int i = r0; i < r1; ++i) v[i] = sc[4 * i + 1] - sc[4 * i + 2] * Lprev - sc[4 * i + 3] * Fq;
+            for (int i = r0; i < r1; ++i) {
+                const int at = (i - r0) * P;
+                v[i] = sy[at] - sv[at] * Lprev - sw[at] * Fafter;
+            }
         }
     }
 }
@@ -275,7 +361,7 @@ __global__ void __launch_bounds__(kSolveThreads) gram_solve_kernel(ProjectPlan p
         const double* x = p.knots + k0;
         const double2* lr = p.lr + (k0 - f);
         double* A;
-        if (use_smem) A = s_cr; else A = p.cr + 4 * k0;
+        if (use_smem) A = s_cr; else A = p.cr + solver_scratch(k0, f);
         double* B = A + n;
         double* C = B + n;
         double* D = C + n;
@@ -326,10 +412,12 @@ __global__ void __launch_bounds__(kSolveThreads) gram_solve_kernel(ProjectPlan p
     }
 }
 
-__global__ void single_project_setup_kernel(pwl_func F, int64_t N, pwl_func* funcs, int64_t* koff)
+__global__ void single_project_setup_kernel(pwl_func F, FuncValueF G, int64_t N, pwl_func* funcs, FuncValueF* funcs_f,
+                                            int64_t* koff)
 {
     if (threadIdx.x == 0 && blockIdx.x == 0) {
         funcs[0] = F;
+        funcs_f[0] = G;
         koff[0] = 0;
         koff[1] = N + 1;
     }
@@ -401,8 +489,9 @@ const GaussLegendre& gauss_legendre_rule(int Q)
 
 size_t project_scratch_bytes(int64_t total_knots, int64_t total_intervals)
 {
+    // (total_knots - total_intervals functions)
     return align256(sizeof(double2) * (size_t)total_intervals) +
-           align256(sizeof(double) * 4 * (size_t)total_knots);
+           align256(sizeof(double) * 4 * (size_t)(total_knots + 32 * (total_knots - total_intervals)));
 }
 
 void project_carve_scratch(ProjectPlan& p, void* scratch)
@@ -435,21 +524,24 @@ pwl_status project_launch(const ProjectPlan& p, const GaussLegendre& gl, cudaStr
         }
         return PWL_OK;
     }
-    const int grid = (int)std::min<int64_t>((p.total_intervals + 127) / 128, (int64_t)di.sms * 16);
+    // 16 lanes per interval while one thread each would leave SMs with few warps;
+    // beyond, their shuffled sums cost more than the spread gives (82,000
+    // intervals: 122 us against 86)
+    const bool nodes = p.precision != PWL_PREC_FP32 && p.total_intervals <= (int64_t)di.sms * 256;
+    const int64_t per_cta = nodes ? 8 : 128;
+    const int grid = (int)std::min<int64_t>((p.total_intervals + per_cta - 1) / per_cta, (int64_t)di.sms * 16);
     const int kinds = plan_kinds(p.kinds);
-    if (kinds & kKindsAnalytic) {
+    for (const bool sampled : {false, true}) {
+        if (!(kinds & (sampled ? kKindsSampled : kKindsAnalytic))) continue;
+        void (*kern)(ProjectPlan, const GaussLegendre);
         if (p.precision == PWL_PREC_FP32)
-            hat_integrals_kernel<float, false><<<grid, 128, 0, s>>>(p, gl);
+            kern = sampled ? hat_integrals_f_kernel<true> : hat_integrals_f_kernel<false>;
+        else if (nodes)
+            kern = sampled ? hat_nodes_kernel<true> : hat_nodes_kernel<false>;
         else
-            hat_integrals_kernel<double, false><<<grid, 128, 0, s>>>(p, gl);
-        PWL_CHECK_LAUNCH("hat_integrals_kernel");
-    }
-    if (kinds & kKindsSampled) {
-        if (p.precision == PWL_PREC_FP32)
-            hat_integrals_kernel<float, true><<<grid, 128, 0, s>>>(p, gl);
-        else
-            hat_integrals_kernel<double, true><<<grid, 128, 0, s>>>(p, gl);
-        PWL_CHECK_LAUNCH("hat_integrals_kernel");
+            kern = sampled ? hat_integrals_kernel<true> : hat_integrals_kernel<false>;
+        kern<<<grid, 128, 0, s>>>(p, gl);
+        PWL_CHECK_LAUNCH("hat integrals kernel");
     }
     if (p.solver == 1) {
         // two warps (functions) per CTA, so that a few hundred functions
@@ -518,12 +610,14 @@ pwl_status pwl_project(const pwl_func* f, const double* d_knots, int64_t n_inter
     p.total_intervals = n_intervals;
     p.funcs = reinterpret_cast<pwl_func*>(w);
     p.koff = reinterpret_cast<int64_t*>(w + 128);
+    p.funcs_f = reinterpret_cast<FuncValueF*>(w + 160);
+    static_assert(sizeof(pwl_func) <= 128 && 160 + sizeof(FuncValueF) <= kProjMeta, "workspace head");
     p.knots = d_knots;
     p.values = d_values;
     project_carve_scratch(p, w + kProjMeta);
     cudaStream_t s = as_stream(stream);
-    single_project_setup_kernel<<<1, 1, 0, s>>>(*f, n_intervals, const_cast<pwl_func*>(p.funcs),
-                                                const_cast<int64_t*>(p.koff));
+    single_project_setup_kernel<<<1, 1, 0, s>>>(prepared(*f), func_value_params(*f), n_intervals, const_cast<pwl_func*>(p.funcs),
+                                                const_cast<FuncValueF*>(p.funcs_f), const_cast<int64_t*>(p.koff));
     PWL_CHECK_LAUNCH("single_project_setup_kernel");
     return project_launch(p, gauss_legendre_rule(quad_points), s);
 }
