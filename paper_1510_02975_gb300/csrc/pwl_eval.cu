@@ -198,6 +198,97 @@ __global__ void __launch_bounds__(1024, MINB) eval_kernel(const EvalArgs args, c
     }
 }
 
+// ---- 16-bit queries by table of all their values ------------------------------
+// A 16-bit query has 65536 values.  On a large stream every CTA first evaluates
+// all of them (the arithmetic of eval_kernel, the index read from global
+// memory: neighbouring patterns are neighbouring points) into 128 KB of shared
+// memory, and a query is then one 2-byte shared load: ~4 instructions instead
+// of ~20, which bound the 16-bit streams at 4 bytes per query.  J0, N = 1024,
+// BF16: 2^27 queries 147 -> 99 us, 2^28 282 -> 180 us (5.98 TB/s).  The table
+// costs each CTA about 10 us (20 for N = 4096), which repays itself from 2^24
+// queries on (25 -> 23 us; 2^23: 17 -> 20), with the Lorentzian's N = 4096 from
+// 2^25 (54 -> 48 us).  Two vectors in flight per thread: 99 us, four: 106.
+constexpr int kLutUnroll = 2;
+constexpr int64_t kLutQueries = (int64_t)1 << 25;
+constexpr size_t kLutBytes = sizeof(uint16_t) << 16;
+
+template <typename IO, class L>
+__device__ __forceinline__ void fill_lut(uint32_t* lut, const L& f)
+{
+    using V = Vec<IO>;
+    constexpr int U = 4;  // vectors of 8 patterns in flight (their global loads overlap)
+    for (int i = threadIdx.x; i < 65536 / 8; i += U * blockDim.x) {
+        uint4 v[U];
+#pragma unroll
+        for (int u = 0; u < U; ++u) {
+            const uint32_t b = 8 * (i + u * blockDim.x);
+            v[u] = make_uint4(b | (b + 1) << 16, (b + 2) | (b + 3) << 16, (b + 4) | (b + 5) << 16, (b + 6) | (b + 7) << 16);
+            v[u] = V::apply(v[u], f);
+        }
+#pragma unroll
+        for (int u = 0; u < U; ++u)
+            if (i + u * blockDim.x < 65536 / 8) reinterpret_cast<uint4*>(lut)[i + u * blockDim.x] = v[u];
+    }
+}
+
+__device__ __forceinline__ uint32_t lut_pair(const uint16_t* lut, uint32_t w)
+{
+    return lut[w & 0xffffu] | (uint32_t)lut[w >> 16] << 16;
+}
+
+template <typename IO, int LAYOUT>
+__global__ void __launch_bounds__(1024, 1) eval_lut_kernel(const EvalArgs args, const IO* x, IO* y, int64_t m)
+{
+    extern __shared__ float4 s_fwd[];
+    uint16_t* lut = reinterpret_cast<uint16_t*>(s_fwd);
+    {
+        uint32_t* lut32 = reinterpret_cast<uint32_t*>(s_fwd);
+        EvalArgs p = args;
+        if (LAYOUT == 1) {
+            const int n_chain = p.hdr->n_chain_b;
+            p.max_chain = p.hdr->max_chain_b;
+            p.n_smem = p.K + n_chain;  // every record from the one (global) array
+            if (n_chain == 0)
+                fill_lut<IO>(lut32, Lerp16<false>{p.rec16, p});
+            else
+                fill_lut<IO>(lut32, Lerp16<true>{p.rec16, p});
+        } else {
+            const int n_chain = p.hdr->n_chain_f;
+            p.max_chain = p.hdr->max_chain_f;
+            p.s_staged = 0;
+            const float2* side = LAYOUT == 2 ? p.recS8 : p.recS;
+            if (n_chain == 0)
+                fill_lut<IO>(lut32, Lerp8<false, false, LAYOUT == 2>{p.recP, side, p});
+            else
+                fill_lut<IO>(lut32, Lerp8<true, false, LAYOUT == 2>{p.recP, side, p});
+        }
+    }
+    __syncthreads();
+    const int64_t nthr = (int64_t)gridDim.x * blockDim.x;
+    const int64_t tid = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    const uint16_t* xs = reinterpret_cast<const uint16_t*>(x);
+    uint16_t* ys = reinterpret_cast<uint16_t*>(y);
+    const uint4* xv = reinterpret_cast<const uint4*>(x + args.head);
+    uint4* yv = reinterpret_cast<uint4*>(y + args.head);
+    constexpr int U = kLutUnroll;
+    int64_t i = tid;
+    for (; i + (U - 1) * nthr < args.nvec; i += U * nthr) {
+        uint4 v[U];
+#pragma unroll
+        for (int u = 0; u < U; ++u) v[u] = ld_stream(xv + i + u * nthr);
+#pragma unroll
+        for (int u = 0; u < U; ++u)
+            st_stream(yv + i + u * nthr, make_uint4(lut_pair(lut, v[u].x), lut_pair(lut, v[u].y), lut_pair(lut, v[u].z),
+                                                    lut_pair(lut, v[u].w)));
+    }
+    for (; i < args.nvec; i += nthr) {
+        const uint4 v = ld_stream(xv + i);
+        st_stream(yv + i, make_uint4(lut_pair(lut, v.x), lut_pair(lut, v.y), lut_pair(lut, v.z), lut_pair(lut, v.w)));
+    }
+    for (int64_t j = tid; j < args.head; j += nthr) ys[j] = lut[xs[j]];
+    for (int64_t j = args.head + args.nvec * 8 + tid; j < m; j += nthr) ys[j] = lut[xs[j]];
+}
+
 // ---- compute ceiling: queries generated in registers (pwl_stream.cuh) ------
 // Algorithm 1 on m generated queries: no query loaded, no result stored;
 // every CTA adds the sum of its results to *sum (FP64).  The staging and the
@@ -456,6 +547,17 @@ pwl_status launch_eval(pwl_table t, int layout, const IO* x, IO* y, int64_t m, c
     stream_split<IO>(x, y, m, &p.head, &p.nvec);
     const DeviceInfo& di = device_info();
     if (smem > di.smem_optin) return fail(PWL_ENOTSUP, "forward index of %zu bytes does not fit one CTA", smem);
+    if constexpr (sizeof(IO) == 2) {
+        if (m >= kLutQueries) {
+            void (*kern)(const EvalArgs, const IO*, IO*, int64_t) =
+                layout == 0 ? eval_lut_kernel<IO, 0> : (layout == 2 ? eval_lut_kernel<IO, 2> : eval_lut_kernel<IO, 1>);
+            int grid = 0;
+            PWL_CUDA_TRY(occupancy_grid(kern, 1024, kLutBytes, &grid));
+            kern<<<grid, 1024, kLutBytes, s>>>(p, x, y, m);
+            PWL_CHECK_LAUNCH("eval_lut_kernel");
+            return PWL_OK;
+        }
+    }
     const bool two = di.smem_per_sm >= 2 * (smem + 1024);
     void (*kern)(const EvalArgs, const IO*, IO*, int64_t);
     if (layout == 0)
