@@ -29,19 +29,37 @@ __all__ = [
 ]
 
 
+_TORCH = None
+
+
 def _torch():
-    import torch
-    return torch
+    global _TORCH
+    if _TORCH is None:
+        import torch
+        _TORCH = torch
+    return _TORCH
+
+
+_RAW_STREAM = None  # (current stream's handle by device, current device) of torch._C, or () without them
 
 
 def _stream(stream=None):
+    """The raw handle of `stream`, or of the current stream of the current device."""
+    global _RAW_STREAM
+    if stream is not None:
+        return stream.cuda_stream
     torch = _torch()
-    s = torch.cuda.current_stream() if stream is None else stream
-    return ctypes.c_void_p(s.cuda_stream)
+    if _RAW_STREAM is None:
+        calls = [getattr(torch._C, n, None) for n in ("_cuda_getCurrentRawStream", "_cuda_getDevice")]
+        _RAW_STREAM = () if None in calls else tuple(calls)
+    if _RAW_STREAM and torch.cuda.is_initialized():
+        # without building a torch.cuda.Stream object, which takes 3 us
+        return _RAW_STREAM[0](_RAW_STREAM[1]())
+    return torch.cuda.current_stream().cuda_stream
 
 
 def _ptr(t):
-    return ctypes.c_void_p(t.data_ptr()) if t is not None else None
+    return t.data_ptr() if t is not None else None
 
 
 def _require(t, dtype, name, numel=None):
@@ -116,28 +134,33 @@ def pwl_table_update(handle, knots, values, stream=None) -> None:
     torch = _torch()
     _require(knots, torch.float64, "knots")
     _require(values, torch.float64, "values", knots.numel())
-    check(load().pwl_table_update(ctypes.c_void_p(handle), _ptr(knots), _ptr(values), _stream(stream)),
+    check(load().pwl_table_update(handle, _ptr(knots), _ptr(values), _stream(stream)),
           "pwl_table_update")
 
 
 def pwl_table_check(handle, stream=None) -> None:
-    check(load().pwl_table_check(ctypes.c_void_p(handle), _stream(stream)), "pwl_table_check")
+    check(load().pwl_table_check(handle, _stream(stream)), "pwl_table_check")
 
 
 def pwl_table_destroy(handle) -> None:
     if handle:
-        check(load().pwl_table_destroy(ctypes.c_void_p(handle)), "pwl_table_destroy")
+        check(load().pwl_table_destroy(handle), "pwl_table_destroy")
 
 
 def pwl_table_get_info(handle) -> dict:
     info = PwlTableInfo()
-    check(load().pwl_table_get_info(ctypes.c_void_p(handle), ctypes.byref(info)), "pwl_table_get_info")
+    check(load().pwl_table_get_info(handle, ctypes.byref(info)), "pwl_table_get_info")
     return {k: getattr(info, k) for k, _ in PwlTableInfo._fields_}
 
 
+_IO_DTYPES = {}
+
+
 def _io_dtype(t):
-    torch = _torch()
-    return {torch.float32: 0, torch.bfloat16: 1, torch.float16: 2}[t.dtype]
+    if not _IO_DTYPES:
+        torch = _torch()
+        _IO_DTYPES.update({torch.float32: 0, torch.bfloat16: 1, torch.float16: 2})
+    return _IO_DTYPES[t.dtype]
 
 
 def pwl_eval(handle, x, y=None, stream=None):
@@ -149,7 +172,7 @@ def pwl_eval(handle, x, y=None, stream=None):
         raise ValueError("x and y must have the same dtype and size")
     if not (x.is_cuda and y.is_cuda and x.is_contiguous() and y.is_contiguous()):
         raise ValueError("x and y must be contiguous CUDA tensors")
-    check(load().pwl_eval(ctypes.c_void_p(handle), _ptr(x), _ptr(y), x.numel(), _io_dtype(x), _stream(stream)),
+    check(load().pwl_eval(handle, _ptr(x), _ptr(y), x.numel(), _io_dtype(x), _stream(stream)),
           "pwl_eval")
     return y
 
@@ -161,7 +184,7 @@ def pwl_eval_variant(handle, mode: int, x, y=None, stream=None):
     if y is None:
         y = torch.empty_like(x)
     _require(y, torch.float32, "y", x.numel())
-    check(load().pwl_eval_variant(ctypes.c_void_p(handle), mode, _ptr(x), _ptr(y), x.numel(), _stream(stream)),
+    check(load().pwl_eval_variant(handle, mode, _ptr(x), _ptr(y), x.numel(), _stream(stream)),
           "pwl_eval_variant")
     return y
 
@@ -173,7 +196,7 @@ def pwl_eval_synthetic(handle, m: int, seed: int = 0, out=None, stream=None):
     if out is None:
         out = torch.zeros(1, dtype=torch.float64, device="cuda")
     _require(out, torch.float64, "out", 1)
-    check(load().pwl_eval_synthetic(ctypes.c_void_p(handle), int(seed) & 0xFFFFFFFF, int(m), _ptr(out),
+    check(load().pwl_eval_synthetic(handle, int(seed) & 0xFFFFFFFF, int(m), _ptr(out),
                                     _stream(stream)), "pwl_eval_synthetic")
     return out
 
@@ -184,7 +207,7 @@ def pwl_eval_synthetic_variant(handle, mode: int, m: int, seed: int = 0, out=Non
     if out is None:
         out = torch.zeros(1, dtype=torch.float64, device="cuda")
     _require(out, torch.float64, "out", 1)
-    check(load().pwl_eval_synthetic_variant(ctypes.c_void_p(handle), int(mode), int(seed) & 0xFFFFFFFF, int(m),
+    check(load().pwl_eval_synthetic_variant(handle, int(mode), int(seed) & 0xFFFFFFFF, int(m),
                                             _ptr(out), _stream(stream)), "pwl_eval_synthetic_variant")
     return out
 
@@ -263,10 +286,10 @@ def pwl_eval_backward(handle, x, gy, gx=None, g_values=None, g_knots=None, works
     for name, t in (("g_values", g_values), ("g_knots", g_knots)):
         if t is not None:
             _require(t, torch.float32, name)
-    need = lib.pwl_eval_backward_workspace_size(ctypes.c_void_p(handle))
+    need = lib.pwl_eval_backward_workspace_size(handle)
     if workspace is None or workspace.numel() < need:
         workspace = _workspace(need, x.device)
-    check(lib.pwl_eval_backward(ctypes.c_void_p(handle), _ptr(x), _ptr(gy), _ptr(gx), _ptr(g_values),
+    check(lib.pwl_eval_backward(handle, _ptr(x), _ptr(gy), _ptr(gx), _ptr(g_values),
                                 _ptr(g_knots), x.numel(), _ptr(workspace), workspace.numel(), _stream(stream)),
           "pwl_eval_backward")
     return gx
@@ -282,7 +305,7 @@ def pwl_eval_backward_noalloc(handle, x, gy, gx=None, g_values=None, g_knots=Non
     if gx is None:
         gx = torch.empty_like(x)
     _require(gx, torch.float32, "gx", x.numel())
-    check(load().pwl_eval_backward_noalloc(ctypes.c_void_p(handle), _ptr(x), _ptr(gy), _ptr(gx), _ptr(g_values),
+    check(load().pwl_eval_backward_noalloc(handle, _ptr(x), _ptr(gy), _ptr(gx), _ptr(g_values),
                                            _ptr(g_knots), x.numel(), _stream(stream)), "pwl_eval_backward_noalloc")
     return gx
 
@@ -304,44 +327,45 @@ def pwl_batch_create(funcs, n_intervals, m_per_interval: int = 0, cells_per_knot
 
 def pwl_batch_destroy(handle) -> None:
     if handle:
-        check(load().pwl_batch_destroy(ctypes.c_void_p(handle)), "pwl_batch_destroy")
+        check(load().pwl_batch_destroy(handle), "pwl_batch_destroy")
 
 
 def pwl_batch_design(handle, precision: str = "fp64", stream=None) -> None:
-    check(load().pwl_batch_design(ctypes.c_void_p(handle), PRECISIONS[precision], _stream(stream)),
+    check(load().pwl_batch_design(handle, PRECISIONS[precision], _stream(stream)),
           "pwl_batch_design")
 
 
 def pwl_batch_project(handle, form: str = "project", quad_points: int = 8, precision: str = "fp64",
                       stream=None) -> None:
-    check(load().pwl_batch_project(ctypes.c_void_p(handle), FORMS[form], quad_points, PRECISIONS[precision],
+    check(load().pwl_batch_project(handle, FORMS[form], quad_points, PRECISIONS[precision],
                                    _stream(stream)), "pwl_batch_project")
 
 
 def pwl_batch_build(handle, stream=None) -> None:
-    check(load().pwl_batch_build(ctypes.c_void_p(handle), _stream(stream)), "pwl_batch_build")
+    check(load().pwl_batch_build(handle, _stream(stream)), "pwl_batch_build")
 
 
 def pwl_batch_check(handle, stream=None) -> None:
-    check(load().pwl_batch_check(ctypes.c_void_p(handle), _stream(stream)), "pwl_batch_check")
+    check(load().pwl_batch_check(handle, _stream(stream)), "pwl_batch_check")
 
 
 def pwl_batch_plan(handle, query_offsets, shape: int = -1, stage_min: int = -1) -> None:
     """query_offsets: F+1 non-decreasing ints (host sequence), first 0."""
     qo = (ctypes.c_int64 * len(query_offsets))(*[int(q) for q in query_offsets])
-    check(load().pwl_batch_plan(ctypes.c_void_p(handle), qo, shape, stage_min), "pwl_batch_plan")
+    check(load().pwl_batch_plan(handle, qo, shape, stage_min), "pwl_batch_plan")
 
 
 def pwl_batch_eval(handle, x, y=None, stream=None):
     torch = _torch()
     _require(x, torch.float32, "x")
-    planned = pwl_batch_get_info(handle)["total_queries"]
-    if x.numel() < planned:
-        raise ValueError(f"x has {x.numel()} elements; the plan has {planned} queries")
+    info = PwlBatchInfo()
+    check(load().pwl_batch_get_info(handle, ctypes.byref(info)), "pwl_batch_get_info")
+    if x.numel() < info.total_queries:
+        raise ValueError(f"x has {x.numel()} elements; the plan has {info.total_queries} queries")
     if y is None:
         y = torch.empty_like(x)
     _require(y, torch.float32, "y", x.numel())
-    check(load().pwl_batch_eval(ctypes.c_void_p(handle), _ptr(x), _ptr(y), _stream(stream)), "pwl_batch_eval")
+    check(load().pwl_batch_eval(handle, _ptr(x), _ptr(y), _stream(stream)), "pwl_batch_eval")
     return y
 
 
@@ -355,7 +379,7 @@ def pwl_batch_autotune(handle, x, y, reps: int = 3, stream=None) -> dict:
         raise ValueError(f"x has {x.numel()} elements; the plan has {planned} queries")
     _require(y, torch.float32, "y", x.numel())
     t = (ctypes.c_float * 20)()
-    check(load().pwl_batch_autotune(ctypes.c_void_p(handle), _ptr(x), _ptr(y), reps, t, _stream(stream)),
+    check(load().pwl_batch_autotune(handle, _ptr(x), _ptr(y), reps, t, _stream(stream)),
           "pwl_batch_autotune")
     return {(shape, stage_min): float(t[4 * shape + j])
             for shape in range(5) for j, stage_min in enumerate((0, 4, 16, 64))}
@@ -370,13 +394,13 @@ def pwl_test_fail_allocations(succeed_first: int) -> None:
 def pwl_batch_inject_wait_timeout(handle, withhold: bool, wait_limit_ns: int = 0) -> None:
     """Failure injection: the asynchronous batch shape's staging waits run out
     after wait_limit_ns (withhold=True); withhold=False restores them."""
-    check(load().pwl_batch_inject_wait_timeout(ctypes.c_void_p(handle), int(bool(withhold)), int(wait_limit_ns)),
+    check(load().pwl_batch_inject_wait_timeout(handle, int(bool(withhold)), int(wait_limit_ns)),
           "pwl_batch_inject_wait_timeout")
 
 
 def pwl_batch_get_info(handle) -> dict:
     info = PwlBatchInfo()
-    check(load().pwl_batch_get_info(ctypes.c_void_p(handle), ctypes.byref(info)), "pwl_batch_get_info")
+    check(load().pwl_batch_get_info(handle, ctypes.byref(info)), "pwl_batch_get_info")
     return {k: getattr(info, k) for k, _ in PwlBatchInfo._fields_}
 
 

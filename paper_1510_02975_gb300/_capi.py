@@ -110,6 +110,8 @@ def library_path() -> str:
 def load():
     """Load libpwl.so and declare its signatures.  Raises if it is missing."""
     global _lib
+    if _lib is not None:
+        return _lib
     with _lock:
         if _lib is not None:
             return _lib

@@ -56,6 +56,92 @@ cudaError_t dev_malloc(void** p, size_t bytes)
     return cudaMalloc(p, bytes);
 }
 
+// Blocks of destroyed tables, kept for the next build: cudaMalloc and cudaFree
+// take ~30 us each, and a table has two blocks (120 us of the 430 from f to a
+// table and its first evaluation).  A block is kept only once the device has
+// finished everything that might still use it (cudaFree waits the same way),
+// so any stream may write to it afterwards.  At most kCacheBlocks blocks of
+// kCacheBlock bytes at most per device; they go back to the device when an
+// allocation fails.
+namespace {
+constexpr size_t kCacheBlock = (size_t)1 << 20;
+constexpr size_t kCacheBlocks = 16;
+struct CachedBlock {
+    int device;
+    size_t bytes;
+    void* p;
+};
+std::mutex g_cache_mu;
+std::vector<CachedBlock> g_cache;
+
+size_t block_bytes(size_t bytes)
+{
+    size_t b = 4096;
+    while (b < bytes) b *= 2;
+    return bytes <= kCacheBlock ? b : bytes;
+}
+
+// the current device's cached blocks back to the device
+void release_cache(int dev)
+{
+    std::vector<void*> blocks;
+    {
+        std::lock_guard<std::mutex> lk(g_cache_mu);
+        for (size_t i = 0; i < g_cache.size();) {
+            if (g_cache[i].device == dev) {
+                blocks.push_back(g_cache[i].p);
+                g_cache.erase(g_cache.begin() + (ptrdiff_t)i);
+            } else {
+                ++i;
+            }
+        }
+    }
+    for (void* p : blocks) cudaFree(p);
+}
+}  // namespace
+
+cudaError_t table_malloc(void** p, size_t bytes)
+{
+    if (!alloc_allowed()) return cudaErrorMemoryAllocation;
+    const size_t b = block_bytes(bytes);
+    int dev = 0;
+    cudaGetDevice(&dev);
+    {
+        std::lock_guard<std::mutex> lk(g_cache_mu);
+        for (size_t i = 0; i < g_cache.size(); ++i)
+            if (g_cache[i].device == dev && g_cache[i].bytes == b) {
+                *p = g_cache[i].p;
+                g_cache.erase(g_cache.begin() + (ptrdiff_t)i);
+                return cudaSuccess;
+            }
+    }
+    cudaError_t e = cudaMalloc(p, b);
+    if (e == cudaErrorMemoryAllocation) {
+        cudaGetLastError();
+        release_cache(dev);
+        e = cudaMalloc(p, b);
+    }
+    return e;
+}
+
+void table_free(void* p, size_t bytes, int device)
+{
+    if (!p) return;
+    const size_t b = block_bytes(bytes);
+    int dev = -1;
+    cudaGetDevice(&dev);
+    if (b <= kCacheBlock && dev == device && cudaDeviceSynchronize() == cudaSuccess) {
+        std::lock_guard<std::mutex> lk(g_cache_mu);
+        size_t mine = 0;
+        for (const CachedBlock& c : g_cache) mine += c.device == dev;
+        if (mine < kCacheBlocks) {
+            g_cache.push_back(CachedBlock{dev, b, p});
+            return;
+        }
+    }
+    cudaFree(p);
+}
+
 cudaError_t dev_malloc_array(cudaArray_t* a, const cudaChannelFormatDesc* d, size_t width)
 {
     if (!alloc_allowed()) return cudaErrorMemoryAllocation;

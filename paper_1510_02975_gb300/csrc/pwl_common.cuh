@@ -59,6 +59,9 @@ inline cudaStream_t as_stream(void* s) { return reinterpret_cast<cudaStream_t>(s
 // can make them fail (pwl_test_fail_allocations) and see each call that
 // allocates return PWL_ENOMEM and release what it had taken.
 cudaError_t dev_malloc(void** p, size_t bytes);
+// The same for a table's blocks, which are reused by later tables (pwl_capi.cu)
+cudaError_t table_malloc(void** p, size_t bytes);
+void table_free(void* p, size_t bytes, int device);
 cudaError_t dev_malloc_array(cudaArray_t* a, const cudaChannelFormatDesc* d, size_t width);
 
 // ---------------------------------------------------------------------------
@@ -492,7 +495,7 @@ struct TableHeader {
     int32_t max_chain_b; // backward index: most chain hops any query can need
     int32_t n_chain_f;   // forward index: knots that share a cell with the previous knot
     int32_t max_chain_f; // forward index: most extra knots in one cell
-    int32_t pad[2];
+    float a, b;          // the end knots
 };
 
 }  // namespace pwl
@@ -514,6 +517,7 @@ struct pwl_table_s {
     int64_t chain_reserve_b;  // chain records the backward kernel stages in shared memory
     void* buf_base;    // header, knots, values, slopes, build scratch
     void* buf_rec;     // index records
+    size_t bytes_base, bytes_rec;
     pwl::TableHeader* hdr;
     float* xk;
     float* vk;

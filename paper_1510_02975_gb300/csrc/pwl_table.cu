@@ -122,6 +122,8 @@ __global__ void __launch_bounds__(kBuildThreads) table_round_kernel(
         TableHeader h{};
         h.status = s_status;
         h.hmin_bits = s_hmin;
+        h.a = xk[0];
+        h.b = xk[N];
         *hdr = h;
     }
 }
@@ -400,7 +402,8 @@ pwl_status pwl_table_build(const double* d_knots, const double* d_values, int64_
     const size_t o_cj = o_vs + align256(4 * n1);
     const size_t o_cp = o_cj + align256(4 * n1);
     const size_t total = o_cp + align256(4 * n1);
-    cudaError_t e = dev_malloc(&t->buf_base, total);
+    t->bytes_base = total;
+    cudaError_t e = table_malloc(&t->buf_base, total);
     if (e != cudaSuccess) {
         delete t;
         return cuda_fail(e, "cudaMalloc(table)");
@@ -424,24 +427,22 @@ pwl_status pwl_table_build(const double* d_knots, const double* d_values, int64_
                                                    t->vstore, t->slope, t->inv_h, t->hdr, 0, 0.0f, 0.0f);
     if ((e = cudaGetLastError()) != cudaSuccess) return bail(cuda_fail(e, "table_round_kernel"));
     TableHeader h{};
-    float ab[2];
     if ((e = cudaMemcpyAsync(&h, t->hdr, sizeof(h), cudaMemcpyDeviceToHost, s)) != cudaSuccess ||
-        (e = cudaMemcpyAsync(&ab[0], t->xk, 4, cudaMemcpyDeviceToHost, s)) != cudaSuccess ||
-        (e = cudaMemcpyAsync(&ab[1], t->xk + N, 4, cudaMemcpyDeviceToHost, s)) != cudaSuccess ||
         (e = cudaStreamSynchronize(s)) != cudaSuccess)
         return bail(cuda_fail(e, "table build (rounding pass)"));
     pwl_status st = status_error(h);
     if (st != PWL_OK) return bail(st);
     float hmin;
     memcpy(&hmin, &h.hmin_bits, 4);
-    t->a = ab[0];
-    t->b = ab[1];
+    t->a = h.a;
+    t->b = h.b;
     choose_cells(t, hmin, k_cells);
     const size_t bytes_b = align256(sizeof(float4) * ((size_t)t->Kb + n1));
     const size_t bytes_p = align256(sizeof(float2) * (size_t)t->K);
     const size_t bytes_s = align256(sizeof(float2) * 2 * n1);
     const size_t bytes_s8 = align256(sizeof(float2) * n1);
-    if ((e = dev_malloc(&t->buf_rec, 2 * bytes_b + bytes_p + bytes_s + bytes_s8)) != cudaSuccess)
+    t->bytes_rec = 2 * bytes_b + bytes_p + bytes_s + bytes_s8;
+    if ((e = table_malloc(&t->buf_rec, t->bytes_rec)) != cudaSuccess)
         return bail(cuda_fail(e, "cudaMalloc(records)"));
     char* r = static_cast<char*>(t->buf_rec);
     t->rec_b = reinterpret_cast<float4*>(r);
@@ -494,8 +495,8 @@ pwl_status pwl_table_destroy(pwl_table t)
     if (!t) return PWL_OK;
     if (t->tex) cudaDestroyTextureObject(t->tex);
     if (t->tex_array) cudaFreeArray(t->tex_array);
-    if (t->buf_rec) cudaFree(t->buf_rec);
-    if (t->buf_base) cudaFree(t->buf_base);
+    table_free(t->buf_rec, t->bytes_rec, t->device);
+    table_free(t->buf_base, t->bytes_base, t->device);
     delete t;
     return PWL_OK;
 }
