@@ -547,6 +547,7 @@ struct pwl_batch_s {
     float2 *recP, *recS;
     int* status;                // device word: bit 2 = an evaluation wait timed out
     int* order;                 // functions by decreasing intervals (the Gram solves' order)
+    double* delta;              // per function: width of a density cell
     int* tile_func;             // per design tile: its function
     FuncValueF* funcs_f;        // the functions' FP32 parameters
     DesignFunc* ffuncs;         // FP32 design: constants per function (scratch)
@@ -734,7 +735,9 @@ pwl_status pwl_batch_create(const pwl_func* funcs, const int64_t* n_intervals, i
         std::fill(tile_func.begin() + choff[f] / design_chunks(1), tile_func.begin() + choff[f + 1] / design_chunks(1), (int)f);
     std::vector<FuncValueF> funcs_f((size_t)n_funcs);
     std::vector<pwl_func> funcs_d((size_t)n_funcs);
+    std::vector<double> delta((size_t)n_funcs);
     for (int64_t f = 0; f < n_funcs; ++f) {
+        delta[(size_t)f] = (funcs[f].b - funcs[f].a) / (double)(mper * b->N[f]);
         funcs_f[(size_t)f] = func_value_params(funcs[f]);
         funcs_d[(size_t)f] = prepared(funcs[f]);
     }
@@ -762,12 +765,13 @@ pwl_status pwl_batch_create(const pwl_func* funcs, const int64_t* n_intervals, i
                             align256(sizeof(int) * F),
                             align256(sizeof(int) * tile_func.size()),
                             align256(sizeof(DesignFunc) * F),
-                            align256(sizeof(FuncValueF) * F)};
+                            align256(sizeof(FuncValueF) * F),
+                            align256(sizeof(double) * F)};
     void** slots[] = {(void**)&b->funcs, (void**)&b->d_koff, (void**)&b->d_moff, (void**)&b->d_choff,
                       (void**)&b->knots, (void**)&b->values, &b->design_scratch, &b->project_scratch,
                       (void**)&b->bf, (void**)&b->xk, (void**)&b->vk, (void**)&b->slope, (void**)&b->cj,
                       (void**)&b->recP, (void**)&b->recS, (void**)&b->status, (void**)&b->order,
-                      (void**)&b->tile_func, (void**)&b->ffuncs, (void**)&b->funcs_f};
+                      (void**)&b->tile_func, (void**)&b->ffuncs, (void**)&b->funcs_f, (void**)&b->delta};
     static_assert(sizeof(sizes) / sizeof(sizes[0]) == sizeof(slots) / sizeof(slots[0]), "one size per slot");
     size_t total = 0;
     for (size_t s : sizes) total += s;
@@ -788,6 +792,7 @@ pwl_status pwl_batch_create(const pwl_func* funcs, const int64_t* n_intervals, i
         (e = cudaMemcpy(b->bf, bfh.data(), sizeof(BatchFunc) * F, cudaMemcpyHostToDevice)) != cudaSuccess ||
         (e = cudaMemset(b->status, 0, sizeof(int))) != cudaSuccess ||
         (e = cudaMemcpy(b->order, order.data(), sizeof(int) * F, cudaMemcpyHostToDevice)) != cudaSuccess ||
+        (e = cudaMemcpy(b->delta, delta.data(), sizeof(double) * F, cudaMemcpyHostToDevice)) != cudaSuccess ||
         (e = cudaMemcpy(b->funcs_f, funcs_f.data(), sizeof(FuncValueF) * F, cudaMemcpyHostToDevice)) != cudaSuccess ||
         (e = cudaMemcpy(b->tile_func, tile_func.data(), sizeof(int) * tile_func.size(), cudaMemcpyHostToDevice)) != cudaSuccess) {
         batch_free(b);
@@ -824,6 +829,7 @@ pwl_status pwl_batch_design(pwl_batch b, int32_t precision, void* stream)
     p.total_chunks = b->total_chunks;
     p.knots = b->knots;
     design_carve_scratch(p, b->design_scratch);
+    p.delta = b->delta;
     p.tile_func = b->tile_func;
     p.ffuncs = b->ffuncs;
     if (precision == PWL_PREC_FP64) return design_launch(p, as_stream(stream));

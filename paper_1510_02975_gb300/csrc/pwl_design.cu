@@ -100,7 +100,7 @@ __global__ void __launch_bounds__(kDesignThreads, 2) density_chunks_kernel(Desig
         if ((F.kind == PWL_F_SAMPLED) != SAMPLED) continue;  // the other launch's (uniform per CTA)
         const int64_t M = p.moff[f + 1] - p.moff[f];
         const int64_t k = (ch - p.choff[f]) * kChunk + threadIdx.x;
-        const double delta = (F.b - F.a) / (double)M;
+        const double delta = p.delta[f];  // (a division here is a tenth of a Gaussian density's FP64 operations)
         double acc = 0.0;
         if (k < M) {
             acc = cell_density<T, SAMPLED>(F, delta, k);
@@ -127,8 +127,22 @@ __global__ void __launch_bounds__(kDesignThreads, 2) density_chunks_kernel(Desig
     }
 }
 
-// Per function: the exclusive FP64 scan of the chunk sums (cbase, stot) and
-// the last cell of positive density before every chunk (plast, in place).
+// smallest i in [1, N] with tau_i = i G_M / N >= G (N if none below N)
+__device__ __forceinline__ int64_t first_target_at_or_above(double G, double GM, int64_t N)
+{
+    auto tau = [&](int64_t i) { return (double)i * GM / (double)N; };
+    const double e = floor(G / GM * (double)N);
+    int64_t i = (int64_t)fmin(fmax(e, 1.0), (double)N);
+    while (i > 1 && tau(i - 1) >= G) --i;
+    while (i < N && tau(i) < G) ++i;
+    return i;
+}
+
+// Per function: the exclusive FP64 scan of the chunk sums (cbase), the last
+// cell of positive density before every chunk (plast, in place), G_M (stot),
+// and every tile's first target (in its first chunk's csum, which is spent by
+// then): one lane per tile, where two lanes of every tile's CTA held the FP64
+// pipe for as long as whole warps would.
 // kScanPer consecutive chunks per thread, 2048 chunks a round.
 constexpr int kScanPer = 8;
 
@@ -179,19 +193,13 @@ __global__ void __launch_bounds__(kDesignThreads) chunk_scan_kernel(DesignPlan p
             carry += tot;
             __syncthreads();  // s_max is rewritten in the next round
         }
-        if (threadIdx.x == 0) p.stot[f] = carry;
+        const int64_t N = p.koff[f + 1] - p.koff[f] - 1;
+        const double delta = p.delta[f], GM = delta * carry;
+        if (threadIdx.x == 0) p.stot[f] = GM;
+        __syncthreads();  // cbase complete, csum read
+        for (int64_t ch = c0 + (int64_t)threadIdx.x * kTileChunks; ch < c1; ch += kDesignThreads * kTileChunks)
+            reinterpret_cast<int64_t*>(p.csum)[ch] = GM > 0.0 ? first_target_at_or_above(delta * p.cbase[ch], GM, N) : 1;
     }
-}
-
-// smallest i in [1, N] with tau_i = i G_M / N >= G (N if none below N)
-__device__ __forceinline__ int64_t first_target_at_or_above(double G, double GM, int64_t N)
-{
-    auto tau = [&](int64_t i) { return (double)i * GM / (double)N; };
-    const double e = floor(G / GM * (double)N);
-    int64_t i = (int64_t)fmin(fmax(e, 1.0), (double)N);
-    while (i > 1 && tau(i - 1) >= G) --i;
-    while (i < N && tau(i) < G) ++i;
-    return i;
 }
 
 // The knots whose targets fall into a tile of kTileChunks chunks (tau_i at or
@@ -207,7 +215,6 @@ __global__ void __launch_bounds__(kDesignThreads) invert_tiles_kernel(DesignPlan
     __shared__ double s_d[kTile];
     __shared__ double s_S[kDesignThreads];  // tile base + exclusive prefix of the thread partials
     __shared__ double s_warp[kDesignThreads / 32 + 1];
-    __shared__ int64_t s_i[2];
     const int t = threadIdx.x;
     for (int64_t tile = blockIdx.x; tile < p.total_chunks / kTileChunks; tile += gridDim.x) {
         const int64_t ch = tile * kTileChunks;  // the tile's first chunk
@@ -216,8 +223,8 @@ __global__ void __launch_bounds__(kDesignThreads) invert_tiles_kernel(DesignPlan
         const int64_t N = p.koff[f + 1] - p.koff[f] - 1;
         const int64_t c0 = (ch - p.choff[f]) * kChunk;
         const double a = p.funcs[f].a, b = p.funcs[f].b;
-        const double delta = (b - a) / (double)M;
-        const double GM = delta * p.stot[f];
+        const double delta = p.delta[f];
+        const double GM = p.stot[f];
         double* __restrict__ knots = p.knots + p.koff[f];
         if (t == 0 && c0 == 0) {
             knots[0] = a;
@@ -229,16 +236,14 @@ __global__ void __launch_bounds__(kDesignThreads) invert_tiles_kernel(DesignPlan
             continue;
         }
         const double base = p.cbase[ch];
-        // neighbouring tiles evaluate the same expression at their common
-        // boundary, so every knot has exactly one tile
-        if (t == 0) s_i[0] = first_target_at_or_above(delta * base, GM, N);
-        if (t == 32)
-            s_i[1] = c0 + kTile < M ? first_target_at_or_above(delta * p.cbase[ch + kTileChunks], GM, N) : N;
+        // the next tile's first target ends this one's, so every knot has exactly one tile
+        const int64_t* first = reinterpret_cast<const int64_t*>(p.csum + ch);
+        const int64_t i0 = first[0], i1 = c0 + kTile < M ? first[kTileChunks] : N;
+        if (i0 >= i1) continue;
         const int cnt = (int)min((int64_t)kTile, M - c0);
         const double* __restrict__ d = p.d + p.moff[f] + c0;
         for (int i = t; i < kTile; i += kDesignThreads) s_d[i] = i < cnt ? d[i] : 0.0;
         __syncthreads();
-        const int64_t i0 = s_i[0], i1 = s_i[1];
         double run = 0.0;
         for (int r = 0; r < kTilePer; ++r) run += s_d[t * kTilePer + r];
         double tot;
@@ -409,7 +414,7 @@ __global__ void __launch_bounds__(128) tile_setup_f_kernel(DesignPlan p)
     if (tile >= p.total_chunks / kTileChunks) return;
     const int f = p.tile_func[tile];
     const int64_t ch = tile * kTileChunks, c0 = (ch - p.choff[f]) * kChunk;
-    const double a = p.funcs[f].a, delta = (p.funcs[f].b - a) / (double)(p.moff[f + 1] - p.moff[f]);
+    const double a = p.funcs[f].a, delta = p.delta[f];
     *reinterpret_cast<float*>(p.cbase + ch) = (float)(a + (double)c0 * delta);
     if (c0 == 0) {
         const pwl_func F = p.funcs[f];
@@ -631,10 +636,11 @@ __global__ void __launch_bounds__(kDesignThreads, 8) invert_tiles_f_kernel(Desig
 // Writes the descriptor and offsets of a one-function batch into the
 // workspace (kernel parameters, so the call needs no host-to-device copy).
 __global__ void single_setup_kernel(pwl_func F, int64_t N, int64_t M, int64_t chunks, pwl_func* funcs,
-                                    int64_t* koff, int64_t* moff, int64_t* choff)
+                                    int64_t* koff, int64_t* moff, int64_t* choff, double* delta)
 {
     if (threadIdx.x == 0 && blockIdx.x == 0) {
         funcs[0] = F;
+        delta[0] = (F.b - F.a) / (double)M;
         koff[0] = 0;
         koff[1] = N + 1;
         moff[0] = 0;
@@ -731,7 +737,7 @@ pwl_status design_batch_f_launch(const DesignPlan& p, cudaStream_t s)
 using namespace pwl;
 
 namespace {
-constexpr size_t kMetaBytes = 512;  // descriptor + three offset pairs
+constexpr size_t kMetaBytes = 512;  // descriptor, three offset pairs, cell width
 int64_t resolve_cells(int64_t n, int64_t m) { return m > 0 ? m : 64 * n; }
 }  // namespace
 
@@ -775,6 +781,7 @@ pwl_status pwl_design(const pwl_func* f, int64_t n_intervals, int64_t m_cells, i
     p.koff = reinterpret_cast<int64_t*>(w + 128);
     p.moff = reinterpret_cast<int64_t*>(w + 160);
     p.choff = reinterpret_cast<int64_t*>(w + 192);
+    p.delta = reinterpret_cast<double*>(w + 224);
     p.total_knots = n_intervals + 1;
     p.total_cells = M;
     p.total_chunks = design_chunks(M);
@@ -784,7 +791,7 @@ pwl_status pwl_design(const pwl_func* f, int64_t n_intervals, int64_t m_cells, i
     cudaStream_t s = as_stream(stream);
     single_setup_kernel<<<1, 1, 0, s>>>(prepared(*f), n_intervals, M, p.total_chunks, const_cast<pwl_func*>(p.funcs),
                                         const_cast<int64_t*>(p.koff), const_cast<int64_t*>(p.moff),
-                                        const_cast<int64_t*>(p.choff));
+                                        const_cast<int64_t*>(p.choff), const_cast<double*>(p.delta));
     PWL_CHECK_LAUNCH("single_setup_kernel");
     return design_launch(p, s);
 }
