@@ -635,10 +635,10 @@ def small_case(wl, reps: int = 50):
 
 
 def gpu_launches_per_step(wl) -> int:
-    # per (function, N): design 5 (descriptor setup + density, chunk scan,
-    # cumulative, inversion), interpolant values 2, projection 3, two table
-    # rebuilds of 3 kernels, four evaluations
-    per_item = 5 + 2 + 3 + 6 + 4
+    # per (function, N): design 4 (descriptor setup + density, chunk scan,
+    # knots), interpolant values 2, projection 3, two table rebuilds of 3
+    # kernels, four evaluations
+    per_item = 4 + 2 + 3 + 6 + 4
     return per_item * len(wl.items)
 
 
