@@ -50,17 +50,13 @@ static bool alloc_allowed()
     return true;
 }
 
-cudaError_t dev_malloc(void** p, size_t bytes)
-{
-    if (!alloc_allowed()) return cudaErrorMemoryAllocation;
-    return cudaMalloc(p, bytes);
-}
-
-// Blocks of destroyed tables, kept for the next build: cudaMalloc and cudaFree
-// take ~30 us each, and a table has two blocks (120 us of the 430 from f to a
-// table and its first evaluation).  A block is kept only once the device has
-// finished everything that might still use it (cudaFree waits the same way),
-// so any stream may write to it afterwards.  At most kCacheBlocks blocks of
+// Base blocks of destroyed tables, kept for the next build: cudaMalloc and
+// cudaFree take ~30 us each, and a table has two blocks (120 us of the 430 from f
+// to a table and its first evaluation).  The other block, the index, goes back by
+// cudaFree, which waits for everything on the device, so any stream may write to
+// the kept block afterwards.  That wait is not cudaDeviceSynchronize: it would
+// end every graph capture that another thread, or a relaxed one of this thread,
+// has under way, which cudaFree leaves alone.  At most kCacheBlocks blocks of
 // kCacheBlock bytes at most per device; they go back to the device when an
 // allocation fails.
 namespace {
@@ -98,7 +94,26 @@ void release_cache(int dev)
     }
     for (void* p : blocks) cudaFree(p);
 }
+
+cudaError_t malloc_or_release(void** p, size_t bytes, int dev)
+{
+    cudaError_t e = cudaMalloc(p, bytes);
+    if (e == cudaErrorMemoryAllocation) {
+        cudaGetLastError();
+        release_cache(dev);
+        e = cudaMalloc(p, bytes);
+    }
+    return e;
+}
 }  // namespace
+
+cudaError_t dev_malloc(void** p, size_t bytes)
+{
+    if (!alloc_allowed()) return cudaErrorMemoryAllocation;
+    int dev = 0;
+    cudaGetDevice(&dev);
+    return malloc_or_release(p, bytes, dev);
+}
 
 cudaError_t table_malloc(void** p, size_t bytes)
 {
@@ -115,31 +130,25 @@ cudaError_t table_malloc(void** p, size_t bytes)
                 return cudaSuccess;
             }
     }
-    cudaError_t e = cudaMalloc(p, b);
-    if (e == cudaErrorMemoryAllocation) {
-        cudaGetLastError();
-        release_cache(dev);
-        e = cudaMalloc(p, b);
-    }
-    return e;
+    return malloc_or_release(p, b, dev);
 }
 
-void table_free(void* p, size_t bytes, int device)
+void table_free(void* base, size_t bytes, void* index, int device)
 {
-    if (!p) return;
+    // a table without an index (a build that failed) has no wait to rely on
+    const bool idle = index && cudaFree(index) == cudaSuccess;
+    if (!base) return;
     const size_t b = block_bytes(bytes);
-    int dev = -1;
-    cudaGetDevice(&dev);
-    if (b <= kCacheBlock && dev == device && cudaDeviceSynchronize() == cudaSuccess) {
+    if (idle && b <= kCacheBlock) {
         std::lock_guard<std::mutex> lk(g_cache_mu);
         size_t mine = 0;
-        for (const CachedBlock& c : g_cache) mine += c.device == dev;
+        for (const CachedBlock& c : g_cache) mine += c.device == device;
         if (mine < kCacheBlocks) {
-            g_cache.push_back(CachedBlock{dev, b, p});
+            g_cache.push_back(CachedBlock{device, b, base});
             return;
         }
     }
-    cudaFree(p);
+    cudaFree(base);
 }
 
 cudaError_t dev_malloc_array(cudaArray_t* a, const cudaChannelFormatDesc* d, size_t width)

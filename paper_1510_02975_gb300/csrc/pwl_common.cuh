@@ -59,9 +59,10 @@ inline cudaStream_t as_stream(void* s) { return reinterpret_cast<cudaStream_t>(s
 // can make them fail (pwl_test_fail_allocations) and see each call that
 // allocates return PWL_ENOMEM and release what it had taken.
 cudaError_t dev_malloc(void** p, size_t bytes);
-// The same for a table's blocks, which are reused by later tables (pwl_capi.cu)
+// The same for a table's base block, which later tables reuse (pwl_capi.cu), and
+// the release of a table's two blocks.
 cudaError_t table_malloc(void** p, size_t bytes);
-void table_free(void* p, size_t bytes, int device);
+void table_free(void* base, size_t bytes, void* index, int device);
 cudaError_t dev_malloc_array(cudaArray_t* a, const cudaChannelFormatDesc* d, size_t width);
 
 // ---------------------------------------------------------------------------
@@ -517,7 +518,7 @@ struct pwl_table_s {
     int64_t chain_reserve_b;  // chain records the backward kernel stages in shared memory
     void* buf_base;    // header, knots, values, slopes, build scratch
     void* buf_rec;     // index records
-    size_t bytes_base, bytes_rec;
+    size_t bytes_base;
     pwl::TableHeader* hdr;
     float* xk;
     float* vk;

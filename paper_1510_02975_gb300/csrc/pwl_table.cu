@@ -441,8 +441,7 @@ pwl_status pwl_table_build(const double* d_knots, const double* d_values, int64_
     const size_t bytes_p = align256(sizeof(float2) * (size_t)t->K);
     const size_t bytes_s = align256(sizeof(float2) * 2 * n1);
     const size_t bytes_s8 = align256(sizeof(float2) * n1);
-    t->bytes_rec = 2 * bytes_b + bytes_p + bytes_s + bytes_s8;
-    if ((e = table_malloc(&t->buf_rec, t->bytes_rec)) != cudaSuccess)
+    if ((e = dev_malloc(&t->buf_rec, 2 * bytes_b + bytes_p + bytes_s + bytes_s8)) != cudaSuccess)
         return bail(cuda_fail(e, "cudaMalloc(records)"));
     char* r = static_cast<char*>(t->buf_rec);
     t->rec_b = reinterpret_cast<float4*>(r);
@@ -495,8 +494,7 @@ pwl_status pwl_table_destroy(pwl_table t)
     if (!t) return PWL_OK;
     if (t->tex) cudaDestroyTextureObject(t->tex);
     if (t->tex_array) cudaFreeArray(t->tex_array);
-    table_free(t->buf_rec, t->bytes_rec, t->device);
-    table_free(t->buf_base, t->bytes_base, t->device);
+    table_free(t->buf_base, t->bytes_base, t->buf_rec, t->device);
     delete t;
     return PWL_OK;
 }

@@ -62,3 +62,40 @@ def test_threads_with_their_own_streams(pwl):
     for t in threads:
         t.join()
     assert not wrong
+
+
+@pytest.mark.parametrize("where, mode", [("here", "relaxed"), ("thread", "relaxed"), ("thread", "thread_local")])
+@pytest.mark.parametrize("n", [63, 9000])
+def test_destroying_leaves_a_capture_alone(pwl, where, mode, n):
+    """A graph capture goes on while a table is destroyed, in any mode and thread that cudaFree
+    allows, and so does one during which another thread builds, uses and destroys a table."""
+    arrays = _arrays(pwl, n)
+    kept, gone = pwl.Table(*arrays), pwl.Table(*arrays)
+    x = torch.rand(100003, device="cuda") * 8 - 4
+    want = kept(x)
+    y, z = torch.empty_like(x), torch.empty_like(x)
+    torch.cuda.synchronize()
+
+    def destroy():
+        gone.close()
+        if where == "thread":
+            with torch.cuda.stream(torch.cuda.Stream()):
+                for _ in range(3):
+                    t = pwl.Table(*arrays)
+                    t(x, z)
+                    t.close()
+
+    g = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(g, capture_error_mode=mode):
+        kept(x, y)
+        if where == "here":
+            destroy()
+        else:
+            t = threading.Thread(target=destroy)
+            t.start()
+            t.join()
+        y.add_(1.0)
+    g.replay()
+    torch.cuda.synchronize()
+    assert torch.equal(y, want + 1.0)
+    assert where == "here" or torch.equal(z, want)
