@@ -66,7 +66,9 @@ __global__ void interp_values_kernel(ProjectPlan p)
 // At the node t_q = mid + half x_q the hats are phi_{j-1} = (1 - x_q)/2 and
 // phi_j = (1 + x_q)/2, so L_j = half sum_q wl_q f(t_q) and
 // R_j = half sum_q wr_q f(t_q) with the host-side weights wl, wr: no
-// division per node.  FP64 mode: t_q and the sums in FP64.  FP32 mode: t_q
+// division per node.  They are stored six times as large, the scale in which the
+// Gram system needs no products with 1/6 and 1/3 (see gram_spike_kernel): the
+// factor 3 (x_j - x_{j-1}) takes the place of half.  FP64 mode: t_q and the sums in FP64.  FP32 mode: t_q
 // and f(t_q) in FP32 (the argument of an FP32 f is rounded to FP32 anyway),
 // the sums in FP64.
 //
@@ -101,7 +103,8 @@ __global__ void hat_integrals_kernel(ProjectPlan p, const __grid_constant__ Gaus
             L = __fma_rn(gl.wl[q], fv, L);
             R = __fma_rn(gl.wr[q], fv, R);
         }
-        p.lr[g] = make_double2(half * L, half * R);
+        const double h3 = 3.0 * (xr - xl);
+        p.lr[g] = make_double2(h3 * L, h3 * R);
     }
 }
 
@@ -132,7 +135,10 @@ __global__ void __launch_bounds__(128) hat_nodes_kernel(ProjectPlan p, const __g
             L += __shfl_xor_sync(lanes, L, o);
             R += __shfl_xor_sync(lanes, R, o);
         }
-        if (q == 0) p.lr[g] = make_double2(half * L, half * R);
+        if (q == 0) {
+            const double h3 = 3.0 * (xr - xl);
+            p.lr[g] = make_double2(h3 * L, h3 * R);
+        }
     }
 }
 
@@ -141,8 +147,8 @@ __global__ void __launch_bounds__(128) hat_nodes_kernel(ProjectPlan p, const __g
 // recovered by an FMA), each addition compensated.  The FP64 pipe (one
 // instruction takes it for 16 clocks or more per warp) was 78% busy with
 // conversions, of the function's parameters above all: those are FP32 in
-// memory now and the rest go by bit arithmetic, which leaves eight FP64
-// operations per interval (4096 functions, 8.4 M intervals: 388 -> 312 us).
+// memory now and the rest go by bit arithmetic, which leaves seven FP64
+// operations per interval (4096 functions, 8.4 M intervals: 388 -> 309 us).
 template <bool SAMPLED>
 __global__ void __launch_bounds__(128) hat_integrals_f_kernel(ProjectPlan p, const __grid_constant__ GaussLegendre gl)
 {
@@ -155,8 +161,8 @@ __global__ void __launch_bounds__(128) hat_integrals_f_kernel(ProjectPlan p, con
         const int64_t j = g - (p.koff[f] - f) + 1;  // interval index 1..N_f
         const double* x = p.knots + p.koff[f];
         const double xl = x[j - 1], xr = x[j];
-        const double half = 0.5 * (xr - xl);
-        const float midf = narrow_bits(0.5 * (xl + xr)), halff = narrow_bits(half);
+        const double h = xr - xl;
+        const float midf = 0.5f * narrow_bits(xl + xr), halff = 0.5f * narrow_bits(h);
         float Lh = 0.0f, Ll = 0.0f, Rh = 0.0f, Rl = 0.0f;
         auto acc = [](float& h, float& l, float wh, float wlo, float fv) {
             const float p = __fmul_rn(wh, fv);
@@ -176,7 +182,8 @@ __global__ void __launch_bounds__(128) hat_integrals_f_kernel(ProjectPlan p, con
             acc(Lh, Ll, gl.wlh[q], gl.wll[q], fv);
             acc(Rh, Rl, gl.wrh[q], gl.wrl[q], fv);
         }
-        p.lr[g] = make_double2(half * (widen_bits(Lh) + widen_bits(Ll)), half * (widen_bits(Rh) + widen_bits(Rl)));
+        const double h3 = 3.0 * h;
+        p.lr[g] = make_double2(h3 * (widen_bits(Lh) + widen_bits(Ll)), h3 * (widen_bits(Rh) + widen_bits(Rl)));
     }
 }
 
@@ -195,9 +202,9 @@ __global__ void __launch_bounds__(128) hat_integrals_f_kernel(ProjectPlan p, con
 //     magnitude on this diagonally dominant matrix, so every pivot
 //     1 + v0_p beta_{p-1} stays near 1);
 //  3. every lane reconstructs its rows.
-// The rows are assembled on the fly (M_{i,i-1} = h_i/6, M_ii = (h_i +
-// h_{i+1})/3, M_{i,i+1} = h_{i+1}/6, b_i = R_i + L_{i+1}).  About 20 FP64
-// operations per row; no barrier beyond the warp.
+// The rows are assembled on the fly (6 M_{i,i-1} = h_i, 6 M_ii = 2 (h_i +
+// h_{i+1}), 6 M_{i,i+1} = h_{i+1}, 6 b_i = R_i + L_{i+1} as the hat integrals
+// are stored).  About 18 FP64 operations per row; no barrier beyond the warp.
 // Blocks of some dozen rows or more are as good as decoupled beyond their
 // neighbours: the spikes fall by 0.27 per row of a uniform partition, and once
 // every w at its block's first row and v at its last is below kSpikeGone, the
@@ -206,14 +213,14 @@ __global__ void __launch_bounds__(128) hat_integrals_f_kernel(ProjectPlan p, con
 // per block, as many as a row and a half of elimination).
 // The scratch (c', y, v, w per row) is laid out by planes, row-in-block major:
 // the 32 lanes' accesses are consecutive, where rows of 32 bytes at a stride of
-// a block touched a sector each.  4096 functions, 8.4 M rows: 703 -> 477 us.
+// a block touched a sector each.  4096 functions, 8.4 M rows: 703 -> 477 us, and
+// 464 us with the system scaled by six.
 constexpr double kSpikeGone = 1e-30;
 
 __global__ void __launch_bounds__(64) gram_spike_kernel(ProjectPlan p, const int* __restrict__ order)
 {
     const int lane = threadIdx.x & 31;
     const int warps = gridDim.x * (blockDim.x >> 5);
-    constexpr double kSixth = 1.0 / 6.0, kThird = 1.0 / 3.0;
     for (int o = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5); o < p.F; o += warps) {
         const int f = order ? order[o] : o;
         const int64_t k0 = p.koff[f];
@@ -240,13 +247,12 @@ __global__ void __launch_bounds__(64) gram_spike_kernel(ProjectPlan p, const int
                 const double xn = i < N ? x[i + 1] : xi;
                 const double hr = xn - xi;
                 const double rhs = (i > 0 ? lr[i - 1].y : 0.0) + (i < N ? lr[i].x : 0.0);
-                const double lower = i > r0 ? hl * kSixth : 0.0;  // coupling inside the block
-                const double upper = hr * kSixth;
-                const double r = recip_newton((hl + hr) * kThird - lower * cprev);
+                const double lower = i > r0 ? hl : 0.0;  // coupling inside the block
+                const double r = recip_newton(2.0 * (hl + hr) - lower * cprev);
                 const double yv = (rhs - lower * yprev) * r;
-                const double vv = ((i == r0 ? hl * kSixth : 0.0) - lower * vprev) * r;
-                cprev = i + 1 < r1 ? upper * r : 0.0;
-                if (i + 1 == r1) wlast = upper * r;  // w'_{m-1}: the coupling to the next block
+                const double vv = ((i == r0 ? hl : 0.0) - lower * vprev) * r;
+                cprev = i + 1 < r1 ? hr * r : 0.0;
+                if (i + 1 == r1) wlast = hr * r;  // w'_{m-1}: the coupling to the next block
                 const int at = (i - r0) * P;
                 sc[at] = cprev;
                 sy[at] = yv;
@@ -352,9 +358,10 @@ __global__ void __launch_bounds__(64) gram_spike_kernel(ProjectPlan p, const int
 // below kCouplingGone and the rows left are solved at once: 1024 intervals
 // 16.8 -> 14.9 us, 4095 41.5 -> 39.1 us.
 // One CTA solves one function, so the solve runs on a single SM's FP64
-// pipe: the pivots' reciprocals come from recip_newton (five FP64
-// operations) and the entries from products with 1/6 and 1/3, not from
-// FP64 divisions (the bench's design graph 0.495 -> 0.455 ms).
+// pipe: the pivots' reciprocals come from recip_newton (three FP64
+// operations) and the system is solved six times as large, which leaves its
+// entries without products, not from FP64 divisions (the bench's design graph
+// 0.495 -> 0.455 ms).
 constexpr double kCouplingGone = 1e-30;
 
 __global__ void __launch_bounds__(kSolveThreads) gram_solve_kernel(ProjectPlan p, int use_smem)
@@ -374,9 +381,9 @@ __global__ void __launch_bounds__(kSolveThreads) gram_solve_kernel(ProjectPlan p
         for (int i = threadIdx.x; i < n; i += blockDim.x) {
             const double hl = (i > 0) ? x[i] - x[i - 1] : 0.0;
             const double hr = (i < N) ? x[i + 1] - x[i] : 0.0;
-            A[i] = hl * (1.0 / 6.0);
-            B[i] = (hl + hr) * (1.0 / 3.0);
-            C[i] = hr * (1.0 / 6.0);
+            A[i] = hl;
+            B[i] = 2.0 * (hl + hr);
+            C[i] = hr;
             D[i] = ((i > 0) ? lr[i - 1].y : 0.0) + ((i < N) ? lr[i].x : 0.0);
         }
         __syncthreads();
