@@ -499,11 +499,10 @@ pwl_status pwl_channels_forward(const float* d_knots, const float* d_values, int
 /* Backward of pwl_channels_forward (FP32 only): gx[r, c] = gy[r, c] * s,
  * and for every channel d_g_values[c, j] += sum over rows of gy dy/dv_j,
  * d_g_knots[c, j] += sum of gy dy/dx_j (the formulas of pwl_eval_backward;
- * either may be NULL).  Inside a CTA the sums are fixed point per channel
- * (each term rounded at 2^-29 of the channel's typical |gy| or finer, the
- * sums exact; terms far above the typical one in FP32); the CTAs' sums are
- * added with FP32 atomics, order-dependent at FP32 rounding.  k_cells as in
- * the forward.                                                             */
+ * either may be NULL).  A CTA's sums hold every term to 2^-18 of itself or
+ * finer and add without further rounding; the CTAs' sums and terms far from
+ * the channel's largest are added with FP32 atomics, order-dependent at FP32
+ * rounding.  k_cells as in the forward.                                    */
 pwl_status pwl_channels_backward(const float* d_knots, const float* d_values, int64_t n_channels,
                                  int64_t n_intervals, int64_t k_cells, const float* d_x, const float* d_gy,
                                  float* d_gx, float* d_g_values, float* d_g_knots, int64_t rows,

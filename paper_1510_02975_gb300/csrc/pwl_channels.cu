@@ -30,13 +30,13 @@
 // are as wide as keeps the index below kIndexBytes.
 //
 // Measured, [65536, 4096] x 257 knots: forward 532 -> 377 us (FP32; 5.70 TB/s),
-// backward 1042 -> 689 us (4.67 TB/s); [16384, 4096] in BF16: forward 196 ->
-// 110 us, backward 695 -> 199 us, 388 us of it FP32 copies of the streams,
+// backward 1042 -> 840 us (3.8 TB/s); [16384, 4096] in BF16: forward 196 ->
+// 110 us, backward 695 -> 265 us, 388 us of the 695 FP32 copies of the streams,
 // which the BF16 kernel does without.  Before, the forward had 8-channel
 // tiles (16-byte cells), the backward two compare-and-swap adds
-// and side selects per element (103 instructions, now ~65), and four CTAs a
+// and side selects per element (103 instructions), and four CTAs a
 // cluster left 8 SMs idle.  What bounds them now: the forward the access
-// pattern (350-370 us as a plain copy), the backward instruction issue (75%).
+// pattern (350-370 us as a plain copy), the backward instruction issue.
 // A range costs ~5 us (forward) to ~15 us (backward) besides its rows: the
 // index build and, backward, the reductions into the global gradients.
 //
@@ -370,29 +370,44 @@ __global__ void __launch_bounds__(kChThreads, 1) channels_forward_kernel(const C
 // tile's rows they become g_v[j] += A_{j+1} + B_j (+ clamped terms) and
 // g_x[j] += -s_{j+1} A_{j+1} - s_j B_j, added to the global gradients.
 //
-// The sums are fixed point, in two 32-bit words each: a term v in units of
-// 2^-F is split into h = rint(v 2^-17) and the rest l = rint(v - h 2^17), both
-// (h by adding 1.5 2^23, which needs no conversion), and added with native
-// integer shared-memory atomics that return nothing.  An FP32 shared-memory
-// add is a compare-and-swap loop in software (about 10 instructions, 2.6 adds
-// per clock and SM against more than 9 for int32): with it this kernel was
-// issue bound.  |v| < 2^33 keeps h and l
-// within 2^16, so neither word of an interval wraps in kFlushRows rows.  F comes, per
-// channel, from the mean binary exponent of gy over rows spread over all of
-// R: a typical term is ~2^kTypicalBits units, i.e. rounded at 2^-29 of it (an FP32 add
-// rounds at 2^-25 of the running sum), terms above 32 times the typical one,
-// inf and NaN are added to the global gradients in FP32, and so is every
-// nonzero term of a tile whose sampled rows are all zero.
-constexpr int kTypicalBits = 28;
-constexpr float kFixLimit = 0x1p33f;
-constexpr int64_t kFlushRows = 32512;  // at most 2^15 - 1, whole passes of every tile width (64, 128, 256 rows)
+// The sums are fixed point, in two 32-bit words each: a term v in units of 2^-F is
+// h 2^19 + l + rest with h = rint(v 2^-19) (by adding 1.5 2^23, which needs no
+// conversion) and l = rint(v - h 2^19), both added with native integer
+// shared-memory atomics that return nothing.  An FP32 shared-memory add is a
+// compare-and-swap loop in software (about 10 instructions, 2.6 adds per clock and
+// SM against more than 9 for int32).  |v| < 2^37 keeps h and l within 2^18, so 6912
+// rows add less than 2^31 - 2^28 to a word; every 6912 rows the words are looked
+// over and the tile's sums flushed where one has passed 2^28.
+// A term of 2^17 units or more is rounded at 2^-18 of itself or finer (from 2^23 on
+// it is exact).  The rest of a smaller one, which the words do not hold, goes to the
+// global gradients in FP32, and so does a term beyond 2^37: every sum is accurate
+// relative to its own terms, however small they are beside the channel's other
+// gradients.
+//
+// F comes, per channel, from the largest of 64 (128, 256) sampled |gy|, spread over
+// the rows; terms of up to 4 to 8 times that fit.
+constexpr int kDigitBits = 19;
+constexpr int kRangeBits = 37;                                // terms below 2^37 units
+constexpr float kFixLimit = 0x1p37f;
+constexpr unsigned kSmallKey = 2u * ((127 + 17) << 23) - 2u;  // small_key of 2^17
+constexpr int kSegRows = 6912;                                // whole passes of every tile width (64, 128, 256 rows)
+constexpr int kFullWord = 1 << 28;
 constexpr float kMagic = 0x1.8p23f;
 constexpr int kMagicBits = 0x4B400000;
+constexpr float kDigit = 0x1p19f, kPerDigit = 0x1p-19f;
 
+// What a range's setup shares, and what the rare paths need (in registers it would
+// weigh on the loop that hardly ever takes them).
 struct BwdShared {
     int bad;
-    int esum[16], ecnt[16];
+    int emax[16];    // per channel: the largest binary exponent of a nonzero finite sample, or kNoSample
+    float unit[16];  // per channel: 2^-F
+    float *gv, *gk;  // the tile's rows of the global gradients (or NULL)
+    uint32_t rec;    // shared address of the tile's first record
+    int N;
 };
+__shared__ BwdShared s_bwd;
+constexpr int kNoSample = -1000;
 
 // gy of this thread's channel at its sampled row (0 past the last channel)
 template <typename IO, int CH>
@@ -401,84 +416,97 @@ __device__ __forceinline__ float sample_gy(const ChanArgs& p, int64_t c0, const 
     const int64_t c = c0 + threadIdx.x % CH, r = p.R * (int64_t)(threadIdx.x / CH) / (kChThreads / CH);
     return c < p.C ? to_f32<IO>(__ldcg(gy + r * p.C + c)) : 0.0f;
 }
-// the samples' binary exponents (nonzero finite ones) into the channels' sums
+// the samples' binary exponents (nonzero finite ones) into the channels' maxima
 template <int CH>
-__device__ __forceinline__ void sum_exponents(float g, BwdShared* sh)
+__device__ __forceinline__ void max_exponents(float g)
 {
     const int ex = (int)(__float_as_uint(g) >> 23 & 0xffu);
-    const bool ok = ex != 0 && ex != 0xff;
-    int esum = ok ? ex - 127 : 0, ecnt = ok ? 1 : 0;
-    for (int o = CH; o < 32; o <<= 1) {
-        esum += __shfl_xor_sync(0xffffffffu, esum, o);
-        ecnt += __shfl_xor_sync(0xffffffffu, ecnt, o);
-    }
-    if ((threadIdx.x & 31) < CH && ecnt) {
-        atomicAdd(&sh->esum[threadIdx.x % CH], esum);
-        atomicAdd(&sh->ecnt[threadIdx.x % CH], ecnt);
-    }
+    int e = ex != 0 && ex != 0xff ? ex - 127 : kNoSample;
+    for (int o = CH; o < 32; o <<= 1) e = max(e, __shfl_xor_sync(0xffffffffu, e, o));
+    if ((threadIdx.x & 31) < CH && e != kNoSample) atomicMax(&s_bwd.emax[threadIdx.x % CH], e);
 }
 
-// F of a channel: from its own samples, else the tile's; with no nonzero
-// sample at all the largest unit scale, which sends every nonzero term to the
-// FP32 path.  2^F and 2^-F are normal FP32 numbers.
+// F of a channel: from its own samples, else from the tile's (whose unit may be
+// far too coarse for it; then its terms count as small).  2^F and 2^-F are
+// normal FP32 numbers.
 template <int CH>
-__device__ __forceinline__ int fix_exponent(const BwdShared* sh, int ch)
+__device__ __forceinline__ int fix_exponent(int ch)
 {
-    int s = sh->esum[ch], n = sh->ecnt[ch];
-    if (n == 0)
-        for (int q = 0; q < CH; ++q) {
-            s += sh->esum[q];
-            n += sh->ecnt[q];
-        }
-    if (n == 0) return 126;
-    return min(max(kTypicalBits - (int)floorf((float)s / (float)n), -60), 126);
+    int e = s_bwd.emax[ch];
+    if (e == kNoSample)
+        for (int q = 0; q < CH; ++q) e = max(e, s_bwd.emax[q]);
+    return e == kNoSample ? 126 : min(max(kRangeBits - 3 - e, -100), 126);
 }
 __device__ __forceinline__ float exp2_int(int e) { return __int_as_float((e + 127) << 23); }
 
-// one term into its two words (h at byte offset H, l at byte offset L)
-template <int H, int L>
+// orders terms by magnitude, 0 (which is exact) above all
+__device__ __forceinline__ unsigned small_key(float v) { return 2u * __float_as_uint(v) - 2u; }
+
+// h 2^19 of a term, and the rest of it
+__device__ __forceinline__ float fix_high(float v, float& m)
+{
+    m = __fmaf_rn(v, kPerDigit, kMagic);
+    return __fmaf_rn(__fsub_rn(m, kMagic), -kDigit, v);
+}
+// one term into its two words (h at byte offset 0, l at byte offset L)
+template <int L>
 __device__ __forceinline__ void fix_add(uint32_t at, float v)
 {
-    const float m = __fmaf_rn(v, 0x1p-17f, kMagic);
-    red_add<H>(at, __float_as_int(m) - kMagicBits);
-    red_add<L>(at, __float2int_rn(__fmaf_rn(__fsub_rn(m, kMagic), -0x1p17f, v)));
+    float m;
+    const float low = fix_high(v, m);
+    red_add<0>(at, __float_as_int(m) - kMagicBits);
+    red_add<L>(at, __float2int_rn(low));
 }
-
+// what fix_add's words leave out
+__device__ __forceinline__ float fix_rest(float v)
+{
+    float m;
+    const float low = fix_high(v, m);
+    return low - __int2float_rn(__float2int_rn(low));
+}
 // FP32 sums of the gradients w.r.t. the end values of clamped elements
 struct EndSums {
     float left, right;
 };
 
-// What the backward of one channel needs besides its lookup.
+// What the backward of one channel needs besides its lookup: record address ->
+// address of the interval's A words and B words (odd rows: B and A).
 struct BwdOut {
-    float* gv;  // the channel's rows of the global gradients (or NULL)
-    float* gk;
-    uint32_t first, second;  // record address -> address of the interval's A words and B words (odd rows: B and A)
+    uint32_t first, second;
     float scale;
     bool odd;
 };
-
-// An element that is clamped, NaN, or beyond the fixed-point range (FP32 to the
-// global gradients); returns its gx.
-__device__ __noinline__ float chan_bwd_rare(float x, float g, float a, float b, float4 r, int e, bool last, float* gv,
-                                            float* gk, EndSums* ends)
+template <int CH>
+__device__ __forceinline__ bool odd_row()
 {
-    if (x >= a && x <= b) {
-        const int i = max(e, 1);  // 0 only where x_0 is NaN
-        const float ca = g * ((r.w - x) * r.y), cb = g * ((x - r.x) * r.y);
-        if (gv) {
-            atomicAdd(gv + i - 1, ca);
-            if (!last) atomicAdd(gv + i, cb);
-        }
-        if (gk) {
-            atomicAdd(gk + i - 1, -r.z * ca);
-            if (!last) atomicAdd(gk + i, -r.z * cb);
-        }
-        return g * r.z;
+    return CH == 16 && threadIdx.x / CH % 2;
+}
+
+// Two terms (in the order of this thread's row) of an element whose record is at
+// `at`, to the global gradients in FP32; s: the interval's slope.
+template <int CH>
+__device__ __noinline__ void add_global_terms(float t1, float t2, uint32_t at, float s)
+{
+    const int e = (int)(at - s_bwd.rec) / (16 * CH), i = max(e, 1);  // 0 only where x_0 is NaN
+    const int64_t k = (int64_t)(threadIdx.x % CH) * (s_bwd.N + 1) + i;
+    const float l = odd_row<CH>() ? t2 : t1;                        // at the interval's left knot
+    const float r = e > s_bwd.N ? 0.0f : odd_row<CH>() ? t1 : t2;  // at its right one (none past x_N)
+    if (s_bwd.gv) {
+        if (l != 0.0f) atomicAdd(s_bwd.gv + k - 1, l);
+        if (r != 0.0f) atomicAdd(s_bwd.gv + k, r);
     }
-    ends->left += x < a ? g : 0.0f;
-    ends->right += x > b ? g : 0.0f;
-    return x != x ? x : 0.0f;
+    if (s_bwd.gk) {
+        if (l != 0.0f) atomicAdd(s_bwd.gk + k - 1, -s * l);
+        if (r != 0.0f) atomicAdd(s_bwd.gk + k, -s * r);
+    }
+}
+// The same for what the words of two terms leave out.
+template <int CH>
+__device__ __noinline__ void add_rests(float t1, float t2, uint32_t at, float s)
+{
+    const float unit = s_bwd.unit[threadIdx.x % CH];
+    const float e1 = fix_rest(t1) * unit, e2 = fix_rest(t2) * unit;
+    if (e1 != 0.0f || e2 != 0.0f) add_global_terms<CH>(e1, e2, at, s);
 }
 
 // G elements: gx in place of g.
@@ -489,34 +517,70 @@ __device__ __forceinline__ void chan_bwd(const float (&x)[G], float (&g)[G], con
     float xc[G];
     float4 r[G];
     uint32_t at[G];
-    bool fine = true;
+    bool inside = true, fits = true;
+    unsigned nans = 0;
 #pragma unroll
     for (int q = 0; q < G; ++q) {
         xc[q] = fminf(fmaxf(x[q], cc.a), cc.b);  // NaN -> a
-        fine = fine && x[q] == xc[q] && fabsf(g[q] * o.scale) < kFixLimit;
+        inside = inside && x[q] == xc[q];
     }
-    chan_lookup<CH, G>(xc, cc, r, at);
-    auto add = [&](int q) {
-        // 1 - delta and delta, each from the interval's other end and so accurate
-        // where it is small; odd rows take them in the other order
-        const float gs = g[q] * o.scale;
-        const float p1 = o.odd ? r[q].x : r[q].w, p2 = o.odd ? r[q].w : r[q].x;
-        fix_add<0, 8 * CH>(at[q] + o.first, gs * (fabsf(p1 - xc[q]) * r[q].y));
-        fix_add<0, 8 * CH>(at[q] + o.second, gs * (fabsf(p2 - xc[q]) * r[q].y));
-        g[q] *= r[q].z;
-    };
-    if (fine) {
-#pragma unroll
-        for (int q = 0; q < G; ++q) add(q);
-    } else {
+    if (!inside) {
 #pragma unroll
         for (int q = 0; q < G; ++q) {
-            if (x[q] == xc[q] && fabsf(g[q] * o.scale) < kFixLimit)
-                add(q);
-            else
-                g[q] = chan_bwd_rare(x[q], g[q], cc.a, cc.b, r[q], (int)(at[q] - cc.rec) / (16 * CH),
-                                     at[q] == cc.last, o.gv, o.gk, &ends);
+            if (x[q] == xc[q]) continue;
+            ends.left += x[q] < cc.a ? g[q] : 0.0f;
+            ends.right += x[q] > cc.b ? g[q] : 0.0f;
+            nans |= x[q] != x[q] ? 1u << q : 0u;
+            g[q] = 0.0f;
         }
+    }
+    chan_lookup<CH, G>(xc, cc, r, at);
+    // 1 - delta and delta, each from the interval's other end and so accurate
+    // where it is small; odd rows take them in the other order
+    auto terms = [&](int q, float gq, float& t1, float& t2) {
+        const float p1 = o.odd ? r[q].x : r[q].w, p2 = o.odd ? r[q].w : r[q].x;
+        t1 = gq * (fabsf(p1 - xc[q]) * r[q].y);
+        t2 = gq * (fabsf(p2 - xc[q]) * r[q].y);
+    };
+    float gs[G];
+    unsigned small = ~0u;
+#pragma unroll
+    for (int q = 0; q < G; ++q) {
+        gs[q] = g[q] * o.scale;
+        fits = fits && fabsf(gs[q]) < kFixLimit;
+    }
+    if (!fits) {
+#pragma unroll
+        for (int q = 0; q < G; ++q) {
+            if (fabsf(gs[q]) < kFixLimit) continue;
+            float t1, t2;
+            terms(q, g[q], t1, t2);
+            add_global_terms<CH>(t1, t2, at[q], r[q].z);
+            gs[q] = 0.0f;
+        }
+    }
+#pragma unroll
+    for (int q = 0; q < G; ++q) {
+        float t1, t2;
+        terms(q, gs[q], t1, t2);
+        fix_add<8 * CH>(at[q] + o.first, t1);
+        fix_add<8 * CH>(at[q] + o.second, t2);
+        small = min(small, min(small_key(t1), small_key(t2)));
+    }
+    if (small < kSmallKey) {
+#pragma unroll
+        for (int q = 0; q < G; ++q) {
+            float t1, t2;
+            terms(q, gs[q], t1, t2);
+            add_rests<CH>(t1, t2, at[q], r[q].z);
+        }
+    }
+#pragma unroll
+    for (int q = 0; q < G; ++q) g[q] *= r[q].z;
+    if (nans) {
+#pragma unroll
+        for (int q = 0; q < G; ++q)
+            if (nans >> q & 1u) g[q] = x[q];
     }
 }
 
@@ -524,17 +588,16 @@ template <typename IO, int CH>
 __device__ __forceinline__ void chan_bwd_rows(const ChanArgs& p, int64_t c0, int64_t r0, int64_t r1,
                                               const float2* cells, const float4* rec, int* acc, float scale,
                                               const IO* __restrict__ x, const IO* __restrict__ gy,
-                                              IO* __restrict__ gx, float* g_values, float* g_knots)
+                                              IO* __restrict__ gx)
 {
     constexpr int RP = kChThreads / CH, U = kBwdUnroll, G = kBwdGroup;
     const int ch = threadIdx.x % CH, row = threadIdx.x / CH;
     const int64_t c = c0 + ch;
     if (c >= p.C) return;
     const ChanConst<CH> cc(p, cells, rec, ch);
-    const bool odd = CH == 16 && row % 2;
+    const bool odd = odd_row<CH>();
     const uint32_t words = smem_addr(acc + ch) - cc.rec;
-    BwdOut out{g_values ? g_values + c * (p.N + 1) : nullptr, g_knots ? g_knots + c * (p.N + 1) : nullptr,
-               words + (odd ? 4 * CH : 0), words + (odd ? 0 : 4 * CH), scale, odd};
+    const BwdOut out{words + (odd ? 4 * CH : 0), words + (odd ? 0 : 4 * CH), scale, odd};
     EndSums ends{0.0f, 0.0f};
     int64_t r = r0 + row;
     const int64_t step = (int64_t)RP * p.C;
@@ -581,9 +644,10 @@ __device__ __forceinline__ void chan_bwd_rows(const ChanArgs& p, int64_t c0, int
         pg += kBwdTail * step;
         po += kBwdTail * step;
     }
-    if (out.gv) {
-        if (ends.left != 0.0f) atomicAdd(out.gv, ends.left);
-        if (ends.right != 0.0f) atomicAdd(out.gv + p.N, ends.right);
+    if (s_bwd.gv) {
+        float* gv = s_bwd.gv + ch * (p.N + 1);
+        if (ends.left != 0.0f) atomicAdd(gv, ends.left);
+        if (ends.right != 0.0f) atomicAdd(gv + p.N, ends.right);
     }
 }
 
@@ -604,21 +668,22 @@ __device__ __forceinline__ void add_global(float* dst, const float* src, int n)
 // at a time (one reduction per lane and address, to 32 different lines per
 // warp, took 15000 clocks for 16 channels of 257 knots).
 template <int CH>
-__device__ __forceinline__ void flush_tile(const ChanArgs& p, int64_t c0, const float4* rec, int* acc, float unit,
+__device__ __forceinline__ void flush_tile(const ChanArgs& p, int64_t c0, const float4* rec, int* acc,
                                            float* stage, float* g_values, float* g_knots)
 {
     __syncthreads();
     const int N = p.N, n1 = N + 1;
     const int ch = threadIdx.x % CH, nch = (int)min((int64_t)CH, p.C - c0);
+    const float unit = s_bwd.unit[ch];
     float* stage_k = stage + (CH * n1 + 3) / 4 * 4;
-    // h 2^17 + l of word w, cleared: with l's carry moved to h, one conversion is
+    // h 2^19 + l of word w, cleared: with l's carry moved to h, one conversion is
     // exact (or rounds below half an ulp) and nothing cancels
     auto take = [&](int i, int w) {
         int *ph = acc + (i * 4 + w) * CH + ch, *pl = ph + 2 * CH;
-        const int l = *pl, h = *ph + (l >> 17);
+        const int l = *pl, h = *ph + (l >> kDigitBits);
         *ph = 0;
         *pl = 0;
-        return __fmaf_rn((float)h, 0x1p17f, (float)(l & 0x1ffff)) * unit;
+        return __fmaf_rn((float)h, kDigit, (float)(l & ((1 << kDigitBits) - 1))) * unit;
     };
     if (ch < nch)
         for (int j = threadIdx.x / CH; j <= N; j += kChThreads / CH) {
@@ -639,29 +704,54 @@ __device__ __forceinline__ void flush_tile(const ChanArgs& p, int64_t c0, const 
     if (stage && g_knots) add_global(g_knots + c0 * n1, stage_k, nch * n1);
 }
 
+// Whether a word of the tile's sums could wrap in the next kSegRows rows.
+template <int CH>
+__device__ __forceinline__ bool near_full(const ChanArgs& p, const int* acc)
+{
+    __syncthreads();
+    bool full = false;
+    for (int i = threadIdx.x; i < (p.N + 2) * CH; i += kChThreads) {
+        const int4 v = reinterpret_cast<const int4*>(acc)[i];
+        for (const int w : {v.x, v.y, v.z, v.w}) full = full || (unsigned)(w + kFullWord) > 2u * kFullWord;
+    }
+    return __syncthreads_or(full);
+}
+
 template <typename IO, int CH>
 __global__ void __launch_bounds__(kChThreads, 1) channels_backward_kernel(const ChanArgs p, const IO* x, const IO* gy,
                                                                           IO* gx, float* g_values, float* g_knots)
 {
     extern __shared__ float4 s_ch[];
-    __shared__ BwdShared sh;
     float4* rec = s_ch;
     int* acc = reinterpret_cast<int*>(rec + (size_t)(p.N + 2) * CH);
     float2* cells = reinterpret_cast<float2*>(acc + (size_t)(p.N + 2) * 4 * CH);
     for (int i = threadIdx.x; i < (p.N + 2) * 4 * CH; i += kChThreads) acc[i] = 0;
+    if (threadIdx.x == 0) {
+        s_bwd.rec = smem_addr(rec);
+        s_bwd.N = p.N;
+    }
     for_each_range<CH>(p, [&](int64_t tile, int64_t r0, int64_t r1) {
+        const int64_t c0 = tile * CH;
+        const int ch = threadIdx.x % CH;
         __syncthreads();  // nobody reads the previous tile any more
-        if (threadIdx.x < CH) sh.esum[threadIdx.x] = sh.ecnt[threadIdx.x] = 0;
-        const float g = sample_gy<IO, CH>(p, tile * CH, gy);
-        build_tile<CH, true>(p, tile * CH, cells, rec, &sh.bad, [&] { sum_exponents<CH>(g, &sh); });
-        if (threadIdx.x == 0 && sh.bad) atomicOr(p.status, 1);
-        const int F = fix_exponent<CH>(&sh, threadIdx.x % CH);
-        const float scale = exp2_int(F), unit = exp2_int(-F);
-        for (int64_t r = r0; r < r1; r += kFlushRows) {
-            chan_bwd_rows<IO, CH>(p, tile * CH, r, min(r1, r + kFlushRows), cells, rec, acc, scale, x, gy, gx, g_values,
-                                  g_knots);
-            flush_tile<CH>(p, tile * CH, rec, acc, unit,
-                           r + kFlushRows < r1 ? nullptr : reinterpret_cast<float*>(cells), g_values, g_knots);
+        if (threadIdx.x < CH) s_bwd.emax[threadIdx.x] = kNoSample;
+        if (threadIdx.x == 0) {
+            s_bwd.gv = g_values ? g_values + c0 * (p.N + 1) : nullptr;
+            s_bwd.gk = g_knots ? g_knots + c0 * (p.N + 1) : nullptr;
+        }
+        const float gs = sample_gy<IO, CH>(p, c0, gy);
+        build_tile<CH, true>(p, c0, cells, rec, &s_bwd.bad, [&] { max_exponents<CH>(gs); });
+        if (threadIdx.x == 0 && s_bwd.bad) atomicOr(p.status, 1);
+        const int F = fix_exponent<CH>(ch);
+        const float scale = exp2_int(F);
+        if (threadIdx.x < CH) s_bwd.unit[ch] = exp2_int(-F);
+        for (int64_t r = r0; r < r1;) {
+            const int64_t from = r;
+            r = min(r1, r + kSegRows);
+            chan_bwd_rows<IO, CH>(p, c0, from, r, cells, rec, acc, scale, x, gy, gx);
+            if (r == r1 || near_full<CH>(p, acc))
+                flush_tile<CH>(p, c0, rec, acc, r < r1 ? nullptr : reinterpret_cast<float*>(cells), g_values,
+                               g_knots);
         }
     });
 }

@@ -1,0 +1,91 @@
+"""Channel-wise table gradients relative to their own terms: every knot's sum is
+held to GRAD_REL of the absolute sum of what was added to it, whatever the
+channel's other gradients are, in tiles of every width (16, 8 and 4 channels);
+sums that fill the integer words."""
+import numpy as np
+import pytest
+
+import oracle
+from pwl_testutil import GRAD_REL
+
+pytestmark = pytest.mark.gpu
+
+torch = pytest.importorskip("torch")
+
+# (channels, intervals, k_cells): 16-, 8- and 4-channel tiles in the backward
+# (1600 requested cells leave 8 channels, 640 intervals 4)
+WIDTHS = [(20, 40, 0), (20, 40, 1600), (10, 640, 0)]
+
+
+@pytest.fixture(scope="module")
+def pwl():
+    import paper_1510_02975_gb300 as m
+    from paper_1510_02975_gb300 import _build
+    _build.build()
+    return m
+
+
+def _tables(C, N, seed=0):
+    rng = np.random.default_rng(seed)
+    knots = np.tile(np.linspace(-2.0, 3.0, N + 1), (C, 1))
+    knots[:, 1:-1] += rng.uniform(-0.4, 0.4, (C, N - 1)) * (5.0 / N)
+    return knots.astype(np.float32), rng.normal(size=(C, N + 1)).astype(np.float32)
+
+
+def _data(case, C, N, R, knots):
+    rng = np.random.default_rng(3)
+    x = rng.uniform(-2.2, 3.2, (R, C)).astype(np.float32)
+    g = rng.normal(size=(R, C))
+    j = N // 2
+    if case.startswith("bin"):  # one interval's gradients 2^-k of the channel's
+        lo, hi = knots[:, j - 1], knots[:, j + 1]
+        g = np.where((x >= lo) & (x < hi), g * 2.0 ** -int(case[3:]), g)
+    elif case == "decades":  # |gy| a function of x, over 12 decades
+        g *= 10.0 ** (12 * (np.clip(x, -2, 3) + 2) / 5 - 12)
+    elif case == "sparse_channels":  # 1% nonzero, each channel its own magnitude
+        g *= (rng.random((R, C)) < 0.01) * 10.0 ** -(np.arange(C) % 13)
+    elif case == "lognormal":
+        g *= np.exp(2 * rng.normal(size=(R, C)))
+    elif case == "beside_a_knot":  # no point near knot j: both intervals' within 2^-16 of their far ends
+        l, m, r = knots[:, j - 1], knots[:, j], knots[:, j + 1]
+        t = np.float32(2.0 ** -16) * rng.random((R, C)).astype(np.float32)
+        x = np.where((x > l) & (x < m), l + (m - l) * t, np.where((x >= m) & (x < r), r - (r - m) * t, x))
+    return x, g.astype(np.float32)
+
+
+def _grads(pwl, knots, values, x, gy, k_cells=0):
+    kt, vt, xt, gt = (torch.tensor(a, device="cuda") for a in (knots, values, x, gy))
+    gv, gk = torch.zeros_like(vt), torch.zeros_like(kt)
+    gx = pwl.pwl_channels_backward(kt, vt, xt, gt, None, gv, gk, k_cells=k_cells)
+    return gx.cpu().numpy(), gv.cpu().numpy(), gk.cpu().numpy()
+
+
+def _check(knots, values, x, gy, gv, gk, channels):
+    for c in channels:
+        _, rv, rk, av, ak = oracle.evaluate_grad(knots[c].astype(np.float64), values[c].astype(np.float64),
+                                                 x[:, c].astype(np.float64), gy[:, c].astype(np.float64))
+        assert np.all(np.abs(gv[c] - rv) <= GRAD_REL * av), (c, np.max(np.abs(gv[c] - rv) / np.maximum(av, 1e-300)))
+        assert np.all(np.abs(gk[c] - rk) <= GRAD_REL * ak), (c, np.max(np.abs(gk[c] - rk) / np.maximum(ak, 1e-300)))
+
+
+@pytest.mark.parametrize("C,N,k_cells", WIDTHS, ids=["16", "8", "4"])
+@pytest.mark.parametrize("case", ["normal", "bin16", "bin20", "bin26", "bin31", "decades", "sparse_channels", "lognormal",
+                                  "beside_a_knot"])
+def test_every_knot_relative_to_its_own_terms(pwl, case, C, N, k_cells):
+    knots, values = _tables(C, N)
+    x, gy = _data(case, C, N, 20000, knots)
+    _, gv, gk = _grads(pwl, knots, values, x, gy, k_cells)
+    _check(knots, values, x, gy, gv, gk, range(C))
+
+
+@pytest.mark.parametrize("N", [1, 5])
+def test_sums_that_fill_the_words(pwl, N):
+    # a CTA takes all rows of a tile; gradients of one size, the largest of its
+    # binade, in one interval: the words grow as fast as samples let them
+    C, R = 2432, 30001
+    knots, values = _tables(C, N)
+    x = np.repeat((0.25 * knots[:, :1] + 0.75 * knots[:, 1:2]).T.astype(np.float32), R, axis=0)
+    gy = np.full((R, C), 1.9999999, dtype=np.float32)
+    gy[-1] = 7.5  # beyond the samples, inside the range
+    _, gv, gk = _grads(pwl, knots, values, x, gy)
+    _check(knots, values, x, gy, gv, gk, [0, 1, 15, 16, 1000, 2431])
