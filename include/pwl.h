@@ -500,9 +500,10 @@ pwl_status pwl_channels_forward(const float* d_knots, const float* d_values, int
  * and for every channel d_g_values[c, j] += sum over rows of gy dy/dv_j,
  * d_g_knots[c, j] += sum of gy dy/dx_j (the formulas of pwl_eval_backward;
  * either may be NULL).  A CTA's sums hold every term to 2^-18 of itself or
- * finer and add without further rounding; the CTAs' sums and terms far from
- * the channel's largest are added with FP32 atomics, order-dependent at FP32
- * rounding.  k_cells as in the forward.                                    */
+ * finer and add without further rounding, or are FP32 sums; the CTAs' sums
+ * and terms far from the channel's largest are added with FP32 atomics,
+ * order-dependent at FP32 rounding.  d_gx may be d_gy.  k_cells as in the
+ * forward.                                                                 */
 pwl_status pwl_channels_backward(const float* d_knots, const float* d_values, int64_t n_channels,
                                  int64_t n_intervals, int64_t k_cells, const float* d_x, const float* d_gy,
                                  float* d_gx, float* d_g_values, float* d_g_knots, int64_t rows,

@@ -370,28 +370,45 @@ __global__ void __launch_bounds__(kChThreads, 1) channels_forward_kernel(const C
 // tile's rows they become g_v[j] += A_{j+1} + B_j (+ clamped terms) and
 // g_x[j] += -s_{j+1} A_{j+1} - s_j B_j, added to the global gradients.
 //
-// The sums are fixed point, in two 32-bit words each: a term v in units of 2^-F is
-// h 2^19 + l + rest with h = rint(v 2^-19) (by adding 1.5 2^23, which needs no
-// conversion) and l = rint(v - h 2^19), both added with native integer
-// shared-memory atomics that return nothing.  An FP32 shared-memory add is a
-// compare-and-swap loop in software (about 10 instructions, 2.6 adds per clock and
-// SM against more than 9 for int32).  |v| < 2^37 keeps h and l within 2^18, so 6912
-// rows add less than 2^31 - 2^28 to a word; every 6912 rows the words are looked
-// over and the tile's sums flushed where one has passed 2^28.
-// A term of 2^17 units or more is rounded at 2^-18 of itself or finer (from 2^23 on
-// it is exact).  The rest of a smaller one, which the words do not hold, goes to the
-// global gradients in FP32, and so does a term beyond 2^37: every sum is accurate
-// relative to its own terms, however small they are beside the channel's other
-// gradients.
+// An FP32 shared-memory add is a compare-and-swap loop in software (about 10
+// instructions, 2.6 adds per clock and SM against more than 9 for int32), so a
+// range of rows takes one of two forms of the sums:
 //
-// F comes, per channel, from the largest of 64 (128, 256) sampled |gy|, spread over
-// the rows; terms of up to 4 to 8 times that fit.
+//   fixed point, two 32-bit words per sum: a term v in units of 2^-F is
+//     h 2^19 + l + rest with h = rint(v 2^-19) (by adding 1.5 2^23, which needs
+//     no conversion) and l = rint(v - h 2^19), both added with native integer
+//     atomics that return nothing.  |v| < 2^37 keeps h and l within 2^18, so
+//     6912 rows add less than 2^31 - 2^28 to a word; every 6912 rows the words
+//     are looked over and the tile's sums flushed where one has passed 2^28.
+//     A term of 2^17 units or more is rounded at 2^-18 of itself or finer (from
+//     2^23 on it is exact).  The rest of a smaller one, which the words do not
+//     hold, goes to the global gradients in FP32, and so does a term beyond 2^37:
+//     every sum is accurate relative to its own terms, however small they are
+//     beside the channel's other gradients.
+//   FP32, one word per sum: where more than kSlowSamples of the range's 1024
+//     sampled elements have such a term, or none is nonzero.
+//
+// F comes, per channel, from the largest of 64 (128, 256) sampled |gy|, spread
+// over the range's rows at irregular distances (the first rows of sequences and
+// the like are not typical); terms of up to 4 to 8 times that fit.
+//
+// [65536, 4096] x 257 knots: 840 us with normal gradients, the same where half or
+// 99% are zero or every 1024th row is, 890-950 log-normal (sigma 1 to 3), over 10
+// decades along x, with one interval's 2^-26 as large, 99.9% zero or a third of the
+// points outside.  (One unit from the mean exponent of the rows R k / 64, four
+// global adds for every element above it: 690, but 1860-3410 log-normal, 6300 where
+// those rows are zero, 1480 with a third outside.)  In FP32 alone: 850-895 for every
+// distribution, but 2860 where all points of a channel fall into one interval (840
+// in fixed point), 1565 with 7 intervals (790), and 5 to 27 times the rounding
+// error (6e-8).  Of the 840, the test for small terms takes 55 and the look at the
+// words 35.
 constexpr int kDigitBits = 19;
 constexpr int kRangeBits = 37;                                // terms below 2^37 units
 constexpr float kFixLimit = 0x1p37f;
 constexpr unsigned kSmallKey = 2u * ((127 + 17) << 23) - 2u;  // small_key of 2^17
 constexpr int kSegRows = 6912;                                // whole passes of every tile width (64, 128, 256 rows)
 constexpr int kFullWord = 1 << 28;
+constexpr int kSlowSamples = 6;  // (log-normal of sigma 2: 1320 us with 16)
 constexpr float kMagic = 0x1.8p23f;
 constexpr int kMagicBits = 0x4B400000;
 constexpr float kDigit = 0x1p19f, kPerDigit = 0x1p-19f;
@@ -409,12 +426,21 @@ struct BwdShared {
 __shared__ BwdShared s_bwd;
 constexpr int kNoSample = -1000;
 
-// gy of this thread's channel at its sampled row (0 past the last channel)
+// This thread's sampled element: its channel, a row of its stratum of [r0, r1).
+// The rows are the CTA's own, so that gx may overwrite gy.
 template <typename IO, int CH>
-__device__ __forceinline__ float sample_gy(const ChanArgs& p, int64_t c0, const IO* gy)
+__device__ __forceinline__ void sample(const ChanArgs& p, int64_t c0, int64_t r0, int64_t r1, const IO* x,
+                                       const IO* gy, float& xs, float& gs)
 {
-    const int64_t c = c0 + threadIdx.x % CH, r = p.R * (int64_t)(threadIdx.x / CH) / (kChThreads / CH);
-    return c < p.C ? to_f32<IO>(__ldcg(gy + r * p.C + c)) : 0.0f;
+    constexpr int S = kChThreads / CH;
+    const int64_t c = c0 + threadIdx.x % CH, n = r1 - r0, s = threadIdx.x / CH;
+    xs = gs = 0.0f;
+    if (c >= p.C) return;
+    const unsigned h = ((unsigned)c0 * 1024u + threadIdx.x) * 0x9E3779B9u;  // multiples of the golden ratio mod 1
+    const int64_t lo = n * s / S, w = min(n * (s + 1) / S - lo, (int64_t)0x7fffffff);
+    const int64_t at = (r0 + lo + (int64_t)((uint64_t)h * (uint64_t)w >> 32)) * p.C + c;
+    xs = to_f32<IO>(__ldcg(x + at));
+    gs = to_f32<IO>(__ldcg(gy + at));
 }
 // the samples' binary exponents (nonzero finite ones) into the channels' maxima
 template <int CH>
@@ -428,14 +454,14 @@ __device__ __forceinline__ void max_exponents(float g)
 
 // F of a channel: from its own samples, else from the tile's (whose unit may be
 // far too coarse for it; then its terms count as small).  2^F and 2^-F are
-// normal FP32 numbers.
+// normal FP32 numbers.  kNoSample if the tile has no nonzero sample.
 template <int CH>
 __device__ __forceinline__ int fix_exponent(int ch)
 {
     int e = s_bwd.emax[ch];
     if (e == kNoSample)
         for (int q = 0; q < CH; ++q) e = max(e, s_bwd.emax[q]);
-    return e == kNoSample ? 126 : min(max(kRangeBits - 3 - e, -100), 126);
+    return e == kNoSample ? kNoSample : min(max(kRangeBits - 3 - e, -100), 126);
 }
 __device__ __forceinline__ float exp2_int(int e) { return __int_as_float((e + 127) << 23); }
 
@@ -464,6 +490,11 @@ __device__ __forceinline__ float fix_rest(float v)
     const float low = fix_high(v, m);
     return low - __int2float_rn(__float2int_rn(low));
 }
+__device__ __forceinline__ void float_add(uint32_t at, float v)
+{
+    if (v != 0.0f) asm volatile("red.shared.add.f32 [%0], %1;" ::"r"(at), "f"(v) : "memory");
+}
+
 // FP32 sums of the gradients w.r.t. the end values of clamped elements
 struct EndSums {
     float left, right;
@@ -510,7 +541,7 @@ __device__ __noinline__ void add_rests(float t1, float t2, uint32_t at, float s)
 }
 
 // G elements: gx in place of g.
-template <int CH, int G>
+template <int CH, int G, bool FLOAT>
 __device__ __forceinline__ void chan_bwd(const float (&x)[G], float (&g)[G], const ChanConst<CH>& cc, const BwdOut& o,
                                          EndSums& ends)
 {
@@ -542,37 +573,47 @@ __device__ __forceinline__ void chan_bwd(const float (&x)[G], float (&g)[G], con
         t1 = gq * (fabsf(p1 - xc[q]) * r[q].y);
         t2 = gq * (fabsf(p2 - xc[q]) * r[q].y);
     };
-    float gs[G];
-    unsigned small = ~0u;
-#pragma unroll
-    for (int q = 0; q < G; ++q) {
-        gs[q] = g[q] * o.scale;
-        fits = fits && fabsf(gs[q]) < kFixLimit;
-    }
-    if (!fits) {
+    if constexpr (FLOAT) {
 #pragma unroll
         for (int q = 0; q < G; ++q) {
-            if (fabsf(gs[q]) < kFixLimit) continue;
             float t1, t2;
             terms(q, g[q], t1, t2);
-            add_global_terms<CH>(t1, t2, at[q], r[q].z);
-            gs[q] = 0.0f;
+            float_add(at[q] + o.first, t1);
+            float_add(at[q] + o.second, t2);
         }
-    }
+    } else {
+        float gs[G];
+        unsigned small = ~0u;
 #pragma unroll
-    for (int q = 0; q < G; ++q) {
-        float t1, t2;
-        terms(q, gs[q], t1, t2);
-        fix_add<8 * CH>(at[q] + o.first, t1);
-        fix_add<8 * CH>(at[q] + o.second, t2);
-        small = min(small, min(small_key(t1), small_key(t2)));
-    }
-    if (small < kSmallKey) {
+        for (int q = 0; q < G; ++q) {
+            gs[q] = g[q] * o.scale;
+            fits = fits && fabsf(gs[q]) < kFixLimit;
+        }
+        if (!fits) {
+#pragma unroll
+            for (int q = 0; q < G; ++q) {
+                if (fabsf(gs[q]) < kFixLimit) continue;
+                float t1, t2;
+                terms(q, g[q], t1, t2);
+                add_global_terms<CH>(t1, t2, at[q], r[q].z);
+                gs[q] = 0.0f;
+            }
+        }
 #pragma unroll
         for (int q = 0; q < G; ++q) {
             float t1, t2;
             terms(q, gs[q], t1, t2);
-            add_rests<CH>(t1, t2, at[q], r[q].z);
+            fix_add<8 * CH>(at[q] + o.first, t1);
+            fix_add<8 * CH>(at[q] + o.second, t2);
+            small = min(small, min(small_key(t1), small_key(t2)));
+        }
+        if (small < kSmallKey) {
+#pragma unroll
+            for (int q = 0; q < G; ++q) {
+                float t1, t2;
+                terms(q, gs[q], t1, t2);
+                add_rests<CH>(t1, t2, at[q], r[q].z);
+            }
         }
     }
 #pragma unroll
@@ -584,7 +625,19 @@ __device__ __forceinline__ void chan_bwd(const float (&x)[G], float (&g)[G], con
     }
 }
 
-template <typename IO, int CH>
+// Whether the fixed-point form of a sampled element needs a global add.
+template <int CH>
+__device__ __forceinline__ bool slow_sample(float x, float g, const ChanConst<CH>& cc, float scale)
+{
+    float xc[1] = {fminf(fmaxf(x, cc.a), cc.b)};
+    float4 r[1];
+    uint32_t at[1];
+    chan_lookup<CH, 1>(xc, cc, r, at);
+    const float gs = g * scale, t1 = gs * (fabsf(r[0].w - xc[0]) * r[0].y), t2 = gs * (fabsf(r[0].x - xc[0]) * r[0].y);
+    return x == xc[0] && (!(fabsf(gs) < kFixLimit) || min(small_key(t1), small_key(t2)) < kSmallKey);
+}
+
+template <typename IO, int CH, bool FLOAT>
 __device__ __forceinline__ void chan_bwd_rows(const ChanArgs& p, int64_t c0, int64_t r0, int64_t r1,
                                               const float2* cells, const float4* rec, int* acc, float scale,
                                               const IO* __restrict__ x, const IO* __restrict__ gy,
@@ -619,7 +672,7 @@ __device__ __forceinline__ void chan_bwd_rows(const ChanArgs& p, int64_t c0, int
                 xf[q] = to_f32<IO>(xv[u + q]);
                 gf[q] = to_f32<IO>(gv[u + q]);
             }
-            chan_bwd<CH, G>(xf, gf, cc, out, ends);
+            chan_bwd<CH, G, FLOAT>(xf, gf, cc, out, ends);
 #pragma unroll
             for (int q = 0; q < G; ++q) st_cs(po + (u + q) * step, from_f32<IO>(gf[q]));
         }
@@ -636,7 +689,7 @@ __device__ __forceinline__ void chan_bwd_rows(const ChanArgs& p, int64_t c0, int
             xf[u] = u < rem ? to_f32<IO>(__ldcg(px + u * step)) : cc.a;
             gf[u] = u < rem ? to_f32<IO>(__ldcg(pg + u * step)) : 0.0f;
         }
-        chan_bwd<CH, kBwdTail>(xf, gf, cc, out, ends);
+        chan_bwd<CH, kBwdTail, FLOAT>(xf, gf, cc, out, ends);
 #pragma unroll
         for (int u = 0; u < kBwdTail; ++u)
             if (u < rem) st_cs(po + u * step, from_f32<IO>(gf[u]));
@@ -649,6 +702,15 @@ __device__ __forceinline__ void chan_bwd_rows(const ChanArgs& p, int64_t c0, int
         if (ends.left != 0.0f) atomicAdd(gv, ends.left);
         if (ends.right != 0.0f) atomicAdd(gv + p.N, ends.right);
     }
+}
+
+// (out of line: inlined, it costs the fixed-point loop registers)
+template <typename IO, int CH>
+__device__ __noinline__ void chan_bwd_rows_float(const ChanArgs& p, int64_t c0, int64_t r0, int64_t r1,
+                                                 const float2* cells, const float4* rec, int* acc, const IO* x,
+                                                 const IO* gy, IO* gx)
+{
+    chan_bwd_rows<IO, CH, true>(p, c0, r0, r1, cells, rec, acc, 1.0f, x, gy, gx);
 }
 
 // n floats from shared memory (16-byte aligned) added to global ones, whole
@@ -668,7 +730,7 @@ __device__ __forceinline__ void add_global(float* dst, const float* src, int n)
 // at a time (one reduction per lane and address, to 32 different lines per
 // warp, took 15000 clocks for 16 channels of 257 knots).
 template <int CH>
-__device__ __forceinline__ void flush_tile(const ChanArgs& p, int64_t c0, const float4* rec, int* acc,
+__device__ __forceinline__ void flush_tile(const ChanArgs& p, int64_t c0, const float4* rec, int* acc, bool flt,
                                            float* stage, float* g_values, float* g_knots)
 {
     __syncthreads();
@@ -676,13 +738,15 @@ __device__ __forceinline__ void flush_tile(const ChanArgs& p, int64_t c0, const 
     const int ch = threadIdx.x % CH, nch = (int)min((int64_t)CH, p.C - c0);
     const float unit = s_bwd.unit[ch];
     float* stage_k = stage + (CH * n1 + 3) / 4 * 4;
-    // h 2^19 + l of word w, cleared: with l's carry moved to h, one conversion is
-    // exact (or rounds below half an ulp) and nothing cancels
+    // a sum, cleared: its FP32 word, or h 2^19 + l of its two words (with l's carry
+    // moved to h, one conversion is exact, or rounds below half an ulp, and nothing
+    // cancels)
     auto take = [&](int i, int w) {
         int *ph = acc + (i * 4 + w) * CH + ch, *pl = ph + 2 * CH;
-        const int l = *pl, h = *ph + (l >> kDigitBits);
+        const int hi = *ph, l = *pl, h = hi + (l >> kDigitBits);
         *ph = 0;
         *pl = 0;
+        if (flt) return __int_as_float(hi);
         return __fmaf_rn((float)h, kDigit, (float)(l & ((1 << kDigitBits) - 1))) * unit;
     };
     if (ch < nch)
@@ -739,18 +803,25 @@ __global__ void __launch_bounds__(kChThreads, 1) channels_backward_kernel(const 
             s_bwd.gv = g_values ? g_values + c0 * (p.N + 1) : nullptr;
             s_bwd.gk = g_knots ? g_knots + c0 * (p.N + 1) : nullptr;
         }
-        const float gs = sample_gy<IO, CH>(p, c0, gy);
+        float xs, gs;
+        sample<IO, CH>(p, c0, r0, r1, x, gy, xs, gs);
         build_tile<CH, true>(p, c0, cells, rec, &s_bwd.bad, [&] { max_exponents<CH>(gs); });
         if (threadIdx.x == 0 && s_bwd.bad) atomicOr(p.status, 1);
         const int F = fix_exponent<CH>(ch);
-        const float scale = exp2_int(F);
-        if (threadIdx.x < CH) s_bwd.unit[ch] = exp2_int(-F);
+        bool slow = F == kNoSample;
+        const float scale = slow ? 1.0f : exp2_int(F);
+        if (threadIdx.x < CH) s_bwd.unit[ch] = slow ? 1.0f : exp2_int(-F);
+        if (c0 + ch < p.C && !slow) slow = slow_sample<CH>(xs, gs, ChanConst<CH>(p, cells, rec, ch), scale);
+        const bool flt = __syncthreads_count(slow) > kSlowSamples;
         for (int64_t r = r0; r < r1;) {
             const int64_t from = r;
-            r = min(r1, r + kSegRows);
-            chan_bwd_rows<IO, CH>(p, c0, from, r, cells, rec, acc, scale, x, gy, gx);
+            r = flt ? r1 : min(r1, r + kSegRows);
+            if (flt)
+                chan_bwd_rows_float<IO, CH>(p, c0, from, r, cells, rec, acc, x, gy, gx);
+            else
+                chan_bwd_rows<IO, CH, false>(p, c0, from, r, cells, rec, acc, scale, x, gy, gx);
             if (r == r1 || near_full<CH>(p, acc))
-                flush_tile<CH>(p, c0, rec, acc, r < r1 ? nullptr : reinterpret_cast<float*>(cells), g_values,
+                flush_tile<CH>(p, c0, rec, acc, flt, r < r1 ? nullptr : reinterpret_cast<float*>(cells), g_values,
                                g_knots);
         }
     });

@@ -1,7 +1,7 @@
 """Channel-wise table gradients relative to their own terms: every knot's sum is
 held to GRAD_REL of the absolute sum of what was added to it, whatever the
 channel's other gradients are, in tiles of every width (16, 8 and 4 channels);
-sums that fill the integer words."""
+sums that fill the integer words; gx written over gy."""
 import numpy as np
 import pytest
 
@@ -53,10 +53,10 @@ def _data(case, C, N, R, knots):
     return x, g.astype(np.float32)
 
 
-def _grads(pwl, knots, values, x, gy, k_cells=0):
+def _grads(pwl, knots, values, x, gy, k_cells=0, out=None):
     kt, vt, xt, gt = (torch.tensor(a, device="cuda") for a in (knots, values, x, gy))
     gv, gk = torch.zeros_like(vt), torch.zeros_like(kt)
-    gx = pwl.pwl_channels_backward(kt, vt, xt, gt, None, gv, gk, k_cells=k_cells)
+    gx = pwl.pwl_channels_backward(kt, vt, xt, gt, gt if out == "gy" else None, gv, gk, k_cells=k_cells)
     return gx.cpu().numpy(), gv.cpu().numpy(), gk.cpu().numpy()
 
 
@@ -89,3 +89,52 @@ def test_sums_that_fill_the_words(pwl, N):
     gy[-1] = 7.5  # beyond the samples, inside the range
     _, gv, gk = _grads(pwl, knots, values, x, gy)
     _check(knots, values, x, gy, gv, gk, [0, 1, 15, 16, 1000, 2431])
+
+
+def test_gx_over_gy(pwl):
+    C, N, R = 200, 30, 40000
+    knots, values = _tables(C, N)
+    values *= 1e7  # gx far from gy in size
+    x, gy = _data("normal", C, N, R, knots)
+    ref = _grads(pwl, knots, values, x, gy)
+    gx, gv, gk = _grads(pwl, knots, values, x, gy, out="gy")
+    assert np.array_equal(gx, ref[0])
+    _check(knots, values, x, gy, gv, gk, range(0, C, 7))
+
+
+@pytest.mark.parametrize("case", ["lognormal", "first_rows_zero", "sparse", "very_sparse", "small_bin", "outside"])
+def test_time_does_not_hang_on_the_gradients(pwl, case):
+    # events around the backward of [65536, 1024] x 257 knots: other distributions of gy, and a
+    # third of the points outside the domain, within half as much again as N(0, 1) gradients
+    C, N, R = 1024, 256, 65536
+    knots, values = (torch.tensor(a, device="cuda") for a in _tables(C, N))
+    g = torch.Generator(device="cuda").manual_seed(1)
+    x = torch.randn(R, C, generator=g, device="cuda")
+    gy = torch.randn(R, C, generator=g, device="cuda")
+    gx, gv, gk = torch.empty_like(x), torch.zeros_like(values), torch.zeros_like(knots)
+
+    def us(x, gy):
+        times = []
+        for _ in range(8):
+            a, b = (torch.cuda.Event(enable_timing=True) for _ in range(2))
+            a.record()
+            pwl.pwl_channels_backward(knots, values, x, gy, gx, gv, gk)
+            b.record()
+            torch.cuda.synchronize()
+            times.append(a.elapsed_time(b) * 1e3)
+        return sorted(times)[3]
+
+    x.clamp_(-1.99, 2.99)
+    base = us(x, gy)
+    if case == "lognormal":
+        gy *= torch.exp(2 * torch.randn(R, C, generator=g, device="cuda"))
+    elif case == "first_rows_zero":
+        gy.view(-1, 1024, C)[:, 0] = 0
+    elif case in ("sparse", "very_sparse"):
+        gy *= torch.rand(R, C, generator=g, device="cuda") < (0.01 if case == "sparse" else 0.001)
+    elif case == "small_bin":
+        gy[(x > 0.5) & (x < 0.6)] *= 2.0 ** -26
+    else:
+        x[torch.rand(R, C, generator=g, device="cuda") < 0.33] = 5.0
+    t = us(x, gy)
+    assert t <= 1.5 * base, (t, base)
