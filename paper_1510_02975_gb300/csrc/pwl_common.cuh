@@ -178,11 +178,12 @@ inline pwl_func prepared(const pwl_func& f)
     return g;
 }
 // a / s from r = 1/s rounded: the product and one correction by its remainder,
-// three FP64 operations (a division's rounding, for about ten)
+// three FP64 operations (a division's rounding, for about ten).  A quotient beyond
+// the range is the division's infinity: its remainder would be NaN.
 __device__ __forceinline__ double ratio(double a, double s, double r)
 {
-    if (__double2hiint(r) == 0) return a / s;
     const double q = a * r;
+    if (__double2hiint(r) == 0 || (__double2hiint(q) & 0x7ff00000) == 0x7ff00000) return a / s;
     return fma(fma(-q, s, a), r, q);
 }
 __device__ __forceinline__ float ratio(float a, float s, double) { return a / s; }
