@@ -88,7 +88,7 @@ struct ProjectPlan {
     const double* knots;
     double* values;
     double2* lr;           // per interval: (int f phi_left, int f phi_right)
-    double* cr;            // solver scratch: 4 doubles per knot and 128 per function
+    double* cr;            // solver scratch: 4 doubles per knot (and 128 per function of several)
     int solver;            // 0: cyclic reduction, one CTA per function; 1: partitioned Thomas, one warp per function
     const int* order;      // solver 1: the order in which warps take the functions (NULL: 0..F-1)
 };

@@ -507,9 +507,11 @@ const GaussLegendre& gauss_legendre_rule(int Q)
 
 size_t project_scratch_bytes(int64_t total_knots, int64_t total_intervals)
 {
-    // (total_knots - total_intervals functions)
+    // the padding of solver_scratch() for more than one function only: what a
+    // single projection asks of its caller stays 4 doubles per row
+    const int64_t F = total_knots - total_intervals;
     return align256(sizeof(double2) * (size_t)total_intervals) +
-           align256(sizeof(double) * 4 * (size_t)(total_knots + 32 * (total_knots - total_intervals)));
+           align256(sizeof(double) * 4 * (size_t)(total_knots + (F > 1 ? 32 * F : 0)));
 }
 
 void project_carve_scratch(ProjectPlan& p, void* scratch)
