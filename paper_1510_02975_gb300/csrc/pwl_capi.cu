@@ -52,18 +52,26 @@ static bool alloc_allowed()
 
 // Base blocks of destroyed tables, kept for the next build: cudaMalloc and
 // cudaFree take ~30 us each, and a table has two blocks (120 us of the 430 from f
-// to a table and its first evaluation).  The other block, the index, goes back by
-// cudaFree, which waits for everything on the device, so any stream may write to
-// the kept block afterwards.  That wait is not cudaDeviceSynchronize: it would
-// end every graph capture that another thread, or a relaxed one of this thread,
-// has under way, which cudaFree leaves alone.  At most kCacheBlocks blocks of
-// kCacheBlock bytes at most per device; they go back to the device when an
-// allocation fails.
+// to a table and its first evaluation).  At most kCacheBlocks blocks of kCacheBlock
+// bytes at most per context; they go back when an allocation fails.
+//
+// A kept block may be written from any stream at once, so nothing may be running
+// on it any more.  That rests on cudaFree of the table's other block, the index:
+// managing memory with cudaMalloc and cudaFree synchronizes across all executing
+// streams of the context (the CUDA programming guide, where it introduces the
+// stream-ordered allocator; the tables' tests run with evaluations in flight on
+// other streams).  cudaDeviceSynchronize would also end every graph capture that
+// another thread, or a relaxed one of this thread, has under way, which cudaFree
+// leaves alone.  Both the wait and the address hold for one context only: a block
+// is kept and reused where the current context is the one the table was built in
+// (not another device's or another context of the same device, nor the one that
+// follows a cudaDeviceReset), known by the driver's context id, which no later
+// context gets again.
 namespace {
 constexpr size_t kCacheBlock = (size_t)1 << 20;
 constexpr size_t kCacheBlocks = 16;
 struct CachedBlock {
-    int device;
+    unsigned long long context;
     size_t bytes;
     void* p;
 };
@@ -77,14 +85,32 @@ size_t block_bytes(size_t bytes)
     return bytes <= kCacheBlock ? b : bytes;
 }
 
-// the current device's cached blocks back to the device
-void release_cache(int dev)
+// the current context's id, 0 if there is none
+unsigned long long context_id()
 {
+    typedef int (*GetId)(void* context, unsigned long long* id);
+    static const GetId get = [] {
+        void* fn = nullptr;
+        cudaDriverEntryPointQueryResult found;
+        if (cudaGetDriverEntryPointByVersion("cuCtxGetId", &fn, 12000, cudaEnableDefault, &found) != cudaSuccess) {
+            cudaGetLastError();
+            fn = nullptr;
+        }
+        return reinterpret_cast<GetId>(fn);
+    }();
+    unsigned long long id = 0;
+    return get && get(nullptr, &id) == 0 ? id : 0;
+}
+
+// the current context's kept blocks back to the device
+void release_cache()
+{
+    const unsigned long long context = context_id();
     std::vector<void*> blocks;
     {
         std::lock_guard<std::mutex> lk(g_cache_mu);
         for (size_t i = 0; i < g_cache.size();) {
-            if (g_cache[i].device == dev) {
+            if (g_cache[i].context == context) {
                 blocks.push_back(g_cache[i].p);
                 g_cache.erase(g_cache.begin() + (ptrdiff_t)i);
             } else {
@@ -95,13 +121,15 @@ void release_cache(int dev)
     for (void* p : blocks) cudaFree(p);
 }
 
-cudaError_t malloc_or_release(void** p, size_t bytes, int dev)
+// alloc(), once more with the kept blocks given back where memory is short
+template <class Alloc>
+cudaError_t alloc_or_release(const Alloc& alloc)
 {
-    cudaError_t e = cudaMalloc(p, bytes);
+    cudaError_t e = alloc();
     if (e == cudaErrorMemoryAllocation) {
         cudaGetLastError();
-        release_cache(dev);
-        e = cudaMalloc(p, bytes);
+        release_cache();
+        e = alloc();
     }
     return e;
 }
@@ -110,41 +138,40 @@ cudaError_t malloc_or_release(void** p, size_t bytes, int dev)
 cudaError_t dev_malloc(void** p, size_t bytes)
 {
     if (!alloc_allowed()) return cudaErrorMemoryAllocation;
-    int dev = 0;
-    cudaGetDevice(&dev);
-    return malloc_or_release(p, bytes, dev);
+    return alloc_or_release([&] { return cudaMalloc(p, bytes); });
 }
 
-cudaError_t table_malloc(void** p, size_t bytes)
+cudaError_t table_malloc(void** p, size_t bytes, unsigned long long* context)
 {
     if (!alloc_allowed()) return cudaErrorMemoryAllocation;
     const size_t b = block_bytes(bytes);
-    int dev = 0;
-    cudaGetDevice(&dev);
-    {
+    *context = context_id();
+    if (*context) {
         std::lock_guard<std::mutex> lk(g_cache_mu);
         for (size_t i = 0; i < g_cache.size(); ++i)
-            if (g_cache[i].device == dev && g_cache[i].bytes == b) {
+            if (g_cache[i].context == *context && g_cache[i].bytes == b) {
                 *p = g_cache[i].p;
                 g_cache.erase(g_cache.begin() + (ptrdiff_t)i);
                 return cudaSuccess;
             }
     }
-    return malloc_or_release(p, b, dev);
+    const cudaError_t e = alloc_or_release([&] { return cudaMalloc(p, b); });
+    *context = context_id();  // (a thread's first call makes its context)
+    return e;
 }
 
-void table_free(void* base, size_t bytes, void* index, int device)
+void table_free(void* base, size_t bytes, void* index, unsigned long long context)
 {
     // a table without an index (a build that failed) has no wait to rely on
     const bool idle = index && cudaFree(index) == cudaSuccess;
     if (!base) return;
     const size_t b = block_bytes(bytes);
-    if (idle && b <= kCacheBlock) {
+    if (idle && b <= kCacheBlock && context != 0 && context == context_id()) {
         std::lock_guard<std::mutex> lk(g_cache_mu);
         size_t mine = 0;
-        for (const CachedBlock& c : g_cache) mine += c.device == device;
+        for (const CachedBlock& c : g_cache) mine += c.context == context;
         if (mine < kCacheBlocks) {
-            g_cache.push_back(CachedBlock{device, b, base});
+            g_cache.push_back(CachedBlock{context, b, base});
             return;
         }
     }
@@ -154,7 +181,7 @@ void table_free(void* base, size_t bytes, void* index, int device)
 cudaError_t dev_malloc_array(cudaArray_t* a, const cudaChannelFormatDesc* d, size_t width)
 {
     if (!alloc_allowed()) return cudaErrorMemoryAllocation;
-    return cudaMallocArray(a, d, width, 0);
+    return alloc_or_release([&] { return cudaMallocArray(a, d, width, 0); });
 }
 
 const DeviceInfo& device_info()

@@ -61,8 +61,8 @@ inline cudaStream_t as_stream(void* s) { return reinterpret_cast<cudaStream_t>(s
 cudaError_t dev_malloc(void** p, size_t bytes);
 // The same for a table's base block, which later tables reuse (pwl_capi.cu), and
 // the release of a table's two blocks.
-cudaError_t table_malloc(void** p, size_t bytes);
-void table_free(void* base, size_t bytes, void* index, int device);
+cudaError_t table_malloc(void** p, size_t bytes, unsigned long long* context);
+void table_free(void* base, size_t bytes, void* index, unsigned long long context);
 cudaError_t dev_malloc_array(cudaArray_t* a, const cudaChannelFormatDesc* d, size_t width);
 
 // ---------------------------------------------------------------------------
@@ -520,6 +520,7 @@ struct pwl_table_s {
     void* buf_base;    // header, knots, values, slopes, build scratch
     void* buf_rec;     // index records
     size_t bytes_base;
+    unsigned long long context;  // that buf_base was allocated in
     pwl::TableHeader* hdr;
     float* xk;
     float* vk;

@@ -403,7 +403,7 @@ pwl_status pwl_table_build(const double* d_knots, const double* d_values, int64_
     const size_t o_cp = o_cj + align256(4 * n1);
     const size_t total = o_cp + align256(4 * n1);
     t->bytes_base = total;
-    cudaError_t e = table_malloc(&t->buf_base, total);
+    cudaError_t e = table_malloc(&t->buf_base, total, &t->context);
     if (e != cudaSuccess) {
         delete t;
         return cuda_fail(e, "cudaMalloc(table)");
@@ -494,7 +494,7 @@ pwl_status pwl_table_destroy(pwl_table t)
     if (!t) return PWL_OK;
     if (t->tex) cudaDestroyTextureObject(t->tex);
     if (t->tex_array) cudaFreeArray(t->tex_array);
-    table_free(t->buf_base, t->bytes_base, t->buf_rec, t->device);
+    table_free(t->buf_base, t->bytes_base, t->buf_rec, t->context);
     delete t;
     return PWL_OK;
 }
