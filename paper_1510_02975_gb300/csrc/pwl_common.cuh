@@ -516,6 +516,7 @@ struct pwl_table_s {
     int64_t Kb;
     float inv_w_b, off_b;
     int64_t n_chain_b;      // at the last synchronous build
+    int max_chain_f, max_chain_b;  // likewise
     int64_t chain_reserve_b;  // chain records the backward kernel stages in shared memory
     void* buf_base;    // header, knots, values, slopes, build scratch
     void* buf_rec;     // index records

@@ -208,6 +208,14 @@ __global__ void __launch_bounds__(1024, MINB) eval_kernel(const EvalArgs args, c
 // costs each CTA about 10 us (20 for N = 4096), which repays itself from 2^24
 // queries on (25 -> 23 us; 2^23: 17 -> 20), with the Lorentzian's N = 4096 from
 // 2^25 (54 -> 48 us).  Two vectors in flight per thread: 99 us, four: 106.
+//
+// Every pattern is looked up, also those that no query has, and half of all
+// patterns lie within 2 of 0: where a cell there holds many knots (knots spaced by
+// the logarithm) every CTA would walk them tens of thousands of times.  Tables with
+// more than kLutChain knots past the first in a cell keep to the index (2^25
+// queries, such knots in one cell: 41 of them 60 us by table and 72 through the
+// index, 84: 82 and 80, 1565: 749 and 417).
+constexpr int kLutChain = 32;
 constexpr int kLutUnroll = 2;
 constexpr int64_t kLutQueries = (int64_t)1 << 25;
 constexpr size_t kLutBytes = sizeof(uint16_t) << 16;
@@ -248,6 +256,7 @@ __global__ void __launch_bounds__(1024, 1) eval_lut_kernel(const EvalArgs args, 
             const int n_chain = p.hdr->n_chain_b;
             p.max_chain = p.hdr->max_chain_b;
             p.n_smem = p.K + n_chain;  // every record from the one (global) array
+            if (p.max_chain > kLutChain) return eval_body<IO, 1>(p, Lerp16<true>{p.rec16, p}, x, y, m);  // since an update
             if (n_chain == 0)
                 fill_lut<IO>(lut32, Lerp16<false>{p.rec16, p});
             else
@@ -257,6 +266,8 @@ __global__ void __launch_bounds__(1024, 1) eval_lut_kernel(const EvalArgs args, 
             p.max_chain = p.hdr->max_chain_f;
             p.s_staged = 0;
             const float2* side = LAYOUT == 2 ? p.recS8 : p.recS;
+            if (p.max_chain > kLutChain)
+                return eval_body<IO, 1>(p, Lerp8<true, true, LAYOUT == 2>{p.recP, side, p}, x, y, m);
             if (n_chain == 0)
                 fill_lut<IO>(lut32, Lerp8<false, false, LAYOUT == 2>{p.recP, side, p});
             else
@@ -548,7 +559,7 @@ pwl_status launch_eval(pwl_table t, int layout, const IO* x, IO* y, int64_t m, c
     const DeviceInfo& di = device_info();
     if (smem > di.smem_optin) return fail(PWL_ENOTSUP, "forward index of %zu bytes does not fit one CTA", smem);
     if constexpr (sizeof(IO) == 2) {
-        if (m >= kLutQueries) {
+        if (m >= kLutQueries && (layout == 1 ? t->max_chain_b : t->max_chain_f) <= kLutChain) {
             void (*kern)(const EvalArgs, const IO*, IO*, int64_t) =
                 layout == 0 ? eval_lut_kernel<IO, 0> : (layout == 2 ? eval_lut_kernel<IO, 2> : eval_lut_kernel<IO, 1>);
             int grid = 0;

@@ -455,6 +455,8 @@ pwl_status pwl_table_build(const double* d_knots, const double* d_values, int64_
         return bail(cuda_fail(e, "table build (index pass)"));
     t->n_chain_b = h.n_chain_b;
     t->n_chain_f = h.n_chain_f;
+    t->max_chain_f = h.max_chain_f;
+    t->max_chain_b = h.max_chain_b;
     // chains in the 16-byte index (cells holding several knots) cost more than
     // the 8-byte index's single-CTA occupancy when the latter has none
     if (t->layout == 1 && k_cells == 0 && t->n_chain_b > 0 && t->n_chain_f == 0) t->layout = 0;
