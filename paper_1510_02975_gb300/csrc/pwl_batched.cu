@@ -550,6 +550,7 @@ struct pwl_batch_s {
     int64_t m_per;
     std::vector<int64_t> N;     // intervals per function
     int64_t n_max;              // the largest of them
+    size_t index_smem;          // shared memory of the index build (0: through global memory)
     std::vector<int64_t> koff;  // knot offsets
     std::vector<int64_t> K;     // cells per function
     int64_t total_knots, total_cells_design, total_chunks, total_cells_index;
@@ -715,6 +716,8 @@ pwl_status pwl_batch_create(const pwl_func* funcs, const int64_t* n_intervals, i
     b->m_per = mper;
     b->N.assign(n_intervals, n_intervals + n_funcs);
     b->n_max = *std::max_element(b->N.begin(), b->N.end());
+    b->index_smem = 16 * (size_t)(b->n_max + 2);
+    if (b->index_smem + 1024 > device_info().smem_optin) b->index_smem = 0;
     b->koff.resize(n_funcs + 1);
     b->K.resize(n_funcs);
     // the largest index one CTA can stage (shape 0: one CTA per SM)
@@ -777,8 +780,9 @@ pwl_status pwl_batch_create(const pwl_func* funcs, const int64_t* n_intervals, i
                             align256(sizeof(BatchFunc) * F),
                             align256(4 * T),
                             align256(4 * T),
-                            align256(4 * (size_t)soff),
-                            align256(4 * T),
+                            // slopes and cells of the knots: in shared memory where they fit
+                            b->index_smem ? 0 : align256(4 * (size_t)soff),
+                            b->index_smem ? 0 : align256(4 * T),
                             align256(8 * (size_t)poff),
                             align256(16 * T),
                             align256(sizeof(int)),
@@ -889,15 +893,13 @@ pwl_status pwl_batch_build(pwl_batch b, void* stream)
 {
     clear_error();
     if (!b) return fail(PWL_EINVAL, "batch is NULL");
-    const DeviceInfo& di = device_info();
-    const size_t smem = 16 * (size_t)(b->n_max + 2);
-    const bool staged = smem + 1024 <= di.smem_optin;
+    const bool staged = b->index_smem != 0;
     void (*kern)(int, const int*, const double*, const double*, BatchFunc*, float*, float*, float*, int*, float2*,
                  float2*) = staged ? batch_index_kernel<true> : batch_index_kernel<false>;
     int grid = 0;
-    PWL_CUDA_TRY(occupancy_grid(kern, kIndexThreads, staged ? smem : 0, &grid));
+    PWL_CUDA_TRY(occupancy_grid(kern, kIndexThreads, b->index_smem, &grid));
     // the largest functions first, in strides of the grid
-    kern<<<(int)std::min<int64_t>(b->F, grid), kIndexThreads, staged ? smem : 0, as_stream(stream)>>>(
+    kern<<<(int)std::min<int64_t>(b->F, grid), kIndexThreads, b->index_smem, as_stream(stream)>>>(
         (int)b->F, b->order, b->knots, b->values, b->bf, b->xk, b->vk, b->slope, b->cj, b->recP, b->recS);
     PWL_CHECK_LAUNCH("batch_index_kernel");
     return PWL_OK;
