@@ -849,6 +849,7 @@ pwl_status pwl_batch_design(pwl_batch b, int32_t precision, void* stream)
     p.moff = b->d_moff;
     p.choff = b->d_choff;
     p.total_knots = b->total_knots;
+    p.n_max = b->n_max;
     p.total_cells = b->total_cells_design;
     p.total_chunks = b->total_chunks;
     p.knots = b->knots;

@@ -210,79 +210,120 @@ __global__ void __launch_bounds__(kDesignThreads) chunk_scan_kernel(DesignPlan p
 // positive density, and x_i = a + k delta + (tau_i - G_k) / d_k.  It reads 8
 // bytes per cell; writing G to memory and searching it there took 24 bytes
 // per cell and a chain of ~17 dependent L2 reads per knot.
-__global__ void __launch_bounds__(kDesignThreads) invert_tiles_kernel(DesignPlan p)
+//
+// Targets can crowd (few cells per knot, or a peak that a fraction of the cells
+// holds), so a tile's knots go to `slices` CTAs, 256 at a time in turn; slices
+// without a knot are passed over, 256 at a time, without reading their tile.
+// 2^20 intervals on 2048 cells 0.18 ms (18.1 with one CTA per tile), 100000 with a
+// peak of 1e-4 of the domain 0.76 ms (2.31).
+struct TileItem {
+    int64_t tile, i0, i1;  // the tile and its knots (i0 <= i < i1)
+    int f, slice;
+    __device__ __forceinline__ TileItem(const DesignPlan& p, int64_t item)
+    {
+        const int64_t tiles = p.total_chunks / kTileChunks, ch = (tile = item % tiles) * kTileChunks;
+        slice = (int)(item / tiles);
+        f = p.tile_func ? p.tile_func[tile] : 0;
+        const int64_t c0 = (ch - p.choff[f]) * kChunk, N = p.koff[f + 1] - p.koff[f] - 1;
+        if (p.stot[f] > 0.0) {
+            // the next tile's first target ends this one's, so every knot has exactly one tile
+            const int64_t* first = reinterpret_cast<const int64_t*>(p.csum + ch);
+            i0 = first[0];
+            i1 = c0 + kTile < p.moff[f + 1] - p.moff[f] ? first[kTileChunks] : N;
+        } else {  // f linear on I (or no finite density): the uniform partition, by the first tile
+            i0 = 1;
+            i1 = c0 == 0 ? N : 1;
+        }
+    }
+    // whether the item has anything to write (the first one of a function the end knots)
+    __device__ __forceinline__ bool any(const DesignPlan& p) const
+    {
+        return i0 + slice * kDesignThreads < i1 || (slice == 0 && tile * kTileChunks == p.choff[f]);
+    }
+};
+
+__global__ void __launch_bounds__(kDesignThreads) invert_tiles_kernel(DesignPlan p, int slices)
 {
     __shared__ double s_d[kTile];
     __shared__ double s_S[kDesignThreads];  // tile base + exclusive prefix of the thread partials
     __shared__ double s_warp[kDesignThreads / 32 + 1];
+    __shared__ int s_items[kDesignThreads];
+    __shared__ int s_count;
     const int t = threadIdx.x;
-    for (int64_t tile = blockIdx.x; tile < p.total_chunks / kTileChunks; tile += gridDim.x) {
-        const int64_t ch = tile * kTileChunks;  // the tile's first chunk
-        const int f = p.tile_func ? p.tile_func[tile] : 0;
-        const int64_t M = p.moff[f + 1] - p.moff[f];
-        const int64_t N = p.koff[f + 1] - p.koff[f] - 1;
-        const int64_t c0 = (ch - p.choff[f]) * kChunk;
-        const double a = p.funcs[f].a, b = p.funcs[f].b;
-        const double delta = p.delta[f];
-        const double GM = p.stot[f];
-        double* __restrict__ knots = p.knots + p.koff[f];
-        if (t == 0 && c0 == 0) {
-            knots[0] = a;
-            knots[N] = b;
-        }
-        if (!(GM > 0.0)) {  // f linear on I (or no finite density): the uniform partition
-            if (c0 == 0)
-                for (int64_t i = 1 + t; i < N; i += kDesignThreads) knots[i] = a + (double)i * (b - a) / (double)N;
-            continue;
-        }
-        const double base = p.cbase[ch];
-        // the next tile's first target ends this one's, so every knot has exactly one tile
-        const int64_t* first = reinterpret_cast<const int64_t*>(p.csum + ch);
-        const int64_t i0 = first[0], i1 = c0 + kTile < M ? first[kTileChunks] : N;
-        if (i0 >= i1) continue;
-        const int cnt = (int)min((int64_t)kTile, M - c0);
-        const double* __restrict__ d = p.d + p.moff[f] + c0;
-        for (int i = t; i < kTile; i += kDesignThreads) s_d[i] = i < cnt ? d[i] : 0.0;
+    const int64_t items = p.total_chunks / kTileChunks * slices, step = (int64_t)gridDim.x * kDesignThreads;
+    for (int64_t base_item = blockIdx.x; base_item < items; base_item += step) {
+        if (t == 0) s_count = 0;
         __syncthreads();
-        double run = 0.0;
-        for (int r = 0; r < kTilePer; ++r) run += s_d[t * kTilePer + r];
-        double tot;
-        s_S[t] = base + block_exclusive_scan(run, s_warp, &tot);
+        const int64_t mine = base_item + (int64_t)t * gridDim.x;
+        if (mine < items && TileItem(p, mine).any(p)) s_items[atomicAdd(&s_count, 1)] = t;
         __syncthreads();
-        const int U = (cnt + kTilePer - 1) / kTilePer;  // threads holding cells
-        for (int64_t i = i0 + t; i < i1; i += kDesignThreads) {
-            const double tau = (double)i * GM / (double)N;
-            int lo = 0, hi = U - 1;  // largest u with G at its first cell <= tau (u = 0 is)
-            while (lo < hi) {
-                const int mid = (lo + hi + 1) >> 1;
-                if (delta * s_S[mid] <= tau) lo = mid; else hi = mid - 1;
+        for (int n = 0; n < s_count; ++n) {
+            const TileItem it(p, base_item + (int64_t)s_items[n] * gridDim.x);
+            const int64_t ch = it.tile * kTileChunks;  // the tile's first chunk
+            const int f = it.f;
+            const int64_t M = p.moff[f + 1] - p.moff[f];
+            const int64_t N = p.koff[f + 1] - p.koff[f] - 1;
+            const int64_t c0 = (ch - p.choff[f]) * kChunk;
+            const int64_t i_first = it.i0 + it.slice * kDesignThreads + t, i_step = (int64_t)slices * kDesignThreads;
+            const double a = p.funcs[f].a, b = p.funcs[f].b;
+            const double delta = p.delta[f];
+            const double GM = p.stot[f];
+            double* __restrict__ knots = p.knots + p.koff[f];
+            if (t == 0 && c0 == 0 && it.slice == 0) {
+                knots[0] = a;
+                knots[N] = b;
             }
-            const int nr = min(kTilePer, cnt - lo * kTilePer);
-            double acc = 0.0, Gk = delta * s_S[lo];
-            int kl = lo * kTilePer;
-            for (int r = 1; r < nr; ++r) {  // the thread's last cell with G <= tau (G does not decrease)
-                acc += s_d[lo * kTilePer + r - 1];
-                const double Gr = delta * (s_S[lo] + acc);
-                if (!(Gr <= tau)) break;
-                kl = lo * kTilePer + r;
-                Gk = Gr;
+            if (!(GM > 0.0)) {
+                for (int64_t i = i_first; i < it.i1; i += i_step) knots[i] = a + (double)i * (b - a) / (double)N;
+                continue;
             }
-            int kk = kl;  // largest cell <= kl of positive density
-            while (kk >= 0 && !(s_d[kk] > 0.0)) --kk;
-            double x;
-            if (kk == kl) {
-                x = __dadd_rn(a, __dmul_rn((double)(c0 + kk), delta));
-                x = __dadd_rn(x, fmin(fmax((tau - Gk) / s_d[kk], 0.0), delta));
-            } else {
-                // no density between the last positive cell (in the tile or before
-                // it) and here, so tau is at or past G at that cell's end: its
-                // right edge
-                const int64_t e = kk >= 0 ? c0 + kk : p.plast[ch];
-                x = e < 0 ? a : __dadd_rn(__dadd_rn(a, __dmul_rn((double)e, delta)), delta);
+            const double base = p.cbase[ch];
+            if (it.i0 >= it.i1) continue;  // (only the end knots)
+            const int cnt = (int)min((int64_t)kTile, M - c0);
+            const double* __restrict__ d = p.d + p.moff[f] + c0;
+            for (int i = t; i < kTile; i += kDesignThreads) s_d[i] = i < cnt ? d[i] : 0.0;
+            __syncthreads();
+            double run = 0.0;
+            for (int r = 0; r < kTilePer; ++r) run += s_d[t * kTilePer + r];
+            double tot;
+            s_S[t] = base + block_exclusive_scan(run, s_warp, &tot);
+            __syncthreads();
+            const int U = (cnt + kTilePer - 1) / kTilePer;  // threads holding cells
+            for (int64_t i = i_first; i < it.i1; i += i_step) {
+                const double tau = (double)i * GM / (double)N;
+                int lo = 0, hi = U - 1;  // largest u with G at its first cell <= tau (u = 0 is)
+                while (lo < hi) {
+                    const int mid = (lo + hi + 1) >> 1;
+                    if (delta * s_S[mid] <= tau) lo = mid; else hi = mid - 1;
+                }
+                const int nr = min(kTilePer, cnt - lo * kTilePer);
+                double acc = 0.0, Gk = delta * s_S[lo];
+                int kl = lo * kTilePer;
+                for (int r = 1; r < nr; ++r) {  // the thread's last cell with G <= tau (G does not decrease)
+                    acc += s_d[lo * kTilePer + r - 1];
+                    const double Gr = delta * (s_S[lo] + acc);
+                    if (!(Gr <= tau)) break;
+                    kl = lo * kTilePer + r;
+                    Gk = Gr;
+                }
+                int kk = kl;  // largest cell <= kl of positive density
+                while (kk >= 0 && !(s_d[kk] > 0.0)) --kk;
+                double x;
+                if (kk == kl) {
+                    x = __dadd_rn(a, __dmul_rn((double)(c0 + kk), delta));
+                    x = __dadd_rn(x, fmin(fmax((tau - Gk) / s_d[kk], 0.0), delta));
+                } else {
+                    // no density between the last positive cell (in the tile or before
+                    // it) and here, so tau is at or past G at that cell's end: its
+                    // right edge
+                    const int64_t e = kk >= 0 ? c0 + kk : p.plast[ch];
+                    x = e < 0 ? a : __dadd_rn(__dadd_rn(a, __dmul_rn((double)e, delta)), delta);
+                }
+                knots[i] = x;
             }
-            knots[i] = x;
+            __syncthreads();  // the shared arrays are rewritten for the next tile
         }
-        __syncthreads();  // the shared arrays are rewritten for the next tile
+        __syncthreads();  // (nobody reads the list any more)
     }
 }
 
@@ -698,6 +739,7 @@ void design_carve_scratch(DesignPlan& p, void* scratch)
 pwl_status design_launch(const DesignPlan& p, cudaStream_t s)
 {
     const DeviceInfo& di = device_info();
+    const int64_t tiles = p.total_chunks / kTileChunks;
     const int grid_chunks = (int)std::min<int64_t>(p.total_chunks, (int64_t)di.sms * 16);
     const int kinds = plan_kinds(p.kinds);
     if (kinds & kKindsAnalytic) {
@@ -716,8 +758,12 @@ pwl_status design_launch(const DesignPlan& p, cudaStream_t s)
     }
     chunk_scan_kernel<<<(int)std::min<int64_t>(p.F, 65535), kDesignThreads, 0, s>>>(p);
     PWL_CHECK_LAUNCH("chunk_scan_kernel");
-    const int grid_tiles = (int)std::min<int64_t>(p.total_chunks / kTileChunks, (int64_t)di.sms * 16);
-    invert_tiles_kernel<<<grid_tiles, kDesignThreads, 0, s>>>(p);
+    // enough slices that a tile holding every knot is done in two rounds of its
+    // CTAs, as far as a CTA passes over a few batches of empty ones
+    const int64_t slices = std::max<int64_t>(
+        1, std::min<int64_t>(p.n_max / (2 * kDesignThreads), (int64_t)di.sms * 8 * kDesignThreads * 8 / tiles));
+    const int grid_items = (int)std::min<int64_t>(tiles * slices, (int64_t)di.sms * 16);
+    invert_tiles_kernel<<<grid_items, kDesignThreads, 0, s>>>(p, (int)slices);
     PWL_CHECK_LAUNCH("invert_tiles_kernel");
     return PWL_OK;
 }
@@ -795,6 +841,7 @@ pwl_status pwl_design(const pwl_func* f, int64_t n_intervals, int64_t m_cells, i
     p.moff = reinterpret_cast<int64_t*>(w + 160);
     p.choff = reinterpret_cast<int64_t*>(w + 192);
     p.delta = reinterpret_cast<double*>(w + 224);
+    p.n_max = n_intervals;
     p.total_knots = n_intervals + 1;
     p.total_cells = M;
     p.total_chunks = design_chunks(M);

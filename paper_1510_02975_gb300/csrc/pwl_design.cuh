@@ -53,6 +53,7 @@ struct DesignPlan {
     const int64_t* koff;
     const int64_t* moff;
     const int64_t* choff;
+    int64_t n_max;         // the most intervals of a function
     int64_t total_knots, total_cells, total_chunks;
     const double* delta;   // F cell widths (b - a) / M
     const int* tile_func;  // per tile of 8 chunks: its function (NULL: one function)
@@ -62,7 +63,7 @@ struct DesignPlan {
     double* cbase;   // total_chunks exclusive chunk bases
     int64_t* plast;  // per chunk: its last cell of positive density, then (after the scan) the last one before
                      // it, or -1
-    double* stot;    // per function: FP64 path G_M = delta sum d, FP32 path sum d
+    double* stot;    // per function: G_M = delta sum d (not in the FP32 mode of a batch)
     double* knots;   // total_knots output
 };
 
