@@ -127,6 +127,54 @@ __global__ void __launch_bounds__(kDesignThreads, 2) density_chunks_kernel(Desig
     }
 }
 
+// The same by whole tiles, one function, 8 cells per thread: one partial per tile (in
+// its first chunk; the others' are 0).  A chunk's sum takes 5 additions per lane, which
+// FP64 densities hardly notice but FP32 ones do, and so they do the parameters'
+// conversions in every cell: a whole FP32 design on 2^24 cells 614 us, by chunks 855.
+// For tiles enough to fill the chip.
+template <typename T, bool SAMPLED>
+__global__ void __launch_bounds__(kDesignThreads) density_tiles_kernel(DesignPlan p)
+{
+    __shared__ double s_red[kDesignThreads / 32];
+    __shared__ int s_last[kDesignThreads / 32];
+    const pwl_func F = p.funcs[0];
+    const double delta = p.delta[0];
+    const int64_t M = p.moff[1];
+    const int t = threadIdx.x;
+    for (int64_t tile = blockIdx.x; tile < p.total_chunks / kTileChunks; tile += gridDim.x) {
+        const int64_t c0 = tile * kTile, ch = tile * kTileChunks;
+        double acc = 0.0;
+        int last = -1;
+#pragma unroll 2
+        for (int r = 0; r < kTilePer; ++r) {
+            const int64_t k = c0 + r * kDesignThreads + t;
+            if (k >= M) break;
+            const double v = cell_density<T, SAMPLED>(F, delta, k);
+            p.d[k] = v;
+            acc += v;
+            if (v > 0.0) last = r * kDesignThreads + t;
+        }
+        acc = warp_sum(acc);
+        last = __reduce_max_sync(0xffffffffu, last);
+        if ((t & 31) == 0) {
+            s_red[t >> 5] = acc;
+            s_last[t >> 5] = last;
+        }
+        __syncthreads();
+        if (t < kTileChunks) {
+            double sum = 0.0;
+            int m = -1;
+            for (int w = 0; w < kDesignThreads / 32; ++w) {
+                sum += s_red[w];
+                m = max(m, s_last[w]);
+            }
+            p.csum[ch + t] = t == 0 ? sum : 0.0;
+            p.plast[ch + t] = t > 0 || m < 0 ? -1 : c0 + m;
+        }
+        __syncthreads();
+    }
+}
+
 // smallest i in [1, N] with tau_i = i G_M / N >= G (N if none below N)
 __device__ __forceinline__ int64_t first_target_at_or_above(double G, double GM, int64_t N)
 {
@@ -741,16 +789,22 @@ pwl_status design_launch(const DesignPlan& p, cudaStream_t s)
     const DeviceInfo& di = device_info();
     const int64_t tiles = p.total_chunks / kTileChunks;
     const int grid_chunks = (int)std::min<int64_t>(p.total_chunks, (int64_t)di.sms * 16);
+    const int grid_tiles = (int)std::min<int64_t>(tiles, (int64_t)di.sms * 16);
+    const bool by_tiles = p.precision == PWL_PREC_FP32 && p.F == 1 && tiles >= (int64_t)di.sms * 8;
     const int kinds = plan_kinds(p.kinds);
     if (kinds & kKindsAnalytic) {
-        if (p.precision == PWL_PREC_FP32)
+        if (by_tiles)
+            density_tiles_kernel<float, false><<<grid_tiles, kDesignThreads, 0, s>>>(p);
+        else if (p.precision == PWL_PREC_FP32)
             density_chunks_kernel<float, false><<<grid_chunks, kDesignThreads, 0, s>>>(p);
         else
             density_chunks_kernel<double, false><<<grid_chunks, kDesignThreads, 0, s>>>(p);
         PWL_CHECK_LAUNCH("density_chunks_kernel");
     }
     if (kinds & kKindsSampled) {
-        if (p.precision == PWL_PREC_FP32)
+        if (by_tiles)
+            density_tiles_kernel<float, true><<<grid_tiles, kDesignThreads, 0, s>>>(p);
+        else if (p.precision == PWL_PREC_FP32)
             density_chunks_kernel<float, true><<<grid_chunks, kDesignThreads, 0, s>>>(p);
         else
             density_chunks_kernel<double, true><<<grid_chunks, kDesignThreads, 0, s>>>(p);

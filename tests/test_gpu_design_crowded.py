@@ -1,5 +1,6 @@
 """Designs whose knots crowd into few density cells (few cells per knot, narrow
-peaks) or spread evenly (no curvature), with tiles shared by several CTAs: parity with the oracle, every knot written once, and
+peaks) or spread evenly (no curvature), with tiles shared by several CTAs and
+densities by whole tiles: parity with the oracle, every knot written once, and
 a time that does not hang on where the knots lie."""
 import numpy as np
 import pytest
@@ -39,6 +40,16 @@ def test_knots(pwl, f, n, m):
     assert np.all(np.diff(k) >= 0)
 
 
+def test_fp32_densities_by_tiles(pwl):
+    # more tiles than eight per SM: FP32 densities eight cells per thread
+    f, n = _peak(0.2), 2000
+    m = 1217 * 2048 - 777
+    k = pwl.pwl_design(f, n, m, precision="fp32").cpu().numpy()
+    ref = oracle.design(f, n, m)
+    h = np.diff(ref)
+    assert np.all(np.abs(k - ref) <= 2e-3 * np.minimum(np.r_[h[0], h], np.r_[h, h[-1]]))
+
+
 def _us(call):
     call()
     times = []
@@ -64,3 +75,9 @@ def test_time_of_few_cells_per_knot(pwl, precision):
 def test_time_of_a_peak(pwl, n):
     wide, peak = (_us(lambda: pwl.pwl_design(_peak(s), n)) for s in (0.3, 1e-4))
     assert peak <= 1.5 * wide, (peak, wide)
+
+
+def test_time_of_fp32_densities(pwl):
+    # an FP32 cell takes a fraction of an FP64 one: 16 M cells, few knots
+    fp64, fp32 = (_us(lambda: pwl.pwl_design(_peak(0.3), 4096, 1 << 24, precision=q)) for q in ("fp64", "fp32"))
+    assert fp32 <= 0.32 * fp64, (fp32, fp64)
