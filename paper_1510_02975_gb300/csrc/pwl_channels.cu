@@ -30,8 +30,8 @@
 // are as wide as keeps the index below kIndexBytes.
 //
 // Measured, [65536, 4096] x 257 knots: forward 532 -> 377 us (FP32; 5.70 TB/s),
-// backward 1042 -> 840 us (3.8 TB/s); [16384, 4096] in BF16: forward 196 ->
-// 110 us, backward 695 -> 265 us, 388 us of the 695 FP32 copies of the streams,
+// backward 1042 -> 800 us (4.0 TB/s); [16384, 4096] in BF16: forward 196 ->
+// 110 us, backward 695 -> 250 us, 388 us of the 695 FP32 copies of the streams,
 // which the BF16 kernel does without.  Before, the forward had 8-channel
 // tiles (16-byte cells), the backward two compare-and-swap adds
 // and side selects per element (103 instructions), and four CTAs a
@@ -378,13 +378,13 @@ __global__ void __launch_bounds__(kChThreads, 1) channels_forward_kernel(const C
 //     h 2^19 + l + rest with h = rint(v 2^-19) (by adding 1.5 2^23, which needs
 //     no conversion) and l = rint(v - h 2^19), both added with native integer
 //     atomics that return nothing.  |v| < 2^37 keeps h and l within 2^18, so
-//     6912 rows add less than 2^31 - 2^28 to a word; every 6912 rows the words
+//     6144 rows add less than 2^31 - 2^28 to a word; every 6144 rows the words
 //     are looked over and the tile's sums flushed where one has passed 2^28.
 //     A term of 2^17 units or more is rounded at 2^-18 of itself or finer (from
 //     2^23 on it is exact).  The rest of a smaller one, which the words do not
-//     hold, goes to the global gradients in FP32, and so does a term beyond 2^37:
-//     every sum is accurate relative to its own terms, however small they are
-//     beside the channel's other gradients.
+//     hold, goes to the global gradients in FP32, and so does a term beyond 2^37
+//     (taken out of the words again): every sum is accurate relative to its own
+//     terms, however small they are beside the channel's other gradients.
 //   FP32, one word per sum: where more than kSlowSamples of the range's 1024
 //     sampled elements have such a term, or none is nonzero.
 //
@@ -392,25 +392,25 @@ __global__ void __launch_bounds__(kChThreads, 1) channels_forward_kernel(const C
 // over the range's rows at irregular distances (the first rows of sequences and
 // the like are not typical); terms of up to 4 to 8 times that fit.
 //
-// [65536, 4096] x 257 knots: 840 us with normal gradients, the same where half or
-// 99% are zero or every 1024th row is, 890-950 log-normal (sigma 1 to 3), over 10
-// decades along x, with one interval's 2^-26 as large, 99.9% zero or a third of the
-// points outside.  (One unit from the mean exponent of the rows R k / 64, four
-// global adds for every element above it: 690, but 1860-3410 log-normal, 6300 where
-// those rows are zero, 1480 with a third outside.)  In FP32 alone: 850-895 for every
-// distribution, but 2860 where all points of a channel fall into one interval (840
-// in fixed point), 1565 with 7 intervals (790), and 5 to 27 times the rounding
-// error (6e-8).  Of the 840, the test for small terms takes 55 and the look at the
-// words 35.
+// [65536, 4096] x 257 knots: 800 us with normal gradients, the same where half are
+// zero or every 1024th row is, 860-920 log-normal (sigma 1 to 3), over 10 decades
+// along x, with one interval's 2^-26 as large, 99% zero or a third of the points
+// outside.  (One unit from the mean exponent of the rows R k / 64, four global adds
+// for every element above it: 690, but 1860-3410 log-normal, 6300 where those rows
+// are zero, 1480 with a third outside.)  In FP32 alone: 850-895 for every
+// distribution, but 2860 where all points of a channel fall into one interval (800
+// in fixed point), 1565 with 7 intervals (760), and 5 to 27 times the rounding
+// error (6e-8).  Of the 800, the test for small terms takes 20 and the look at the
+// words 30 (the barriers' waits).
 constexpr int kDigitBits = 19;
 constexpr int kRangeBits = 37;                                // terms below 2^37 units
 constexpr float kFixLimit = 0x1p37f;
 constexpr unsigned kSmallKey = 2u * ((127 + 17) << 23) - 2u;  // small_key of 2^17
-constexpr int kSegRows = 6912;                                // whole passes of every tile width (64, 128, 256 rows)
+constexpr int kSegRows = 6144;                                // whole unrolled passes of every tile width
 constexpr int kFullWord = 1 << 28;
 constexpr int kSlowSamples = 6;  // (log-normal of sigma 2: 1320 us with 16)
 constexpr float kMagic = 0x1.8p23f;
-constexpr int kMagicBits = 0x4B400000;
+constexpr unsigned kMagicBits = 0x4B400000u;
 constexpr float kDigit = 0x1p19f, kPerDigit = 0x1p-19f;
 
 // What a range's setup shares, and what the rare paths need (in registers it would
@@ -475,13 +475,13 @@ __device__ __forceinline__ float fix_high(float v, float& m)
     return __fmaf_rn(__fsub_rn(m, kMagic), -kDigit, v);
 }
 // one term into its two words (h at byte offset 0, l at byte offset L)
-template <int L>
+template <int L, int SIGN = 1>
 __device__ __forceinline__ void fix_add(uint32_t at, float v)
 {
     float m;
     const float low = fix_high(v, m);
-    red_add<0>(at, __float_as_int(m) - kMagicBits);
-    red_add<L>(at, __float2int_rn(low));
+    red_add<0>(at, (int)(SIGN * (__float_as_uint(m) - kMagicBits)));
+    red_add<L>(at, (int)(SIGN * (unsigned)__float2int_rn(low)));
 }
 // what fix_add's words leave out
 __device__ __forceinline__ float fix_rest(float v)
@@ -540,30 +540,33 @@ __device__ __noinline__ void add_rests(float t1, float t2, uint32_t at, float s)
     if (e1 != 0.0f || e2 != 0.0f) add_global_terms<CH>(e1, e2, at, s);
 }
 
-// G elements: gx in place of g.
+// Two terms out of range, whose words hold nonsense: out of the words again (integer
+// adds are exact modulo 2^32) and to the global gradients.
+template <int CH>
+__device__ __noinline__ void add_instead(float v1, float v2, float t1, float t2, uint32_t at, float s, uint32_t first,
+                                         uint32_t second)
+{
+    fix_add<8 * CH, -1>(at + first, v1);  // (as they were added, in units)
+    fix_add<8 * CH, -1>(at + second, v2);
+    add_global_terms<CH>(t1, t2, at, s);
+}
+
+// G elements: gx in place of g.  One branch per group: what elements outside the
+// domain, small terms and terms out of range need comes after the adds (a branch for
+// each of the three, two of them before the adds: 840 us instead of 800).
 template <int CH, int G, bool FLOAT>
 __device__ __forceinline__ void chan_bwd(const float (&x)[G], float (&g)[G], const ChanConst<CH>& cc, const BwdOut& o,
                                          EndSums& ends)
 {
-    float xc[G];
+    float xc[G], gs[G];
     float4 r[G];
     uint32_t at[G];
     bool inside = true, fits = true;
-    unsigned nans = 0;
 #pragma unroll
     for (int q = 0; q < G; ++q) {
         xc[q] = fminf(fmaxf(x[q], cc.a), cc.b);  // NaN -> a
         inside = inside && x[q] == xc[q];
-    }
-    if (!inside) {
-#pragma unroll
-        for (int q = 0; q < G; ++q) {
-            if (x[q] == xc[q]) continue;
-            ends.left += x[q] < cc.a ? g[q] : 0.0f;
-            ends.right += x[q] > cc.b ? g[q] : 0.0f;
-            nans |= x[q] != x[q] ? 1u << q : 0u;
-            g[q] = 0.0f;
-        }
+        gs[q] = x[q] == xc[q] ? (FLOAT ? g[q] : g[q] * o.scale) : 0.0f;
     }
     chan_lookup<CH, G>(xc, cc, r, at);
     // 1 - delta and delta, each from the interval's other end and so accurate
@@ -573,56 +576,47 @@ __device__ __forceinline__ void chan_bwd(const float (&x)[G], float (&g)[G], con
         t1 = gq * (fabsf(p1 - xc[q]) * r[q].y);
         t2 = gq * (fabsf(p2 - xc[q]) * r[q].y);
     };
-    if constexpr (FLOAT) {
+    unsigned small = ~0u;
 #pragma unroll
-        for (int q = 0; q < G; ++q) {
-            float t1, t2;
-            terms(q, g[q], t1, t2);
+    for (int q = 0; q < G; ++q) {
+        float t1, t2;
+        terms(q, gs[q], t1, t2);
+        if constexpr (FLOAT) {
             float_add(at[q] + o.first, t1);
             float_add(at[q] + o.second, t2);
-        }
-    } else {
-        float gs[G];
-        unsigned small = ~0u;
-#pragma unroll
-        for (int q = 0; q < G; ++q) {
-            gs[q] = g[q] * o.scale;
-            fits = fits && fabsf(gs[q]) < kFixLimit;
-        }
-        if (!fits) {
-#pragma unroll
-            for (int q = 0; q < G; ++q) {
-                if (fabsf(gs[q]) < kFixLimit) continue;
-                float t1, t2;
-                terms(q, g[q], t1, t2);
-                add_global_terms<CH>(t1, t2, at[q], r[q].z);
-                gs[q] = 0.0f;
-            }
-        }
-#pragma unroll
-        for (int q = 0; q < G; ++q) {
-            float t1, t2;
-            terms(q, gs[q], t1, t2);
+        } else {
             fix_add<8 * CH>(at[q] + o.first, t1);
             fix_add<8 * CH>(at[q] + o.second, t2);
             small = min(small, min(small_key(t1), small_key(t2)));
+            fits = fits && fabsf(gs[q]) < kFixLimit;
         }
-        if (small < kSmallKey) {
+    }
+    if (!inside || !fits || small < kSmallKey) {
+        if (!fits || small < kSmallKey) {
 #pragma unroll
             for (int q = 0; q < G; ++q) {
                 float t1, t2;
                 terms(q, gs[q], t1, t2);
-                add_rests<CH>(t1, t2, at[q], r[q].z);
+                if (fabsf(gs[q]) < kFixLimit) {
+                    add_rests<CH>(t1, t2, at[q], r[q].z);
+                } else {
+                    float u1, u2;
+                    terms(q, g[q], u1, u2);
+                    add_instead<CH>(t1, t2, u1, u2, at[q], r[q].z, o.first, o.second);
+                }
             }
         }
+#pragma unroll
+        for (int q = 0; q < G; ++q) {
+            const bool in = x[q] == xc[q];
+            ends.left += x[q] < cc.a ? g[q] : 0.0f;
+            ends.right += x[q] > cc.b ? g[q] : 0.0f;
+            g[q] = in ? g[q] * r[q].z : x[q] != x[q] ? x[q] : 0.0f;
+        }
+        return;
     }
 #pragma unroll
     for (int q = 0; q < G; ++q) g[q] *= r[q].z;
-    if (nans) {
-#pragma unroll
-        for (int q = 0; q < G; ++q)
-            if (nans >> q & 1u) g[q] = x[q];
-    }
 }
 
 // Whether the fixed-point form of a sampled element needs a global add.

@@ -46,6 +46,9 @@ def _data(case, C, N, R, knots):
         g *= (rng.random((R, C)) < 0.01) * 10.0 ** -(np.arange(C) % 13)
     elif case == "lognormal":
         g *= np.exp(2 * rng.normal(size=(R, C)))
+    elif case == "outliers":  # a few elements far beyond what the samples suggest
+        g[777::4999] *= 1e9
+        g[1234] *= 1e33
     elif case == "beside_a_knot":  # no point near knot j: both intervals' within 2^-16 of their far ends
         l, m, r = knots[:, j - 1], knots[:, j], knots[:, j + 1]
         t = np.float32(2.0 ** -16) * rng.random((R, C)).astype(np.float32)
@@ -70,7 +73,7 @@ def _check(knots, values, x, gy, gv, gk, channels):
 
 @pytest.mark.parametrize("C,N,k_cells", WIDTHS, ids=["16", "8", "4"])
 @pytest.mark.parametrize("case", ["normal", "bin16", "bin20", "bin26", "bin31", "decades", "sparse_channels", "lognormal",
-                                  "beside_a_knot"])
+                                  "outliers", "beside_a_knot"])
 def test_every_knot_relative_to_its_own_terms(pwl, case, C, N, k_cells):
     knots, values = _tables(C, N)
     x, gy = _data(case, C, N, 20000, knots)
