@@ -30,8 +30,8 @@
 // are as wide as keeps the index below kIndexBytes.
 //
 // Measured, [65536, 4096] x 257 knots: forward 532 -> 377 us (FP32; 5.70 TB/s),
-// backward 1042 -> 800 us (4.0 TB/s); [16384, 4096] in BF16: forward 196 ->
-// 110 us, backward 695 -> 250 us, 388 us of the 695 FP32 copies of the streams,
+// backward 1042 -> 780 us (4.1 TB/s); [16384, 4096] in BF16: forward 196 ->
+// 110 us, backward 695 -> 238 us, 388 us of the 695 FP32 copies of the streams,
 // which the BF16 kernel does without.  Before, the forward had 8-channel
 // tiles (16-byte cells), the backward two compare-and-swap adds
 // and side selects per element (103 instructions), and four CTAs a
@@ -392,15 +392,15 @@ __global__ void __launch_bounds__(kChThreads, 1) channels_forward_kernel(const C
 // over the range's rows at irregular distances (the first rows of sequences and
 // the like are not typical); terms of up to 4 to 8 times that fit.
 //
-// [65536, 4096] x 257 knots: 800 us with normal gradients, the same where half are
-// zero or every 1024th row is, 860-920 log-normal (sigma 1 to 3), over 10 decades
+// [65536, 4096] x 257 knots: 780 us with normal gradients, the same where half are
+// zero or every 1024th row is, 840-910 log-normal (sigma 1 to 3), over 10 decades
 // along x, with one interval's 2^-26 as large, 99% zero or a third of the points
 // outside.  (One unit from the mean exponent of the rows R k / 64, four global adds
 // for every element above it: 690, but 1860-3410 log-normal, 6300 where those rows
 // are zero, 1480 with a third outside.)  In FP32 alone: 850-895 for every
-// distribution, but 2860 where all points of a channel fall into one interval (800
-// in fixed point), 1565 with 7 intervals (760), and 5 to 27 times the rounding
-// error (6e-8).  Of the 800, the test for small terms takes 20 and the look at the
+// distribution, but 2860 where all points of a channel fall into one interval (776
+// in fixed point), 1565 with 7 intervals (740), and 5 to 27 times the rounding
+// error (6e-8).  Of the 780, the test for small terms takes 20 and the look at the
 // words 30 (the barriers' waits).
 constexpr int kDigitBits = 19;
 constexpr int kRangeBits = 37;                                // terms below 2^37 units
@@ -436,7 +436,9 @@ __device__ __forceinline__ void sample(const ChanArgs& p, int64_t c0, int64_t r0
     const int64_t c = c0 + threadIdx.x % CH, n = r1 - r0, s = threadIdx.x / CH;
     xs = gs = 0.0f;
     if (c >= p.C) return;
-    const unsigned h = ((unsigned)c0 * 1024u + threadIdx.x) * 0x9E3779B9u;  // multiples of the golden ratio mod 1
+    // multiples of the golden ratio mod 1; one row for the tile's channels (a row each
+    // read 16 times the sectors, 0.08 of the 0.66 GB of a call at 16384 rows)
+    const unsigned h = (unsigned)(c0 / CH * S + s) * 0x9E3779B9u;
     const int64_t lo = n * s / S, w = min(n * (s + 1) / S - lo, (int64_t)0x7fffffff);
     const int64_t at = (r0 + lo + (int64_t)((uint64_t)h * (uint64_t)w >> 32)) * p.C + c;
     xs = to_f32<IO>(__ldcg(x + at));
