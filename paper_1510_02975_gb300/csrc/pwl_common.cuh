@@ -318,13 +318,16 @@ __device__ __forceinline__ float func_value_f(const FuncValueF& F, float x)
 }
 
 // FP64 <-> FP32 without the FP64 pipe (normal FP32 magnitudes and zero by bit
-// arithmetic, the rest by conversion): narrowing rounds to nearest even.
+// arithmetic, the rest by conversion): narrowing rounds to nearest even.  HALVE: of v / 2
+// (v may be beyond FP32).
+template <int HALVE = 0>
 __device__ __forceinline__ float narrow_bits(double v)
 {
     const uint32_t h = (uint32_t)__double2hiint(v), l = (uint32_t)__double2loint(v);
     const uint32_t e = h >> 20 & 0x7ffu;
-    if (e < 897 || e > 1149) return (h << 1 | l) == 0 ? 0.0f : __double2float_rn(v);
-    const uint32_t m = (e - 896) << 23 | (h << 3 & 0x7ffff8u) | l >> 29;
+    if (e < 897 + HALVE || e > 1149 + HALVE)
+        return (h << 1 | l) == 0 ? 0.0f : __double2float_rn(HALVE ? 0.5 * v : v);
+    const uint32_t m = (e - 896 - HALVE) << 23 | (h << 3 & 0x7ffff8u) | l >> 29;
     const uint32_t rest = l << 3;  // the 29 bits below, at the top
     const uint32_t up = rest > 0x80000000u || (rest == 0x80000000u && (m & 1u)) ? 1u : 0u;
     return __uint_as_float((h & 0x80000000u) | (m + up));

@@ -162,7 +162,7 @@ __global__ void __launch_bounds__(128) hat_integrals_f_kernel(ProjectPlan p, con
         const double* x = p.knots + p.koff[f];
         const double xl = x[j - 1], xr = x[j];
         const double h = xr - xl;
-        const float midf = 0.5f * narrow_bits(xl + xr), halff = 0.5f * narrow_bits(h);
+        const float midf = narrow_bits<1>(xl + xr), halff = narrow_bits<1>(h);
         float Lh = 0.0f, Ll = 0.0f, Rh = 0.0f, Rl = 0.0f;
         auto acc = [](float& h, float& l, float wh, float wlo, float fv) {
             const float p = __fmul_rn(wh, fv);
