@@ -300,13 +300,17 @@ __global__ void __launch_bounds__(kDesignThreads) invert_tiles_kernel(DesignPlan
     const int t = threadIdx.x;
     const int64_t items = p.total_chunks / kTileChunks * slices, step = (int64_t)gridDim.x * kDesignThreads;
     for (int64_t base_item = blockIdx.x; base_item < items; base_item += step) {
-        if (t == 0) s_count = 0;
-        __syncthreads();
-        const int64_t mine = base_item + (int64_t)t * gridDim.x;
-        if (mine < items && TileItem(p, mine).any(p)) s_items[atomicAdd(&s_count, 1)] = t;
-        __syncthreads();
-        for (int n = 0; n < s_count; ++n) {
-            const TileItem it(p, base_item + (int64_t)s_items[n] * gridDim.x);
+        const bool list = items > gridDim.x;  // (else one item per CTA)
+        if (list) {
+            if (t == 0) s_count = 0;
+            __syncthreads();
+            const int64_t mine = base_item + (int64_t)t * gridDim.x;
+            if (mine < items && TileItem(p, mine).any(p)) s_items[atomicAdd(&s_count, 1)] = t;
+            __syncthreads();
+        }
+        for (int n = 0; n < (list ? s_count : 1); ++n) {
+            const TileItem it(p, list ? base_item + (int64_t)s_items[n] * gridDim.x : base_item);
+            if (!list && !it.any(p)) continue;
             const int64_t ch = it.tile * kTileChunks;  // the tile's first chunk
             const int f = it.f;
             const int64_t M = p.moff[f + 1] - p.moff[f];
