@@ -27,7 +27,7 @@
 // copy of that access pattern reaches also depends on the L1 the index
 // leaves: 16-channel tiles 360 us up to 132 KB of shared memory, 370 at 164
 // KB, 500 at 198 KB and beyond; 8-channel tiles 503, 578 and 665.  So tiles
-// are as wide as keeps the index below kIndexBytes.
+// are wide and, where that allows it, the index below kIndexBytes.
 //
 // Measured, [65536, 4096] x 257 knots: forward 532 -> 377 us (FP32; 5.70 TB/s),
 // backward 1042 -> 780 us (4.1 TB/s); [16384, 4096] in BF16: forward 196 ->
@@ -388,7 +388,7 @@ __global__ void __launch_bounds__(kChThreads, 1) channels_forward_kernel(const C
 //   FP32, one word per sum: where more than kSlowSamples of the range's 1024
 //     sampled elements have such a term, or none is nonzero.
 //
-// F comes, per channel, from the largest of 64 (128, 256) sampled |gy|, spread
+// F comes, per channel, from the largest of 64 (128) sampled |gy|, spread
 // over the range's rows at irregular distances (the first rows of sequences and
 // the like are not typical); terms of up to 4 to 8 times that fit.
 //
@@ -827,9 +827,9 @@ __global__ void __launch_bounds__(kChThreads, 1) channels_backward_kernel(const 
 // The sizes the calls accept are those of one CTA holding 8 channels' 16-byte
 // cells, knots, values and slopes (forward) or 16 channels' 8-byte cells,
 // 8-byte interval records, two sums and knots (backward), plus a little for
-// scalars; every accepted size fits the tiles below (a 4-channel tile takes
-// less for the same N and K).  Without k_cells, that index may shrink to its
-// remainder of 16 cells.
+// scalars; every accepted size fits the tiles below (4 channels forward and 8
+// backward take less for the same N and K).  Without k_cells, that index may shrink to
+// its remainder of 16 cells.
 size_t accepted_bytes(int64_t N, int64_t K, bool backward)
 {
     const size_t n1 = (size_t)(N + 1), n2 = (size_t)(N + 2);
@@ -846,26 +846,37 @@ size_t tile_bytes(int64_t N, int64_t K, int CH, bool backward)
 // Shared memory of a CTA that leaves the L1 at least ~60 KB (a carve-out of
 // 196 KB) for the rows in flight.
 constexpr size_t kIndexBytes = 196 * 1024 - 1024 - 512;
-constexpr int64_t kFwdCells = 2, kBwdCells = 2;  // cells per knot where they fit
+constexpr int64_t kCells = 2;  // cells per knot where they fit
 
 struct ChanShape {
     int CH, K;
     size_t smem;
 };
 
-// The widest tile whose index fits kIndexBytes with the wanted cells (at least
-// kBwdCells per knot), else the narrowest.
+// The widest tile whose index holds at least one cell per knot (or what the caller
+// asked for) within kIndexBytes or, before the tile is narrowed, the whole shared
+// memory: few cells and little L1 cost less than 32-byte row segments.
+//   Forward, [65536, 2048] FP32: 16 channels up to N = 517 205-226 us, with all of the
+//   shared memory up to 602 279, 8 channels up to 1036 313-318, with all up to 1206 374,
+//   then 4 channels 666-726.  (With 2 cells per knot as the least: 288 from 388 on, 614
+//   from 777.)
+//   Backward, [65536, 4096]: 16 channels up to N = 309 780-798, with all up to 360 943,
+//   8 channels up to 620 1258-1318, then with all 1540 (1245 from 258 on, 2530 from 518).
 ChanShape choose_shape(int64_t N, int64_t k_cells, bool backward)
 {
-    const int64_t want = k_cells > 0 ? k_cells : (backward ? kBwdCells : kFwdCells) * (N + 1);
-    const int64_t need = k_cells > 0 ? k_cells : kBwdCells * (N + 1);
-    const size_t optin = device_info().smem_optin - 512;
+    const int64_t want = k_cells > 0 ? k_cells : kCells * (N + 1);
+    const int64_t need = k_cells > 0 ? k_cells : N + 1;
+    const size_t optin = device_info().smem_optin - 512, part = std::min(kIndexBytes, optin);
+    const struct {
+        int CH;
+        size_t budget;
+    } candidates[] = {{16, part}, {16, optin}, {8, part}, {8, optin}, {4, optin}};
     ChanShape s{};
-    for (int CH : {16, 8, 4}) {
-        const size_t budget = CH == 4 ? optin : std::min(kIndexBytes, optin);
-        const size_t recs = 16 * (size_t)(N + 2) * (size_t)CH * (backward ? 2 : 1);
-        const int64_t room = budget > recs ? (int64_t)((budget - recs) / (8 * (size_t)CH)) : 0;
-        s.CH = CH;
+    for (int i = 0; i < (backward ? 4 : 5); ++i) {  // (no accepted backward needs 4 channels)
+        const auto& c = candidates[i];
+        const size_t recs = 16 * (size_t)(N + 2) * (size_t)c.CH * (backward ? 2 : 1);
+        const int64_t room = c.budget > recs ? (int64_t)((c.budget - recs) / (8 * (size_t)c.CH)) : 0;
+        s.CH = c.CH;
         s.K = (int)std::min(want, std::max<int64_t>(room, 1));
         if (room >= std::max<int64_t>(need, stage_pitch((int)N))) break;
     }
@@ -946,10 +957,8 @@ pwl_status launch_backward(ChanArgs p, const ChanShape& sh, const void* x, const
     switch (sh.CH) {
     case 16:
         return launch(p, 16, sh.smem, channels_backward_kernel<IO, 16>, s, xi, gi, go, g_values, g_knots);
-    case 8:
-        return launch(p, 8, sh.smem, channels_backward_kernel<IO, 8>, s, xi, gi, go, g_values, g_knots);
     default:
-        return launch(p, 4, sh.smem, channels_backward_kernel<IO, 4>, s, xi, gi, go, g_values, g_knots);
+        return launch(p, 8, sh.smem, channels_backward_kernel<IO, 8>, s, xi, gi, go, g_values, g_knots);
     }
 }
 

@@ -1,20 +1,20 @@
 """Channel-wise table gradients relative to their own terms: every knot's sum is
 held to GRAD_REL of the absolute sum of what was added to it, whatever the
-channel's other gradients are, in tiles of every width (16, 8 and 4 channels);
+channel's other gradients are, in tiles of every shape (16 and 8 channels);
 sums that fill the integer words; gx written over gy."""
 import numpy as np
 import pytest
 
 import oracle
-from pwl_testutil import GRAD_REL
+from pwl_testutil import EVAL_REL, GRAD_REL
 
 pytestmark = pytest.mark.gpu
 
 torch = pytest.importorskip("torch")
 
-# (channels, intervals, k_cells): 16-, 8- and 4-channel tiles in the backward
-# (1600 requested cells leave 8 channels, 640 intervals 4)
-WIDTHS = [(20, 40, 0), (20, 40, 1600), (10, 640, 0)]
+# (channels, intervals, k_cells): 16- and 8-channel tiles in the backward, each in the
+# part of shared memory that leaves the L1 room and in all of it
+WIDTHS = [(20, 40, 0), (20, 330, 0), (20, 40, 1700), (10, 640, 0)]
 
 
 @pytest.fixture(scope="module")
@@ -71,7 +71,7 @@ def _check(knots, values, x, gy, gv, gk, channels):
         assert np.all(np.abs(gk[c] - rk) <= GRAD_REL * ak), (c, np.max(np.abs(gk[c] - rk) / np.maximum(ak, 1e-300)))
 
 
-@pytest.mark.parametrize("C,N,k_cells", WIDTHS, ids=["16", "8", "4"])
+@pytest.mark.parametrize("C,N,k_cells", WIDTHS, ids=["16", "16_all", "8", "8_all"])
 @pytest.mark.parametrize("case", ["normal", "bin16", "bin20", "bin26", "bin31", "decades", "sparse_channels", "lognormal",
                                   "outliers", "beside_a_knot"])
 def test_every_knot_relative_to_its_own_terms(pwl, case, C, N, k_cells):
@@ -79,6 +79,21 @@ def test_every_knot_relative_to_its_own_terms(pwl, case, C, N, k_cells):
     x, gy = _data(case, C, N, 20000, knots)
     _, gv, gk = _grads(pwl, knots, values, x, gy, k_cells)
     _check(knots, values, x, gy, gv, gk, range(C))
+
+
+@pytest.mark.parametrize("N", [387, 388, 517, 518, 602, 603, 1036, 1037, 1206, 1207, 1790])
+def test_forward_shapes(pwl, N):
+    # the edges of the forward's tile shapes, one cell per knot at each
+    C, R = 21, 700
+    knots, values = _tables(C, N)
+    x = _data("normal", C, N, R, knots)[0]
+    x[:3] = knots[:, [0, N // 2, N]].T
+    kt, vt, xt = (torch.tensor(a, device="cuda") for a in (knots, values, x))
+    y = pwl.pwl_channels_forward(kt, vt, xt).cpu().numpy().astype(np.float64)
+    for c in range(C):
+        v = values[c].astype(np.float64)
+        ref = oracle.evaluate(knots[c].astype(np.float64), v, x[:, c].astype(np.float64))
+        assert np.abs(y[:, c] - ref).max() <= EVAL_REL * np.abs(v).max(), c
 
 
 @pytest.mark.parametrize("N", [1, 5])
@@ -141,3 +156,29 @@ def test_time_does_not_hang_on_the_gradients(pwl, case):
         x[torch.rand(R, C, generator=g, device="cuda") < 0.33] = 5.0
     t = us(x, gy)
     assert t <= 1.5 * base, (t, base)
+
+
+@pytest.mark.parametrize("N,factor", [(300, 1.35), (512, 2.0), (600, 2.0)])
+def test_time_of_large_tables(pwl, N, factor):
+    # beyond the sizes that two cells per knot leave 16 channels (257 intervals) or 8 (517)
+    C, R = 1024, 65536
+    g = torch.Generator(device="cuda").manual_seed(1)
+    x = torch.randn(R, C, generator=g, device="cuda").clamp_(-1.99, 2.99)
+    gy = torch.randn(R, C, generator=g, device="cuda")
+    gx = torch.empty_like(x)
+
+    def us(n):
+        knots, values = (torch.tensor(a, device="cuda") for a in _tables(C, n))
+        gv, gk = torch.zeros_like(values), torch.zeros_like(knots)
+        times = []
+        for _ in range(8):
+            a, b = (torch.cuda.Event(enable_timing=True) for _ in range(2))
+            a.record()
+            pwl.pwl_channels_backward(knots, values, x, gy, gx, gv, gk)
+            b.record()
+            torch.cuda.synchronize()
+            times.append(a.elapsed_time(b) * 1e3)
+        return sorted(times)[3]
+
+    t, base = us(N), us(256)
+    assert t <= factor * base, (t, base)
