@@ -67,7 +67,7 @@ __device__ __forceinline__ int lower_bound_int(const int* c, int n, int v)
 // and each knot writes its own cell's record and those of the cells up to the
 // next knot's (every cell is written whatever the knots are).  Through global
 // memory, with a bisection per cell, the kernel waited on the L1 (4096
-// functions, 25 M cells: 302 us; staged 211 us; by knot 170 us, of which what
+// functions, 25 M cells: 302 us; staged 211 us; by knot 164 us, of which what
 // it must move takes about 80).  An interval of more than kOwnCells cells is
 // finished by its warp (4096 functions with one over most of the domain, 33 M
 // cells: 209 us, by one thread 2.27 ms; one function of 1.3 M cells 1.0 and 23.5

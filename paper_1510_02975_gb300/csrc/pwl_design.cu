@@ -7,8 +7,8 @@
 // (descriptors and CSR offsets of knots, cells and 256-cell chunks, the
 // chunks of a function padded to whole tiles of 8); a single function is a
 // batch of one.  Three launches:
-//   densities       d_k = |f''(t_k)|^{2/5} and one partial sum per chunk (FP64)
-//                   or tile (FP32 mode of a batch)
+//   densities       d_k = |f''(t_k)|^{2/5} and one partial sum per chunk, or per
+//                   tile (FP32 mode of a batch, and of one function of many cells)
 //   scan            exclusive FP64 scan of the partial sums, per function
 //   knots           per tile of 2048 cells: the in-tile prefix of the
 //                   densities and the knots whose targets tau_i = i G_M / N
@@ -17,7 +17,7 @@
 // per function waits for its largest function and for the barriers of every
 // tile in turn.  40 functions of up to 4095 intervals at 64 cells per
 // interval, FP64: 25.2 ms that way (which also computed the densities twice),
-// 1.12 ms this way (density 1.03).
+// 0.82 ms this way (density 0.755).
 #include <math.h>
 
 #include <algorithm>
@@ -402,8 +402,8 @@ __device__ __forceinline__ float fused_density_f(const FuncF& G, const pwl_func&
 //     thread per tile: an FP64 instruction occupies the pipe for the whole warp
 //     however few of its lanes run it, and done by one lane, or by every thread,
 //     of each tile's CTA these took most of the time (design of 4096 functions
-//     1.79 ms, 1.25 ms by one CTA per function, 0.96 ms now; 40 functions
-//     209 -> 42 us);
+//     1.79 ms, 1.25 ms by one CTA per function, 0.94 ms now; 40 functions
+//     209 -> 36 us);
 //   - the densities go to scratch and come back in 16-byte vectors; cell
 //     midpoints are formed in FP32 from the tile start (the FP32 f'' rounds its
 //     argument to FP32 anyway);
@@ -643,7 +643,8 @@ __global__ void __launch_bounds__(kDesignThreads, SAMPLED ? 4 : 8) density_tiles
 }
 
 // 8 CTAs per SM: the kernel waits on the chain of loads that starts a tile and
-// on the scan's barriers (4 CTAs per SM 586 us, 6 480 us, 8 414 us).
+// on the scan's barriers (4 CTAs per SM 586 us, 6 480 us, 8 414 us, and 398 us since
+// the thread sums do without renormalising).
 __global__ void __launch_bounds__(kDesignThreads, 8) invert_tiles_f_kernel(DesignPlan p)
 {
     __shared__ float4 s_d4[kTile / 4];
