@@ -62,7 +62,8 @@ constexpr int kFwdTail = 4;       // rows per predicated batch of a range's tail
 constexpr int kBwdUnroll = 8;     // rows of x and gy in flight per thread (64 KB per SM in FP32)
 constexpr int kBwdTail = 2;
 constexpr int kFwdGroup = 4;      // elements looked up together (their shared loads overlap, one chain test)
-constexpr int kBwdGroup = 2;
+constexpr int kBwdGroup = 2;      // (fixed-point sums)
+constexpr int kFloatGroup = 4;    // (FP32 sums; 2: 880 instead of 940 us, but 1181 instead of 862 at one point)
 constexpr int kStage = 4;         // knots and values in flight per thread while a tile is staged
 
 template <typename IO>
@@ -388,27 +389,32 @@ __global__ void __launch_bounds__(kChThreads, 1) channels_forward_kernel(const C
 //   FP32, one word per sum: where more than kSlowSamples of the range's 1024
 //     sampled elements have such a term, or none is nonzero.
 //
-// F comes, per channel, from the largest of 64 (128) sampled |gy|, spread
-// over the range's rows at irregular distances (the first rows of sequences and
-// the like are not typical); terms of up to 4 to 8 times that fit.
+// F comes, per channel, from 64 (128) sampled |gy|, spread over the range's rows at
+// irregular distances (the first rows of sequences and the like are not typical);
+// terms of up to 4 to 8 times their largest fit (see fix_exponent).
 //
-// [65536, 4096] x 257 knots: 780 us with normal gradients, the same where half are
-// zero or every 1024th row is, 840-910 log-normal (sigma 1 to 3), over 10 decades
-// along x, with one interval's 2^-26 as large, 99% zero or a third of the points
-// outside.  (One unit from the mean exponent of the rows R k / 64, four global adds
-// for every element above it: 690, but 1860-3410 log-normal, 6300 where those rows
-// are zero, 1480 with a third outside.)  In FP32 alone: 850-895 for every
-// distribution, but 2860 where all points of a channel fall into one interval (776
-// in fixed point), 1565 with 7 intervals (740), and 5 to 27 times the rounding
-// error (6e-8).  Of the 780, the test for small terms takes 20 and the look at the
-// words 30 (the barriers' waits).
+// [65536, 4096] x 257 knots, us (the FP32 atomics before; one unit from the mean exponent
+// of the rows R k / 64 and four global adds for every element above it; now):
+//   normal gradients                                    1009    694    785
+//   log-normal, sigma 1 / 1.6 / 2 / 3                   1009   1858+   870 / 1110 / 940 / 940
+//   every 1024th row zero                               1010   6315    785
+//   half / 97% / 99.9% zero                         917-968    695    785 / 785 / 842
+//   0.1% / 1% of them 2^10 as large                     1009           874 / 1344
+//   over 10 decades along x, one interval's 2^-26       1010   2820+   940
+//   a third of the points outside                        943   1490    912
+//   all points of a channel / half of all in an interval 3090   690    784 / 785
+//   half of them within 2^-10 of a knot in some channels 2416          1250
+// In FP32 alone: 850-895 for every distribution, but 2860 where all points of a channel
+// fall into one interval, 1565 with 7 intervals (740), and 5 to 27 times the rounding error
+// (6e-8).  Of the 785, the test for small terms takes 20 and the look at the words 30
+// (the barriers' waits).
 constexpr int kDigitBits = 19;
 constexpr int kRangeBits = 37;                                // terms below 2^37 units
 constexpr float kFixLimit = 0x1p37f;
 constexpr unsigned kSmallKey = 2u * ((127 + 17) << 23) - 2u;  // small_key of 2^17
 constexpr int kSegRows = 6144;                                // whole unrolled passes of every tile width
 constexpr int kFullWord = 1 << 28;
-constexpr int kSlowSamples = 6;  // (log-normal of sigma 2: 1320 us with 16)
+constexpr int kSlowSamples = 4;  // (log-normal, sigma 2: 940 us, with 6 1356; with 3 some normal ranges take FP32 sums)
 constexpr float kMagic = 0x1.8p23f;
 constexpr unsigned kMagicBits = 0x4B400000u;
 constexpr float kDigit = 0x1p19f, kPerDigit = 0x1p-19f;
@@ -417,7 +423,9 @@ constexpr float kDigit = 0x1p19f, kPerDigit = 0x1p-19f;
 // weigh on the loop that hardly ever takes them).
 struct BwdShared {
     int bad;
-    int emax[16];    // per channel: the largest binary exponent of a nonzero finite sample, or kNoSample
+    // per channel, of the nonzero finite samples: the largest binary exponent (kNoSample
+    // if none), the exponents' sum, their number
+    int emax[16], esum[16], ecnt[16];
     float unit[16];  // per channel: 2^-F
     float *gv, *gk;  // the tile's rows of the global gradients (or NULL)
     uint32_t rec;    // shared address of the tile's first record
@@ -444,26 +452,42 @@ __device__ __forceinline__ void sample(const ChanArgs& p, int64_t c0, int64_t r0
     xs = to_f32<IO>(__ldcg(x + at));
     gs = to_f32<IO>(__ldcg(gy + at));
 }
-// the samples' binary exponents (nonzero finite ones) into the channels' maxima
+// the samples' binary exponents (nonzero finite ones) into the channels' figures
 template <int CH>
-__device__ __forceinline__ void max_exponents(float g)
+__device__ __forceinline__ void add_exponents(float g)
 {
     const int ex = (int)(__float_as_uint(g) >> 23 & 0xffu);
-    int e = ex != 0 && ex != 0xff ? ex - 127 : kNoSample;
-    for (int o = CH; o < 32; o <<= 1) e = max(e, __shfl_xor_sync(0xffffffffu, e, o));
-    if ((threadIdx.x & 31) < CH && e != kNoSample) atomicMax(&s_bwd.emax[threadIdx.x % CH], e);
+    const bool ok = ex != 0 && ex != 0xff;
+    int top = ok ? ex - 127 : kNoSample, sum = ok ? ex - 127 : 0, cnt = ok ? 1 : 0;
+    for (int o = CH; o < 32; o <<= 1) {
+        top = max(top, __shfl_xor_sync(0xffffffffu, top, o));
+        sum += __shfl_xor_sync(0xffffffffu, sum, o);
+        cnt += __shfl_xor_sync(0xffffffffu, cnt, o);
+    }
+    if ((threadIdx.x & 31) < CH && cnt) {
+        atomicMax(&s_bwd.emax[threadIdx.x % CH], top);
+        atomicAdd(&s_bwd.esum[threadIdx.x % CH], sum);
+        atomicAdd(&s_bwd.ecnt[threadIdx.x % CH], cnt);
+    }
 }
 
-// F of a channel: from its own samples, else from the tile's (whose unit may be
-// far too coarse for it; then its terms count as small).  2^F and 2^-F are
-// normal FP32 numbers.  kNoSample if the tile has no nonzero sample.
+// F of a channel, from its largest sample, but no more than 2^7 of the mean (a single
+// outlier would leave the others few bits).  Few samples say little: with less than 8
+// nonzero ones the tile's largest counts too, up to 2^10 above the channel's own, and
+// with none it stands alone (where it is far too coarse, the channel's terms count as
+// small).  2^F and 2^-F are normal FP32 numbers.  kNoSample if the tile has no nonzero
+// sample.
 template <int CH>
 __device__ __forceinline__ int fix_exponent(int ch)
 {
-    int e = s_bwd.emax[ch];
-    if (e == kNoSample)
-        for (int q = 0; q < CH; ++q) e = max(e, s_bwd.emax[q]);
-    return e == kNoSample ? kNoSample : min(max(kRangeBits - 3 - e, -100), 126);
+    const int n = s_bwd.ecnt[ch];
+    int e = n > 0 ? min(s_bwd.emax[ch], (int)floorf((float)s_bwd.esum[ch] / (float)n) + 7) : kNoSample;
+    if (n < 8) {
+        int top = kNoSample;
+        for (int q = 0; q < CH; ++q) top = max(top, s_bwd.emax[q]);
+        e = n > 0 ? max(e, min(top, e + 10)) : top;
+    }
+    return e == kNoSample ? kNoSample : min(max(kRangeBits - (n < 16 ? 4 : 3) - e, -100), 126);
 }
 __device__ __forceinline__ float exp2_int(int e) { return __int_as_float((e + 127) << 23); }
 
@@ -579,14 +603,28 @@ __device__ __forceinline__ void chan_bwd(const float (&x)[G], float (&g)[G], con
         t2 = gq * (fabsf(p2 - xc[q]) * r[q].y);
     };
     unsigned small = ~0u;
+    if constexpr (FLOAT) {
+        // elements of one interval added up first: adds to one address wait for each other
+        float t1[G], t2[G];
 #pragma unroll
-    for (int q = 0; q < G; ++q) {
-        float t1, t2;
-        terms(q, gs[q], t1, t2);
-        if constexpr (FLOAT) {
-            float_add(at[q] + o.first, t1);
-            float_add(at[q] + o.second, t2);
-        } else {
+        for (int q = 0; q < G; ++q) terms(q, gs[q], t1[q], t2[q]);
+#pragma unroll
+        for (int q = 1; q < G; ++q)
+            if (at[q] == at[0]) {
+                t1[0] += t1[q];
+                t2[0] += t2[q];
+                t1[q] = t2[q] = 0.0f;
+            }
+#pragma unroll
+        for (int q = 0; q < G; ++q) {
+            float_add(at[q] + o.first, t1[q]);
+            float_add(at[q] + o.second, t2[q]);
+        }
+    } else {
+#pragma unroll
+        for (int q = 0; q < G; ++q) {
+            float t1, t2;
+            terms(q, gs[q], t1, t2);
             fix_add<8 * CH>(at[q] + o.first, t1);
             fix_add<8 * CH>(at[q] + o.second, t2);
             small = min(small, min(small_key(t1), small_key(t2)));
@@ -600,7 +638,7 @@ __device__ __forceinline__ void chan_bwd(const float (&x)[G], float (&g)[G], con
                 float t1, t2;
                 terms(q, gs[q], t1, t2);
                 if (fabsf(gs[q]) < kFixLimit) {
-                    add_rests<CH>(t1, t2, at[q], r[q].z);
+                    if (min(small_key(t1), small_key(t2)) < kSmallKey) add_rests<CH>(t1, t2, at[q], r[q].z);
                 } else {
                     float u1, u2;
                     terms(q, g[q], u1, u2);
@@ -639,7 +677,7 @@ __device__ __forceinline__ void chan_bwd_rows(const ChanArgs& p, int64_t c0, int
                                               const IO* __restrict__ x, const IO* __restrict__ gy,
                                               IO* __restrict__ gx)
 {
-    constexpr int RP = kChThreads / CH, U = kBwdUnroll, G = kBwdGroup;
+    constexpr int RP = kChThreads / CH, U = kBwdUnroll, G = FLOAT ? kFloatGroup : kBwdGroup;
     const int ch = threadIdx.x % CH, row = threadIdx.x / CH;
     const int64_t c = c0 + ch;
     if (c >= p.C) return;
@@ -794,14 +832,17 @@ __global__ void __launch_bounds__(kChThreads, 1) channels_backward_kernel(const 
         const int64_t c0 = tile * CH;
         const int ch = threadIdx.x % CH;
         __syncthreads();  // nobody reads the previous tile any more
-        if (threadIdx.x < CH) s_bwd.emax[threadIdx.x] = kNoSample;
+        if (threadIdx.x < CH) {
+            s_bwd.emax[threadIdx.x] = kNoSample;
+            s_bwd.esum[threadIdx.x] = s_bwd.ecnt[threadIdx.x] = 0;
+        }
         if (threadIdx.x == 0) {
             s_bwd.gv = g_values ? g_values + c0 * (p.N + 1) : nullptr;
             s_bwd.gk = g_knots ? g_knots + c0 * (p.N + 1) : nullptr;
         }
         float xs, gs;
         sample<IO, CH>(p, c0, r0, r1, x, gy, xs, gs);
-        build_tile<CH, true>(p, c0, cells, rec, &s_bwd.bad, [&] { max_exponents<CH>(gs); });
+        build_tile<CH, true>(p, c0, cells, rec, &s_bwd.bad, [&] { add_exponents<CH>(gs); });
         if (threadIdx.x == 0 && s_bwd.bad) atomicOr(p.status, 1);
         const int F = fix_exponent<CH>(ch);
         bool slow = F == kNoSample;

@@ -120,7 +120,8 @@ def test_gx_over_gy(pwl):
     _check(knots, values, x, gy, gv, gk, range(0, C, 7))
 
 
-@pytest.mark.parametrize("case", ["lognormal", "first_rows_zero", "sparse", "very_sparse", "small_bin", "outside"])
+@pytest.mark.parametrize("case", ["lognormal", "first_rows_zero", "sparse", "very_sparse", "small_bin", "outliers",
+                                  "outside"])
 def test_time_does_not_hang_on_the_gradients(pwl, case):
     # events around the backward of [65536, 1024] x 257 knots: other distributions of gy, and a
     # third of the points outside the domain, within half as much again as N(0, 1) gradients
@@ -152,6 +153,8 @@ def test_time_does_not_hang_on_the_gradients(pwl, case):
         gy *= torch.rand(R, C, generator=g, device="cuda") < (0.01 if case == "sparse" else 0.001)
     elif case == "small_bin":
         gy[(x > 0.5) & (x < 0.6)] *= 2.0 ** -26
+    elif case == "outliers":
+        gy[torch.rand(R, C, generator=g, device="cuda") < 0.001] *= 2.0 ** 10
     else:
         x[torch.rand(R, C, generator=g, device="cuda") < 0.33] = 5.0
     t = us(x, gy)
